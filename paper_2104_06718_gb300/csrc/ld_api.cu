@@ -1181,17 +1181,19 @@ ld_status ld_intermediate_bounds_split(ld_net* net, const float* lb0, const floa
 
 namespace {
 
-// Workspace of the propagation kernels for up to max_rows objective rows
-// (plus `extra` bytes for the caller, returned at the end of the block via
-// A.mu_b + ... -- see ib_extra), grown on demand; fills the workspace part of A.
-ld_status ib_args(ld_net* net, size_t max_rows, size_t extra, ld::IbLayerArgs& A, char** extra_ptr = nullptr) {
-  int max_w = 1;
-  for (int k = 1; k < net->n; ++k) max_w = std::max(max_w, layer(net, k).n_out);
-  const size_t mu_cap = (size_t)256 << 20;   // both coefficient buffers together
-  int64_t chunk = (int64_t)std::max<size_t>(1, mu_cap / (2 * sizeof(float) * (size_t)max_w));
-  if ((size_t)chunk > max_rows) chunk = (int64_t)std::max<size_t>(max_rows, 1);
-  const size_t acc_b = align256(24 * std::max<size_t>(max_rows, 1)), mu_b = align256(sizeof(float) * (size_t)chunk * max_w);
-  const size_t need = acc_b + 2 * mu_b + align256(extra);
+// Workspace of the propagation kernels for the bounds of layers k_lo..k_hi of
+// n_owners owners (plus `extra` bytes for the caller, at *extra_ptr), grown on
+// demand; fills the workspace part of A.
+ld_status ib_args(ld_net* net, int k_lo, int k_hi, int n_owners, int n_rules, int n_signs, size_t extra,
+                  ld::IbLayerArgs& A, char** extra_ptr = nullptr) {
+  size_t acc_b = 0, mu_b = 0, part_b = 0;
+  for (int k = k_lo; k <= k_hi; ++k) {
+    const ld::IbSpace sp = ld::ib_space(net->L, k, n_owners, n_rules, n_signs);
+    acc_b = std::max(acc_b, align256(sp.acc));
+    mu_b = std::max(mu_b, align256(sp.mu));
+    part_b = std::max(part_b, align256(sp.part));
+  }
+  const size_t need = acc_b + 2 * mu_b + part_b + align256(extra);
   if (need > net->ib_bytes) {
     cudaDeviceSynchronize();
     if (net->ib_ws) cudaFree(net->ib_ws);
@@ -1212,9 +1214,9 @@ ld_status ib_args(ld_net* net, size_t max_rows, size_t extra, ld::IbLayerArgs& A
   A.acc = reinterpret_cast<double*>(c);
   A.mu_a = reinterpret_cast<float*>(c + acc_b);
   A.mu_b = reinterpret_cast<float*>(c + acc_b + mu_b);
-  A.chunk_rows = chunk;
+  A.part = reinterpret_cast<double*>(c + acc_b + 2 * mu_b);
   A.gamma_M = ld::final_gamma(2.0 * (double)(net->N + net->n0) + 8.0);
-  if (extra_ptr) *extra_ptr = c + acc_b + 2 * mu_b;
+  if (extra_ptr) *extra_ptr = c + acc_b + 2 * mu_b + part_b;
   return LD_OK;
 }
 
@@ -1522,10 +1524,8 @@ ld_status ld_intermediate_bounds_propagated(ld_net* net, const float* lb0, const
                        net->d_status, s, rows);
   if (n <= 2) return last_error();
   const int n_rules = rules == (LD_IB_CROWN | LD_IB_WK) ? 2 : 1;
-  size_t max_rows = 0;
-  for (int k = 2; k < n; ++k) max_rows = std::max(max_rows, (size_t)n_rows * ld::ib_rows_per_owner(net->L, k, n_rules));
   ld::IbLayerArgs A{};
-  if ((st = ib_args(net, max_rows, 0, A)) != LD_OK) return st;
+  if ((st = ib_args(net, 2, n - 1, n_rows, n_rules, 2, 0, A)) != LD_OK) return st;
   A.n_owners = n_rows;
   A.n_rules = n_rules;
   A.rule0 = rules == LD_IB_WK ? 1 : 0;
@@ -1606,7 +1606,7 @@ ld_status ld_branch(ld_net* net, const float* lb0, const float* ub0, const float
   const size_t extra = b_cand + b_box + b_out + 2 * b_bnd;
   ld::IbLayerArgs A{};
   char* x = nullptr;
-  if ((st = ib_args(net, owners * 2 * 2, extra, A, &x)) != LD_OK) return st;
+  if ((st = ib_args(net, net->n, net->n, (int)owners, 2, 1, extra, A, &x)) != LD_OK) return st;
   int32_t* cand = reinterpret_cast<int32_t*>(x);
   int32_t* box = reinterpret_cast<int32_t*>(x + b_cand);
   double* child = reinterpret_cast<double*>(x + b_cand + b_box);

@@ -697,14 +697,21 @@ struct IbLayerArgs {
   const int32_t* box_row;   // [owners] box of each owner, or nullptr (owner = box row; box 0 with one box)
   int n_boxes;
   const int8_t* mask;       // [owners, N] split masks or nullptr
-  double* acc;              // [owners x rules x 2 x n_k, 3]
-  float* mu_a;              // [chunk_rows, max hidden width] x 2
+  double* acc;              // [owners x rules x signs x n_k, 3]: value, sum |terms|, error bound of a row
+  float* mu_a;              // coefficients of a chunk of groups, twice
   float* mu_b;
-  int64_t chunk_rows;
+  double* part;             // partial sums of a chunk of groups
   double gamma_M;           // FP64 constant of the per-row sums
   double* out_lb;           // layer k = n (the output): lower bound per owner [owners] instead of lbk/ubk
 };
-size_t ib_rows_per_owner(const std::vector<LayerDev>& Ls, int k, int n_rules);
+// Bytes of acc, of each of mu_a and mu_b, and of part for layer k's bounds
+// (n_signs: 2, or 1 when only the lower bounds are formed: out_lb), and the
+// groups of 32 rows that a chunk holds.
+struct IbSpace {
+  size_t acc, mu, part;
+  int64_t chunk_groups;
+};
+IbSpace ib_space(const std::vector<LayerDev>& Ls, int k, int n_owners, int n_rules, int n_signs);
 cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLayerArgs& A, cudaStream_t s);
 
 // FP64 final bound (ld_final.cu).

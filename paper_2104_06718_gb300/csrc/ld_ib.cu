@@ -16,49 +16,83 @@
 // WK a_low = a_bar (the WK relaxation quoted in Sec. 4.1).  Layer 1 is the
 // exact range of an affine map over the box (the interval bound of layer 1).
 //
-// Every objective row (owner x rule x sign x neuron) is one CTA.  Its dense
-// coefficient vector is staged in shared memory and each transposed pass
-// a = W^T mu runs in FP32 as a compensated dot product (each product split
-// exactly into value and error by an FMA, the running sum by TwoSum, the
-// errors summed alongside: Ogita, Rump and Oishi's Dot2), with a sum of
-// |W||mu| rounded upward beside it.  The result's error is at most
+// Rows (owner x rule x sign x neuron) run in groups of 32, one row per lane of
+// a warp, with the coefficient vectors of a group stored coefficient-major
+// (the 32 rows of a coefficient side by side in 128 bytes).  Every lane of a
+// warp then forms the same element of its own row: the weight is one
+// broadcast load for 32 rows, the coefficients are one coalesced load shared
+// by up to four channels, and no lane waits for another's sparsity.
+//   * Rows of a conv layer: a group is one output position of one owner, its
+//     lanes the (rule, sign, channel) combinations, so all 32 rows reach the
+//     same window of every layer below; only that window is stored and
+//     visited (its size is the same for every position; positions of it
+//     outside the plane are skipped).
+//   * Rows of an FC layer reach everything: lanes are consecutive rows.
+//   * An element whose ReLU is blocking in every row of the group relaxes to a
+//     zero coefficient whatever its sum is, so the sum is not formed; a
+//     coefficient that is zero in every row is skipped (it would add exact
+//     zeros).  Rows of one owner share both patterns, so these tests are
+//     uniform and cost one vote.
+//
+// Each transposed pass a = W^T mu is a compensated FP32 dot product (each
+// product split exactly into value and error by an FMA, the running sum by
+// TwoSum, the errors summed alongside: Ogita, Rump and Oishi's Dot2), with a
+// sum of |w mu| rounded upward beside it.  The result's error is at most
 // u |a| + gamma_K^2 sum|W||mu| (u = 2^-24, K = terms per sum), and since a
 // multiplies x_{j-1} in the substitution, the bound is lowered by that error
 // times max|x_{j-1}|.  (A plain FP32 sum would carry gamma_K sum|W||mu|,
 // which over a deep chain of substitutions loosens the bounds by ~1e-3.)
-// The relaxation slopes are
-// rounded in the direction that keeps each relaxation valid (a_bar upward,
-// b_bar upward; any lower slope in [0,1] is valid), a rounded mu_j product
-// lowers the bound by its rounding error times max|x_hat_j|, and every scalar
-// term is added in FP64 (exact products of FP32 values), whose summation error
-// is bounded by gamma_M times the sum of |terms|.  So the returned bounds
+// The relaxation slopes are rounded in the direction that keeps each
+// relaxation valid (a_bar upward, b_bar upward; any lower slope in [0,1] is
+// valid), and a rounded mu_j product lowers the bound by its rounding error
+// times max|x_hat_j|.  The scalar terms of a row (box, bias and intercept
+// products) are exact FP32 product pairs summed by the same Dot2 for at most
+// kFlush terms, then added in FP64: GB300 runs 2 FP64 operations per clock
+// and SM against 128 FP32 ones, and an FP64 epilogue cost more than the sums.
+// The error of that is at most gamma_32^2 of a block's |terms| (FP32 gamma)
+// plus gamma_M (FP64) times the sum of |terms|; the error bounds and the sum
+// of |terms| themselves are FP32 sums rounded upward.  So the returned bounds
 // contain the exact CROWN/WK bounds (outward), like the interval bounds.
-#include <climits>
+//
+// A row's value does not depend on the other rows of a call: the elements of a
+// layer are dealt to CTAs and warps by the layer's geometry alone.
+#include <algorithm>
 
 #include "ld_common.cuh"
 
 namespace ld {
 namespace {
 
-constexpr int NT = 256;
+constexpr int NW = 8;              // warps per CTA
+constexpr int NT = 32 * NW;
+constexpr int kUnitC = 4;          // elements per unit (channels of a position / consecutive FC inputs)
+constexpr int kUnitsPerCta = 32;   // units of a CTA, until a layer has more than kMaxChunks of them
+constexpr int kMaxChunks = 64;
+constexpr int kFlush = 2;          // units between FP64 flushes: at most 2 * kUnitC * kFlush = 16 terms
+constexpr float kTwoU = 1.1920928955078125e-07f;  // 2^-23, twice the FP32 unit roundoff
+
+// Window of a group's nonzero coefficients on a plane: full, or hh x ww from
+// (oy * mul - sub, ox * mul - sub) for the group's position (oy, ox).
+struct IbWin {
+  int full;
+  int hh, ww;
+  int mul, sub;
+};
 
 struct IbStep {
   LayerDev L;               // layer j: this launch computes a_{j-1} = W_j^T mu_j
   int seed;                 // 1: mu_j is the row's objective (+-e_i, layer k = j): a is a row of W_k, exact
   int box;                  // 1: j == 1, the epilogue adds the box term
-  const float* mu_in;       // [rows of the chunk, L.n_out] (unused when seed)
-  float* mu_out;            // [rows of the chunk, L.n_in]  (unused when box)
-  const float* bias_cur;    // seed: bias of layer k, plane_cur outputs per channel
-  int plane_cur;
+  IbWin win, wout;          // windows of mu_j (unused when seed) and of mu_{j-1}
+  int in_elems, out_elems;  // coefficients of a group in each
+  const float* mu_in;       // [groups of the chunk][in_elems][32]
+  float* mu_out;            // [groups of the chunk][out_elems][32] (unused when box)
   const float* bias_prev;   // hidden epilogue: bias of layer j-1 (plane_prev outputs per channel)
   int plane_prev;
   int prev_r_off;           // layer j-1 in the flat ReLU vector
-  float gamma_K;            // FP32 gamma of this pass's sums (its square bounds Dot2's error; 0 when seed)
-  // rows
-  int n_k;                  // neurons of the layer being bounded
-  int n_rules;              // 1 or 2
-  int rule0;                // rule of rule index 0: 0 CROWN, 1 WK (index 1 is WK)
-  int64_t row0;             // first row of this chunk
+  float g2;                 // upper bound on 2 gamma_K^2 of this pass's sums (0 when seed)
+  int chunks, units, units_per_cta;
+  int slot;                 // this launch's first partial-sum slot
   // bounds of the layers before k, per owner [owners, N], already clamped; boxes
   const float* lbk;
   const float* ubk;
@@ -68,17 +102,64 @@ struct IbStep {
   int n0;
   const int32_t* box_row;   // owner -> box row (nullptr: box_of_owner = owner, or 0 with one box)
   int n_boxes;
-  double* acc;              // [rows, 3]: value, sum |terms| (up), error bound (up)
+  double* part;             // [slots, 32 * groups of the chunk, 3]: value, sum |terms| (up), error bound (up)
 };
 
-__device__ __forceinline__ void decode_row(const IbStep& st, int64_t r, int& owner, int& rule, float& sign, int& i) {
-  const int64_t per_owner = (int64_t)st.n_rules * 2 * st.n_k;
-  owner = (int)(r / per_owner);
-  const int64_t rem = r % per_owner;
-  const int q = (int)(rem / (2 * st.n_k));
-  rule = q == 0 ? st.rule0 : 1;
-  sign = ((rem / st.n_k) % 2) == 0 ? 1.f : -1.f;
-  i = (int)(rem % st.n_k);
+// Rows of the layer being bounded and their order in groups of 32.
+struct IbRowMap {
+  int conv;                 // 1: groups are (owner, output position, block of 32 combinations)
+  int n_k;                  // neurons of the layer
+  int cout, wo, hw;         // conv: channels, output width, positions
+  int n_rules, n_signs;
+  int rule0;                // rule of rule index 0: 0 CROWN, 1 WK (index 1 is WK)
+  int per_pos, gpp;         // conv: combinations of a position, groups of a position
+  int64_t rows;             // owners * n_rules * n_signs * n_k
+  int64_t group0;           // first group of this chunk
+  int n_groups;             // groups of this chunk
+};
+
+struct IbRow {
+  bool valid;
+  int owner, rule, i;
+  int oy, ox;               // conv: the group's position (uniform over a warp)
+  float sign;
+  int64_t acc;              // row index, owner-major: ((owner * rules + rule) * signs + sign) * n_k + i
+};
+
+__device__ __forceinline__ IbRow ib_row(const IbRowMap& M, int64_t g, int lane) {
+  IbRow r;
+  int q, sg;
+  r.oy = r.ox = 0;
+  if (M.conv) {
+    const int64_t per_owner = (int64_t)M.hw * M.gpp;
+    r.owner = (int)(g / per_owner);
+    const int rem = (int)(g % per_owner);
+    const int pos = rem / M.gpp;
+    int t = (rem % M.gpp) * 32 + lane;
+    r.valid = t < M.per_pos;
+    if (!r.valid) t = 0;
+    const int o = t % M.cout;
+    t /= M.cout;
+    sg = t % M.n_signs;
+    q = t / M.n_signs;
+    r.oy = pos / M.wo;
+    r.ox = pos - r.oy * M.wo;
+    r.i = o * M.hw + pos;
+  } else {
+    int64_t e = g * 32 + lane;
+    r.valid = e < M.rows;
+    if (!r.valid) e = M.rows - 1;
+    r.i = (int)(e % M.n_k);
+    e /= M.n_k;
+    sg = (int)(e % M.n_signs);
+    e /= M.n_signs;
+    q = (int)(e % M.n_rules);
+    r.owner = (int)(e / M.n_rules);
+  }
+  r.rule = q == 0 ? M.rule0 : 1;
+  r.sign = sg == 0 ? 1.f : -1.f;
+  r.acc = (((int64_t)r.owner * M.n_rules + q) * M.n_signs + sg) * M.n_k + r.i;
+  return r;
 }
 
 __device__ __forceinline__ int box_of(const IbStep& st, int owner) {
@@ -90,7 +171,7 @@ __device__ __forceinline__ int box_of(const IbStep& st, int owner) {
 }
 
 // Compensated dot product state: running sum p, accumulated errors c, and
-// s >= sum |w m| (rounded up).
+// s >= (sum |w m|) / (1 + u) (the rounded products' sizes, rounded up).
 struct Dot2 {
   float p = 0.f, c = 0.f, s = 0.f;
   __device__ __forceinline__ void add(float w, float m) {
@@ -102,223 +183,266 @@ struct Dot2 {
     const float q = __fadd_rn(__fsub_rn(p, av), __fsub_rn(h, bv));
     p = t;
     c = __fadd_rn(c, __fadd_rn(q, r));
-    s = __fmaf_ru(fabsf(w), fabsf(m), s);
+    s = __fadd_ru(s, fabsf(h));
+  }
+  __device__ __forceinline__ float value() const { return __fadd_rn(p, c); }
+  __device__ __forceinline__ float size() const { return __fmul_ru(s, 1.f + 2.f * kTwoU); }
+};
+
+// A row's scalar terms: the pair (d.p, d.c) of the current block, the FP64
+// sum of the finished ones, sum |terms| and the error bound (FP32, rounded up).
+struct RowSum {
+  Dot2 d;
+  double v = 0.0;
+  float e = 0.f;
+  __device__ __forceinline__ void flush() {
+    v += (double)d.p;
+    v += (double)d.c;
+    d.p = d.c = 0.f;
   }
 };
 
-// a = (W^T mu)[ii] by Dot2 and s >= sum |W| |mu| (FP32, rounded up), mu in shared memory.
-// A zero mu term is skipped: it would add an exact zero to the running sum,
-// to its error and to s, so the result is the same (a row's mu is sparse: a
-// conv neuron's objective reaches only its receptive field, and blocking
-// ReLUs relax to zero).
-__device__ __forceinline__ void transposed_elem(const LayerDev& L, const float* mu, int ii, float& a, float& s) {
-  Dot2 d;
-  if (L.kind == LD_LAYER_FC) {
-    const float* w = L.W + ii;
-    for (int o = 0; o < L.n_out; ++o) {
-      const float m = mu[o];
-      if (m != 0.f) d.add(__ldg(w + (size_t)o * L.n_in), m);
-    }
-    a = __fadd_rn(d.p, d.c);
-    s = d.s;
-    return;
-  }
-  const int hw = L.h * L.w;
-  const int c = ii / hw, rem = ii % hw, y = rem / L.w, x = rem % L.w;
-  for (int ki = 0; ki < L.kh; ++ki) {
-    const int ty = y + L.pad - ki;
-    if (ty < 0 || ty % L.stride) continue;
-    const int oy = ty / L.stride;
-    if (oy >= L.ho) continue;
-    for (int kj = 0; kj < L.kw; ++kj) {
-      const int tx = x + L.pad - kj;
-      if (tx < 0 || tx % L.stride) continue;
-      const int ox = tx / L.stride;
-      if (ox >= L.wo) continue;
-      for (int o = 0; o < L.cout; ++o) {
-        const float m = mu[((size_t)o * L.ho + oy) * L.wo + ox];
-        if (m != 0.f) d.add(__ldg(L.W + (((size_t)o * L.cin + c) * L.kh + ki) * L.kw + kj), m);
-      }
-    }
-  }
-  a = __fadd_rn(d.p, d.c);
-  s = d.s;
-}
-
-// (A warp whose values are all zero skips its FP64 shuffle tree: its sum is
-// that zero, and FP64 additions are GB300's scarce unit.)
-__device__ __forceinline__ double block_sum(double v, double* red, bool up) {
-  if (__any_sync(0xffffffffu, v != 0.0))
-    for (int o = 16; o > 0; o >>= 1) {
-      const double w = __shfl_down_sync(0xffffffffu, v, o);
-      v = up ? __dadd_ru(v, w) : v + w;
-    }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < NT / 32; ++w) t = up ? __dadd_ru(t, red[w]) : t + red[w];
-  return t;
-}
-
-// Seed pass: a = W_k^T (sign e_i) is sign times row i of W_k (a conv row:
-// the kernel taps of output neuron i that land on input element ii), exact.
-__device__ __forceinline__ float seed_elem(const LayerDev& L, int i, float sign, int ii) {
-  if (L.kind == LD_LAYER_FC) return sign * __ldg(L.W + (size_t)i * L.n_in + ii);
-  const int hw = L.ho * L.wo;
-  const int o = i / hw, orem = i % hw, oy = orem / L.wo, ox = orem % L.wo;
-  const int hwi = L.h * L.w;
-  const int c = ii / hwi, rem = ii % hwi, y = rem / L.w, x = rem % L.w;
-  const int ky = y + L.pad - oy * L.stride, kx = x + L.pad - ox * L.stride;
-  if (ky < 0 || ky >= L.kh || kx < 0 || kx >= L.kw) return 0.f;
-  return sign * __ldg(L.W + (((size_t)o * L.cin + c) * L.kh + ky) * L.kw + kx);
-}
-
-__global__ void __launch_bounds__(NT) ib_step_kernel(IbStep st) {
-  extern __shared__ float mu[];
-  __shared__ double red[NT / 32];
-  const int64_t rl = blockIdx.x;
-  const int64_t r = st.row0 + rl;
-  int owner, rule, i;
-  float sign;
-  decode_row(st, r, owner, rule, sign, i);
+// a = (W^T mu) of NA channels c[0..NA) at the plane position (y, x) of the
+// input of conv layer L, for the lane's row.
+template <int NA>
+__device__ __forceinline__ void conv_dots(const IbStep& st, const float* __restrict__ mu, int wy0, int wx0, int y,
+                                          int x, const int* c, Dot2* d) {
   const LayerDev& L = st.L;
-  if (!st.seed) {
-    const float* src = st.mu_in + (size_t)rl * L.n_out;
-    for (int o = threadIdx.x; o < L.n_out; o += NT) mu[o] = src[o];
-  }
-  __syncthreads();
-  double v = 0.0, av = 0.0, e = 0.0;
-  if (st.seed && threadIdx.x == 0) {
-    const double bb = (double)sign * (double)st.bias_cur[i / st.plane_cur];
-    v = bb;
-    av = fabs(bb);
-  }
-  // Conv layers: the window of the input plane that the nonzero mu reach
-  // (output rows oy feed input rows oy*stride - pad .. + kh - 1, and the same
-  // for columns); an element outside it meets only zero terms, a = 0 and
-  // s = 0, and is skipped as such below.
-  __shared__ int win[4];
-  bool windowed = false;
-  if (!st.seed && L.kind == LD_LAYER_CONV) {
-    windowed = true;
-    if (threadIdx.x == 0) {
-      win[0] = INT_MAX;
-      win[1] = -1;
-      win[2] = INT_MAX;
-      win[3] = -1;
-    }
-    __syncthreads();
-    int y0 = INT_MAX, y1 = -1, x0 = INT_MAX, x1 = -1;
-    const int hwo = L.ho * L.wo;
-    for (int o = threadIdx.x; o < L.n_out; o += NT)
-      if (mu[o] != 0.f) {
-        const int r = o % hwo, oy = r / L.wo, ox = r - oy * L.wo;
-        y0 = min(y0, oy);
-        y1 = max(y1, oy);
-        x0 = min(x0, ox);
-        x1 = max(x1, ox);
-      }
-    if (y1 >= 0) {
-      atomicMin(&win[0], y0);
-      atomicMax(&win[1], y1);
-      atomicMin(&win[2], x0);
-      atomicMax(&win[3], x1);
-    }
-    __syncthreads();
-  }
-  int wy0 = 0, wy1 = -1, wx0 = 0, wx1 = -1;
-  if (windowed && win[1] >= 0) {
-    wy0 = max(0, win[0] * L.stride - L.pad);
-    wy1 = min(L.h - 1, win[1] * L.stride - L.pad + L.kh - 1);
-    wx0 = max(0, win[2] * L.stride - L.pad);
-    wx1 = min(L.w - 1, win[3] * L.stride - L.pad + L.kw - 1);
-  }
-  const int bx = st.box ? box_of(st, owner) : 0;
-  const double g2 = 2.0 * (double)st.gamma_K * (double)st.gamma_K;
-  for (int ii = threadIdx.x; ii < L.n_in; ii += NT) {
-    float a, s;
-    if (st.seed) {
-      a = seed_elem(L, i, sign, ii);
-      s = fabsf(a);
-    } else {
-      if (windowed) {
-        const int rem = ii % (L.h * L.w), y = rem / L.w, x = rem - y * L.w;
-        if (y < wy0 || y > wy1 || x < wx0 || x > wx1) {
-          if (!st.box) st.mu_out[(size_t)rl * L.n_in + ii] = 0.f;
-          continue;
+  const int estep = st.win.hh * st.win.ww * 32;
+  const size_t wstep = (size_t)L.kh * L.kw * L.cin;
+  for (int ki = (y + L.pad) % L.stride; ki < L.kh; ki += L.stride) {
+    const int oy = (y + L.pad - ki) / L.stride;     // y + pad - ki is a multiple of stride here
+    if (y + L.pad < ki) break;
+    const int wy = oy - wy0;
+    if (oy >= L.ho || wy < 0 || wy >= st.win.hh) continue;
+    for (int kj = (x + L.pad) % L.stride; kj < L.kw; kj += L.stride) {
+      if (x + L.pad < kj) break;
+      const int ox = (x + L.pad - kj) / L.stride;
+      const int wx = ox - wx0;
+      if (ox >= L.wo || wx < 0 || wx >= st.win.ww) continue;
+      const float* mp = mu + (wy * st.win.ww + wx) * 32;
+      const float* wp = L.Wt + ((size_t)ki * L.kw + kj) * L.cin;
+      int o = 0;
+      for (; o + 4 <= L.cout; o += 4) {
+        float m[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) m[q] = __ldg(mp + (size_t)(o + q) * estep);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (!__any_sync(0xffffffffu, m[q] != 0.f)) continue;
+          const float* w = wp + (size_t)(o + q) * wstep;
+#pragma unroll
+          for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m[q]);
         }
       }
-      transposed_elem(L, mu, ii, a, s);
-    }
-    if (a == 0.f && s == 0.f) {
-      // no term reached this element: it adds nothing to the bound, its
-      // error or its relaxation (mu = 0 for the next pass)
-      if (!st.box) st.mu_out[(size_t)rl * L.n_in + ii] = 0.f;
-      continue;
-    }
-    // bound on |a - W^T mu| (Dot2): u |a| + gamma_K^2 sum|W||mu|, with margin; 0 for the exact seed
-    const double da = st.seed ? 0.0 : __dadd_ru(__dmul_ru(1.1920928955078125e-07, fabs((double)a)), __dmul_ru(g2, (double)s));
-    if (st.box) {
-      const double l = (double)st.l0[(size_t)bx * st.n0 + ii], u = (double)st.u0[(size_t)bx * st.n0 + ii];
-      const double t = fmin((double)a * l, (double)a * u);
-      v += t;
-      av = __dadd_ru(av, fabs(t));
-      e = __dadd_ru(e, __dmul_ru(da, fmax(fabs(l), fabs(u))));
-      continue;
-    }
-    const size_t j = (size_t)owner * st.N + st.prev_r_off + ii;
-    const float l = st.lbk[j], u = st.ubk[j];
-    float m = 0.f;
-    if (u <= 0.f) {
-      m = 0.f;                          // blocking: x = 0, nothing to relax
-    } else if (l >= 0.f) {
-      m = a;                            // passing: x = x_hat
-    } else {
-      const float ab = __fdiv_ru(u, __fsub_rd(u, l));  // upper slope, rounded up (still a valid relaxation)
-      if (a >= 0.f) {
-        const float slo = rule == 0 ? (u >= -l ? 1.f : 0.f) : fminf(ab, 1.f);
-        m = slo * a;
-      } else {
-        m = ab * a;
-        const float bb = __fmul_ru(-l, ab);           // upper intercept, rounded up
-        const double t = (double)a * (double)bb;
-        v += t;
-        av = __dadd_ru(av, fabs(t));
+      for (; o < L.cout; ++o) {
+        const float m = __ldg(mp + (size_t)o * estep);
+        if (!__any_sync(0xffffffffu, m != 0.f)) continue;
+        const float* w = wp + (size_t)o * wstep;
+#pragma unroll
+        for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m);
       }
-      // rounding of the product mu = slope * a, times max |x_hat|
-      e = __dadd_ru(e, __dmul_ru(__dmul_ru(1.1920928955078125e-07, fabs((double)m)), fmax(-(double)l, (double)u)));
     }
-    if (u > 0.f) {
-      const double t = (double)m * (double)st.bias_prev[ii / st.plane_prev];
-      v += t;
-      av = __dadd_ru(av, fabs(t));
-      // the pass's own rounding, times max x_{j-1} = max(u, 0)
-      e = __dadd_ru(e, __dmul_ru(da, (double)u));
-    }
-    st.mu_out[(size_t)rl * L.n_in + ii] = m;
   }
-  v = block_sum(v, red, false);
-  av = block_sum(av, red, true);
-  e = block_sum(e, red, true);
-  if (threadIdx.x == 0) {
-    double* p = st.acc + (size_t)r * 3;
-    if (st.seed) {
-      p[0] = v;
-      p[1] = av;
-      p[2] = e;
+}
+
+// a = (W^T mu) of the NA inputs c[0..NA) of FC layer L.
+template <int NA>
+__device__ __forceinline__ void fc_dots(const LayerDev& L, const float* __restrict__ mu, const int* c, Dot2* d) {
+  int o = 0;
+  for (; o + 4 <= L.n_out; o += 4) {
+    float m[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) m[q] = __ldg(mu + (size_t)(o + q) * 32);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (!__any_sync(0xffffffffu, m[q] != 0.f)) continue;
+      const float* w = L.W + (size_t)(o + q) * L.n_in;
+#pragma unroll
+      for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m[q]);
+    }
+  }
+  for (; o < L.n_out; ++o) {
+    const float m = __ldg(mu + (size_t)o * 32);
+    if (!__any_sync(0xffffffffu, m != 0.f)) continue;
+    const float* w = L.W + (size_t)o * L.n_in;
+#pragma unroll
+    for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m);
+  }
+}
+
+// One element's contribution to the row and its coefficient for the next
+// pass: a with error bound da, on the input interval [l, u] (box) or through
+// the relaxation of a ReLU with bounds [l, u] and bias b.
+__device__ __forceinline__ void box_term(RowSum& R, float a, float da, float l, float u) {
+  const float x = a >= 0.f ? l : u;                 // min(a l, a u)
+  R.d.add(x, a);
+  R.e = __fmaf_ru(da, fmaxf(fabsf(l), fabsf(u)), R.e);
+}
+
+__device__ __forceinline__ float relu_term(RowSum& R, float a, float da, float l, float u, float b, int rule) {
+  if (u <= 0.f) return 0.f;                         // blocking: x = 0, nothing to relax
+  float m = a;                                      // passing: x = x_hat
+  if (l < 0.f) {
+    const float ab = __fdiv_ru(u, __fsub_rd(u, l));  // upper slope, rounded up (still a valid relaxation)
+    if (a >= 0.f) {
+      const float slo = rule == 0 ? (u >= -l ? 1.f : 0.f) : fminf(ab, 1.f);
+      m = slo * a;
     } else {
-      p[0] += v;
-      p[1] = __dadd_ru(p[1], av);
-      p[2] = __dadd_ru(p[2], e);
+      m = ab * a;
+      R.d.add(__fmul_ru(-l, ab), a);                // upper intercept, rounded up
     }
+    // rounding of the product mu = slope * a, times max |x_hat|
+    R.e = __fmaf_ru(__fmul_ru(kTwoU, fabsf(m)), fmaxf(-l, u), R.e);
   }
+  R.d.add(b, m);
+  // the pass's own rounding, times max x_{j-1} = max(u, 0)
+  R.e = __fmaf_ru(da, u, R.e);
+  return m;
+}
+
+// One CTA: units [chunk * units_per_cta, ...) of one group of 32 rows; a unit
+// is kUnitC channels of one position (conv) or kUnitC consecutive inputs (FC).
+__global__ void __launch_bounds__(NT) ib_step_kernel(IbStep st, IbRowMap M) {
+  __shared__ double red[NW][32][3];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gl = blockIdx.x / st.chunks, chunk = blockIdx.x % st.chunks;
+  const IbRow r = ib_row(M, M.group0 + gl, lane);
+  const LayerDev& L = st.L;
+  const bool conv = L.kind == LD_LAYER_CONV;
+  const float* mu = st.mu_in + (size_t)gl * st.in_elems * 32 + lane;
+  float* out = st.mu_out + (size_t)gl * st.out_elems * 32 + lane;
+  const int iy0 = st.win.full ? 0 : r.oy * st.win.mul - st.win.sub;
+  const int ix0 = st.win.full ? 0 : r.ox * st.win.mul - st.win.sub;
+  const int oy0 = st.wout.full ? 0 : r.oy * st.wout.mul - st.wout.sub;
+  const int ox0 = st.wout.full ? 0 : r.ox * st.wout.mul - st.wout.sub;
+  const int cb = conv ? (L.cin + kUnitC - 1) / kUnitC : 0;
+  const int so = conv ? r.i / (L.ho * L.wo) : 0;    // seed: the row's output channel
+  const size_t lo_off = st.box ? (size_t)box_of(st, r.owner) * st.n0 : (size_t)r.owner * st.N + st.prev_r_off;
+  const float* lp = (st.box ? st.l0 : st.lbk) + lo_off;
+  const float* up = (st.box ? st.u0 : st.ubk) + lo_off;
+  RowSum R;
+  const int u_lo = chunk * st.units_per_cta, u_hi = min(st.units, u_lo + st.units_per_cta);
+  int done = 0;
+  for (int un = u_lo + warp; un < u_hi; un += NW) {
+    int wy = 0, wx = 0, y = 0, x = 0, c0, nc;
+    if (conv) {
+      const int pos = un / cb;
+      c0 = (un - pos * cb) * kUnitC;
+      nc = min(kUnitC, L.cin - c0);
+      wy = pos / st.wout.ww;
+      wx = pos - wy * st.wout.ww;
+      y = oy0 + wy;
+      x = ox0 + wx;
+      if (y < 0 || y >= L.h || x < 0 || x >= L.w) continue;
+    } else {
+      c0 = un * kUnitC;
+      nc = min(kUnitC, L.n_in - c0);
+    }
+    // the elements' bounds; those that some row of the group needs
+    float l[kUnitC], u[kUnitC];
+    int act[kUnitC] = {0, 0, 0, 0}, na = 0;
+#pragma unroll
+    for (int q = 0; q < kUnitC; ++q) {
+      l[q] = u[q] = 0.f;
+      if (q < nc) {
+        const int ii = conv ? ((c0 + q) * L.h + y) * L.w + x : c0 + q;
+        l[q] = __ldg(lp + ii);
+        u[q] = __ldg(up + ii);
+      }
+      if (q < nc && __any_sync(0xffffffffu, st.box || u[q] > 0.f)) {
+#pragma unroll
+        for (int k = 0; k < kUnitC; ++k)
+          if (na == k) act[k] = c0 + q;
+        ++na;
+      }
+    }
+    Dot2 d[kUnitC];
+    if (st.seed) {
+      const float sg = r.valid ? r.sign : 0.f;
+      const int ky = y + L.pad - r.oy * L.stride, kx = x + L.pad - r.ox * L.stride;
+#pragma unroll
+      for (int q = 0; q < kUnitC; ++q) {
+        if (q >= nc) continue;
+        float a = 0.f;
+        if (!conv) a = sg * __ldg(L.W + (size_t)r.i * L.n_in + c0 + q);
+        else if (ky >= 0 && ky < L.kh && kx >= 0 && kx < L.kw)
+          a = sg * __ldg(L.W + (((size_t)so * L.cin + c0 + q) * L.kh + ky) * L.kw + kx);
+        d[q].p = a;
+      }
+    } else if (na > 0) {
+      Dot2 t[kUnitC];
+      if (conv) {
+        if (na == 1) conv_dots<1>(st, mu, iy0, ix0, y, x, act, t);
+        else if (na == 2) conv_dots<2>(st, mu, iy0, ix0, y, x, act, t);
+        else if (na == 3) conv_dots<3>(st, mu, iy0, ix0, y, x, act, t);
+        else conv_dots<4>(st, mu, iy0, ix0, y, x, act, t);
+      } else {
+        if (na == 1) fc_dots<1>(L, mu, act, t);
+        else if (na == 2) fc_dots<2>(L, mu, act, t);
+        else if (na == 3) fc_dots<3>(L, mu, act, t);
+        else fc_dots<4>(L, mu, act, t);
+      }
+      // back to their channels
+#pragma unroll
+      for (int k = 0; k < kUnitC; ++k)
+#pragma unroll
+        for (int q = k; q < kUnitC; ++q)
+          if (k < na && act[k] == c0 + q) d[q] = t[k];
+    }
+#pragma unroll
+    for (int q = 0; q < kUnitC; ++q) {
+      if (q >= nc) continue;
+      const float a = d[q].value();
+      const float da = st.seed ? 0.f : __fmaf_ru(st.g2, d[q].size(), __fmul_ru(kTwoU, fabsf(a)));
+      if (st.box) {
+        box_term(R, a, da, l[q], u[q]);
+      } else {
+        const int ii = conv ? ((c0 + q) * L.h + y) * L.w + x : c0 + q;
+        const float m = (a == 0.f && d[q].s == 0.f)
+                            ? 0.f
+                            : relu_term(R, a, da, l[q], u[q], __ldg(st.bias_prev + ii / st.plane_prev), r.rule);
+        const int e = conv ? ((c0 + q) * st.wout.hh + wy) * st.wout.ww + wx : c0 + q;
+        out[(size_t)e * 32] = m;
+      }
+    }
+    if (++done % kFlush == 0) R.flush();
+  }
+  R.flush();
+  red[warp][lane][0] = R.v;
+  red[warp][lane][1] = (double)R.d.size();
+  red[warp][lane][2] = (double)R.e;
+  __syncthreads();
+  if (threadIdx.x < 96) {
+    const int q = threadIdx.x / 32;
+    double t = red[0][lane][q];
+    for (int w = 1; w < NW; ++w) t = q == 0 ? t + red[w][lane][q] : __dadd_ru(t, red[w][lane][q]);
+    st.part[(((size_t)st.slot + chunk) * M.n_groups * 32 + (size_t)gl * 32 + lane) * 3 + q] = t;
+  }
+}
+
+// Sums a chunk's slots per row (fixed order), with the objective's bias term.
+__global__ void __launch_bounds__(NT) ib_collect_kernel(IbRowMap M, int slots, const double* part, const float* bias,
+                                                        int plane, double* acc) {
+  const int64_t t = blockIdx.x * (int64_t)NT + threadIdx.x;
+  if (t >= (int64_t)M.n_groups * 32) return;
+  const IbRow r = ib_row(M, M.group0 + t / 32, (int)(t % 32));
+  if (!r.valid) return;
+  double v = (double)r.sign * (double)bias[r.i / plane], av = fabs(v), e = 0.0;
+  for (int s = 0; s < slots; ++s) {
+    const double* p = part + ((size_t)s * M.n_groups * 32 + t) * 3;
+    v += p[0];
+    av = __dadd_ru(av, p[1]);
+    e = __dadd_ru(e, p[2]);
+  }
+  double* a = acc + (size_t)r.acc * 3;
+  a[0] = v;
+  a[1] = av;
+  a[2] = e;
 }
 
 struct IbFinish {
-  int n_owners, n_k, n_rules, N, r_off;
+  int n_owners, n_k, n_rules, n_signs, N, r_off;
   const double* acc;
   double gamma_M;
   const int8_t* mask;       // [owners, N] or nullptr
@@ -336,8 +460,8 @@ __global__ void ib_finish_kernel(IbFinish f) {
     const int owner = (int)(t / f.n_k), i = (int)(t % f.n_k);
     double lo = -INFINITY, up = INFINITY;
     for (int q = 0; q < f.n_rules; ++q)
-      for (int sg = 0; sg < 2; ++sg) {
-        const int64_t r = (((int64_t)owner * f.n_rules + q) * 2 + sg) * f.n_k + i;
+      for (int sg = 0; sg < f.n_signs; ++sg) {
+        const int64_t r = (((int64_t)owner * f.n_rules + q) * f.n_signs + sg) * f.n_k + i;
         const double* p = f.acc + (size_t)r * 3;
         const double b = __dsub_rd(__dsub_rd(p[0], p[2]), __dmul_ru(f.gamma_M, p[1]));
         if (sg == 0) lo = fmax(lo, b);
@@ -359,29 +483,94 @@ __global__ void ib_finish_kernel(IbFinish f) {
   }
 }
 
-float gamma32(int K) {
+double gamma32(int K) {
   const double u = 5.9604644775390625e-08;  // 2^-24
-  const double g = K * u / (1.0 - K * u) * (1.0 + 1e-6);
-  return (float)g * (1.0f + 1e-6f);
+  return K * u / (1.0 - K * u) * (1.0 + 1e-6);
+}
+
+// Geometry of the substitution of layer k's rows, layer by layer.
+struct IbGeo {
+  IbWin w[kMaxLayers + 1];   // w[j]: window on layer j's output plane (j < k)
+  int elems[kMaxLayers + 1];
+  int units[kMaxLayers + 1], chunks[kMaxLayers + 1], per_cta[kMaxLayers + 1];  // of the launch that forms a_j
+  int slots, width;          // partial-sum slots of a chunk, widest hidden level
+};
+
+IbGeo ib_geo(const std::vector<LayerDev>& Ls, int k) {
+  IbGeo g{};
+  int mul = 1, sub = 0, hh = 1, ww = 1;
+  bool full = Ls[k - 1].kind == LD_LAYER_FC;
+  for (int j = k - 1; j >= 0; --j) {
+    const LayerDev& up = Ls[j];  // layer j+1, whose input plane this is
+    if (up.kind == LD_LAYER_CONV && !full) {
+      // positions [y0, y0 + hh) of its output reach [y0 s - p, (y0 + hh - 1) s - p + k) of its input
+      hh = (hh - 1) * up.stride + up.kh;
+      ww = (ww - 1) * up.stride + up.kw;
+      mul *= up.stride;
+      sub = sub * up.stride + up.pad;
+      // the whole plane once the window is no smaller, or where an FC layer reads it flat
+      if (hh >= up.h || ww >= up.w || (j >= 1 && Ls[j - 1].kind == LD_LAYER_FC)) full = true;
+    }
+    g.w[j] = full ? IbWin{1, up.h, up.w, 0, 0} : IbWin{0, hh, ww, mul, sub};  // full: as layer j+1 sees it
+    const bool conv = up.kind == LD_LAYER_CONV;
+    g.elems[j] = conv ? up.cin * g.w[j].hh * g.w[j].ww : up.n_in;
+    g.units[j] = conv ? g.w[j].hh * g.w[j].ww * ((up.cin + kUnitC - 1) / kUnitC) : (up.n_in + kUnitC - 1) / kUnitC;
+    g.per_cta[j] = std::max(kUnitsPerCta, (g.units[j] + kMaxChunks - 1) / kMaxChunks);
+    g.chunks[j] = (g.units[j] + g.per_cta[j] - 1) / g.per_cta[j];
+    g.slots += g.chunks[j];
+    if (j >= 1) g.width = std::max(g.width, g.elems[j]);
+  }
+  return g;
+}
+
+IbRowMap ib_rows(const LayerDev& Lk, int n_owners, int n_rules, int n_signs, int rule0) {
+  IbRowMap M{};
+  M.conv = Lk.kind == LD_LAYER_CONV;
+  M.n_k = Lk.n_out;
+  M.cout = Lk.cout;
+  M.wo = Lk.wo;
+  M.hw = Lk.ho * Lk.wo;
+  M.n_rules = n_rules;
+  M.n_signs = n_signs;
+  M.rule0 = rule0;
+  M.per_pos = n_rules * n_signs * Lk.cout;
+  M.gpp = (M.per_pos + 31) / 32;
+  M.rows = (int64_t)n_owners * n_rules * n_signs * Lk.n_out;
+  return M;
+}
+
+int64_t ib_groups(const IbRowMap& M, int n_owners) {
+  return M.conv ? (int64_t)n_owners * M.hw * M.gpp : (M.rows + 31) / 32;
 }
 
 }  // namespace
 
-size_t ib_rows_per_owner(const std::vector<LayerDev>& Ls, int k, int n_rules) {
-  return (size_t)n_rules * 2 * Ls[k - 1].n_out;
+// Workspace of layer k's bounds for n_owners: row sums, the partial sums and
+// the two coefficient buffers of a chunk of groups (at most kMuCap together).
+IbSpace ib_space(const std::vector<LayerDev>& Ls, int k, int n_owners, int n_rules, int n_signs) {
+  constexpr size_t kMuCap = (size_t)256 << 20;
+  const IbGeo g = ib_geo(Ls, k);
+  const IbRowMap M = ib_rows(Ls[k - 1], n_owners, n_rules, n_signs, 0);
+  const size_t per_group = sizeof(float) * 32 * (size_t)g.width;
+  IbSpace sp;
+  const int64_t cap = std::max<int64_t>(1, (int64_t)(kMuCap / (2 * per_group)));
+  sp.chunk_groups = std::max<int64_t>(1, std::min<int64_t>({cap, ib_groups(M, n_owners), int64_t(1) << 24}));
+  sp.acc = 24 * (size_t)std::max<int64_t>(1, M.rows);
+  sp.mu = per_group * (size_t)sp.chunk_groups;
+  sp.part = 24 * 32 * (size_t)g.slots * (size_t)sp.chunk_groups;
+  return sp;
 }
 
-// Bounds of layer k (2 <= k <= n-1) for every owner, from the bounds of the
+// Bounds of layer k (2 <= k <= n) for every owner, from the bounds of the
 // layers before it (already in lbk/ubk, clamped); see IbLayerArgs.
 cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLayerArgs& A, cudaStream_t s) {
   const LayerDev& Lk = Ls[k - 1];
-  const int n_k = Lk.n_out;
-  const int64_t rows = (int64_t)A.n_owners * A.n_rules * 2 * n_k;
-  if (rows == 0) return cudaSuccess;
+  const int n_signs = A.out_lb ? 1 : 2;
+  IbRowMap M = ib_rows(Lk, A.n_owners, A.n_rules, n_signs, A.rule0);
+  if (M.rows == 0) return cudaSuccess;
+  const IbGeo g = ib_geo(Ls, k);
+  const int64_t groups = ib_groups(M, A.n_owners);
   IbStep st{};
-  st.n_k = n_k;
-  st.n_rules = A.n_rules;
-  st.rule0 = A.rule0;
   st.lbk = A.lbk;
   st.ubk = A.ubk;
   st.N = A.N;
@@ -390,20 +579,28 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
   st.n0 = A.n0;
   st.box_row = A.box_row;
   st.n_boxes = A.n_boxes;
-  st.acc = A.acc;
-  for (int64_t r0 = 0; r0 < rows; r0 += A.chunk_rows) {
-    const int64_t nr = rows - r0 < A.chunk_rows ? rows - r0 : A.chunk_rows;
+  st.part = A.part;
+  const int plane_k = Lk.kind == LD_LAYER_FC ? 1 : Lk.ho * Lk.wo;
+  const int64_t chunk = ib_space(Ls, k, A.n_owners, A.n_rules, n_signs).chunk_groups;
+  for (int64_t g0 = 0; g0 < groups; g0 += chunk) {
+    M.group0 = g0;
+    M.n_groups = (int)std::min(chunk, groups - g0);
     float* cur = A.mu_a;
     float* nxt = A.mu_b;
+    st.slot = 0;
     for (int j = k; j >= 1; --j) {
       const LayerDev& L = Ls[j - 1];
       st.L = L;
       st.seed = j == k;
       st.box = j == 1;
+      st.win = j == k ? IbWin{1, 1, 1, 0, 0} : g.w[j];
+      if (st.win.full) st.win = IbWin{1, L.ho, L.wo, 0, 0};
+      st.wout = g.w[j - 1];
+      if (st.wout.full) st.wout = IbWin{1, L.h, L.w, 0, 0};
+      st.in_elems = st.seed ? 0 : g.elems[j];
+      st.out_elems = g.elems[j - 1];
       st.mu_in = cur;
       st.mu_out = nxt;
-      st.bias_cur = Lk.b;
-      st.plane_cur = Lk.kind == LD_LAYER_FC ? 1 : Lk.ho * Lk.wo;
       if (j >= 2) {
         const LayerDev& Lp = Ls[j - 2];
         st.bias_prev = Lp.b;
@@ -414,20 +611,27 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
         st.plane_prev = 1;
         st.prev_r_off = 0;
       }
-      st.gamma_K = j == k ? 0.f : gamma32(L.fan_t);
-      st.row0 = r0;
-      const size_t smem = j == k ? 0 : sizeof(float) * (size_t)L.n_out;
+      const double gk = st.seed ? 0.0 : gamma32(L.fan_t);
+      st.g2 = (float)(2.0 * gk * gk * (1.0 + 1e-6));
+      st.chunks = g.chunks[j - 1];
+      st.units = g.units[j - 1];
+      st.units_per_cta = g.per_cta[j - 1];
       count_launch();
-      ib_step_kernel<<<(unsigned)nr, NT, smem, s>>>(st);
+      ib_step_kernel<<<(unsigned)(M.n_groups * (int64_t)st.chunks), NT, 0, s>>>(st, M);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
-      float* t = cur;
-      cur = nxt;
-      nxt = t;
+      st.slot += st.chunks;
+      std::swap(cur, nxt);
     }
+    count_launch();
+    ib_collect_kernel<<<(unsigned)((M.n_groups * 32LL + NT - 1) / NT), NT, 0, s>>>(M, g.slots, A.part, Lk.b, plane_k,
+                                                                                 A.acc);
   }
-  IbFinish f{A.n_owners, n_k, A.n_rules, A.N, Lk.r_out_off, A.acc, A.gamma_M, A.mask, A.lbk, A.ubk, A.out_lb};
-  const int64_t total = (int64_t)A.n_owners * n_k;
+  // FP64 sums, plus Dot2's gamma_32^2 (FP32) of the blocks of at most 16 terms
+  const double gd = gamma32(2 * kUnitC * kFlush);
+  IbFinish f{A.n_owners, Lk.n_out, A.n_rules, n_signs, A.N, Lk.r_out_off, A.acc, A.gamma_M + 2.0 * gd * gd, A.mask,
+             A.lbk, A.ubk, A.out_lb};
+  const int64_t total = (int64_t)A.n_owners * Lk.n_out;
   const int grid = (int)((total + 255) / 256 < 65535 ? (total + 255) / 256 : 65535);
   count_launch();
   ib_finish_kernel<<<grid > 0 ? grid : 1, 256, 0, s>>>(f);
