@@ -9,65 +9,103 @@
 //     x_hat_A,k+1 = W_{k+1} x_k^* + b_{k+1}             -> supergradient, Adam on rho_{k+1}
 //
 // FC layers are SIMT GEMMs with the subdomain batch as the M dimension in
-// 32 x 32 tiles, so one weight tile serves 32 subdomains; the forward FC pass
+// 32 x 32 tiles, so one weight tile serves 32 subdomains, with up to 128 of K staged at once; the forward FC pass
 // splits K across blocks when the output is small and the last block of a tile
 // reduces the partial sums in a fixed order (deterministic) before the
 // epilogue.  4x4/stride-2 and 3x3/stride-1 convs take register-blocked kernels
-// (several channels per thread, compile-time taps, transposed conv split by
-// stride phase); other geometries take direct loops.
+// on operand rows staged in shared memory (several channels per thread,
+// compile-time taps, transposed conv split by stride phase); other geometries
+// take direct loops.
+#include <algorithm>
+
 #include "ld_common.cuh"
 
 namespace ld {
 namespace {
 
-constexpr int TM = 32, TN = 32, TK = 16, NT = 256;
+constexpr int TM = 32, TN = 32, NT = 256;
+constexpr int TK = 128;    // K staged at once: the hidden FC widths and the split-K ranges of these nets in one round
+constexpr int kSplitStep = 16;  // split-K ranges are multiples of this
 
-// Accumulates C[m0 + ty + 16r][n0 + tx + 16c] (r, c in {0,1}) over k in [k_lo, k_hi):
+// Accumulates C[m0 + ty + 16r][n0 + 2 tx + c] (r, c in {0,1}) over k in [k_lo, k_hi):
 //   C[m, n] = sum_k A[m*lda + k] * Bop(k, n)
 //   W_KN:  Bop(k, n) = W[k*ldw + n]   (transposed pass: W[o, i], k = o, n = i)
 //   !W_KN: Bop(k, n) = W[n*ldw + k]   (forward pass:    W[o, i], k = i, n = o)
+// each output one chain of FMAs in the order of k.  The tiles are far too
+// small to hide a load behind the products, so what bounds a tile is the
+// number of load rounds: all of K (up to TK) is staged in one round, every
+// thread's 32 loads in flight together (with 16 per round the 100 rows of the
+// Base FC layer took 7 rounds of load, barrier, 16 products).
 template <bool W_KN>
 __device__ __forceinline__ void gemm_tile(int m0, int n0, int M, int Ncol, int k_lo, int k_hi,
                                           const float* __restrict__ A, int lda, const float* __restrict__ W, int ldw,
                                           float acc[2][2]) {
-  __shared__ float As[TK][TM + 1];
-  __shared__ float Bs[TK][TN + 1];
+  __shared__ float As[TM][TK + 1];
+  __shared__ __align__(16) float Bs[TK][TN + 2];
   const int t = threadIdx.x, tx = t % 16, ty = t / 16;
   for (int k0 = k_lo; k0 < k_hi; k0 += TK) {
+    const int kn = min(TK, k_hi - k0);
+    float av[TM * TK / NT], bv[TN * TK / NT];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int idx = t + e * NT;
-      const int mm = idx / TK, kk = idx % TK;
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < M && gk < k_hi) ? __ldg(A + (size_t)gm * lda + gk) : 0.f;
+    for (int e = 0; e < TM * TK / NT; ++e) {
+      const int idx = t + e * NT, mm = idx / TK, kk = idx % TK;
+      av[e] = (m0 + mm < M && kk < kn) ? __ldg(A + (size_t)(m0 + mm) * lda + k0 + kk) : 0.f;
     }
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < TN * TK / NT; ++e) {
       const int idx = t + e * NT;
-      int kk, nn;
-      if (W_KN) {
-        kk = idx / TN;
-        nn = idx % TN;
-      } else {
-        nn = idx / TK;
-        kk = idx % TK;
+      const int kk = W_KN ? idx / TN : idx % TK, nn = W_KN ? idx % TN : idx / TK;
+      bv[e] = (kk < kn && n0 + nn < Ncol)
+                  ? (W_KN ? __ldg(W + (size_t)(k0 + kk) * ldw + n0 + nn) : __ldg(W + (size_t)(n0 + nn) * ldw + k0 + kk))
+                  : 0.f;
+    }
+    if (k0 > k_lo) __syncthreads();
+#pragma unroll
+    for (int e = 0; e < TM * TK / NT; ++e) {
+      const int idx = t + e * NT;
+      As[idx / TK][idx % TK] = av[e];
+    }
+#pragma unroll
+    for (int e = 0; e < TN * TK / NT; ++e) {
+      const int idx = t + e * NT;
+      Bs[W_KN ? idx / TN : idx % TK][W_KN ? idx % TN : idx / TK] = bv[e];
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int kk = 0; kk < kn; ++kk) {
+      const float a0 = As[ty][kk], a1 = As[ty + 16][kk];
+      const float2 w = *reinterpret_cast<const float2*>(&Bs[kk][2 * tx]);
+      acc[0][0] = fmaf(a0, w.x, acc[0][0]);
+      acc[0][1] = fmaf(a0, w.y, acc[0][1]);
+      acc[1][0] = fmaf(a1, w.x, acc[1][0]);
+      acc[1][1] = fmaf(a1, w.y, acc[1][1]);
+    }
+  }
+}
+
+// Applies the epilogue to a thread's outputs of a tile; a reducing epilogue's
+// row sums are added over the 16 threads that share a row first.
+template <class Epi>
+__device__ __forceinline__ void gemm_epilogue(int m0, int n0, int M, int Ncol, const float (&acc)[2][2], const Epi& epi) {
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int m = m0 + ty + 16 * r;
+    double q = 0.0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int n = n0 + 2 * tx + c;
+      if (m < M && n < Ncol) {
+        if constexpr (Epi::kReduce)
+          q += epi(m, n, acc[r][c]);
+        else
+          epi(m, n, acc[r][c]);
       }
-      const int gk = k0 + kk, gn = n0 + nn;
-      float v = 0.f;
-      if (gk < k_hi && gn < Ncol) v = W_KN ? __ldg(W + (size_t)gk * ldw + gn) : __ldg(W + (size_t)gn * ldw + gk);
-      Bs[kk][nn] = v;
     }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      const float a0 = As[kk][ty], a1 = As[kk][ty + 16];
-      const float b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      acc[0][0] = fmaf(a0, b0, acc[0][0]);
-      acc[0][1] = fmaf(a0, b1, acc[0][1]);
-      acc[1][0] = fmaf(a1, b0, acc[1][0]);
-      acc[1][1] = fmaf(a1, b1, acc[1][1]);
+    if constexpr (Epi::kReduce) {
+      for (int o = 8; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o, 16);
+      if (tx == 0 && m < M) epi.finish(m, q);
     }
-    __syncthreads();
   }
 }
 
@@ -78,14 +116,7 @@ __global__ void __launch_bounds__(NT) gemm_kernel(int M, int Ncol, int K, const 
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
   float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
   gemm_tile<W_KN>(m0, n0, M, Ncol, 0, K, A, lda, W, ldw, acc);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int m = m0 + ty + 16 * r, n = n0 + tx + 16 * c;
-      if (m < M && n < Ncol) epi(m, n, acc[r][c]);
-    }
+  gemm_epilogue(m0, n0, M, Ncol, acc, epi);
 }
 
 // Split-K forward GEMM: block z covers K range [z*kc, (z+1)*kc); partial sums go
@@ -104,7 +135,7 @@ __global__ void __launch_bounds__(NT) gemm_splitk_kernel(int M, int Ncol, int K,
   for (int r = 0; r < 2; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int m = m0 + ty + 16 * r, n = n0 + tx + 16 * c;
+      const int m = m0 + ty + 16 * r, n = n0 + 2 * tx + c;
       if (m < M && n < Ncol) part[((size_t)z * M + m) * Ncol + n] = acc[r][c];
     }
   __threadfence();
@@ -119,118 +150,213 @@ __global__ void __launch_bounds__(NT) gemm_splitk_kernel(int M, int Ncol, int K,
   for (int r = 0; r < 2; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int m = m0 + ty + 16 * r, n = n0 + tx + 16 * c;
-      if (m < M && n < Ncol) {
-        float s = 0.f;
-        for (int q = 0; q < splits; ++q) s += __ldcg(part + ((size_t)q * M + m) * Ncol + n);
-        epi(m, n, s);
-      }
+      const int m = m0 + ty + 16 * r, n = n0 + 2 * tx + c;
+      acc[r][c] = 0.f;
+      if (m < M && n < Ncol)
+        for (int q = 0; q < splits; ++q) acc[r][c] += __ldcg(part + ((size_t)q * M + m) * Ncol + n);
     }
+  gemm_epilogue(m0, n0, M, Ncol, acc, epi);
   if (threadIdx.x == 0) count[tile] = 0;
 }
 
-// Transposed conv, blocked (k4 s2 / k3 s1): thread = one input position of one
-// stride phase and G channels; g[b, c, yy, xx] = sum_{o,i,j} W[o,c,i,j] r[b, o, y, x]
-// over the taps of the phase.  Weights in shared memory as [o][i][j][c].
-template <int KH, int KW, int ST, int G, class Epi>
-__global__ void __launch_bounds__(NT) conv_t_fast_kernel(LayerDev L, const float* __restrict__ r, int rs, Epi epi) {
-  extern __shared__ float sW[];
-  const int nw = L.cout * L.cin * KH * KW;
-  for (int e = threadIdx.x; e < nw; e += NT) sW[e] = L.Wt[e];
+// One CTA's outputs of a conv pass belong to one subdomain: adds a reducing
+// epilogue's sums over the CTA (fixed order, in the launch's dynamic shared
+// memory, whose operands are done with) and hands them over once.
+constexpr size_t kFinishSmem = sizeof(double) * NT;
+template <class Epi>
+__device__ __forceinline__ void cta_finish(int b, double q, float* smem, const Epi& epi) {
+  if constexpr (Epi::kReduce) {
+    double* red = reinterpret_cast<double*>(smem);
+    __syncthreads();
+    red[threadIdx.x] = q;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      double t = 0.0;
+      for (int w = 0; w < NT / 32; ++w) t += red[w * 32 + threadIdx.x];
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (threadIdx.x == 0) epi.finish(b, t);
+    }
+  }
+}
+
+// Shared-memory tile of the blocked conv passes: the weights, then the rows of
+// the operand plane that a band of outputs reads, zero outside the plane (a
+// tap there adds an exact zero to the chain), rows split by column phase for a
+// stride-2 forward pass so that consecutive outputs read consecutive words.
+struct ConvTile {
+  int bands, bh;        // bands of bh rows (transposed pass: rows of a stride phase)
+  int rows, pitch;      // staged rows per channel and their pitch (floats)
+  int y_off, x_off;     // plane row / column of the tile's first, relative to the band's first row * stride
+  int w_floats, wc;     // floats of the staged weights; transposed: channels per tap in them (cin padded to 4)
+  size_t smem;
+};
+
+__device__ __forceinline__ void stage16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void stage4(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void stage_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const int b = blockIdx.y;
-  const float* rb = r + (size_t)b * rs;
+}
+
+// Transposed conv, blocked (k4 s2 / k3 s1): a CTA takes one subdomain and a
+// band of positions of every stride phase; a thread one position of one phase
+// and G channels; g[b, c, yy, xx] = sum_{o,i,j} W[o,c,i,j] r[b, o, y, x] over
+// the taps of the phase, one chain of FMAs per output in the order (i, j, o).
+// Operands come from shared memory (direct global reads left each thread
+// waiting for one load per product: 12-14 us for 256 Base subdomains).
+template <int KH, int KW, int ST, int G, class Epi>
+__global__ void __launch_bounds__(NT) conv_t_fast_kernel(LayerDev L, ConvTile T, const float* __restrict__ r, int rs,
+                                                         Epi epi) {
+  extern __shared__ __align__(16) float sm[];
+  float* sR = sm + T.w_floats;
+  const int b = blockIdx.x / T.bands, band = blockIdx.x % T.bands;
   const int qh = L.h / ST, qw = L.w / ST, ncg = L.cin / G, hw_o = L.ho * L.wo;
-  const int items = ST * ST * ncg * qh * qw;
-  for (int e = blockIdx.x * NT + threadIdx.x; e < items; e += gridDim.x * NT) {
+  const int q0 = band * T.bh, nq = min(T.bh, qh - q0);
+  const int nw = L.cout * L.cin * KH * KW;
+  if (T.wc == L.cin) {
+    for (int e = threadIdx.x; e < nw / 4; e += NT) stage16(sm + 4 * e, L.Wt + 4 * e);
+    for (int e = (nw & ~3) + threadIdx.x; e < nw; e += NT) stage4(sm + e, L.Wt + e, true);
+  } else {
+    for (int e = threadIdx.x; e < nw; e += NT) stage4(sm + e / L.cin * T.wc + e % L.cin, L.Wt + e, true);
+  }
+  const float* rb = r + (size_t)b * rs;
+  const int plane = T.rows * T.pitch, n = L.cout * plane;
+  for (int e = threadIdx.x; e < n; e += NT) {
+    const int o = e / plane, rem = e - o * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
+    const int y = q0 + yy + T.y_off, x = xx + T.x_off;
+    const bool in = y >= 0 && y < L.ho && x >= 0 && x < L.wo;
+    stage4(sR + e, rb + (in ? o * hw_o + y * L.wo + x : 0), in);
+  }
+  stage_wait();
+  const int items = ST * ST * ncg * nq * qw;
+  for (int e = threadIdx.x; e < items; e += NT) {
     int q = e;
+    const int rx = q % ST;
+    q /= ST;
     const int qx = q % qw;
     q /= qw;
-    const int qy = q % qh;
-    q /= qh;
-    const int cg = q % ncg;
-    q /= ncg;
-    const int rx = q % ST;
-    const int ry = q / ST;
+    const int qy = q % nq;
+    q /= nq;
+    const int ry = q % ST;
+    const int cg = q / ST;
     const int i0 = (ry + L.pad) % ST, j0 = (rx + L.pad) % ST;
     const int dy0 = (ry + L.pad - i0) / ST, dx0 = (rx + L.pad - j0) / ST;
     float acc[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) acc[g] = 0.f;
+    const float* rp = sR + (qy + dy0 - T.y_off) * T.pitch + qx + dx0 - T.x_off;
+    const float* wp = sm + (i0 * KW + j0) * T.wc + cg * G;
 #pragma unroll
-    for (int a = 0; a < KH / ST; ++a) {
-      const int y = qy + dy0 - a;
-      if (y < 0 || y >= L.ho) continue;
+    for (int a = 0; a < KH / ST; ++a)
 #pragma unroll
       for (int bb = 0; bb < KW / ST; ++bb) {
-        const int x = qx + dx0 - bb;
-        if (x < 0 || x >= L.wo) continue;
-        const float* rp = rb + y * L.wo + x;
-        const float* wp = sW + ((i0 + ST * a) * KW + j0 + ST * bb) * L.cin + cg * G;
+        const float* ra = rp - a * T.pitch - bb;
+        const float* wa = wp + (ST * a * KW + ST * bb) * T.wc;
+#pragma unroll 8
         for (int o = 0; o < L.cout; ++o) {
-          const float rv = __ldg(rp + (size_t)o * hw_o);
-          const float* w = wp + o * KH * KW * L.cin;
-#pragma unroll
-          for (int g = 0; g < G; ++g) acc[g] = fmaf(w[g], rv, acc[g]);
+          const float rv = ra[o * plane];
+          const float4 w = *reinterpret_cast<const float4*>(wa + o * KH * KW * T.wc);
+          acc[0] = fmaf(w.x, rv, acc[0]);
+          acc[1] = fmaf(w.y, rv, acc[1]);
+          acc[2] = fmaf(w.z, rv, acc[2]);
+          if (G == 4) acc[G - 1] = fmaf(w.w, rv, acc[G - 1]);
         }
       }
-    }
-    const int yy = ry + ST * qy, xx = rx + ST * qx;
+    const int yy = ry + ST * (q0 + qy), xx = rx + ST * qx;
 #pragma unroll
     for (int g = 0; g < G; ++g) epi(b, ((cg * G + g) * L.h + yy) * L.w + xx, acc[g]);
   }
 }
 
-// Forward conv, blocked (k4 s2 / k3 s1): thread = one output position and GF
-// output channels.  Weights in shared memory as [c][i][j][o].
+// Forward conv, blocked (k4 s2 / k3 s1): a CTA takes one subdomain and a band
+// of output rows; a thread one output position and GF output channels, one
+// chain of FMAs per output in the order (c, i, j).
 template <int KH, int KW, int ST, int GF, class Epi>
-__global__ void __launch_bounds__(NT) conv_fwd_fast_kernel(LayerDev L, const float* __restrict__ x, int xs, Epi epi) {
-  extern __shared__ float sW[];
+__global__ void __launch_bounds__(NT) conv_fwd_fast_kernel(LayerDev L, ConvTile T, const float* __restrict__ x, int xs,
+                                                           Epi epi) {
+  extern __shared__ __align__(16) float sm[];
+  float* sX = sm + T.w_floats;
+  const int b = blockIdx.x / T.bands, band = blockIdx.x % T.bands;
+  const int y0 = band * T.bh, ny = min(T.bh, L.ho - y0);
   const int nw = L.cout * L.cin * KH * KW;
-  for (int e = threadIdx.x; e < nw; e += NT) sW[e] = L.Wf[e];
-  __syncthreads();
-  const int b = blockIdx.y;
+  for (int e = threadIdx.x; e < nw / 4; e += NT) stage16(sm + 4 * e, L.Wf + 4 * e);
+  for (int e = (nw & ~3) + threadIdx.x; e < nw; e += NT) stage4(sm + e, L.Wf + e, true);
   const float* xb = x + (size_t)b * xs;
-  const int nog = L.cout / GF, hw_o = L.ho * L.wo, hw_i = L.h * L.w;
-  const int items = nog * hw_o;
-  for (int e = blockIdx.x * NT + threadIdx.x; e < items; e += gridDim.x * NT) {
-    const int og = e / hw_o, rem = e % hw_o, yo = rem / L.wo, xo = rem % L.wo;
+  const int hw_o = L.ho * L.wo, hw_i = L.h * L.w, half = T.pitch / ST;
+  const int plane = T.rows * T.pitch, n = L.cin * plane;
+  for (int e = threadIdx.x; e < n; e += NT) {
+    const int c = e / plane, rem = e - c * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
+    const int y = y0 * ST + yy + T.y_off, xi = xx + T.x_off;
+    const bool in = y >= 0 && y < L.h && xi >= 0 && xi < L.w;
+    // column xx of the padded row: phase xx % ST, place xx / ST
+    stage4(sX + c * plane + yy * T.pitch + (xx % ST) * half + xx / ST, xb + (in ? c * hw_i + y * L.w + xi : 0), in);
+  }
+  stage_wait();
+  const int nog = L.cout / GF, items = nog * ny * L.wo;
+  double q = 0.0;
+  for (int e = threadIdx.x; e < items; e += NT) {
+    int r = e;
+    const int xo = r % L.wo;
+    r /= L.wo;
+    const int yo = r % ny;
+    const int og = r / ny;
     float acc[GF];
 #pragma unroll
     for (int g = 0; g < GF; ++g) acc[g] = 0.f;
-    for (int c = 0; c < L.cin; ++c) {
-      const float* xc = xb + (size_t)c * hw_i;
-      const float* wc = sW + c * KH * KW * L.cout + og * GF;
+    const float* xc = sX + yo * ST * T.pitch + xo;
+    const float* wc = sm + og * GF;
+#pragma unroll 2
+    for (int c = 0; c < L.cin; ++c, xc += plane, wc += KH * KW * L.cout) {
 #pragma unroll
-      for (int i = 0; i < KH; ++i) {
-        const int yy = yo * ST - L.pad + i;
-        if (yy < 0 || yy >= L.h) continue;
+      for (int i = 0; i < KH; ++i)
 #pragma unroll
         for (int j = 0; j < KW; ++j) {
-          const int xx = xo * ST - L.pad + j;
-          if (xx < 0 || xx >= L.w) continue;
-          const float xv = __ldg(xc + yy * L.w + xx);
+          const float xv = xc[i * T.pitch + (j % ST) * half + j / ST];
           const float* w = wc + (i * KW + j) * L.cout;
-#pragma unroll
-          for (int g = 0; g < GF; ++g) acc[g] = fmaf(w[g], xv, acc[g]);
+          if (GF == 4) {
+            const float4 w4 = *reinterpret_cast<const float4*>(w);
+            acc[0] = fmaf(w4.x, xv, acc[0]);
+            acc[1] = fmaf(w4.y, xv, acc[1]);
+            acc[GF - 2] = fmaf(w4.z, xv, acc[GF - 2]);
+            acc[GF - 1] = fmaf(w4.w, xv, acc[GF - 1]);
+          } else {
+            const float2 w2 = *reinterpret_cast<const float2*>(w);
+            acc[0] = fmaf(w2.x, xv, acc[0]);
+            acc[1] = fmaf(w2.y, xv, acc[1]);
+          }
         }
-      }
     }
 #pragma unroll
-    for (int g = 0; g < GF; ++g) epi(b, (og * GF + g) * hw_o + rem, acc[g]);
+    for (int g = 0; g < GF; ++g) {
+      const int i = (og * GF + g) * hw_o + (y0 + yo) * L.wo + xo;
+      if constexpr (Epi::kReduce)
+        q += epi(b, i, acc[g]);
+      else
+        epi(b, i, acc[g]);
+    }
   }
+  cta_finish(b, q, sm, epi);
 }
 
 // Forward conv, direct: out[b, o, y, x] = sum_{c,i,j} W[o,c,i,j] x[b, c, y*s-p+i, x*s-p+j]
 template <class Epi>
 __global__ void __launch_bounds__(NT) conv_fwd_kernel(LayerDev L, const float* __restrict__ x, int xs, Epi epi) {
-  extern __shared__ float sW[];
+  extern __shared__ __align__(16) float sm[];
+  float* sW = sm;
   const int nw = L.cout * L.cin * L.kh * L.kw;
   for (int e = threadIdx.x; e < nw; e += blockDim.x) sW[e] = L.W[e];
   __syncthreads();
   const int b = blockIdx.y;
   const float* xb = x + (size_t)b * xs;
   const int hw_o = L.ho * L.wo, plane = L.cout * hw_o;
+  double q = 0.0;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < plane; e += gridDim.x * blockDim.x) {
     const int o = e / hw_o, rem = e % hw_o, y = rem / L.wo, xo = rem % L.wo;
     float acc = 0.f;
@@ -247,15 +373,20 @@ __global__ void __launch_bounds__(NT) conv_fwd_kernel(LayerDev L, const float* _
         }
       }
     }
-    epi(b, e, acc);
+    if constexpr (Epi::kReduce)
+      q += epi(b, e, acc);
+    else
+      epi(b, e, acc);
   }
+  cta_finish(b, q, sW, epi);
 }
 
 // Transposed conv, direct: g[b, c, yy, xx] = sum_{o,i,j} W[o,c,i,j] r[b, o, y, x] over
 // the (y, x) with y*s - p + i = yy and x*s - p + j = xx.
 template <class Epi>
 __global__ void __launch_bounds__(NT) conv_t_kernel(LayerDev L, const float* __restrict__ r, int rs, Epi epi) {
-  extern __shared__ float sW[];
+  extern __shared__ __align__(16) float sm[];
+  float* sW = sm;
   const int nw = L.cout * L.cin * L.kh * L.kw;
   for (int e = threadIdx.x; e < nw; e += blockDim.x) sW[e] = L.W[e];
   __syncthreads();
@@ -338,6 +469,28 @@ inline int conv_geo(const LayerDev& L) {
   return 0;
 }
 
+// Shared memory of a blocked conv CTA: two of them still share an SM.
+constexpr size_t kConvSmem = 96 * 1024;
+
+// Launches a blocked conv kernel, raising its shared-memory limit where needed.
+template <class K, class... A>
+void launch_blocked(K kernel, unsigned grid, size_t smem, cudaStream_t s, A... args) {
+  if (smem > 44 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
+  kernel<<<grid, NT, smem, s>>>(args...);
+}
+
+// Rows per band of a blocked conv pass: the whole plane while the batch alone
+// gives every SM several CTAs; fewer (at least one round of items per CTA) for
+// small batches, and what fits kConvSmem with the weights (row_bytes per
+// operand row; a band of bh rows stages bh * st + extra of them).  0: not even
+// one row fits.
+int conv_band(int rows, int items_per_row, int B, size_t w_bytes, size_t row_bytes, int st, int extra) {
+  int bh = rows;
+  while (bh > 1 && (size_t)B * ((rows + bh - 1) / bh) < 4 * 152 && (bh + 1) / 2 * items_per_row >= NT) bh = (bh + 1) / 2;
+  while (bh > 0 && w_bytes + row_bytes * (size_t)(bh * st + extra) > kConvSmem) bh = bh > 1 ? (bh + 1) / 2 : 0;
+  return bh;
+}
+
 template <class Epi>
 void transposed(const LayerDev& L, const Problem& P, const float* rho, Epi epi, cudaStream_t s) {
   // g over the inputs of layer L (= the neurons of the layer below it).
@@ -353,20 +506,33 @@ void transposed(const LayerDev& L, const Problem& P, const float* rho, Epi epi, 
   const int st = L.stride;
   if (geo && L.h % st == 0 && L.w % st == 0 && L.Wt && (L.cin % 4 == 0 || L.cin == 3)) {
     const int G = L.cin == 3 ? 3 : 4;
-    const int items = st * st * (L.cin / G) * (L.h / st) * (L.w / st);
-    dim3 grid((items + NT - 1) / NT, P.B);
-    if (geo == 1) {
-      if (G == 3)
-        conv_t_fast_kernel<4, 4, 2, 3, Epi><<<grid, NT, smem, s>>>(L, r, P.N, epi);
-      else
-        conv_t_fast_kernel<4, 4, 2, 4, Epi><<<grid, NT, smem, s>>>(L, r, P.N, epi);
-    } else {
-      if (G == 3)
-        conv_t_fast_kernel<3, 3, 1, 3, Epi><<<grid, NT, smem, s>>>(L, r, P.N, epi);
-      else
-        conv_t_fast_kernel<3, 3, 1, 4, Epi><<<grid, NT, smem, s>>>(L, r, P.N, epi);
+    // rows / columns of r around a position's own: taps reach dy0 - (k/s - 1) .. dy0
+    const int dlo = L.pad / st - (L.kh / st - 1), dhi = (st - 1 + L.pad) / st;
+    const int nt = st * st * (L.cin / G) * (L.w / st);  // items of one row
+    ConvTile T{};
+    T.wc = (L.cin + 3) & ~3;
+    T.w_floats = L.cout * L.kh * L.kw * T.wc;
+    T.y_off = T.x_off = dlo;
+    T.pitch = L.w / st + dhi - dlo;
+    T.bh = conv_band(L.h / st, nt, P.B, sizeof(float) * T.w_floats, sizeof(float) * L.cout * T.pitch, 1, dhi - dlo);
+    if (T.bh > 0) {
+      T.bands = (L.h / st + T.bh - 1) / T.bh;
+      T.rows = T.bh + dhi - dlo;
+      T.smem = sizeof(float) * ((size_t)T.w_floats + (size_t)L.cout * T.rows * T.pitch);
+      const unsigned grid = (unsigned)P.B * T.bands;
+      if (geo == 1) {
+        if (G == 3)
+          launch_blocked(conv_t_fast_kernel<4, 4, 2, 3, Epi>, grid, T.smem, s, L, T, r, P.N, epi);
+        else
+          launch_blocked(conv_t_fast_kernel<4, 4, 2, 4, Epi>, grid, T.smem, s, L, T, r, P.N, epi);
+      } else {
+        if (G == 3)
+          launch_blocked(conv_t_fast_kernel<3, 3, 1, 3, Epi>, grid, T.smem, s, L, T, r, P.N, epi);
+        else
+          launch_blocked(conv_t_fast_kernel<3, 3, 1, 4, Epi>, grid, T.smem, s, L, T, r, P.N, epi);
+      }
+      return;
     }
-    return;
   }
   const int plane = L.cin * L.h * L.w;
   dim3 grid((plane + NT - 1) / NT, P.B);
@@ -391,7 +557,7 @@ void forward(const LayerDev& L, const Problem& P, const float* x, Epi epi, cudaS
       dim3 grid(tiles_n, tiles_m);
       gemm_kernel<false, Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, xin, P.XS, L.W, L.n_in, epi);
     } else {
-      const int kc = ((L.n_in + splits - 1) / splits + TK - 1) / TK * TK;
+      const int kc = ((L.n_in + splits - 1) / splits + kSplitStep - 1) / kSplitStep * kSplitStep;
       splits = (L.n_in + kc - 1) / kc;
       dim3 grid(tiles_n, tiles_m, splits);
       gemm_splitk_kernel<Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, kc, xin, P.XS, L.W, L.n_in, P.splitk_part,
@@ -399,26 +565,35 @@ void forward(const LayerDev& L, const Problem& P, const float* x, Epi epi, cudaS
     }
     return;
   }
-  const size_t smem = sizeof(float) * L.cout * L.cin * L.kh * L.kw;
+  const size_t smem = std::max(sizeof(float) * L.cout * L.cin * L.kh * L.kw, Epi::kReduce ? kFinishSmem : 0);
   const int geo = conv_geo(L);
   if (geo && L.Wf && L.cout % 2 == 0) {
-    const int hw_o = L.ho * L.wo;
-    // four output channels per thread unless that leaves the GPU under-filled
-    const int GF = (L.cout % 4 == 0 && (size_t)(L.cout / 4) * hw_o * P.B >= 152 * 4 * NT) ? 4 : 2;
-    const int items = (L.cout / GF) * hw_o;
-    dim3 grid((items + NT - 1) / NT, P.B);
-    if (geo == 1) {
-      if (GF == 4)
-        conv_fwd_fast_kernel<4, 4, 2, 4, Epi><<<grid, NT, smem, s>>>(L, xin, P.XS, epi);
-      else
-        conv_fwd_fast_kernel<4, 4, 2, 2, Epi><<<grid, NT, smem, s>>>(L, xin, P.XS, epi);
-    } else {
-      if (GF == 4)
-        conv_fwd_fast_kernel<3, 3, 1, 4, Epi><<<grid, NT, smem, s>>>(L, xin, P.XS, epi);
-      else
-        conv_fwd_fast_kernel<3, 3, 1, 2, Epi><<<grid, NT, smem, s>>>(L, xin, P.XS, epi);
+    const int st = L.stride, GF = L.cout % 4 == 0 ? 4 : 2;
+    ConvTile T{};
+    T.w_floats = (L.cout * L.cin * L.kh * L.kw + 3) & ~3;
+    T.y_off = T.x_off = -L.pad;
+    T.pitch = ((L.wo - 1) * st + L.kw + st - 1) / st * st;
+    T.bh = conv_band(L.ho, (L.cout / GF) * L.wo, P.B, sizeof(float) * T.w_floats, sizeof(float) * L.cin * T.pitch, st,
+                     L.kh - st);
+    if (T.bh > 0) {
+      T.bands = (L.ho + T.bh - 1) / T.bh;
+      T.rows = T.bh * st + L.kh - st;
+      T.smem = std::max(sizeof(float) * ((size_t)T.w_floats + (size_t)L.cin * T.rows * T.pitch),
+                        Epi::kReduce ? kFinishSmem : 0);
+      const unsigned grid = (unsigned)P.B * T.bands;
+      if (geo == 1) {
+        if (GF == 4)
+          launch_blocked(conv_fwd_fast_kernel<4, 4, 2, 4, Epi>, grid, T.smem, s, L, T, xin, P.XS, epi);
+        else
+          launch_blocked(conv_fwd_fast_kernel<4, 4, 2, 2, Epi>, grid, T.smem, s, L, T, xin, P.XS, epi);
+      } else {
+        if (GF == 4)
+          launch_blocked(conv_fwd_fast_kernel<3, 3, 1, 4, Epi>, grid, T.smem, s, L, T, xin, P.XS, epi);
+        else
+          launch_blocked(conv_fwd_fast_kernel<3, 3, 1, 2, Epi>, grid, T.smem, s, L, T, xin, P.XS, epi);
+      }
+      return;
     }
-    return;
   }
   const int plane = L.cout * L.ho * L.wo;
   dim3 grid((plane + NT - 1) / NT, P.B);
