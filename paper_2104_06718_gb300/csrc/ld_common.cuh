@@ -58,6 +58,14 @@ struct Problem {
   const float* ball_eps = nullptr;
 };
 
+// The double of a float by its bits: FP64 instructions, conversions among
+// them, issue at 2 lanes per clock and SM on GB300, integer ones at 64.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+  if (m - 1u < 0x7fffffu || m >= 0x7f800000u) return (double)f;  // subnormals, infinities, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+}
+
 // Property of subdomain b; an out-of-range index is clamped here (so no
 // access leaves the per-property arrays) and reported by the pre-pass.
 __device__ __forceinline__ int prop_of(const Problem& P, int b) {
@@ -654,6 +662,16 @@ void launch_fsb_pick(int B, int C, const int32_t* cand, const double* child, int
 // Arrays: lam [B, N] (lambda), pi [B, N] (momentum), xB [B, N] and xA [B, N + 1]
 // (the primal blocks; xA's last column is x_hat_A,n), zB [B, N] and zA [B, N + 1]
 // (the conditional gradient), lp [B, N] (lambda' = lambda + (xB - xA) / eta).
+// Schedule of a call and, in device memory, where it stands: the captured
+// graph of one iteration reads eta from there.
+struct ProxSchedule {
+  double eta0, eta_end;
+  int T;
+};
+struct ProxIter {
+  int t;
+  float eta, eta_next;
+};
 struct ProxState {
   float* lam;
   float* pi;
@@ -662,19 +680,21 @@ struct ProxState {
   float* zB;
   float* zA;
   float* lp;
+  ProxIter* it;
 };
-// lambda' of the neurons [off, off + n) of every subdomain.
-void launch_prox_dual_prime(const Problem& P, const ProxState& S, int off, int n, float eta, cudaStream_t s);
+// The iteration state: iteration 0 (start = 1), or one iteration on.
+void launch_prox_step(const ProxSchedule& c, const ProxState& S, int start, cudaStream_t s);
+// lambda' of every neuron.
+void launch_prox_dual_prime(const Problem& P, const ProxState& S, cudaStream_t s);
 // Block k's optimal step (Eq. optimal-gamma-gauss) per subdomain and its
 // convex-combination update of (x_hat_B,k, x_hat_A,k+1); layer k at offset
 // off_k (n_k neurons; k = 0: none), layer k+1 at off_k1 (n_k1 neurons), last:
 // layer k+1 is the output (x_hat_A,n at column N, eta_n = infinity).
 void launch_prox_block_update(const Problem& P, const ProxState& S, int off_k, int n_k, int off_k1, int n_k1,
-                              int last, float eta, cudaStream_t s);
-// Dual update with momentum (Eq. momentum_updates; mu = 0: Eq. lambda_updates).
-// eta_next > 0: also forms lambda' for the next iteration's eta.
-void launch_prox_dual_update(const Problem& P, const ProxState& S, float eta, float mu, float eta_next,
-                             cudaStream_t s);
+                              int last, cudaStream_t s);
+// Dual update with momentum (Eq. momentum_updates; mu = 0: Eq. lambda_updates),
+// and lambda' for the next iteration's eta.
+void launch_prox_dual_update(const Problem& P, const ProxState& S, float mu, cudaStream_t s);
 
 // Feasibility pre-pass and box checks (ld_passes.cu).
 void launch_empty_flags(const Problem& P, int8_t* empty, int* status, cudaStream_t s);

@@ -21,7 +21,7 @@
 // (the 32 rows of a coefficient side by side in 128 bytes).  Every lane of a
 // warp then forms the same element of its own row: the weight is one
 // broadcast load for 32 rows, the coefficients are one coalesced load shared
-// by up to four channels, and no lane waits for another's sparsity.
+// by up to eight channels, and no lane waits for another's sparsity.
 //   * Rows of a conv layer: a group is one output position of one owner, its
 //     lanes the (rule, sign, channel) combinations, so all 32 rows reach the
 //     same window of every layer below; only that window is stored and
@@ -46,8 +46,8 @@
 // relaxation valid (a_bar upward, b_bar upward; any lower slope in [0,1] is
 // valid), and a rounded mu_j product lowers the bound by its rounding error
 // times max|x_hat_j|.  The scalar terms of a row (box, bias and intercept
-// products) are exact FP32 product pairs summed by the same Dot2 for at most
-// kFlush terms, then added in FP64: GB300 runs 2 FP64 operations per clock
+// products) are exact FP32 product pairs summed by the same Dot2 for one unit's
+// terms (at most 16), then added in FP64: GB300 runs 2 FP64 operations per clock
 // and SM against 128 FP32 ones, and an FP64 epilogue cost more than the sums.
 // The error of that is at most gamma_32^2 of a block's |terms| (FP32 gamma)
 // plus gamma_M (FP64) times the sum of |terms|; the error bounds and the sum
@@ -65,10 +65,13 @@ namespace {
 
 constexpr int NW = 8;              // warps per CTA
 constexpr int NT = 32 * NW;
-constexpr int kUnitC = 4;          // elements per unit (channels of a position / consecutive FC inputs)
-constexpr int kUnitsPerCta = 32;   // units of a CTA, until a layer has more than kMaxChunks of them
-constexpr int kMaxChunks = 64;
-constexpr int kFlush = 2;          // units between FP64 flushes: at most 2 * kUnitC * kFlush = 16 terms
+constexpr int kUnitC = 8;          // elements per unit (channels of a position / consecutive FC inputs)
+constexpr int kPairs = kUnitC / 2;
+constexpr int kTerms = 16;         // most scalar terms of a row between two FP64 flushes (a unit has up to 2 kUnitC)
+constexpr int kMaxChunks = 64;     // CTAs of a group
+constexpr int kWarpWork = 1024;    // terms a warp should have (2 to 8 units): its fixed cost is a few hundred instructions
+constexpr int kFcRows = 128;       // FC weight rows staged at once (a CTA has one unit per warp)
+constexpr unsigned kFull = 0xffffffffu;
 constexpr float kTwoU = 1.1920928955078125e-07f;  // 2^-23, twice the FP32 unit roundoff
 
 // Window of a group's nonzero coefficients on a plane: full, or hh x ww from
@@ -92,6 +95,8 @@ struct IbStep {
   int prev_r_off;           // layer j-1 in the flat ReLU vector
   float g2;                 // upper bound on 2 gamma_K^2 of this pass's sums (0 when seed)
   int chunks, units, units_per_cta;
+  int cp;                   // floats of a staged weight row (conv: cin rounded up)
+  int flush;                // units between FP64 flushes of the scalar terms
   int slot;                 // this launch's first partial-sum slot
   // bounds of the layers before k, per owner [owners, N], already clamped; boxes
   const float* lbk;
@@ -189,6 +194,61 @@ struct Dot2 {
   __device__ __forceinline__ float size() const { return __fmul_ru(s, 1.f + 2.f * kTwoU); }
 };
 
+// b - a by one packed instruction (a packed add takes no negated operand; the
+// product with -1 is exact, so the rounding is that of the subtraction).
+__device__ __forceinline__ float2 sub2(float2 b, float2 a) { return __ffma2_rn(a, make_float2(-1.f, -1.f), b); }
+
+// The dot products of a unit's needed elements, two per packed instruction
+// (half the issue slots of two Dot2, which leaves them to loads and votes) and
+// a last odd one by itself; pairs past np are not touched.
+struct UnitSums {
+  float2 p[kPairs], c[kPairs], s[kPairs];
+  Dot2 one;
+  int wa[kPairs], wb[kPairs], w1;    // the elements' places in a staged weight row
+  int np;
+  bool odd;
+  // Dot2::add of pair K, with nh = -h and nb = -bv.
+  template <int K>
+  __device__ __forceinline__ void pair(const float* ws, float2 m, float2 nm) {
+    const float2 v = make_float2(ws[wa[K]], ws[wb[K]]);
+    const float2 nh = __fmul2_rn(v, nm);
+    const float2 r = __ffma2_rn(v, m, nh);
+    const float2 t = sub2(p[K], nh);
+    const float2 nb = sub2(p[K], t);
+    const float2 q = __fadd2_rn(sub2(p[K], __fadd2_rn(t, nb)), sub2(nb, nh));
+    p[K] = t;
+    c[K] = __fadd2_rn(c[K], __fadd2_rn(q, r));
+    s[K] = make_float2(__fadd_ru(s[K].x, fabsf(nh.x)), __fadd_ru(s[K].y, fabsf(nh.y)));
+  }
+  __device__ __forceinline__ void add(const float* ws, float m1) {
+    const float2 m = make_float2(m1, m1), nm = make_float2(-m1, -m1);
+    if (np > 0) pair<0>(ws, m, nm);
+    if (np > 1) pair<1>(ws, m, nm);
+    if (np > 2) pair<2>(ws, m, nm);
+    if (np > 3) pair<3>(ws, m, nm);
+    if (odd) one.add(ws[w1], m1);
+  }
+  // Adds n terms: m at mp + k mstep (one coalesced load for all elements), the
+  // weights at ws + k CP.  A coefficient that is zero in every row is skipped.
+  template <int CP>
+  __device__ __forceinline__ void run(const float* __restrict__ mp, int mstep, const float* ws, int cp, int n) {
+    const int wstep = CP ? CP : cp;
+    int k = 0;
+    for (; k + 4 <= n; k += 4, mp += 4 * (size_t)mstep, ws += 4 * wstep) {
+      const float m0 = __ldg(mp), m1 = __ldg(mp + mstep), m2 = __ldg(mp + 2 * (size_t)mstep),
+                  m3 = __ldg(mp + 3 * (size_t)mstep);
+      if (__any_sync(kFull, m0 != 0.f)) add(ws, m0);
+      if (__any_sync(kFull, m1 != 0.f)) add(ws + wstep, m1);
+      if (__any_sync(kFull, m2 != 0.f)) add(ws + 2 * wstep, m2);
+      if (__any_sync(kFull, m3 != 0.f)) add(ws + 3 * wstep, m3);
+    }
+    for (; k < n; ++k, mp += mstep, ws += wstep) {
+      const float m = __ldg(mp);
+      if (__any_sync(kFull, m != 0.f)) add(ws, m);
+    }
+  }
+};
+
 // A row's scalar terms: the pair (d.p, d.c) of the current block, the FP64
 // sum of the finished ones, sum |terms| and the error bound (FP32, rounded up).
 struct RowSum {
@@ -196,80 +256,11 @@ struct RowSum {
   double v = 0.0;
   float e = 0.f;
   __device__ __forceinline__ void flush() {
-    v += (double)d.p;
-    v += (double)d.c;
+    v += widen(d.p);
+    v += widen(d.c);
     d.p = d.c = 0.f;
   }
 };
-
-// a = (W^T mu) of NA channels c[0..NA) at the plane position (y, x) of the
-// input of conv layer L, for the lane's row.
-template <int NA>
-__device__ __forceinline__ void conv_dots(const IbStep& st, const float* __restrict__ mu, int wy0, int wx0, int y,
-                                          int x, const int* c, Dot2* d) {
-  const LayerDev& L = st.L;
-  const int estep = st.win.hh * st.win.ww * 32;
-  const size_t wstep = (size_t)L.kh * L.kw * L.cin;
-  for (int ki = (y + L.pad) % L.stride; ki < L.kh; ki += L.stride) {
-    const int oy = (y + L.pad - ki) / L.stride;     // y + pad - ki is a multiple of stride here
-    if (y + L.pad < ki) break;
-    const int wy = oy - wy0;
-    if (oy >= L.ho || wy < 0 || wy >= st.win.hh) continue;
-    for (int kj = (x + L.pad) % L.stride; kj < L.kw; kj += L.stride) {
-      if (x + L.pad < kj) break;
-      const int ox = (x + L.pad - kj) / L.stride;
-      const int wx = ox - wx0;
-      if (ox >= L.wo || wx < 0 || wx >= st.win.ww) continue;
-      const float* mp = mu + (wy * st.win.ww + wx) * 32;
-      const float* wp = L.Wt + ((size_t)ki * L.kw + kj) * L.cin;
-      int o = 0;
-      for (; o + 4 <= L.cout; o += 4) {
-        float m[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) m[q] = __ldg(mp + (size_t)(o + q) * estep);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (!__any_sync(0xffffffffu, m[q] != 0.f)) continue;
-          const float* w = wp + (size_t)(o + q) * wstep;
-#pragma unroll
-          for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m[q]);
-        }
-      }
-      for (; o < L.cout; ++o) {
-        const float m = __ldg(mp + (size_t)o * estep);
-        if (!__any_sync(0xffffffffu, m != 0.f)) continue;
-        const float* w = wp + (size_t)o * wstep;
-#pragma unroll
-        for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m);
-      }
-    }
-  }
-}
-
-// a = (W^T mu) of the NA inputs c[0..NA) of FC layer L.
-template <int NA>
-__device__ __forceinline__ void fc_dots(const LayerDev& L, const float* __restrict__ mu, const int* c, Dot2* d) {
-  int o = 0;
-  for (; o + 4 <= L.n_out; o += 4) {
-    float m[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) m[q] = __ldg(mu + (size_t)(o + q) * 32);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (!__any_sync(0xffffffffu, m[q] != 0.f)) continue;
-      const float* w = L.W + (size_t)(o + q) * L.n_in;
-#pragma unroll
-      for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m[q]);
-    }
-  }
-  for (; o < L.n_out; ++o) {
-    const float m = __ldg(mu + (size_t)o * 32);
-    if (!__any_sync(0xffffffffu, m != 0.f)) continue;
-    const float* w = L.W + (size_t)o * L.n_in;
-#pragma unroll
-    for (int a = 0; a < NA; ++a) d[a].add(__ldg(w + c[a]), m);
-  }
-}
 
 // One element's contribution to the row and its coefficient for the next
 // pass: a with error bound da, on the input interval [l, u] (box) or through
@@ -303,13 +294,29 @@ __device__ __forceinline__ float relu_term(RowSum& R, float a, float da, float l
 
 // One CTA: units [chunk * units_per_cta, ...) of one group of 32 rows; a unit
 // is kUnitC channels of one position (conv) or kUnitC consecutive inputs (FC).
-__global__ void __launch_bounds__(NT) ib_step_kernel(IbStep st, IbRowMap M) {
+// The elements that some row needs are summed together from one stream of
+// coefficients, the weights in shared memory (conv: [tap][o][cp] channels; FC:
+// up to kFcRows rows of the CTA's inputs at a time).  Bound by the FP32 pipe:
+// 11 operations a term and element; with one or two elements per stream the
+// loads, votes and addresses were most of the instructions.
+// CP: floats of a staged weight row where it is one of the usual sizes (the
+// four rows of an unrolled step are then immediate offsets), else 0.
+template <int CP>
+__global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
+  extern __shared__ float sw[];
   __shared__ double red[NW][32][3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gl = blockIdx.x / st.chunks, chunk = blockIdx.x % st.chunks;
   const IbRow r = ib_row(M, M.group0 + gl, lane);
   const LayerDev& L = st.L;
   const bool conv = L.kind == LD_LAYER_CONV;
+  if (conv && !st.seed) {
+    for (int e = threadIdx.x; e < L.cout * L.kh * L.kw * st.cp; e += NT) {
+      const int c = e % st.cp, q = e / st.cp, o = q % L.cout, tap = q / L.cout;
+      sw[e] = c < L.cin ? __ldg(L.Wt + ((size_t)o * L.kh * L.kw + tap) * L.cin + c) : 0.f;
+    }
+    __syncthreads();
+  }
   const float* mu = st.mu_in + (size_t)gl * st.in_elems * 32 + lane;
   float* out = st.mu_out + (size_t)gl * st.out_elems * 32 + lane;
   const int iy0 = st.win.full ? 0 : r.oy * st.win.mul - st.win.sub;
@@ -317,96 +324,126 @@ __global__ void __launch_bounds__(NT) ib_step_kernel(IbStep st, IbRowMap M) {
   const int oy0 = st.wout.full ? 0 : r.oy * st.wout.mul - st.wout.sub;
   const int ox0 = st.wout.full ? 0 : r.ox * st.wout.mul - st.wout.sub;
   const int cb = conv ? (L.cin + kUnitC - 1) / kUnitC : 0;
-  const int so = conv ? r.i / (L.ho * L.wo) : 0;    // seed: the row's output channel
   const size_t lo_off = st.box ? (size_t)box_of(st, r.owner) * st.n0 : (size_t)r.owner * st.N + st.prev_r_off;
   const float* lp = (st.box ? st.l0 : st.lbk) + lo_off;
   const float* up = (st.box ? st.u0 : st.ubk) + lo_off;
+  // seed: the row's output channel and sign (0: a lane without a row)
+  const int so = conv ? r.i / (L.ho * L.wo) : 0;
+  const float sg = r.valid ? r.sign : 0.f;
+  const int hw = conv ? L.h * L.w : 1, ostep = conv ? st.wout.hh * st.wout.ww : 1;
   RowSum R;
-  const int u_lo = chunk * st.units_per_cta, u_hi = min(st.units, u_lo + st.units_per_cta);
   int done = 0;
-  for (int un = u_lo + warp; un < u_hi; un += NW) {
-    int wy = 0, wx = 0, y = 0, x = 0, c0, nc;
+  const int u_lo = chunk * st.units_per_cta, u_hi = min(st.units, u_lo + st.units_per_cta);
+  for (int ub = u_lo; ub < u_hi; ub += NW) {
+    const int un = ub + warp;
+    // element c (channel / input) of the unit: flat index ib + c hw, coefficient eb + c ostep
+    int y = 0, x = 0, c0 = un * kUnitC, nc = min(kUnitC, L.n_in - c0), ib = 0, eb = 0;
+    bool in = un < u_hi;
     if (conv) {
-      const int pos = un / cb;
+      const int pos = un / cb, wy = pos / st.wout.ww, wx = pos - wy * st.wout.ww;
       c0 = (un - pos * cb) * kUnitC;
       nc = min(kUnitC, L.cin - c0);
-      wy = pos / st.wout.ww;
-      wx = pos - wy * st.wout.ww;
       y = oy0 + wy;
       x = ox0 + wx;
-      if (y < 0 || y >= L.h || x < 0 || x >= L.w) continue;
-    } else {
-      c0 = un * kUnitC;
-      nc = min(kUnitC, L.n_in - c0);
+      in = in && y >= 0 && y < L.h && x >= 0 && x < L.w;
+      ib = y * L.w + x;
+      eb = pos;
     }
-    // the elements' bounds; those that some row of the group needs
-    float l[kUnitC], u[kUnitC];
-    int act[kUnitC] = {0, 0, 0, 0}, na = 0;
+    unsigned act = in ? (1u << nc) - 1u : 0u;
+    if (in && !st.box) {
+      // elements blocking in every row relax to zero whatever their sum is
+      float u[kUnitC];
 #pragma unroll
-    for (int q = 0; q < kUnitC; ++q) {
-      l[q] = u[q] = 0.f;
-      if (q < nc) {
-        const int ii = conv ? ((c0 + q) * L.h + y) * L.w + x : c0 + q;
-        l[q] = __ldg(lp + ii);
-        u[q] = __ldg(up + ii);
+      for (int q = 0; q < kUnitC; ++q) u[q] = q < nc ? __ldg(up + ib + (c0 + q) * hw) : 0.f;
+#pragma unroll
+      for (int q = 0; q < kUnitC; ++q)
+        if (q < nc && !__any_sync(kFull, u[q] > 0.f)) {
+          act &= ~(1u << q);
+          out[(size_t)(eb + (c0 + q) * ostep) * 32] = 0.f;
+        }
+    }
+    UnitSums S;
+    S.np = __popc(act) / 2;
+    S.odd = __popc(act) & 1;
+    {
+      const int wb = conv ? c0 : warp * kUnitC;   // the unit's first element in a staged weight row
+      unsigned rest = act;
+#pragma unroll
+      for (int k = 0; k < kPairs; ++k) {
+        S.p[k] = S.c[k] = S.s[k] = make_float2(0.f, 0.f);
+        S.wa[k] = S.wb[k] = 0;
+        if (k < S.np) {
+          const int a = __ffs(rest) - 1;
+          rest &= rest - 1;
+          const int b = __ffs(rest) - 1;
+          rest &= rest - 1;
+          S.wa[k] = wb + a;
+          S.wb[k] = wb + b;
+        }
       }
-      if (q < nc && __any_sync(0xffffffffu, st.box || u[q] > 0.f)) {
-#pragma unroll
-        for (int k = 0; k < kUnitC; ++k)
-          if (na == k) act[k] = c0 + q;
-        ++na;
+      S.w1 = S.odd ? wb + __ffs(rest) - 1 : 0;
+    }
+    if (!st.seed && conv) {
+      const int estep = st.win.hh * st.win.ww * 32, ys = y + L.pad, xs = x + L.pad;
+      // taps i0 + t stride read row (y + pad - i0) / stride - t
+      const int i0 = ys % L.stride, j0 = xs % L.stride;
+      const int oy = ys / L.stride, ox = xs / L.stride;
+      if (act)
+        for (int i = i0, qy = oy; i < L.kh && qy >= 0; i += L.stride, --qy) {
+          const int wy = qy - iy0;
+          if (qy >= L.ho || wy < 0 || wy >= st.win.hh) continue;
+          for (int j = j0, qx = ox; j < L.kw && qx >= 0; j += L.stride, --qx) {
+            const int wx = qx - ix0;
+            if (qx >= L.wo || wx < 0 || wx >= st.win.ww) continue;
+            S.run<CP>(mu + (wy * st.win.ww + wx) * 32, estep, sw + (i * L.kw + j) * L.cout * st.cp, st.cp, L.cout);
+          }
+        }
+    } else if (!st.seed) {
+      constexpr int kCols = NW * kUnitC;
+      for (int o0 = 0; o0 < L.n_out; o0 += kFcRows) {
+        const int nr = min(kFcRows, L.n_out - o0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nr * kCols; e += NT) {
+          const int o = e / kCols, i = ub * kUnitC + e % kCols;
+          sw[e] = i < L.n_in ? __ldg(L.W + (size_t)(o0 + o) * L.n_in + i) : 0.f;
+        }
+        __syncthreads();
+        if (act) S.run<CP>(mu + (size_t)o0 * 32, 32, sw, kCols, nr);
       }
     }
-    Dot2 d[kUnitC];
-    if (st.seed) {
-      const float sg = r.valid ? r.sign : 0.f;
-      const int ky = y + L.pad - r.oy * L.stride, kx = x + L.pad - r.ox * L.stride;
+    const int ky = y + L.pad - r.oy * L.stride, kx = x + L.pad - r.ox * L.stride;
+    for (int e = 0; act; ++e) {
+      const int c = c0 + __ffs(act) - 1, ii = ib + c * hw;
+      act &= act - 1;
+      // the element's sum: half e % 2 of pair e / 2, or the odd one
+      Dot2 d = S.one;
 #pragma unroll
-      for (int q = 0; q < kUnitC; ++q) {
-        if (q >= nc) continue;
-        float a = 0.f;
-        if (!conv) a = sg * __ldg(L.W + (size_t)r.i * L.n_in + c0 + q);
+      for (int k = 0; k < kPairs; ++k) {
+        const bool lo = k < S.np && e == 2 * k, hi = k < S.np && e == 2 * k + 1;
+        d.p = lo ? S.p[k].x : hi ? S.p[k].y : d.p;
+        d.c = lo ? S.c[k].x : hi ? S.c[k].y : d.c;
+        d.s = lo ? S.s[k].x : hi ? S.s[k].y : d.s;
+      }
+      if (st.seed) {
+        if (!conv) d.p = sg * __ldg(L.W + (size_t)r.i * L.n_in + c);
         else if (ky >= 0 && ky < L.kh && kx >= 0 && kx < L.kw)
-          a = sg * __ldg(L.W + (((size_t)so * L.cin + c0 + q) * L.kh + ky) * L.kw + kx);
-        d[q].p = a;
+          d.p = sg * __ldg(L.W + (((size_t)so * L.cin + c) * L.kh + ky) * L.kw + kx);
+        else
+          d.p = 0.f;
       }
-    } else if (na > 0) {
-      Dot2 t[kUnitC];
-      if (conv) {
-        if (na == 1) conv_dots<1>(st, mu, iy0, ix0, y, x, act, t);
-        else if (na == 2) conv_dots<2>(st, mu, iy0, ix0, y, x, act, t);
-        else if (na == 3) conv_dots<3>(st, mu, iy0, ix0, y, x, act, t);
-        else conv_dots<4>(st, mu, iy0, ix0, y, x, act, t);
-      } else {
-        if (na == 1) fc_dots<1>(L, mu, act, t);
-        else if (na == 2) fc_dots<2>(L, mu, act, t);
-        else if (na == 3) fc_dots<3>(L, mu, act, t);
-        else fc_dots<4>(L, mu, act, t);
-      }
-      // back to their channels
-#pragma unroll
-      for (int k = 0; k < kUnitC; ++k)
-#pragma unroll
-        for (int q = k; q < kUnitC; ++q)
-          if (k < na && act[k] == c0 + q) d[q] = t[k];
-    }
-#pragma unroll
-    for (int q = 0; q < kUnitC; ++q) {
-      if (q >= nc) continue;
-      const float a = d[q].value();
-      const float da = st.seed ? 0.f : __fmaf_ru(st.g2, d[q].size(), __fmul_ru(kTwoU, fabsf(a)));
+      const float l = __ldg(lp + ii), u = __ldg(up + ii);
+      const float a = d.value();
+      const float da = st.seed ? 0.f : __fmaf_ru(st.g2, d.size(), __fmul_ru(kTwoU, fabsf(a)));
       if (st.box) {
-        box_term(R, a, da, l[q], u[q]);
+        box_term(R, a, da, l, u);
       } else {
-        const int ii = conv ? ((c0 + q) * L.h + y) * L.w + x : c0 + q;
-        const float m = (a == 0.f && d[q].s == 0.f)
+        const float m = (a == 0.f && d.s == 0.f)
                             ? 0.f
-                            : relu_term(R, a, da, l[q], u[q], __ldg(st.bias_prev + ii / st.plane_prev), r.rule);
-        const int e = conv ? ((c0 + q) * st.wout.hh + wy) * st.wout.ww + wx : c0 + q;
-        out[(size_t)e * 32] = m;
+                            : relu_term(R, a, da, l, u, __ldg(st.bias_prev + ii / st.plane_prev), r.rule);
+        out[(size_t)(eb + c * ostep) * 32] = m;
       }
     }
-    if (++done % kFlush == 0) R.flush();
+    if (++done % st.flush == 0) R.flush();
   }
   R.flush();
   red[warp][lane][0] = R.v;
@@ -515,7 +552,9 @@ IbGeo ib_geo(const std::vector<LayerDev>& Ls, int k) {
     const bool conv = up.kind == LD_LAYER_CONV;
     g.elems[j] = conv ? up.cin * g.w[j].hh * g.w[j].ww : up.n_in;
     g.units[j] = conv ? g.w[j].hh * g.w[j].ww * ((up.cin + kUnitC - 1) / kUnitC) : (up.n_in + kUnitC - 1) / kUnitC;
-    g.per_cta[j] = std::max(kUnitsPerCta, (g.units[j] + kMaxChunks - 1) / kMaxChunks);
+    const int unit_terms = up.fan_t * std::min(kUnitC, conv ? up.cin : up.n_in);
+    g.per_cta[j] = NW * std::max(std::min(8, std::max(2, kWarpWork / unit_terms)),
+                                 (g.units[j] + NW * kMaxChunks - 1) / (NW * kMaxChunks));
     g.chunks[j] = (g.units[j] + g.per_cta[j] - 1) / g.per_cta[j];
     g.slots += g.chunks[j];
     if (j >= 1) g.width = std::max(g.width, g.elems[j]);
@@ -616,8 +655,24 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
       st.chunks = g.chunks[j - 1];
       st.units = g.units[j - 1];
       st.units_per_cta = g.per_cta[j - 1];
+      const bool conv = L.kind == LD_LAYER_CONV;
+      st.cp = conv ? (L.cin <= 4 ? 4 : L.cin <= 8 ? 8 : L.cin <= 16 ? 16 : (L.cin + 1) & ~1) : NW * kUnitC;
+      const int terms = (st.box ? 1 : 2) * std::min(kUnitC, conv ? L.cin : L.n_in);
+      st.flush = std::max(1, kTerms / terms);
+      const size_t smem = sizeof(float) * (size_t)st.cp * (st.seed ? 0
+                                                           : conv  ? L.cout * L.kh * L.kw
+                                                                   : std::min(kFcRows, L.n_out));
+      auto kernel = st.cp == 4    ? ib_step_kernel<4>
+                    : st.cp == 8  ? ib_step_kernel<8>
+                    : st.cp == 16 ? ib_step_kernel<16>
+                    : st.cp == 64 ? ib_step_kernel<64>
+                                  : ib_step_kernel<0>;
+      if (smem > 40 * 1024) {
+        const cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+        if (ea != cudaSuccess) return ea;
+      }
       count_launch();
-      ib_step_kernel<<<(unsigned)(M.n_groups * (int64_t)st.chunks), NT, 0, s>>>(st, M);
+      kernel<<<(unsigned)(M.n_groups * (int64_t)st.chunks), NT, smem, s>>>(st, M);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
       st.slot += st.chunks;
@@ -627,8 +682,8 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
     ib_collect_kernel<<<(unsigned)((M.n_groups * 32LL + NT - 1) / NT), NT, 0, s>>>(M, g.slots, A.part, Lk.b, plane_k,
                                                                                  A.acc);
   }
-  // FP64 sums, plus Dot2's gamma_32^2 (FP32) of the blocks of at most 16 terms
-  const double gd = gamma32(2 * kUnitC * kFlush);
+  // FP64 sums, plus Dot2's gamma_32^2 (FP32) of the blocks of at most kTerms terms
+  const double gd = gamma32(kTerms);
   IbFinish f{A.n_owners, Lk.n_out, A.n_rules, n_signs, A.N, Lk.r_out_off, A.acc, A.gamma_M + 2.0 * gd * gd, A.mask,
              A.lbk, A.ubk, A.out_lb};
   const int64_t total = (int64_t)A.n_owners * Lk.n_out;
