@@ -415,23 +415,31 @@ ld_status run_iterations(ld_net* net, const Problem& P, const ld_opts& o, int n_
 // Runs launches(stream) captured into a CUDA graph that is then launched on s
 // (one launch instead of one per kernel; the executable graph is updated in
 // place when only kernel arguments changed), or directly on s when s is
-// itself being captured or capture is unavailable.
+// itself being captured or capture is unavailable; `times` such launches in a
+// row (an iteration whose parameters are kept on the device: capturing and
+// updating the 2600 kernels of 100 proximal iterations took longer than
+// running them).
 template <class F>
-ld_status run_graphed(ld_net* net, cudaStream_t s, F launches) {
+ld_status run_graphed(ld_net* net, cudaStream_t s, F launches, int times = 1) {
+  const auto direct = [&] {
+    ld_status st = LD_OK;
+    for (int i = 0; i < times && st == LD_OK; ++i) st = launches(s);
+    return st;
+  };
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (!net->graphs || cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
-    return launches(s);
+    return direct();
   }
   if (!net->cap_stream && cudaStreamCreateWithFlags(&net->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     net->graphs = false;
-    return launches(s);
+    return direct();
   }
   if (cudaStreamBeginCapture(net->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
     net->graphs = false;
-    return launches(s);
+    return direct();
   }
   const ld_status st = launches(net->cap_stream);
   cudaGraph_t g = nullptr;
@@ -441,7 +449,7 @@ ld_status run_graphed(ld_net* net, cudaStream_t s, F launches) {
     cudaGetLastError();
     if (st != LD_OK) return st;
     net->graphs = false;  // nothing ran: launch directly from now on
-    return launches(s);
+    return direct();
   }
   if (net->iter_exec) {
     cudaGraphExecUpdateResultInfo info;
@@ -456,10 +464,15 @@ ld_status run_graphed(ld_net* net, cudaStream_t s, F launches) {
     cudaGraphDestroy(g);
     net->iter_exec = nullptr;
     net->graphs = false;
-    return launches(s);
+    return direct();
   }
+  size_t nodes = 0;
+  if (times > 1 && cudaGraphGetNodes(g, nullptr, &nodes) == cudaSuccess)
+    ld::count_launch((int)nodes * (times - 1));  // the capture counted one pass
   cudaGraphDestroy(g);
-  return cuda_status(cudaGraphLaunch(net->iter_exec, s));
+  cudaError_t le = cudaSuccess;
+  for (int i = 0; i < times && le == cudaSuccess; ++i) le = cudaGraphLaunch(net->iter_exec, s);
+  return cuda_status(le);
 }
 
 // Tensor-core plan and shadow buffers for B subdomains and n_props properties.
@@ -1240,11 +1253,10 @@ ld_status ensure_prox_ws(ld_net* net, int B) {
   const size_t a = align256(4 * Bn * (N + 1)), l = align256(4 * Bn * N);
   cudaDeviceSynchronize();
   if (net->prox_ws) cudaFree(net->prox_ws);
-  if (net->dsg_ws) cudaFree(net->dsg_ws);
   net->prox_ws = nullptr;
   net->prox_B = -1;
   void* p = nullptr;
-  const cudaError_t e = ld::dev_malloc(&p, 2 * a + l);
+  const cudaError_t e = ld::dev_malloc(&p, 2 * a + l + align256(sizeof(ld::ProxIter)));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cuda_status(e);
@@ -1266,6 +1278,7 @@ ld::ProxState prox_state(ld_net* net) {
   S.xA = reinterpret_cast<float*>(c);
   S.zA = reinterpret_cast<float*>(c + a);
   S.lp = reinterpret_cast<float*>(c + 2 * a);
+  S.it = reinterpret_cast<ld::ProxIter*>(c + 2 * a + align256(4 * Bn * N));
   return S;
 }
 
@@ -1285,39 +1298,32 @@ void prox_init_primal(ld_net* net, const Problem& P, const ld::ProxState& S, cud
   }
 }
 
-// T outer iterations of Algorithm 2: J block-coordinate Frank-Wolfe sweeps
+// One outer iteration of Algorithm 2: J block-coordinate Frank-Wolfe sweeps
 // (blocks k = 0..n-1: lambda' of layers k and k+1, the conditional gradient
 // by the transposed pass of layer k+1 with the vertex choice of layer k and
 // the forward pass of layer k+1, then the optimal step and the block's move),
-// then the dual update.
-ld_status run_prox_iterations(ld_net* net, const Problem& P, const ld::ProxState& S, const ld_prox_opts& o,
-                              int n_iters, cudaStream_t s) {
+// then the dual update.  lambda' is kept current by the block moves and the
+// dual updates.
+ld_status run_prox_iteration(ld_net* net, const Problem& P, const ld::ProxState& S, const ld_prox_opts& o,
+                             const ld::ProxSchedule& sched, cudaStream_t s) {
   const int n = net->n;
-  auto eta_of = [&](int t) {
-    return (float)((double)o.eta0 + ((double)o.eta_end - (double)o.eta0) * t / std::max(n_iters - 1, 1));
-  };
-  // lambda' of every layer at the first eta; from then on the block moves and
-  // the dual updates keep it current
-  if (n_iters > 0) ld::launch_prox_dual_prime(P, S, 0, net->N, eta_of(0), s);
-  for (int t = 0; t < n_iters; ++t) {
-    const float eta = eta_of(t);
-    for (int j = 0; j < o.J; ++j) {
-      for (int k = 0; k < n; ++k) {
-        ld::EpiArgmin ea{P, k, r_off(net, k), x_off(net, k), S.lp, net->x, S.zB, nullptr, nullptr};
-        if (k == n - 1)
-          ld::launch_top_argmin(layer(net, n), P, ea, s);
-        else
-          ld::launch_transposed_argmin(layer(net, k + 1), nullptr, P, S.lp, ea, s);
-        const LayerDev& Lk1 = layer(net, k + 1);
-        ld::EpiStore es{P, Lk1.r_out_off, plane_of(Lk1), k + 1 == n ? 1 : 0, Lk1.b, S.zA};
-        ld::launch_forward_store(Lk1, P, net->x, es, s);
-        ld::launch_prox_block_update(P, S, k >= 1 ? r_off(net, k) : 0, k >= 1 ? layer(net, k).n_out : 0,
-                                     k + 1 <= n - 1 ? r_off(net, k + 1) : 0, k + 1 <= n - 1 ? Lk1.n_out : 1,
-                                     k + 1 == n ? 1 : 0, eta, s);
-      }
+  for (int j = 0; j < o.J; ++j) {
+    for (int k = 0; k < n; ++k) {
+      ld::EpiArgmin ea{P, k, r_off(net, k), x_off(net, k), S.lp, net->x, S.zB, nullptr, nullptr};
+      if (k == n - 1)
+        ld::launch_top_argmin(layer(net, n), P, ea, s);
+      else
+        ld::launch_transposed_argmin(layer(net, k + 1), nullptr, P, S.lp, ea, s);
+      const LayerDev& Lk1 = layer(net, k + 1);
+      ld::EpiStore es{P, Lk1.r_out_off, plane_of(Lk1), k + 1 == n ? 1 : 0, Lk1.b, S.zA};
+      ld::launch_forward_store(Lk1, P, net->x, es, s);
+      ld::launch_prox_block_update(P, S, k >= 1 ? r_off(net, k) : 0, k >= 1 ? layer(net, k).n_out : 0,
+                                   k + 1 <= n - 1 ? r_off(net, k + 1) : 0, k + 1 <= n - 1 ? Lk1.n_out : 1,
+                                   k + 1 == n ? 1 : 0, s);
     }
-    ld::launch_prox_dual_update(P, S, eta, o.mu, t + 1 < n_iters ? eta_of(t + 1) : 0.f, s);
   }
+  ld::launch_prox_dual_update(P, S, o.mu, s);
+  ld::launch_prox_step(sched, S, 0, s);
   return last_error();
 }
 
@@ -1483,7 +1489,10 @@ ld_status ld_bound_proximal(ld_net* net, const float* lb0, const float* ub0, con
   }
   if (n_iters > 0) {
     PhaseMark pm(net, LD_PHASE_ITER, s);
-    st = run_graphed(net, s, [&](cudaStream_t cs) { return run_prox_iterations(net, P, PS, o, n_iters, cs); });
+    const ld::ProxSchedule sched{(double)o.eta0, (double)o.eta_end, n_iters};
+    ld::launch_prox_step(sched, PS, 1, s);
+    ld::launch_prox_dual_prime(P, PS, s);
+    st = run_graphed(net, s, [&](cudaStream_t cs) { return run_prox_iteration(net, P, PS, o, sched, cs); }, n_iters);
     if (st != LD_OK) return st;
   }
   {
