@@ -1309,17 +1309,8 @@ ld_status run_prox_iteration(ld_net* net, const Problem& P, const ld::ProxState&
   const int n = net->n;
   for (int j = 0; j < o.J; ++j) {
     for (int k = 0; k < n; ++k) {
-      ld::EpiArgmin ea{P, k, r_off(net, k), x_off(net, k), S.lp, net->x, S.zB, nullptr, nullptr};
-      if (k == n - 1)
-        ld::launch_top_argmin(layer(net, n), P, ea, s);
-      else
-        ld::launch_transposed_argmin(layer(net, k + 1), nullptr, P, S.lp, ea, s);
-      const LayerDev& Lk1 = layer(net, k + 1);
-      ld::EpiStore es{P, Lk1.r_out_off, plane_of(Lk1), k + 1 == n ? 1 : 0, Lk1.b, S.zA};
-      ld::launch_forward_store(Lk1, P, net->x, es, s);
-      ld::launch_prox_block_update(P, S, k >= 1 ? r_off(net, k) : 0, k >= 1 ? layer(net, k).n_out : 0,
-                                   k + 1 <= n - 1 ? r_off(net, k + 1) : 0, k + 1 <= n - 1 ? Lk1.n_out : 1,
-                                   k + 1 == n ? 1 : 0, s);
+      ld::launch_prox_block(k >= 1 ? &layer(net, k) : nullptr, layer(net, k + 1), k, n, P, S, net->x, x_off(net, k),
+                            net->smem_optin, s);
     }
   }
   ld::launch_prox_dual_update(P, S, o.mu, s);

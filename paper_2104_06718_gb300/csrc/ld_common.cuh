@@ -634,6 +634,13 @@ void launch_forward_adam(const LayerDev& L, const Problem& P, const float* x, Ep
 void launch_forward_record(const LayerDev& L, const Problem& P, const float* x, EpiRecord epi,
                            cudaStream_t s);
 void launch_forward_store(const LayerDev& L, const Problem& P, const float* x, EpiStore epi, cudaStream_t s);
+// Split-K ranges of the forward pass of FC layer L; its partial sums alone,
+// into P.splitk_part [splits][B][n_out] (false, nothing launched: no room).
+struct SplitK {
+  int splits, kc;
+};
+SplitK forward_split(const LayerDev& L, const Problem& P);
+bool launch_forward_partials(const LayerDev& L, const Problem& P, const float* x, SplitK& k, cudaStream_t s);
 void launch_transposed_scores(const LayerDev& L, const Problem& P, const float* mu, EpiScores epi, cudaStream_t s);
 void launch_top_scores(const LayerDev& Ln, const Problem& P, EpiScores epi, cudaStream_t s);
 void launch_forward_eval(const LayerDev& L, const Problem& P, const float* x, EpiEval epi, cudaStream_t s);
@@ -686,12 +693,12 @@ struct ProxState {
 void launch_prox_step(const ProxSchedule& c, const ProxState& S, int start, cudaStream_t s);
 // lambda' of every neuron.
 void launch_prox_dual_prime(const Problem& P, const ProxState& S, cudaStream_t s);
-// Block k's optimal step (Eq. optimal-gamma-gauss) per subdomain and its
-// convex-combination update of (x_hat_B,k, x_hat_A,k+1); layer k at offset
-// off_k (n_k neurons; k = 0: none), layer k+1 at off_k1 (n_k1 neurons), last:
-// layer k+1 is the output (x_hat_A,n at column N, eta_n = infinity).
-void launch_prox_block_update(const Problem& P, const ProxState& S, int off_k, int n_k, int off_k1, int n_k1,
-                              int last, cudaStream_t s);
+// One Frank-Wolfe step of block k = (x_hat_B,k, x_hat_A,k+1), Lk1 = layer k+1:
+// the conditional gradient at lambda', the optimal step of Eq.
+// (optimal-gamma-gauss) per subdomain and the convex combination.  Lk: layer k
+// (nullptr: k = 0); x: the x buffer; x_off: layer k's offset in it.
+void launch_prox_block(const LayerDev* Lk, const LayerDev& Lk1, int k, int n, const Problem& P, const ProxState& S,
+                       float* x, int x_off, size_t smem_limit, cudaStream_t s);
 // Dual update with momentum (Eq. momentum_updates; mu = 0: Eq. lambda_updates),
 // and lambda' for the next iteration's eta.
 void launch_prox_dual_update(const Problem& P, const ProxState& S, float mu, cudaStream_t s);

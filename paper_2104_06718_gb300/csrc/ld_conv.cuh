@@ -1,0 +1,206 @@
+// The blocked conv passes (k4 s2 / k3 s1) on operands staged in shared memory:
+// device code shared by the layerwise kernels (ld_passes.cu) and the proximal
+// solver's block kernel (ld_prox.cu), and the host's choice of their tiles.
+#pragma once
+#include <algorithm>
+
+#include "ld_common.cuh"
+
+namespace ld {
+namespace {
+
+// Shared-memory tile of the blocked conv passes: the weights, then the rows of
+// the operand plane that a band of outputs reads, zero outside the plane (a
+// tap there adds an exact zero to the chain), rows split by column phase for a
+// stride-2 forward pass so that consecutive outputs read consecutive words.
+struct ConvTile {
+  int bands, bh;        // bands of bh rows (transposed pass: rows of a stride phase)
+  int rows, pitch;      // staged rows per channel and their pitch (floats)
+  int y_off, x_off;     // plane row / column of the tile's first, relative to the band's first row * stride
+  int w_floats, wc;     // floats of the staged weights; transposed: channels per tap in them (cin padded to 4)
+  size_t smem;
+};
+
+__device__ __forceinline__ void stage16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void stage4(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void stage_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+}
+__device__ __forceinline__ void stage_floats(float* dst, const float* src, int n, int nt) {
+  for (int e = threadIdx.x; e < n / 4; e += nt) stage16(dst + 4 * e, src + 4 * e);
+  for (int e = (n & ~3) + threadIdx.x; e < n; e += nt) stage4(dst + e, src + e, true);
+}
+
+// Weights of the transposed pass: [o][i][j][wc].
+__device__ __forceinline__ void conv_t_weights(const LayerDev& L, const ConvTile& T, float* sW, int nt) {
+  const int nw = L.cout * L.cin * L.kh * L.kw;
+  if (T.wc == L.cin) {
+    stage_floats(sW, L.Wt, nw, nt);
+  } else {
+    for (int e = threadIdx.x; e < nw; e += nt) stage4(sW + e / L.cin * T.wc + e % L.cin, L.Wt + e, true);
+  }
+}
+
+// The rows of r (one subdomain's [cout, ho, wo]) read by the band from phase row q0.
+__device__ __forceinline__ void conv_t_rows(const LayerDev& L, const ConvTile& T, float* sR, const float* rb, int q0,
+                                            int nt) {
+  const int plane = T.rows * T.pitch, n = L.cout * plane, hw_o = L.ho * L.wo;
+  for (int e = threadIdx.x; e < n; e += nt) {
+    const int o = e / plane, rem = e - o * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
+    const int y = q0 + yy + T.y_off, x = xx + T.x_off;
+    const bool in = y >= 0 && y < L.ho && x >= 0 && x < L.wo;
+    stage4(sR + e, rb + (in ? o * hw_o + y * L.wo + x : 0), in);
+  }
+}
+
+// f(channel, y, x, g) for every output of the band: a thread takes one
+// position of one stride phase and G channels; g[c, yy, xx] = sum_{o,i,j}
+// W[o,c,i,j] r[o, y, x] over the taps of the phase, one chain of FMAs per
+// output in the order (i, j, o).
+template <int KH, int KW, int ST, int G, class F>
+__device__ __forceinline__ void conv_t_items(const LayerDev& L, const ConvTile& T, const float* sW, const float* sR,
+                                             int q0, int nq, int nt, F f) {
+  const int qw = L.w / ST, ncg = L.cin / G, plane = T.rows * T.pitch;
+  const int items = ST * ST * ncg * nq * qw;
+  for (int e = threadIdx.x; e < items; e += nt) {
+    int q = e;
+    const int rx = q % ST;
+    q /= ST;
+    const int qx = q % qw;
+    q /= qw;
+    const int qy = q % nq;
+    q /= nq;
+    const int ry = q % ST;
+    const int cg = q / ST;
+    const int i0 = (ry + L.pad) % ST, j0 = (rx + L.pad) % ST;
+    const int dy0 = (ry + L.pad - i0) / ST, dx0 = (rx + L.pad - j0) / ST;
+    float acc[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) acc[g] = 0.f;
+    const float* rp = sR + (qy + dy0 - T.y_off) * T.pitch + qx + dx0 - T.x_off;
+    const float* wp = sW + (i0 * KW + j0) * T.wc + cg * G;
+#pragma unroll
+    for (int a = 0; a < KH / ST; ++a)
+#pragma unroll
+      for (int bb = 0; bb < KW / ST; ++bb) {
+        const float* ra = rp - a * T.pitch - bb;
+        const float* wa = wp + (ST * a * KW + ST * bb) * T.wc;
+#pragma unroll 8
+        for (int o = 0; o < L.cout; ++o) {
+          const float rv = ra[o * plane];
+          const float4 w = *reinterpret_cast<const float4*>(wa + o * KH * KW * T.wc);
+          acc[0] = fmaf(w.x, rv, acc[0]);
+          acc[1] = fmaf(w.y, rv, acc[1]);
+          acc[2] = fmaf(w.z, rv, acc[2]);
+          if (G == 4) acc[G - 1] = fmaf(w.w, rv, acc[G - 1]);
+        }
+      }
+    const int yy = ry + ST * (q0 + qy), xx = rx + ST * qx;
+#pragma unroll
+    for (int g = 0; g < G; ++g) f(cg * G + g, yy, xx, acc[g]);
+  }
+}
+
+// Place of input element (c, row yy of the tile, padded column xx) in the forward tile.
+__device__ __forceinline__ int conv_f_at(const ConvTile& T, int st, int c, int yy, int xx) {
+  return (c * T.rows + yy) * T.pitch + (st == 2 ? (xx & 1) * (T.pitch / 2) + (xx >> 1) : xx);
+}
+
+// f(channel, y, x, acc) for every output of the band of ny rows from y0: a
+// thread takes one output position and GF output channels, one chain of FMAs
+// per output in the order (c, i, j).
+template <int KH, int KW, int ST, int GF, class F>
+__device__ __forceinline__ void conv_f_items(const LayerDev& L, const ConvTile& T, const float* sW, const float* sX,
+                                             int y0, int ny, int nt, F f) {
+  const int nog = L.cout / GF, items = nog * ny * L.wo, plane = T.rows * T.pitch, half = T.pitch / ST;
+  for (int e = threadIdx.x; e < items; e += nt) {
+    int r = e;
+    const int xo = r % L.wo;
+    r /= L.wo;
+    const int yo = r % ny;
+    const int og = r / ny;
+    float acc[GF];
+#pragma unroll
+    for (int g = 0; g < GF; ++g) acc[g] = 0.f;
+    const float* xc = sX + yo * ST * T.pitch + xo;
+    const float* wc = sW + og * GF;
+#pragma unroll 2
+    for (int c = 0; c < L.cin; ++c, xc += plane, wc += KH * KW * L.cout) {
+#pragma unroll
+      for (int i = 0; i < KH; ++i)
+#pragma unroll
+        for (int j = 0; j < KW; ++j) {
+          const float xv = xc[i * T.pitch + (j % ST) * half + j / ST];
+          const float* w = wc + (i * KW + j) * L.cout;
+          if (GF == 4) {
+            const float4 w4 = *reinterpret_cast<const float4*>(w);
+            acc[0] = fmaf(w4.x, xv, acc[0]);
+            acc[1] = fmaf(w4.y, xv, acc[1]);
+            acc[GF - 2] = fmaf(w4.z, xv, acc[GF - 2]);
+            acc[GF - 1] = fmaf(w4.w, xv, acc[GF - 1]);
+          } else {
+            const float2 w2 = *reinterpret_cast<const float2*>(w);
+            acc[0] = fmaf(w2.x, xv, acc[0]);
+            acc[1] = fmaf(w2.y, xv, acc[1]);
+          }
+        }
+    }
+#pragma unroll
+    for (int g = 0; g < GF; ++g) f(og * GF + g, y0 + yo, xo, acc[g]);
+  }
+}
+
+// 1: 4x4 stride 2, 2: 3x3 stride 1 (the blocked passes), 0: other geometries.
+inline int conv_geo(const LayerDev& L) {
+  if (L.kh == 4 && L.kw == 4 && L.stride == 2) return 1;
+  if (L.kh == 3 && L.kw == 3 && L.stride == 1) return 2;
+  return 0;
+}
+// Whether the blocked transposed / forward pass covers the layer.
+inline bool conv_t_covers(const LayerDev& L) {
+  return L.kind == LD_LAYER_CONV && conv_geo(L) && L.h % L.stride == 0 && L.w % L.stride == 0 && L.Wt &&
+         (L.cin % 4 == 0 || L.cin == 3);
+}
+inline bool conv_f_covers(const LayerDev& L) {
+  return L.kind == LD_LAYER_CONV && conv_geo(L) && L.Wf && L.cout % 2 == 0;
+}
+
+// Tiles of the transposed / forward pass with bands of bh rows (bh <= 0: the
+// fixed part only).
+inline ConvTile conv_t_tile(const LayerDev& L, int bh) {
+  const int st = L.stride, dlo = L.pad / st - (L.kh / st - 1), dhi = (st - 1 + L.pad) / st;
+  ConvTile T{};
+  // rows / columns of r around a position's own: taps reach dy0 - (k/s - 1) .. dy0
+  T.wc = (L.cin + 3) & ~3;
+  T.w_floats = L.cout * L.kh * L.kw * T.wc;
+  T.y_off = T.x_off = dlo;
+  T.pitch = L.w / st + dhi - dlo;
+  T.bh = bh;
+  T.rows = bh + dhi - dlo;
+  T.bands = bh > 0 ? (L.h / st + bh - 1) / bh : 0;
+  T.smem = sizeof(float) * ((size_t)T.w_floats + (size_t)L.cout * T.rows * T.pitch);
+  return T;
+}
+inline ConvTile conv_f_tile(const LayerDev& L, int bh) {
+  const int st = L.stride;
+  ConvTile T{};
+  T.w_floats = (L.cout * L.cin * L.kh * L.kw + 3) & ~3;
+  T.y_off = T.x_off = -L.pad;
+  T.pitch = ((L.wo - 1) * st + L.kw + st - 1) / st * st;
+  T.bh = bh;
+  T.rows = bh * st + L.kh - st;
+  T.bands = bh > 0 ? (L.ho + bh - 1) / bh : 0;
+  T.smem = sizeof(float) * ((size_t)T.w_floats + (size_t)L.cin * T.rows * T.pitch);
+  return T;
+}
+
+}  // namespace
+}  // namespace ld

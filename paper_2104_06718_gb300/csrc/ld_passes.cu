@@ -16,9 +16,7 @@
 // on operand rows staged in shared memory (several channels per thread,
 // compile-time taps, transposed conv split by stride phase); other geometries
 // take direct loops.
-#include <algorithm>
-
-#include "ld_common.cuh"
+#include "ld_conv.cuh"
 
 namespace ld {
 namespace {
@@ -119,6 +117,42 @@ __global__ void __launch_bounds__(NT) gemm_kernel(int M, int Ncol, int K, const 
   gemm_epilogue(m0, n0, M, Ncol, acc, epi);
 }
 
+// Ranges of the split-K forward pass of FC layer L for B subdomains: `splits`
+// ranges of kc inputs each (1: no split).
+void split_of(const LayerDev& L, const Problem& P, int& splits, int& kc) {
+  const int tiles_n = (L.n_out + TN - 1) / TN, tiles_m = (P.B + TM - 1) / TM;
+  // split K until the grid covers the GPU about twice (304 blocks)
+  splits = (304 + tiles_n * tiles_m - 1) / (tiles_n * tiles_m);
+  const int kmax = (L.n_in + 63) / 64;
+  if (splits > kmax) splits = kmax;
+  if (splits > 16) splits = 16;
+  if (!P.splitk_part || (size_t)splits * P.B * L.n_out > (size_t)P.splitk_part_cap ||
+      tiles_n * tiles_m > P.splitk_count_cap)
+    splits = 1;
+  kc = L.n_in;
+  if (splits > 1) {
+    kc = ((L.n_in + splits - 1) / splits + kSplitStep - 1) / kSplitStep * kSplitStep;
+    splits = (L.n_in + kc - 1) / kc;
+  }
+}
+
+// The partial sums alone: part[z][m][n] of every range z, for a consumer that
+// adds them itself in the order z = 0, 1, ...
+__global__ void __launch_bounds__(NT) gemm_partials_kernel(int M, int Ncol, int K, int kc, const float* __restrict__ A,
+                                                           int lda, const float* __restrict__ W, int ldw, float* part) {
+  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN, z = blockIdx.z;
+  float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+  gemm_tile<false>(m0, n0, M, Ncol, z * kc, min(K, (z + 1) * kc), A, lda, W, ldw, acc);
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int m = m0 + ty + 16 * r, n = n0 + 2 * tx + c;
+      if (m < M && n < Ncol) part[((size_t)z * M + m) * Ncol + n] = acc[r][c];
+    }
+}
+
 // Split-K forward GEMM: block z covers K range [z*kc, (z+1)*kc); partial sums go
 // to part[z][m][n]; the last block to finish a tile sums the partials in the
 // order z = 0, 1, ... and applies the epilogue, then re-arms the tile counter.
@@ -179,169 +213,47 @@ __device__ __forceinline__ void cta_finish(int b, double q, float* smem, const E
   }
 }
 
-// Shared-memory tile of the blocked conv passes: the weights, then the rows of
-// the operand plane that a band of outputs reads, zero outside the plane (a
-// tap there adds an exact zero to the chain), rows split by column phase for a
-// stride-2 forward pass so that consecutive outputs read consecutive words.
-struct ConvTile {
-  int bands, bh;        // bands of bh rows (transposed pass: rows of a stride phase)
-  int rows, pitch;      // staged rows per channel and their pitch (floats)
-  int y_off, x_off;     // plane row / column of the tile's first, relative to the band's first row * stride
-  int w_floats, wc;     // floats of the staged weights; transposed: channels per tap in them (cin padded to 4)
-  size_t smem;
-};
-
-__device__ __forceinline__ void stage16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void stage4(float* dst, const float* src, bool in) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-               "r"(in ? 4 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void stage_wait() {
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-}
-
 // Transposed conv, blocked (k4 s2 / k3 s1): a CTA takes one subdomain and a
-// band of positions of every stride phase; a thread one position of one phase
-// and G channels; g[b, c, yy, xx] = sum_{o,i,j} W[o,c,i,j] r[b, o, y, x] over
-// the taps of the phase, one chain of FMAs per output in the order (i, j, o).
-// Operands come from shared memory (direct global reads left each thread
-// waiting for one load per product: 12-14 us for 256 Base subdomains).
+// band of positions of every stride phase.  Operands come from shared memory
+// (direct global reads left each thread waiting for one load per product).
 template <int KH, int KW, int ST, int G, class Epi>
 __global__ void __launch_bounds__(NT) conv_t_fast_kernel(LayerDev L, ConvTile T, const float* __restrict__ r, int rs,
                                                          Epi epi) {
   extern __shared__ __align__(16) float sm[];
-  float* sR = sm + T.w_floats;
-  const int b = blockIdx.x / T.bands, band = blockIdx.x % T.bands;
-  const int qh = L.h / ST, qw = L.w / ST, ncg = L.cin / G, hw_o = L.ho * L.wo;
-  const int q0 = band * T.bh, nq = min(T.bh, qh - q0);
-  const int nw = L.cout * L.cin * KH * KW;
-  if (T.wc == L.cin) {
-    for (int e = threadIdx.x; e < nw / 4; e += NT) stage16(sm + 4 * e, L.Wt + 4 * e);
-    for (int e = (nw & ~3) + threadIdx.x; e < nw; e += NT) stage4(sm + e, L.Wt + e, true);
-  } else {
-    for (int e = threadIdx.x; e < nw; e += NT) stage4(sm + e / L.cin * T.wc + e % L.cin, L.Wt + e, true);
-  }
-  const float* rb = r + (size_t)b * rs;
-  const int plane = T.rows * T.pitch, n = L.cout * plane;
-  for (int e = threadIdx.x; e < n; e += NT) {
-    const int o = e / plane, rem = e - o * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
-    const int y = q0 + yy + T.y_off, x = xx + T.x_off;
-    const bool in = y >= 0 && y < L.ho && x >= 0 && x < L.wo;
-    stage4(sR + e, rb + (in ? o * hw_o + y * L.wo + x : 0), in);
-  }
+  const int b = blockIdx.x / T.bands, q0 = (blockIdx.x % T.bands) * T.bh, nq = min(T.bh, L.h / ST - q0);
+  conv_t_weights(L, T, sm, NT);
+  conv_t_rows(L, T, sm + T.w_floats, r + (size_t)b * rs, q0, NT);
   stage_wait();
-  const int items = ST * ST * ncg * nq * qw;
-  for (int e = threadIdx.x; e < items; e += NT) {
-    int q = e;
-    const int rx = q % ST;
-    q /= ST;
-    const int qx = q % qw;
-    q /= qw;
-    const int qy = q % nq;
-    q /= nq;
-    const int ry = q % ST;
-    const int cg = q / ST;
-    const int i0 = (ry + L.pad) % ST, j0 = (rx + L.pad) % ST;
-    const int dy0 = (ry + L.pad - i0) / ST, dx0 = (rx + L.pad - j0) / ST;
-    float acc[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) acc[g] = 0.f;
-    const float* rp = sR + (qy + dy0 - T.y_off) * T.pitch + qx + dx0 - T.x_off;
-    const float* wp = sm + (i0 * KW + j0) * T.wc + cg * G;
-#pragma unroll
-    for (int a = 0; a < KH / ST; ++a)
-#pragma unroll
-      for (int bb = 0; bb < KW / ST; ++bb) {
-        const float* ra = rp - a * T.pitch - bb;
-        const float* wa = wp + (ST * a * KW + ST * bb) * T.wc;
-#pragma unroll 8
-        for (int o = 0; o < L.cout; ++o) {
-          const float rv = ra[o * plane];
-          const float4 w = *reinterpret_cast<const float4*>(wa + o * KH * KW * T.wc);
-          acc[0] = fmaf(w.x, rv, acc[0]);
-          acc[1] = fmaf(w.y, rv, acc[1]);
-          acc[2] = fmaf(w.z, rv, acc[2]);
-          if (G == 4) acc[G - 1] = fmaf(w.w, rv, acc[G - 1]);
-        }
-      }
-    const int yy = ry + ST * (q0 + qy), xx = rx + ST * qx;
-#pragma unroll
-    for (int g = 0; g < G; ++g) epi(b, ((cg * G + g) * L.h + yy) * L.w + xx, acc[g]);
-  }
+  conv_t_items<KH, KW, ST, G>(L, T, sm, sm + T.w_floats, q0, nq, NT,
+                              [&](int c, int y, int x, float g) { epi(b, (c * L.h + y) * L.w + x, g); });
 }
 
 // Forward conv, blocked (k4 s2 / k3 s1): a CTA takes one subdomain and a band
-// of output rows; a thread one output position and GF output channels, one
-// chain of FMAs per output in the order (c, i, j).
+// of output rows.
 template <int KH, int KW, int ST, int GF, class Epi>
 __global__ void __launch_bounds__(NT) conv_fwd_fast_kernel(LayerDev L, ConvTile T, const float* __restrict__ x, int xs,
                                                            Epi epi) {
   extern __shared__ __align__(16) float sm[];
   float* sX = sm + T.w_floats;
-  const int b = blockIdx.x / T.bands, band = blockIdx.x % T.bands;
-  const int y0 = band * T.bh, ny = min(T.bh, L.ho - y0);
-  const int nw = L.cout * L.cin * KH * KW;
-  for (int e = threadIdx.x; e < nw / 4; e += NT) stage16(sm + 4 * e, L.Wf + 4 * e);
-  for (int e = (nw & ~3) + threadIdx.x; e < nw; e += NT) stage4(sm + e, L.Wf + e, true);
+  const int b = blockIdx.x / T.bands, y0 = (blockIdx.x % T.bands) * T.bh, ny = min(T.bh, L.ho - y0);
+  stage_floats(sm, L.Wf, L.cout * L.cin * KH * KW, NT);
   const float* xb = x + (size_t)b * xs;
-  const int hw_o = L.ho * L.wo, hw_i = L.h * L.w, half = T.pitch / ST;
-  const int plane = T.rows * T.pitch, n = L.cin * plane;
+  const int hw_i = L.h * L.w, plane = T.rows * T.pitch, n = L.cin * plane;
   for (int e = threadIdx.x; e < n; e += NT) {
     const int c = e / plane, rem = e - c * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
     const int y = y0 * ST + yy + T.y_off, xi = xx + T.x_off;
     const bool in = y >= 0 && y < L.h && xi >= 0 && xi < L.w;
-    // column xx of the padded row: phase xx % ST, place xx / ST
-    stage4(sX + c * plane + yy * T.pitch + (xx % ST) * half + xx / ST, xb + (in ? c * hw_i + y * L.w + xi : 0), in);
+    stage4(sX + conv_f_at(T, ST, c, yy, xx), xb + (in ? c * hw_i + y * L.w + xi : 0), in);
   }
   stage_wait();
-  const int nog = L.cout / GF, items = nog * ny * L.wo;
   double q = 0.0;
-  for (int e = threadIdx.x; e < items; e += NT) {
-    int r = e;
-    const int xo = r % L.wo;
-    r /= L.wo;
-    const int yo = r % ny;
-    const int og = r / ny;
-    float acc[GF];
-#pragma unroll
-    for (int g = 0; g < GF; ++g) acc[g] = 0.f;
-    const float* xc = sX + yo * ST * T.pitch + xo;
-    const float* wc = sm + og * GF;
-#pragma unroll 2
-    for (int c = 0; c < L.cin; ++c, xc += plane, wc += KH * KW * L.cout) {
-#pragma unroll
-      for (int i = 0; i < KH; ++i)
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-          const float xv = xc[i * T.pitch + (j % ST) * half + j / ST];
-          const float* w = wc + (i * KW + j) * L.cout;
-          if (GF == 4) {
-            const float4 w4 = *reinterpret_cast<const float4*>(w);
-            acc[0] = fmaf(w4.x, xv, acc[0]);
-            acc[1] = fmaf(w4.y, xv, acc[1]);
-            acc[GF - 2] = fmaf(w4.z, xv, acc[GF - 2]);
-            acc[GF - 1] = fmaf(w4.w, xv, acc[GF - 1]);
-          } else {
-            const float2 w2 = *reinterpret_cast<const float2*>(w);
-            acc[0] = fmaf(w2.x, xv, acc[0]);
-            acc[1] = fmaf(w2.y, xv, acc[1]);
-          }
-        }
-    }
-#pragma unroll
-    for (int g = 0; g < GF; ++g) {
-      const int i = (og * GF + g) * hw_o + (y0 + yo) * L.wo + xo;
-      if constexpr (Epi::kReduce)
-        q += epi(b, i, acc[g]);
-      else
-        epi(b, i, acc[g]);
-    }
-  }
+  conv_f_items<KH, KW, ST, GF>(L, T, sm, sX, y0, ny, NT, [&](int o, int y, int xo, float acc) {
+    const int i = (o * L.ho + y) * L.wo + xo;
+    if constexpr (Epi::kReduce)
+      q += epi(b, i, acc);
+    else
+      epi(b, i, acc);
+  });
   cta_finish(b, q, sm, epi);
 }
 
@@ -463,12 +375,6 @@ inline int grid1d(size_t total, int nt = NT) {
   return (int)(g > 65535 * 8 ? 65535 * 8 : (g < 1 ? 1 : g));
 }
 
-inline int conv_geo(const LayerDev& L) {
-  if (L.kh == 4 && L.kw == 4 && L.stride == 2) return 1;
-  if (L.kh == 3 && L.kw == 3 && L.stride == 1) return 2;
-  return 0;
-}
-
 // Shared memory of a blocked conv CTA: two of them still share an SM.
 constexpr size_t kConvSmem = 96 * 1024;
 
@@ -502,23 +408,13 @@ void transposed(const LayerDev& L, const Problem& P, const float* rho, Epi epi, 
     return;
   }
   const size_t smem = sizeof(float) * L.cout * L.cin * L.kh * L.kw;
-  const int geo = conv_geo(L);
-  const int st = L.stride;
-  if (geo && L.h % st == 0 && L.w % st == 0 && L.Wt && (L.cin % 4 == 0 || L.cin == 3)) {
-    const int G = L.cin == 3 ? 3 : 4;
-    // rows / columns of r around a position's own: taps reach dy0 - (k/s - 1) .. dy0
-    const int dlo = L.pad / st - (L.kh / st - 1), dhi = (st - 1 + L.pad) / st;
-    const int nt = st * st * (L.cin / G) * (L.w / st);  // items of one row
-    ConvTile T{};
-    T.wc = (L.cin + 3) & ~3;
-    T.w_floats = L.cout * L.kh * L.kw * T.wc;
-    T.y_off = T.x_off = dlo;
-    T.pitch = L.w / st + dhi - dlo;
-    T.bh = conv_band(L.h / st, nt, P.B, sizeof(float) * T.w_floats, sizeof(float) * L.cout * T.pitch, 1, dhi - dlo);
-    if (T.bh > 0) {
-      T.bands = (L.h / st + T.bh - 1) / T.bh;
-      T.rows = T.bh + dhi - dlo;
-      T.smem = sizeof(float) * ((size_t)T.w_floats + (size_t)L.cout * T.rows * T.pitch);
+  if (conv_t_covers(L)) {
+    const int geo = conv_geo(L), st = L.stride, G = L.cin == 3 ? 3 : 4;
+    const ConvTile T0 = conv_t_tile(L, 0);
+    const int bh = conv_band(L.h / st, st * st * (L.cin / G) * (L.w / st), P.B, sizeof(float) * T0.w_floats,
+                             sizeof(float) * L.cout * T0.pitch, 1, T0.rows);
+    if (bh > 0) {
+      const ConvTile T = conv_t_tile(L, bh);
       const unsigned grid = (unsigned)P.B * T.bands;
       if (geo == 1) {
         if (G == 3)
@@ -545,20 +441,12 @@ void forward(const LayerDev& L, const Problem& P, const float* x, Epi epi, cudaS
   const float* xin = x + L.x_in_off;
   if (L.kind == LD_LAYER_FC) {
     const int tiles_n = (L.n_out + TN - 1) / TN, tiles_m = (P.B + TM - 1) / TM;
-    // split K until the grid covers the GPU about twice (304 blocks)
-    int splits = (304 + tiles_n * tiles_m - 1) / (tiles_n * tiles_m);
-    const int kmax = (L.n_in + 63) / 64;
-    if (splits > kmax) splits = kmax;
-    if (splits > 16) splits = 16;
-    if (!P.splitk_part || (size_t)splits * P.B * L.n_out > (size_t)P.splitk_part_cap ||
-        tiles_n * tiles_m > P.splitk_count_cap)
-      splits = 1;
+    int splits, kc;
+    split_of(L, P, splits, kc);
     if (splits <= 1) {
       dim3 grid(tiles_n, tiles_m);
       gemm_kernel<false, Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, xin, P.XS, L.W, L.n_in, epi);
     } else {
-      const int kc = ((L.n_in + splits - 1) / splits + kSplitStep - 1) / kSplitStep * kSplitStep;
-      splits = (L.n_in + kc - 1) / kc;
       dim3 grid(tiles_n, tiles_m, splits);
       gemm_splitk_kernel<Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, kc, xin, P.XS, L.W, L.n_in, P.splitk_part,
                                                   P.splitk_count, epi);
@@ -566,20 +454,14 @@ void forward(const LayerDev& L, const Problem& P, const float* x, Epi epi, cudaS
     return;
   }
   const size_t smem = std::max(sizeof(float) * L.cout * L.cin * L.kh * L.kw, Epi::kReduce ? kFinishSmem : 0);
-  const int geo = conv_geo(L);
-  if (geo && L.Wf && L.cout % 2 == 0) {
-    const int st = L.stride, GF = L.cout % 4 == 0 ? 4 : 2;
-    ConvTile T{};
-    T.w_floats = (L.cout * L.cin * L.kh * L.kw + 3) & ~3;
-    T.y_off = T.x_off = -L.pad;
-    T.pitch = ((L.wo - 1) * st + L.kw + st - 1) / st * st;
-    T.bh = conv_band(L.ho, (L.cout / GF) * L.wo, P.B, sizeof(float) * T.w_floats, sizeof(float) * L.cin * T.pitch, st,
-                     L.kh - st);
-    if (T.bh > 0) {
-      T.bands = (L.ho + T.bh - 1) / T.bh;
-      T.rows = T.bh * st + L.kh - st;
-      T.smem = std::max(sizeof(float) * ((size_t)T.w_floats + (size_t)L.cin * T.rows * T.pitch),
-                        Epi::kReduce ? kFinishSmem : 0);
+  if (conv_f_covers(L)) {
+    const int geo = conv_geo(L), st = L.stride, GF = L.cout % 4 == 0 ? 4 : 2;
+    const ConvTile T0 = conv_f_tile(L, 0);
+    const int bh = conv_band(L.ho, (L.cout / GF) * L.wo, P.B, sizeof(float) * T0.w_floats,
+                             sizeof(float) * L.cin * T0.pitch, st, T0.rows);
+    if (bh > 0) {
+      ConvTile T = conv_f_tile(L, bh);
+      if (Epi::kReduce) T.smem = std::max(T.smem, kFinishSmem);
       const unsigned grid = (unsigned)P.B * T.bands;
       if (geo == 1) {
         if (GF == 4)
@@ -633,6 +515,22 @@ void launch_forward_record(const LayerDev& L, const Problem& P, const float* x, 
 
 void launch_forward_store(const LayerDev& L, const Problem& P, const float* x, EpiStore epi, cudaStream_t s) {
   forward(L, P, x, epi, s);
+}
+
+SplitK forward_split(const LayerDev& L, const Problem& P) {
+  SplitK k{};
+  split_of(L, P, k.splits, k.kc);
+  return k;
+}
+
+bool launch_forward_partials(const LayerDev& L, const Problem& P, const float* x, SplitK& k, cudaStream_t s) {
+  k = forward_split(L, P);
+  if (!P.splitk_part || (size_t)k.splits * P.B * L.n_out > (size_t)P.splitk_part_cap) return false;
+  count_launch();
+  dim3 grid((L.n_out + TN - 1) / TN, (P.B + TM - 1) / TM, k.splits);
+  gemm_partials_kernel<<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, k.kc, x + L.x_in_off, P.XS, L.W, L.n_in,
+                                           P.splitk_part);
+  return true;
 }
 
 void launch_transposed_scores(const LayerDev& L, const Problem& P, const float* mu, EpiScores epi, cudaStream_t s) {
