@@ -493,6 +493,12 @@ bool fused_ball_fits(const FusedNet& f, int code);
 cudaError_t launch_fused(const FusedNet& f, int code, const Problem& P, float* rho, float* m, float* v,
                          const FusedIter& it, cudaStream_t s);
 
+// The same launch for nets of FC layers whose weights fit in shared memory
+// (ld_mlp.cu): bitwise the results of the launch shape `code`.
+bool mlp_covers(const FusedNet& f);
+cudaError_t launch_mlp(const FusedNet& f, int code, const Problem& P, float* rho, float* m, float* v,
+                       const FusedIter& it, cudaStream_t s);
+
 // ---------------------------------------------------------------- fused tensor-core engine
 // The fused engine with its conv passes on the tensor cores (ld_fused_tc.cu):
 // every conv pass is an implicit GEMM D[rows, N] = A[rows, K] B[N, K]^T read
