@@ -368,20 +368,24 @@ ld::AdamStep adam_step(const ld_opts& o, int tt, int T_sched) {
 bool tile_fits(const ld_net* net, int code) { return ld::fused_smem_bytes(net->fused, code) <= net->smem_optin; }
 
 // Threads of a fused CTA that run the FC passes of an iteration while the
-// others run the conv passes: half the CTA when the net has both kinds of
-// hidden layer (measured on the Base, Wide and Deep nets: 2-11% faster than
-// every pass on all threads; unequal splits leave items unevenly spread and
-// are slower), else none.
+// others run the conv passes, when the net has both kinds of hidden layer
+// (else 0): half the CTA, or a quarter of a 512-thread CTA of one subdomain
+// where the convs have at least kConvHeavy times the products of the FC layers
+// (Deep 8.9: 1024 subdomains, T = 50, 13.53 -> 12.37 ms; Wide 3.5 and Base 2.2
+// keep half: their FC passes are the longer ones with fewer threads).
 int fused_fc_threads(const ld_net* net, int code) {
-  bool fc = false, conv = false;
+  constexpr double kConvHeavy = 6.0;
+  double fc = 0, conv = 0;
   for (int k = 0; k + 1 < net->n; ++k) {
-    if (net->L[k].kind == LD_LAYER_FC)
-      fc = true;
+    const LayerDev& L = net->L[k];
+    if (L.kind == LD_LAYER_FC)
+      fc += (double)L.n_in * L.n_out;
     else
-      conv = true;
+      conv += (double)L.cin * L.kh * L.kw * L.n_out;
   }
-  if (!fc || !conv) return 0;
-  return ((code & ld::kFusedWide) ? 512 : 256) / 2;
+  if (fc == 0 || conv == 0) return 0;
+  if (!(code & ld::kFusedWide)) return 128;
+  return (code & ~ld::kFusedWide) == 1 && conv >= kConvHeavy * fc ? 128 : 256;
 }
 
 // T Adam iterations with the given engine (tile = subdomains per CTA).

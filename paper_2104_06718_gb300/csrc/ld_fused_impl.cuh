@@ -78,10 +78,19 @@ __device__ __forceinline__ IntDiv int_div(int d) { return IntDiv{d, (d & (d - 1)
 __device__ __forceinline__ int div_of(int n, const IntDiv& v) { return v.sh >= 0 ? n >> v.sh : n / v.d; }
 
 // The threads a pass is spread over: this thread's index in the group (-1:
-// not a member) and the group's size (a multiple of 32).
+// not a member) and the group's size (a multiple of 32); split_n: the size by
+// which transposed FC passes decide whether to sum their rows in two halves
+// (a smaller group forms both halves in one thread, with the same sums).
 struct Team {
-  int tid, n;
+  int tid, n, split_n;
 };
+
+// Whether the kernel may run with an FC group smaller than half the CTA (one
+// subdomain per CTA; the code costs the two-subdomain kernel 2%).
+template <int S, bool TC>
+__host__ __device__ constexpr bool quarter_fc() { return S == 1 && !TC; }
+template <int S, bool TC>
+__device__ __forceinline__ int split_size(const Team& tm) { return quarter_fc<S, TC>() ? tm.split_n : tm.n; }
 
 // Barrier over the n threads (whole warps) that execute it with this id
 // (id 0 is __syncthreads).
@@ -378,6 +387,12 @@ __device__ __forceinline__ void tfc_bounds(const Ctx<S, NT, TC>& c, int k, int s
   }
 }
 
+// Whether the pass has a second part after a barrier (tfc_finish).
+template <int S, bool TC>
+__device__ __forceinline__ bool tfc_two_part(const LayerDev& L, const FusedLayer& F, const Team& tm) {
+  return tm.n >= split_size<S, TC>(tm) && tfc_split(L, F, split_size<S, TC>(tm));
+}
+
 // Main part of the transposed FC pass.  Unsplit: the whole pass.  Split:
 // each half streams its rows and publishes its partial sums (slot = half);
 // tfc_finish adds the two slots and runs the epilogue once both are written.
@@ -386,12 +401,28 @@ __device__ void tfc_main(const Ctx<S, NT, TC>& c, const LayerDev& L, const Fused
   const float* __restrict__ W = L.W;
   constexpr int U = tfc_batch_rows<S, TC>();
   if (tm.tid < 0) return;
-  if (tfc_split(L, F, tm.n)) {
+  if (tfc_split(L, F, split_size<S, TC>(tm))) {
     const int n4 = L.n_in / 4, half = tm.n / 2;
+    const int nbat = (L.n_out + U - 1) / U, mid = (nbat + 1) / 2;
+    if (quarter_fc<S, TC>() && tm.n < tm.split_n) {
+      for (int i4 = tm.tid; i4 < n4; i4 += tm.n) {
+        float4 acc[S], hi[S];
+        tfc_rows(c, L, F, i4, 0, mid, acc);
+        tfc_rows(c, L, F, i4, mid, nbat, hi);
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          if (!active(c, s)) continue;
+          float l[4], u[4];
+          tfc_bounds(c, k, s, i4, l, u);
+          tfc_epi(c, F, k, s, i4,
+                  make_float4(acc[s].x + hi[s].x, acc[s].y + hi[s].y, acc[s].z + hi[s].z, acc[s].w + hi[s].w), l, u);
+        }
+      }
+      return;
+    }
     const int part = tm.tid >= half ? 1 : 0;
     const int i4 = tm.tid - part * half;
     if (i4 >= n4) return;
-    const int nbat = (L.n_out + U - 1) / U, mid = (nbat + 1) / 2;
     float4 acc[S];
     tfc_rows(c, L, F, i4, part ? mid : 0, part ? nbat : mid, acc);
     float4* X = reinterpret_cast<float4*>(red_of(c, k)) + part * S * n4;  // slot [part][S][n4]
@@ -441,7 +472,7 @@ __device__ void tfc_main(const Ctx<S, NT, TC>& c, const LayerDev& L, const Fused
 // subdomains s with s % 2 == p (all of them for S = 1) from slot 0 + slot 1.
 template <int S, int NT, bool TC>
 __device__ void tfc_finish(const Ctx<S, NT, TC>& c, const LayerDev& L, const FusedLayer& F, int k, const Team& tm) {
-  if (tm.tid < 0 || !tfc_split(L, F, tm.n)) return;
+  if (tm.tid < 0 || !tfc_two_part<S, TC>(L, F, tm)) return;
   const int n4 = L.n_in / 4, half = tm.n / 2;
   const int part = tm.tid >= half ? 1 : 0;
   const int i4 = tm.tid - part * half;
@@ -463,7 +494,7 @@ __device__ void tfc_finish(const Ctx<S, NT, TC>& c, const LayerDev& L, const Fus
 template <int S, int NT, bool TC>
 __device__ void transposed_fc(const Ctx<S, NT, TC>& c, const LayerDev& L, const FusedLayer& F, int k, const Team& tm) {
   tfc_main(c, L, F, k, tm);
-  if (tfc_split(L, F, tm.n)) {
+  if (tfc_two_part<S, TC>(L, F, tm)) {
     __syncthreads();
     tfc_finish(c, L, F, k, tm);
   }
@@ -788,15 +819,44 @@ __device__ void conv_t_generic(const Ctx<S, NT, TC>& c, const LayerDev& L, const
   }
 }
 
+// Whether a blocked forward conv takes four channels per item (enough items for the
+// group, or with one subdomain per CTA for half the CTA), else two.
+template <int S, int NT, bool TC>
+__device__ __forceinline__ bool conv_fwd_by4(const LayerDev& L, const Team& tm) {
+  return S * (L.ho / 2) * L.wo * (L.cout / 4) >= (quarter_fc<S, TC>() ? NT / 2 : tm.n);
+}
+
+// The conv group's threads for the next pass of a phase: pass after pass, its
+// items start where the last pass's ended, so that a group of more threads
+// than a pass has items still shares the phase's work evenly.
+struct Turn {
+  int next;  // first thread of the next pass
+  __device__ __forceinline__ Team team(const Team& tm, int items) {
+    if (tm.tid < 0) return tm;
+    int t = tm.tid - next;
+    if (t < 0) t += tm.n;
+    next = (next + ((items + 31) & ~31)) % tm.n;
+    return Team{t, tm.n, tm.split_n};
+  }
+};
+template <int S>
+__device__ __forceinline__ int conv_t_count(const LayerDev& L, const FusedLayer& F) {
+  return F.tmode ? S * (L.h / 2) * L.w * (L.cin == 3 ? 1 : L.cin / 4) : L.cin * L.h * L.w;
+}
+template <int S, int NT, bool TC>
+__device__ __forceinline__ int conv_f_count(const LayerDev& L, const FusedLayer& F, const Team& tm) {
+  return F.fmode ? S * (L.ho / 2) * L.wo * (L.cout / (conv_fwd_by4<S, NT, TC>(L, tm) ? 4 : 2)) : L.cout * L.ho * L.wo;
+}
+
 // Forward conv pass of layer L = layer k+1, with the Adam epilogue.
 template <int S, int NT, bool TC>
 __device__ void forward_conv(const Ctx<S, NT, TC>& c, const LayerDev& L, const FusedLayer& F, const FusedIter& it,
                              const AdamStep& st, const Team& tm) {
-  if (F.fmode == 1 && S * (L.ho / 2) * L.wo * (L.cout / 4) >= tm.n)
+  if (F.fmode == 1 && conv_fwd_by4<S, NT, TC>(L, tm))
     conv_fwd_blocked<4, 4, 2, 4>(c, L, F, it, st, tm);
   else if (F.fmode == 1)  // too few 4-channel items to fill the group
     conv_fwd_blocked<4, 4, 2, 2>(c, L, F, it, st, tm);
-  else if (F.fmode == 2 && S * (L.ho / 2) * L.wo * (L.cout / 4) >= tm.n)
+  else if (F.fmode == 2 && conv_fwd_by4<S, NT, TC>(L, tm))
     conv_fwd_blocked<3, 3, 1, 4>(c, L, F, it, st, tm);
   else if (F.fmode == 2)
     conv_fwd_blocked<3, 3, 1, 2>(c, L, F, it, st, tm);
@@ -1227,9 +1287,9 @@ __global__ void __launch_bounds__(NT) fused_kernel(const __grid_constant__ Fused
   // The FC passes of the iterations run on the first fc_threads threads and
   // the conv passes on the rest, side by side (0: every pass on all threads).
   const int nf = it.fc_threads;
-  const Team all{(int)threadIdx.x, NT};
-  const Team tf = nf ? Team{(int)threadIdx.x < nf ? (int)threadIdx.x : -1, nf} : all;
-  const Team tc = nf ? Team{(int)threadIdx.x >= nf ? (int)threadIdx.x - nf : -1, NT - nf} : all;
+  const Team all{(int)threadIdx.x, NT, NT};
+  const Team tf = nf ? Team{(int)threadIdx.x < nf ? (int)threadIdx.x : -1, nf, NT / 2} : all;
+  const Team tc = nf ? Team{(int)threadIdx.x >= nf ? (int)threadIdx.x - nf : -1, NT - nf, NT - nf} : all;
   if (it.crown) {
     // The CROWN start sets rho_k = g_k exactly for passing ReLUs; those ties
     // survive only if the iterations compute g_k with the same sums, so each
@@ -1263,7 +1323,7 @@ __global__ void __launch_bounds__(NT) fused_kernel(const __grid_constant__ Fused
   for (int k = 0; k + 1 < net.n; ++k)
     if (net.L[k].kind == LD_LAYER_FC) {
       any_fc = true;
-      any_split = any_split || tfc_split(net.L[k], net.F[k], tf.n);
+      any_split = any_split || tfc_two_part<S, TC>(net.L[k], net.F[k], tf);
     }
   // One iteration in two phases.  Every transposed pass (and the top
   // subproblem) reads only rho of the previous iteration and writes its own
@@ -1294,8 +1354,11 @@ __global__ void __launch_bounds__(NT) fused_kernel(const __grid_constant__ Fused
           tc_issue(tcp, tcp.t0, tcp.nt, tc.tid / 32, tcp.issuers, false);
         tc_epilogues(c, tcp.t0, tcp.nt, (uint32_t)(t & 1), tc.tid / 32, it, st);
       } else {
+        Turn turn{0};
         for (int k = net.n - 2; k >= 0; --k)
-          if (net.L[k].kind != LD_LAYER_FC) transposed_pass(c, net.L[k], net.F[k], k, tc);
+          if (net.L[k].kind != LD_LAYER_FC)
+            transposed_pass(c, net.L[k], net.F[k], k,
+                            quarter_fc<S, TC>() ? turn.team(tc, conv_t_count<S>(net.L[k], net.F[k])) : tc);
       }
     } else {
       top_pass(c, all);
@@ -1321,8 +1384,11 @@ __global__ void __launch_bounds__(NT) fused_kernel(const __grid_constant__ Fused
         tc_issue(tcp, tcp.f0, tcp.nf, tc.tid / 32, tcp.issuers, false);
       if (tc.tid >= 0) tc_epilogues(c, tcp.f0, tcp.nf, (uint32_t)(t & 1), tc.tid / 32, it, st);
     } else {
+      Turn turn{0};
       for (int k = net.n - 2; k >= 0; --k)
-        if (net.L[k].kind != LD_LAYER_FC) forward_conv(c, net.L[k], net.F[k], it, st, tc);
+        if (net.L[k].kind != LD_LAYER_FC)
+          forward_conv(c, net.L[k], net.F[k], it, st,
+                       quarter_fc<S, TC>() ? turn.team(tc, conv_f_count<S, NT, TC>(net.L[k], net.F[k], tc)) : tc);
     }
     if (!nf && any_fc) {
       __syncthreads();
