@@ -6,47 +6,79 @@
 //   q(rho) = sum_j min_{x0_j in [l0_j,u0_j]} (-g_0[j] x0_j)                    (P0)
 //          + sum_{k=1}^{n-1} sum_i min_{vertices of P_k} (rho_k[i] xB - g_k[i] x) (Pk)
 //          - sum_{k=1}^{n-1} rho_k^T b_k + b_n
-// so the final bound needs only the transposed pass.  Each g_k is summed in
-// FP64 from the FP32 weights and duals (the products are exact in FP64); an
-// upper bound A_i >= sum |W||rho| is summed alongside in FP32 rounded up,
-// which bounds the FP64 summation error by delta_i = gamma_K A_i (Higham,
-// gamma_K = K u / (1 - K u), u = 2^-53).  Every term's value t and an upper
+// so the final bound needs only the transposed pass.  The FP64 pipe of GB300
+// runs 2 operations per clock and SM against 128 FP32 ones, so g_k is summed in
+// FP32 to more than FP64 precision: every product is an exact FP32 pair (FMA),
+// and the pairs are summed on three levels.  Level 1 starts at 1.5 2^a with
+// 2^(a-2) > sum |W||rho| (formed first, rounded up), so that its partial sums
+// keep one exponent, every rounding error is exact and at most 2^(a-24)
+// (Fast2Sum; the extraction sums of Rump, Ogita and Oishi's AccSum); those
+// errors and the products' low parts of a block of k = 64 terms go to level 2,
+// started at 1.5 2^b with 2^(b-1) >= (k + 1) 2^(a-24), whose errors, at most
+// 2^(b-24) each, level 3 sums plainly; levels 2 and 3 are added in FP64 after
+// each block.  So |g - exact| <= delta = (k + k^2) 2^(b-47) a block + 2^-52 |g|,
+// below 2^-48 sum|W||rho| a block, where an FP64 sum has the bound gamma_k =
+// 2^-47 sum|W||rho| for 64 terms.  15 FP32 operations a term take the place of
+// one FP64 one (64 FP32 slots).  Geometries without a blocked path
+// sum in FP64 (the products are exact there) with delta = gamma_K A_i,
+// A_i >= sum |W||rho| in FP32 rounded up (Higham, gamma_K = K u / (1 - K u),
+// u = 2^-53).  Every term's value t and an upper
 // bound e on its error (from delta_i and the rounding of one subtraction and
 // one product) are summed per subdomain; the bound returned is
 //   S - E - gamma_M * sum|t|   (S = sum t, E = sum e, M = number of terms),
-// with E and sum|t| summed rounding upward and scaled by 1 + 2 gamma_M as a
+// with t and S in FP64, and E and sum|t| summed (in FP32 within a block) rounding upward and scaled by 1 + 2 gamma_M as a
 // margin.  Partial sums go to fixed slots that one kernel adds in a fixed
 // order, so the bound does not depend on the order in which blocks run.
-#include "ld_common.cuh"
+#include <cmath>
+
+#include "ld_conv.cuh"
 
 namespace ld {
 namespace {
 
-constexpr int BN = 64, BK = 16, NT = 256;
-constexpr double U52 = 2.220446049250313e-16;  // 2^-52
+constexpr int BN = 64, NT = 256;
+constexpr float kU52 = 2.220446049250313e-16f;  // 2^-52
 
-// Value and error bound of one per-neuron minimum.  box: P0 term with
-// coefficient -g on [l, u].  Otherwise the Pk neuron with rho r.
-__device__ __forceinline__ void final_term(bool box, double r, double g, double delta, double l, double u,
-                                           double& t, double& e) {
-  if (!box && u <= 0.0) {            // blocking: min r*xB over [l,u], exact products
-    t = fmin(r * l, r * u);
-    e = 0.0;
+// Sums of a thread's terms: values, error bounds (up), |values| (up).
+struct TermSum {
+  double t = 0.0;
+  float e = 0.f, a = 0.f;
+};
+
+// |x| rounded up to FP32, by integer instructions (at least 2^-126).
+__device__ __forceinline__ float abs_up(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+  if (hi < 0x38100000u) return hi | lo ? 1.1754943508222875e-38f : 0.f;
+  if (hi >= 0x47e00000u) return x != x ? (float)x : INFINITY;  // beyond FLT_MAX's binade, inf, NaN
+  return __uint_as_float(((hi - 0x38000000u) << 3 | lo >> 29) + 1u);
+}
+
+__device__ __forceinline__ void add_term(TermSum& s, double t, float e) {
+  s.t += t;
+  s.e = __fadd_ru(s.e, e);
+  s.a = __fadd_ru(s.a, abs_up(t));
+}
+
+// One per-neuron minimum, g within delta of the exact value.  box: P0 term
+// with coefficient -g on [l, u]; otherwise the Pk neuron with rho r.
+__device__ __forceinline__ void final_term(TermSum& s, bool box, float r, double g, float delta, float l, float u) {
+  if (!box && u <= 0.f) {             // blocking: min r*xB over [l,u], exact products
+    add_term(s, widen(r) * widen(r >= 0.f ? l : u), 0.f);
     return;
   }
-  const double d = box ? -g : r - g;  // coefficient of xB (and of x) in the box/passing/(u,u) cases
-  const double ad = fabs(d);
-  if (box || l >= 0.0) {              // P0 box, or passing: min d*xB over [l,u]
-    const double tl = d * l, tu = d * u;
-    t = fmin(tl, tu);
-    const double xm = fmax(fabs(l), fabs(u));
-    e = __dadd_ru(__dmul_ru(xm, __dadd_ru(delta, __dmul_ru(U52, ad))), __dmul_ru(U52, fmax(fabs(tl), fabs(tu))));
+  const double d = box ? -g : widen(r) - g;  // coefficient of xB (and of x) in the box/passing/(u,u) cases
+  const float ed = __fmaf_ru(kU52, abs_up(d), delta);
+  if (box || l >= 0.f) {              // P0 box, or passing: min d*xB over [l,u]
+    const double t = d * widen(d >= 0.0 ? l : u);
+    // within delta of d the other end may be the minimum: either product is then within |d|_up max|x| of 0
+    const float xm = fmaxf(fabsf(l), fabsf(u));
+    add_term(s, t, __fmaf_ru(xm, ed, __fmul_ru(kU52, abs_up(t))));
     return;
   }
   // ambiguous: vertices (l,0) -> r*l (exact), (0,0) -> 0, (u,u) -> d*u
-  const double tuu = d * u;
-  t = fmin(fmin(r * l, 0.0), tuu);
-  e = __dadd_ru(__dmul_ru(fabs(u), __dadd_ru(delta, __dmul_ru(U52, ad))), __dmul_ru(U52, fabs(tuu)));
+  const double tuu = d * widen(u);
+  add_term(s, fmin(fmin(widen(r) * widen(l), 0.0), tuu),
+           __fmaf_ru(fabsf(u), ed, __fmul_ru(kU52, abs_up(tuu))));
 }
 
 struct FinalEpi {
@@ -56,32 +88,125 @@ struct FinalEpi {
   const float* rho;
   double gamma_K;
   int ball_norm;       // layer 0, l2 ball: the term is an upper bound on g_0[i]^2 (for ||g_0||)
-  __device__ __forceinline__ void term(int b, int i, double g, float abs_sum, double& t, double& e) const {
-    term_delta(b, i, g, __dmul_ru(gamma_K, (double)abs_sum), t, e);
+  // abs_sum: bound on sum |W||rho| of an FP64 sum g
+  __device__ __forceinline__ void term(int b, int i, double g, float abs_sum, TermSum& s) const {
+    term_delta(b, i, g, __fmul_ru(__double2float_ru(gamma_K), abs_sum), s);
   }
   // delta: bound on |g - exact g|
-  __device__ __forceinline__ void term_delta(int b, int i, double g, double delta, double& t, double& e) const {
+  __device__ __forceinline__ void term_delta(int b, int i, double g, float delta, TermSum& s) const {
     if (layer == 0) {
       if (ball_norm) {
         // |exact g_0[i]| <= |g| + delta: its square, rounded up
-        const double a = __dadd_ru(fabs(g), delta);
-        t = __dmul_ru(a, a);
-        e = 0.0;
+        const double a = __dadd_ru(fabs(g), (double)delta);
+        add_term(s, __dmul_ru(a, a), 0.f);
         return;
       }
       // the box; over an l2 ball l0 = u0 = the centre, which gives the
       // -g_0^T c part of the ball's minimum (the -eps ||g_0|| part is added
       // by the ball pass)
       const int p = prop_of(P, b);
-      final_term(true, 0.0, g, delta, (double)P.l0[(size_t)p * P.n0 + i], (double)P.u0[(size_t)p * P.n0 + i], t, e);
+      final_term(s, true, 0.f, g, delta, P.l0[(size_t)p * P.n0 + i], P.u0[(size_t)p * P.n0 + i]);
       return;
     }
     const int j = r_off + i;
     float l, u;
     clamped_bounds(P, b, j, l, u);
-    final_term(false, (double)rho[(size_t)b * P.N + j], g, delta, (double)l, (double)u, t, e);
+    final_term(s, false, rho[(size_t)b * P.N + j], g, delta, l, u);
   }
 };
+
+// ---------------------------------------------------------------- three-level sums
+// b - a by one packed instruction (the product with -1 is exact).
+__device__ __forceinline__ float2 sub2(float2 b, float2 a) { return __ffma2_rn(a, make_float2(-1.f, -1.f), b); }
+
+// Two sums (packed) of products: start(), size(w, r) for every term, then
+// begin(K) and add(w, r) for every term again.
+constexpr int kBlk = 64;  // terms between two blocks
+struct Sum3x2 {
+  float2 p, q, c;      // levels 1 to 3; p holds the sum of sizes until begin()
+  double g0, g1;       // finished blocks
+  __device__ __forceinline__ void start() { p = make_float2(0.f, 0.f); }
+  __device__ __forceinline__ void size(float2 w, float2 r) {
+    const float2 h = __fmul2_rn(w, r);
+    p = make_float2(__fadd_ru(p.x, fabsf(h.x)), __fadd_ru(p.y, fabsf(h.y)));
+  }
+  // 2^a from the sum of |rounded products|: 2^(a-1) is more than twice the sum,
+  // which leaves room for the products' rounding and the level's own errors;
+  // sums below 2^-40 take that a (their errors are then far below any term's)
+  static __device__ __forceinline__ float top(float s) {
+    const unsigned e = __float_as_uint(fmaxf(s, 9.094947017729282e-13f)) & 0x7f800000u;
+    return __uint_as_float(e) * 8.f;
+  }
+  static __device__ __forceinline__ float binade(float p) { return __uint_as_float(__float_as_uint(p) & 0x7f800000u); }
+  __device__ __forceinline__ void begin(float lvl2) {
+    p = make_float2(1.5f * top(p.x), 1.5f * top(p.y));
+    q = make_float2(p.x * lvl2, p.y * lvl2);
+    c = make_float2(0.f, 0.f);
+    g0 = g1 = 0.0;
+  }
+  // Levels 2 and 3 of a finished block (at most kBlk terms) into FP64; 2^a is
+  // recovered from p, which lies in [2^a, 2^(a+1)).
+  __device__ __forceinline__ void block(float lvl2) {
+    const float2 z = make_float2(1.5f * binade(p.x) * lvl2, 1.5f * binade(p.y) * lvl2);
+    g0 += widen(q.x - z.x) + widen(c.x);
+    g1 += widen(q.y - z.y) + widen(c.y);
+    q = z;
+    c = make_float2(0.f, 0.f);
+  }
+  __device__ __forceinline__ void add(float2 w, float2 r, float2 nr) {
+    const float2 nh = __fmul2_rn(w, nr);
+    const float2 e = __ffma2_rn(w, r, nh);           // w r = -nh + e exactly
+    const float2 t = sub2(p, nh);
+    const float2 n1 = __fadd2_rn(nh, sub2(t, p));    // minus the error of t
+    p = t;
+    const float2 t2 = sub2(q, n1);
+    const float2 n2 = __fadd2_rn(n1, sub2(t2, q));   // minus the error of t2
+    const float2 t3 = __fadd2_rn(t2, e);
+    const float2 e3 = sub2(e, sub2(t3, t2));         // the error of t3
+    q = t3;
+    c = __fadd2_rn(c, sub2(e3, n2));
+  }
+  // Value and bound of half h after the last block.
+  __device__ __forceinline__ void result(int h, float kk, double& g, float& delta) const {
+    const float ph = h ? p.y : p.x, two_a = binade(ph);
+    if (!(two_a < 1.329227995784916e36f)) {          // sums beyond 2^117: no value, an infinite bound (NaN stays)
+      g = ph == ph ? 0.0 : (double)ph;
+      delta = INFINITY;
+      return;
+    }
+    g = widen(ph - 1.5f * two_a) + (h ? g1 : g0);
+    delta = __fmaf_ru(kk, two_a, __fmul_ru(kU52, abs_up(g)));
+  }
+};
+// 2^(b-a) of level 2, 2^(b-1) >= (k + 1) 2^(a-24) for blocks of at most k =
+// min(kBlk, K) terms, and blocks times (k + k^2) 2^(b-47-a).
+struct Sum3Const {
+  float lvl2, kk;
+};
+inline Sum3Const sum3_const(int blocks, int K) {
+  const int k = std::min(kBlk, K);
+  int cl = 0;
+  while ((1 << cl) < k + 1) ++cl;
+  Sum3Const s;
+  s.lvl2 = (float)std::ldexp(1.0, cl - 23);
+  s.kk = (float)(blocks * std::ldexp((double)k + (double)k * k, cl - 23 - 47) * (1.0 + 1e-6));
+  return s;
+}
+// Blocks of a conv sum: `taps` runs of cout terms (in pieces of kBlk), a new
+// block wherever the next run or piece would not fit (as final_conv_fast_kernel).
+inline int sum3_blocks(int taps, int cout) {
+  int blocks = 1, cnt = 0;
+  for (int t = 0; t < taps; ++t)
+    for (int o = 0; o < cout; o += kBlk) {
+      const int n = std::min(kBlk, cout - o);
+      if (cnt + n > kBlk) {
+        ++blocks;
+        cnt = 0;
+      }
+      cnt += n;
+    }
+  return blocks;
+}
 
 // Each (subdomain, slot) partial is written exactly once and the slots are
 // summed in a fixed order by the combine kernel: the final bound does not
@@ -93,124 +218,132 @@ __device__ __forceinline__ void acc_add(FinalAcc a, int slot, int b, double t, d
   p[2] = at;
 }
 
-// FP64 transposed FC pass (A = rho_{k+1} [B, n_out], W [n_out, n_in]).
-// Tile: BM = 16 TM subdomains x BN = 64 columns (TM = 4, or 1 when the
+// Transposed FC pass (A = rho_{k+1} [B, n_out], W [n_out, n_in]) in three-level
+// sums.  Tile: BM = 16 TM subdomains x BN = 64 columns (TM = 4, or 1 when the
 // 64-row grid would leave SMs idle; the column blocks, and so the partial-sum
-// slots, are the same either way).  The operands are converted to double once
-// when a tile is staged (the FP64 pipe is GB300's scarce unit), and their
-// magnitudes kept as floats for the FP32 round-up sum of |W||rho|.
+// slots, are the same either way), a thread TM x 4 of it; up to KS rows of K
+// staged at once.
+constexpr int KS = 128;
 template <int TM>
 __global__ void __launch_bounds__(NT) final_fc_kernel(int M, int Ncol, int K, const float* __restrict__ A, int lda,
                                                       const float* __restrict__ W, int ldw, FinalEpi epi,
-                                                      FinalAcc acc_out) {
+                                                      Sum3Const sc, FinalAcc acc_out) {
   constexpr int BMt = 16 * TM;
-  __shared__ double As[BK][BMt + 1];
-  __shared__ double Bs[BK][BN + 1];
-  __shared__ float Aa[BK][BMt + 4];
-  __shared__ float Ba[BK][BN + 4];
+  extern __shared__ __align__(16) float sm[];
+  float* As = sm;                      // [k][BMt + 1]
+  float* Bs = As + KS * (BMt + 1) + (4 - (KS * (BMt + 1)) % 4) % 4;  // [k][BN]
   const int t = threadIdx.x, tx = t % 16, ty = t / 16;
   const int m0 = blockIdx.y * BMt, n0 = blockIdx.x * BN;
-  double acc[TM][4];
-  float aab[TM][4];
+  Sum3x2 acc[TM][2];
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      acc[i][j] = 0.0;
-      aab[i][j] = 0.f;
-    }
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    for (int idx = t; idx < BMt * BK; idx += NT) {
-      const int mm = idx / BK, kk = idx % BK;
-      const int gm = m0 + mm, gk = k0 + kk;
-      const float v = (gm < M && gk < K) ? A[(size_t)gm * lda + gk] : 0.f;
-      As[kk][mm] = (double)v;
-      Aa[kk][mm] = fabsf(v);
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int idx = t + e * NT;
-      const int kk = idx / BN, nn = idx % BN;
-      const int gk = k0 + kk, gn = n0 + nn;
-      const float v = (gk < K && gn < Ncol) ? W[(size_t)gk * ldw + gn] : 0.f;
-      Bs[kk][nn] = (double)v;
-      Ba[kk][nn] = fabsf(v);
-    }
-    __syncthreads();
+  for (int i = 0; i < TM; ++i) {
+    acc[i][0].start();
+    acc[i][1].start();
+  }
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int k0 = 0; k0 < K; k0 += KS) {
+      const int kn = min(KS, K - k0);
+      if (pass == 0 || K > KS) {
+        __syncthreads();
+        for (int idx = t; idx < BMt * kn; idx += NT) {
+          const int mm = idx / kn, kk = idx - mm * kn;
+          As[kk * (BMt + 1) + mm] = m0 + mm < M ? __ldg(A + (size_t)(m0 + mm) * lda + k0 + kk) : 0.f;
+        }
+        for (int idx = t; idx < BN * kn; idx += NT) {
+          const int kk = idx / BN, nn = idx % BN;
+          Bs[kk * BN + nn] = n0 + nn < Ncol ? __ldg(W + (size_t)(k0 + kk) * ldw + n0 + nn) : 0.f;
+        }
+        __syncthreads();
+      }
+      if (pass == 0) {
 #pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
-      double a[TM], bb[4];
-      float aa[TM], ba[4];
+        for (int kk = 0; kk < kn; ++kk) {
+          const float4 w = *reinterpret_cast<const float4*>(Bs + kk * BN + 4 * tx);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) {
+            const float a = As[kk * (BMt + 1) + ty + 16 * i];
+            acc[i][0].size(make_float2(w.x, w.y), make_float2(a, a));
+            acc[i][1].size(make_float2(w.z, w.w), make_float2(a, a));
+          }
+        }
+        continue;
+      }
+      for (int kb = 0; kb < kn; kb += kBlk) {
+#pragma unroll 2
+        for (int kk = kb; kk < min(kn, kb + kBlk); ++kk) {
+          const float4 w = *reinterpret_cast<const float4*>(Bs + kk * BN + 4 * tx);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) {
+            const float a = As[kk * (BMt + 1) + ty + 16 * i];
+            acc[i][0].add(make_float2(w.x, w.y), make_float2(a, a), make_float2(-a, -a));
+            acc[i][1].add(make_float2(w.z, w.w), make_float2(a, a), make_float2(-a, -a));
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          acc[i][0].block(sc.lvl2);
+          acc[i][1].block(sc.lvl2);
+        }
+      }
+    }
+    if (pass == 0)
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
-        a[i] = As[kk][ty + 16 * i];
-        aa[i] = Aa[kk][ty + 16 * i];
+        acc[i][0].begin(sc.lvl2);
+        acc[i][1].begin(sc.lvl2);
       }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        bb[j] = Bs[kk][tx + 16 * j];
-        ba[j] = Ba[kk][tx + 16 * j];
-      }
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j] = fma(a[i], bb[j], acc[i][j]);
-          aab[i][j] = __fmaf_ru(aa[i], ba[j], aab[i][j]);
-        }
-    }
-    __syncthreads();
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int m = m0 + ty + 16 * i;
-    double st = 0.0, se = 0.0, sa = 0.0;
+    TermSum s;
     if (m < M) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int n = n0 + tx + 16 * j;
-        if (n < Ncol) {
-          double tv, ev;
-          epi.term(m, n, acc[i][j], aab[i][j], tv, ev);
-          st += tv;
-          se = __dadd_ru(se, ev);
-          sa = __dadd_ru(sa, fabs(tv));
-        }
+        const int n = n0 + 4 * tx + j;
+        if (n >= Ncol) continue;
+        double g;
+        float delta;
+        acc[i][j / 2].result(j % 2, sc.kk, g, delta);
+        epi.term_delta(m, n, g, delta, s);
       }
     }
 #pragma unroll
     for (int off = 8; off > 0; off >>= 1) {
-      st += __shfl_xor_sync(0xffffffffu, st, off);
-      se = __dadd_ru(se, __shfl_xor_sync(0xffffffffu, se, off));
-      sa = __dadd_ru(sa, __shfl_xor_sync(0xffffffffu, sa, off));
+      s.t += __shfl_xor_sync(0xffffffffu, s.t, off);
+      s.e = __fadd_ru(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
+      s.a = __fadd_ru(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
     }
-    if (tx == 0 && m < M) acc_add(acc_out, acc_out.slot + blockIdx.x, m, st, se, sa);
+    if (tx == 0 && m < M) acc_add(acc_out, acc_out.slot + blockIdx.x, m, s.t, (double)s.e, (double)s.a);
   }
 }
 
-__device__ __forceinline__ void block_reduce_add(FinalAcc a, int slot, int b, double st, double se, double sa) {
-  __shared__ double red[3][NT / 32];
+__device__ __forceinline__ void block_reduce_add(FinalAcc a, int slot, int b, TermSum s) {
+  __shared__ double rt[NT / 32];
+  __shared__ float re[NT / 32], ra[NT / 32];
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    st += __shfl_xor_sync(0xffffffffu, st, off);
-    se = __dadd_ru(se, __shfl_xor_sync(0xffffffffu, se, off));
-    sa = __dadd_ru(sa, __shfl_xor_sync(0xffffffffu, sa, off));
+    s.t += __shfl_xor_sync(0xffffffffu, s.t, off);
+    s.e = __fadd_ru(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
+    s.a = __fadd_ru(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
   }
   const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (lane == 0) {
-    red[0][w] = st;
-    red[1][w] = se;
-    red[2][w] = sa;
+    rt[w] = s.t;
+    re[w] = s.e;
+    ra[w] = s.a;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+    double t = 0.0;
+    float e = 0.f, at = 0.f;
     for (int i = 0; i < (int)(blockDim.x / 32); ++i) {
-      t0 += red[0][i];
-      t1 = __dadd_ru(t1, red[1][i]);
-      t2 = __dadd_ru(t2, red[2][i]);
+      t += rt[i];
+      e = __fadd_ru(e, re[i]);
+      at = __fadd_ru(at, ra[i]);
     }
-    acc_add(a, slot, b, t0, t1, t2);
+    acc_add(a, slot, b, t, (double)e, (double)at);
   }
 }
 
@@ -224,7 +357,7 @@ __global__ void __launch_bounds__(NT) final_conv_kernel(LayerDev L, const float*
   const int b = blockIdx.y;
   const float* rb = r + (size_t)b * rs;
   const int hw_i = L.h * L.w, plane = L.cin * hw_i, hw_o = L.ho * L.wo;
-  double st = 0.0, se = 0.0, sa = 0.0;
+  TermSum s;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < plane; e += gridDim.x * blockDim.x) {
     const int c = e / hw_i, rem = e % hw_i, yy = rem / L.w, xx = rem % L.w;
     double acc = 0.0;
@@ -248,47 +381,30 @@ __global__ void __launch_bounds__(NT) final_conv_kernel(LayerDev L, const float*
         }
       }
     }
-    double tv, ev;
-    epi.term(b, e, acc, aab, tv, ev);
-    st += tv;
-    se = __dadd_ru(se, ev);
-    sa = __dadd_ru(sa, fabs(tv));
+    epi.term(b, e, acc, aab, s);
   }
-  block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, st, se, sa);
+  block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s);
 }
 
-// FP64 transposed conv by stride phase (k4 s2 / k3 s1), G input channels per
-// thread: g[b, c, yy, xx] = sum over the phase's taps (i, j) and o of
-// W[o, c, i, j] rho[b, o, y, x].  Weights sit in shared memory as doubles and
-// their magnitudes as floats, [o][i][j][c], and so does the subdomain's
-// rho_{k+1} (converted once per block), so one rho load feeds G FP64 FMAs.  Same terms and error bounds as final_conv_kernel; the
-// slots are this grid's blocks.
+// Transposed conv by stride phase (k4 s2 / k3 s1) in three-level sums, G input
+// channels per thread (two packed pairs; G = 3: the fourth has zero weights):
+// g[b, c, yy, xx] = sum over the phase's taps (i, j) and o of W[o, c, i, j]
+// rho[b, o, y, x], weights and the subdomain's rho_{k+1} (with its zero halo) in
+// shared memory.  The slots are this grid's blocks.
 template <int KH, int KW, int ST, int G>
-__global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, const float* __restrict__ r, int rs,
-                                                             FinalEpi epi, FinalAcc acc_out) {
-  extern __shared__ double sWd[];
-  const int nw = L.cout * L.cin * KH * KW;
-  const int hw_o = L.ho * L.wo, slab = L.cout * hw_o;
-  // the subdomain's rho_{k+1} as doubles (converted once) and its magnitudes
-  double* sR = sWd + nw;
-  float* sWa = reinterpret_cast<float*>(sR + slab);
-  float* sRa = sWa + nw;
+__global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, ConvTile T, const float* __restrict__ r, int rs,
+                                                             FinalEpi epi, Sum3Const sc, FinalAcc acc_out) {
+  extern __shared__ __align__(16) float sm[];
+  float* sR = sm + T.w_floats;
   const int b = blockIdx.y;
-  const float* rb = r + (size_t)b * rs;
-  for (int e = threadIdx.x; e < nw; e += NT) {
-    const float w = L.Wt[e];
-    sWd[e] = (double)w;
-    sWa[e] = fabsf(w);
-  }
-  for (int e = threadIdx.x; e < slab; e += NT) {
-    const float v = __ldg(rb + e);
-    sR[e] = (double)v;
-    sRa[e] = fabsf(v);
-  }
-  __syncthreads();
-  const int qh = L.h / ST, qw = L.w / ST, ncg = L.cin / G;
+  if (G == 3)
+    for (int e = threadIdx.x; e < T.w_floats / 4; e += NT) sm[4 * e + 3] = 0.f;
+  conv_t_weights(L, T, sm, NT);
+  conv_t_rows(L, T, sR, r + (size_t)b * rs, 0, NT);
+  stage_wait();
+  const int qh = L.h / ST, qw = L.w / ST, ncg = L.cin / G, plane = T.rows * T.pitch;
   const int items = ST * ST * ncg * qh * qw;
-  double st = 0.0, se = 0.0, sa = 0.0;
+  TermSum s;
   for (int e = blockIdx.x * NT + threadIdx.x; e < items; e += gridDim.x * NT) {
     int q = e;
     const int qx = q % qw;
@@ -301,68 +417,72 @@ __global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, const f
     const int ry = q / ST;
     const int i0 = (ry + L.pad) % ST, j0 = (rx + L.pad) % ST;
     const int dy0 = (ry + L.pad - i0) / ST, dx0 = (rx + L.pad - j0) / ST;
-    double acc[G];
-    float aab[G];
+    const float* rp = sR + (qy + dy0 - T.y_off) * T.pitch + qx + dx0 - T.x_off;
+    const float* wp = sm + (i0 * KW + j0) * T.wc + cg * G;
+    Sum3x2 a0, a1;
+    a0.start();
+    a1.start();
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      acc[g] = 0.0;
-      aab[g] = 0.f;
-    }
-#pragma unroll
-    for (int a = 0; a < KH / ST; ++a) {
-      const int y = qy + dy0 - a;
-      if (y < 0 || y >= L.ho) continue;
+    for (int a = 0; a < KH / ST; ++a)
 #pragma unroll
       for (int bb = 0; bb < KW / ST; ++bb) {
-        const int x = qx + dx0 - bb;
-        if (x < 0 || x >= L.wo) continue;
-        const int rp = y * L.wo + x;
-        const int wo0 = ((i0 + ST * a) * KW + j0 + ST * bb) * L.cin + cg * G;
+        const float* ra = rp - a * T.pitch - bb;
+        const float* wa = wp + (ST * a * KW + ST * bb) * T.wc;
+#pragma unroll 4
         for (int o = 0; o < L.cout; ++o) {
-          const double rd = sR[rp + o * hw_o];
-          const float ra = sRa[rp + o * hw_o];
-          const double* wd = sWd + wo0 + o * KH * KW * L.cin;
-          const float* wa = sWa + wo0 + o * KH * KW * L.cin;
-#pragma unroll
-          for (int g = 0; g < G; ++g) {
-            acc[g] = fma(wd[g], rd, acc[g]);
-            aab[g] = __fmaf_ru(wa[g], ra, aab[g]);
+          const float rv = ra[o * plane];
+          const float4 w = *reinterpret_cast<const float4*>(wa + o * KH * KW * T.wc);
+          a0.size(make_float2(w.x, w.y), make_float2(rv, rv));
+          a1.size(make_float2(w.z, w.w), make_float2(rv, rv));
+        }
+      }
+    a0.begin(sc.lvl2);
+    a1.begin(sc.lvl2);
+    int cnt = 0;
+#pragma unroll 1
+    for (int a = 0; a < KH / ST; ++a)
+#pragma unroll 1
+      for (int bb = 0; bb < KW / ST; ++bb) {
+        const float* ra = rp - a * T.pitch - bb;
+        const float* wa = wp + (ST * a * KW + ST * bb) * T.wc;
+        for (int o0 = 0; o0 < L.cout; o0 += kBlk) {
+          const int on = min(L.cout, o0 + kBlk);
+          if (cnt + on - o0 > kBlk) {
+            a0.block(sc.lvl2);
+            a1.block(sc.lvl2);
+            cnt = 0;
+          }
+          cnt += on - o0;
+#pragma unroll 4
+          for (int o = o0; o < on; ++o) {
+            const float rv = ra[o * plane];
+            const float4 w = *reinterpret_cast<const float4*>(wa + o * KH * KW * T.wc);
+            a0.add(make_float2(w.x, w.y), make_float2(rv, rv), make_float2(-rv, -rv));
+            a1.add(make_float2(w.z, w.w), make_float2(rv, rv), make_float2(-rv, -rv));
           }
         }
       }
-    }
+    a0.block(sc.lvl2);
+    a1.block(sc.lvl2);
     const int yy = ry + ST * qy, xx = rx + ST * qx;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      double tv, ev;
-      epi.term(b, ((cg * G + g) * L.h + yy) * L.w + xx, acc[g], aab[g], tv, ev);
-      st += tv;
-      se = __dadd_ru(se, ev);
-      sa = __dadd_ru(sa, fabs(tv));
+      double gv;
+      float delta;
+      (g / 2 ? a1 : a0).result(g % 2, sc.kk, gv, delta);
+      epi.term_delta(b, ((cg * G + g) * L.h + yy) * L.w + xx, gv, delta, s);
     }
   }
-  block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, st, se, sa);
+  block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s);
 }
 
-// Shared memory of the phase-split FP64 transposed conv: weights and the
-// rho slab, each as double + float magnitude.
-size_t final_fast_smem(const LayerDev& L) {
-  return (size_t)L.cout * L.cin * L.kh * L.kw * 12 + (size_t)L.cout * L.ho * L.wo * 12;
-}
-
-// Geometry and channel blocking of the phase-split FP64 transposed conv, or 0.
+// Geometry and channel blocking of the phase-split transposed conv, or 0.
+constexpr size_t kFinalSmem = 160 * 1024;
 int final_fast_geo(const LayerDev& L, int& G) {
   G = 0;
-  if (!L.Wt || L.h % L.stride || L.w % L.stride) return 0;
-  int geo = 0;
-  if (L.kh == 4 && L.kw == 4 && L.stride == 2) geo = 1;
-  if (L.kh == 3 && L.kw == 3 && L.stride == 1) geo = 2;
-  if (!geo) return 0;
-  if (L.cin % 4 == 0) G = 4;
-  else if (L.cin == 3) G = 3;
-  else return 0;
-  if (final_fast_smem(L) > 200 * 1024) return 0;
-  return geo;
+  if (!conv_t_covers(L) || conv_t_tile(L, L.h / L.stride).smem > kFinalSmem) return 0;
+  G = L.cin == 3 ? 3 : 4;
+  return conv_geo(L);
 }
 
 int final_fast_blocks(const LayerDev& L, int G) {
@@ -380,18 +500,14 @@ __global__ void __launch_bounds__(NT) final_top_kernel(int n, const float* __res
                                                        const double* __restrict__ Wn_err, FinalEpi epi,
                                                        FinalAcc acc_out) {
   const int b = blockIdx.x;
-  double st = 0.0, se = 0.0, sa = 0.0;
+  TermSum s;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double tv, ev;
     if (Wn64)
-      epi.term_delta(b, i, -Wn64[i], Wn_err[i], tv, ev);
+      epi.term_delta(b, i, -Wn64[i], abs_up(Wn_err[i]), s);
     else
-      epi.term(b, i, -(double)Wn[i], 0.f, tv, ev);
-    st += tv;
-    se = __dadd_ru(se, ev);
-    sa = __dadd_ru(sa, fabs(tv));
+      epi.term_delta(b, i, -widen(Wn[i]), 0.f, s);
   }
-  block_reduce_add(acc_out, acc_out.slot, b, st, se, sa);
+  block_reduce_add(acc_out, acc_out.slot, b, s);
 }
 
 struct BiasLayers {
@@ -406,33 +522,37 @@ struct BiasLayers {
 __global__ void __launch_bounds__(NT) final_bias_kernel(Problem P, BiasLayers BL, const float* __restrict__ rho,
                                                         FinalAcc acc_out) {
   const int b = blockIdx.x;
-  double st = 0.0, sa = 0.0;
+  TermSum s;
   for (int k = 0; k < BL.count; ++k)
-    for (int i = threadIdx.x; i < BL.n[k]; i += blockDim.x) {
-      const double tv = -(double)rho[(size_t)b * P.N + BL.r_off[k] + i] * (double)BL.bias[k][i / BL.plane[k]];
-      st += tv;
-      sa = __dadd_ru(sa, fabs(tv));
-    }
-  block_reduce_add(acc_out, acc_out.slot, b, st, 0.0, sa);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < BL.n[k]; i += blockDim.x)
+      add_term(s, -widen(rho[(size_t)b * P.N + BL.r_off[k] + i]) * widen(__ldg(BL.bias[k] + i / BL.plane[k])), 0.f);
+  block_reduce_add(acc_out, acc_out.slot, b, s);
 }
 
+// One warp per subdomain: lane i loads slot i of a round, the slots are added in order.
 __global__ void final_combine_kernel(Problem P, FinalAcc a, double bn, double bn_err, double gamma_M, double inflate,
                                      double* out) {
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < P.B; b += gridDim.x * blockDim.x) {
-    if (P.empty[b]) {
-      out[b] = __longlong_as_double(0x7ff0000000000000LL);  // +inf: empty subdomain
-      continue;
+  const int lane = threadIdx.x & 31, b = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  if (b >= P.B) return;
+  double S = bn, E = bn_err, A = fabs(bn);
+  const double* p = a.slots + (size_t)b * a.n_slots * 3;
+  for (int i0 = 0; i0 < a.n_slots; i0 += 32) {
+    const bool in = i0 + lane < a.n_slots;
+    const double t = in ? p[3 * (i0 + lane)] : 0.0, e = in ? p[3 * (i0 + lane) + 1] : 0.0,
+                 at = in ? p[3 * (i0 + lane) + 2] : 0.0;
+    const int n = min(32, a.n_slots - i0);
+    for (int i = 0; i < n; ++i) {
+      S += __shfl_sync(0xffffffffu, t, i);
+      E = __dadd_ru(E, __shfl_sync(0xffffffffu, e, i));
+      A = __dadd_ru(A, __shfl_sync(0xffffffffu, at, i));
     }
-    double S = bn, E = bn_err, A = fabs(bn);
-    const double* p = a.slots + (size_t)b * a.n_slots * 3;
-    for (int i = 0; i < a.n_slots; ++i) {
-      S += p[3 * i];
-      E = __dadd_ru(E, p[3 * i + 1]);
-      A = __dadd_ru(A, p[3 * i + 2]);
-    }
+  }
+  if (lane == 0) {
     E = __dmul_ru(E, inflate);
     A = __dmul_ru(A, inflate);
-    out[b] = __dsub_rd(__dsub_rd(S, E), __dmul_ru(gamma_M, A));
+    out[b] = P.empty[b] ? __longlong_as_double(0x7ff0000000000000LL)  // +inf: empty subdomain
+                        : __dsub_rd(__dsub_rd(S, E), __dmul_ru(gamma_M, A));
   }
 }
 
@@ -449,15 +569,23 @@ static double gamma_of(double K) {
 }
 
 template <int KH, int KW, int ST, int G>
-void launch_fast(dim3 grid, size_t smem, const LayerDev& L, const float* r, int rs, FinalEpi epi, FinalAcc acc,
-                 cudaStream_t s) {
-  static size_t attr = 0;  // dynamic shared memory opted in for this instantiation
-  if (smem > attr) {
+void launch_fast(dim3 grid, const LayerDev& L, const float* r, int rs, FinalEpi epi, FinalAcc acc, cudaStream_t s) {
+  const ConvTile T = conv_t_tile(L, L.h / ST);
+  if (T.smem > 40 * 1024)
     cudaFuncSetAttribute(final_conv_fast_kernel<KH, KW, ST, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr = smem;
-  }
-  final_conv_fast_kernel<KH, KW, ST, G><<<grid, NT, smem, s>>>(L, r, rs, epi, acc);
+                         (int)kFinalSmem);
+  final_conv_fast_kernel<KH, KW, ST, G><<<grid, NT, T.smem, s>>>(L, T, r, rs, epi, sum3_const(sum3_blocks((KH / ST) * (KW / ST), L.cout), L.fan_t), acc);
+}
+
+template <int TM>
+void launch_fc(const LayerDev& L, const Problem& P, const float* r, const FinalEpi& epi, FinalAcc acc, cudaStream_t s) {
+  constexpr int BMt = 16 * TM;
+  constexpr size_t smem = sizeof(float) * (KS * (BMt + 1) + 4 + KS * BN);
+  if (smem > 40 * 1024)
+    cudaFuncSetAttribute(final_fc_kernel<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  dim3 grid((L.n_in + BN - 1) / BN, (P.B + BMt - 1) / BMt);
+  final_fc_kernel<TM><<<grid, NT, smem, s>>>(P.B, L.n_in, L.n_out, r, P.N, L.W, L.n_in, epi,
+                                             sum3_const((L.n_out + kBlk - 1) / kBlk + L.n_out / KS, L.n_out), acc);
 }
 
 int sm_count() {
@@ -484,25 +612,21 @@ void launch_final_layer(const LayerDev& Lnext, int layer, int r_off, int x_off, 
   const float* r = rho + Lnext.r_out_off;
   if (Lnext.kind == LD_LAYER_FC) {
     const int nb = (Lnext.n_in + BN - 1) / BN;
-    if (nb * ((P.B + 63) / 64) >= 2 * sm_count()) {
-      dim3 grid(nb, (P.B + 63) / 64);
-      final_fc_kernel<4><<<grid, NT, 0, s>>>(P.B, Lnext.n_in, Lnext.n_out, r, P.N, Lnext.W, Lnext.n_in, epi, acc);
-    } else {
-      dim3 grid(nb, (P.B + 15) / 16);
-      final_fc_kernel<1><<<grid, NT, 0, s>>>(P.B, Lnext.n_in, Lnext.n_out, r, P.N, Lnext.W, Lnext.n_in, epi, acc);
-    }
+    if (nb * ((P.B + 63) / 64) >= 2 * sm_count())
+      launch_fc<4>(Lnext, P, r, epi, acc, s);
+    else
+      launch_fc<1>(Lnext, P, r, epi, acc, s);
   } else {
     int G = 0;
     const int geo = final_fast_geo(Lnext, G);
     if (geo) {
       dim3 grid(final_fast_blocks(Lnext, G), P.B);
-      const size_t smem = final_fast_smem(Lnext);
       if (geo == 1) {
-        if (G == 4) launch_fast<4, 4, 2, 4>(grid, smem, Lnext, r, P.N, epi, acc, s);
-        else launch_fast<4, 4, 2, 3>(grid, smem, Lnext, r, P.N, epi, acc, s);
+        if (G == 4) launch_fast<4, 4, 2, 4>(grid, Lnext, r, P.N, epi, acc, s);
+        else launch_fast<4, 4, 2, 3>(grid, Lnext, r, P.N, epi, acc, s);
       } else {
-        if (G == 4) launch_fast<3, 3, 1, 4>(grid, smem, Lnext, r, P.N, epi, acc, s);
-        else launch_fast<3, 3, 1, 3>(grid, smem, Lnext, r, P.N, epi, acc, s);
+        if (G == 4) launch_fast<3, 3, 1, 4>(grid, Lnext, r, P.N, epi, acc, s);
+        else launch_fast<3, 3, 1, 3>(grid, Lnext, r, P.N, epi, acc, s);
       }
       return;
     }
@@ -535,7 +659,7 @@ void launch_final_combine_bn(const Problem& P, FinalAcc acc, double bn, double b
                              double inflate, double* out, cudaStream_t s) {
   if (P.B == 0) return;
   count_launch();
-  final_combine_kernel<<<(P.B + 255) / 256, 256, 0, s>>>(P, acc, bn, bn_err, gamma_M, inflate, out);
+  final_combine_kernel<<<(P.B + 3) / 4, 128, 0, s>>>(P, acc, bn, bn_err, gamma_M, inflate, out);
 }
 
 double final_gamma(double K) { return gamma_of(K); }
