@@ -337,15 +337,31 @@ __global__ void top_kernel(int B, int n, const float* __restrict__ Wn, Epi epi) 
   }
 }
 
-// Subdomain b is empty when some clamped bound pair crosses (l > u).
-__global__ void empty_kernel(Problem P, int8_t* empty, int* status) {
+// Subdomain b is empty when some clamped bound pair crosses (l > u).  One CTA
+// per subdomain: bound by the latency of its loads, so they go kE at a time
+// (17 us for 128 Deep subdomains with one at a time).
+__global__ void __launch_bounds__(NT) empty_kernel(Problem P, int8_t* empty, int* status) {
+  constexpr int kE = 8;
   const int b = blockIdx.x;
   if (threadIdx.x == 0 && P.prop && (P.prop[b] < 0 || P.prop[b] >= P.n_props)) atomicCAS(status, 0, (int)LD_ERR_ARG);
+  const float* lb = P.lbk + (size_t)prop_of(P, b) * P.N;
+  const float* ub = P.ubk + (size_t)prop_of(P, b) * P.N;
+  const int8_t* mask = P.mask ? P.mask + (size_t)b * P.N : nullptr;
   int bad = 0;
-  for (int j = threadIdx.x; j < P.N; j += blockDim.x) {
-    float l, u;
-    clamped_bounds(P, b, j, l, u);
-    bad |= (l > u) ? 1 : 0;
+  for (int j0 = threadIdx.x; j0 < P.N; j0 += kE * NT) {
+    float l[kE], u[kE];
+    int m[kE];
+#pragma unroll
+    for (int e = 0; e < kE; ++e) {
+      const int j = j0 + e * NT;
+      const bool in = j < P.N;
+      l[e] = in ? __ldg(lb + j) : 0.f;
+      u[e] = in ? __ldg(ub + j) : 0.f;
+      m[e] = in && mask ? __ldg(mask + j) : 0;
+    }
+#pragma unroll
+    for (int e = 0; e < kE; ++e)
+      bad |= (m[e] > 0 ? fmaxf(l[e], 0.f) : l[e]) > (m[e] < 0 ? fminf(u[e], 0.f) : u[e]) ? 1 : 0;
   }
   bad = __syncthreads_or(bad);
   if (threadIdx.x == 0) empty[b] = (int8_t)(bad ? 1 : 0);
