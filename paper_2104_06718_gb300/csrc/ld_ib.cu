@@ -167,6 +167,13 @@ __device__ __forceinline__ IbRow ib_row(const IbRowMap& M, int64_t g, int lane) 
   return r;
 }
 
+// Units of ib_box_kernel in one row of a window of ww columns.
+__host__ __device__ __forceinline__ int box_units(int stride, int ww) {
+  return stride * (((ww + stride - 1) / stride + 1) / 2);
+}
+// Whether a_0 of first layer L goes through ib_box_kernel.
+inline bool box_pairs(const LayerDev& L) { return L.kind == LD_LAYER_CONV && L.cin <= 4; }
+
 __device__ __forceinline__ int box_of(const IbStep& st, int owner) {
   if (st.box_row) {
     const int p = st.box_row[owner];
@@ -198,34 +205,36 @@ struct Dot2 {
 // product with -1 is exact, so the rounding is that of the subtraction).
 __device__ __forceinline__ float2 sub2(float2 b, float2 a) { return __ffma2_rn(a, make_float2(-1.f, -1.f), b); }
 
+// Two Dot2 in packed form (with nh = -h and nb = -bv of Dot2::add).
+struct Pair {
+  float2 p = {0.f, 0.f}, c = {0.f, 0.f}, s = {0.f, 0.f};
+  __device__ __forceinline__ void add(float2 v, float2 m, float2 nm) {
+    const float2 nh = __fmul2_rn(v, nm);
+    const float2 r = __ffma2_rn(v, m, nh);
+    const float2 t = sub2(p, nh);
+    const float2 nb = sub2(p, t);
+    const float2 q = __fadd2_rn(sub2(p, __fadd2_rn(t, nb)), sub2(nb, nh));
+    p = t;
+    c = __fadd2_rn(c, __fadd2_rn(q, r));
+    s = make_float2(__fadd_ru(s.x, fabsf(nh.x)), __fadd_ru(s.y, fabsf(nh.y)));
+  }
+};
+
 // The dot products of a unit's needed elements, two per packed instruction
 // (half the issue slots of two Dot2, which leaves them to loads and votes) and
 // a last odd one by itself; pairs past np are not touched.
 struct UnitSums {
-  float2 p[kPairs], c[kPairs], s[kPairs];
+  Pair d[kPairs];
   Dot2 one;
   int wa[kPairs], wb[kPairs], w1;    // the elements' places in a staged weight row
   int np;
   bool odd;
-  // Dot2::add of pair K, with nh = -h and nb = -bv.
-  template <int K>
-  __device__ __forceinline__ void pair(const float* ws, float2 m, float2 nm) {
-    const float2 v = make_float2(ws[wa[K]], ws[wb[K]]);
-    const float2 nh = __fmul2_rn(v, nm);
-    const float2 r = __ffma2_rn(v, m, nh);
-    const float2 t = sub2(p[K], nh);
-    const float2 nb = sub2(p[K], t);
-    const float2 q = __fadd2_rn(sub2(p[K], __fadd2_rn(t, nb)), sub2(nb, nh));
-    p[K] = t;
-    c[K] = __fadd2_rn(c[K], __fadd2_rn(q, r));
-    s[K] = make_float2(__fadd_ru(s[K].x, fabsf(nh.x)), __fadd_ru(s[K].y, fabsf(nh.y)));
-  }
   __device__ __forceinline__ void add(const float* ws, float m1) {
     const float2 m = make_float2(m1, m1), nm = make_float2(-m1, -m1);
-    if (np > 0) pair<0>(ws, m, nm);
-    if (np > 1) pair<1>(ws, m, nm);
-    if (np > 2) pair<2>(ws, m, nm);
-    if (np > 3) pair<3>(ws, m, nm);
+    if (np > 0) d[0].add(make_float2(ws[wa[0]], ws[wb[0]]), m, nm);
+    if (np > 1) d[1].add(make_float2(ws[wa[1]], ws[wb[1]]), m, nm);
+    if (np > 2) d[2].add(make_float2(ws[wa[2]], ws[wb[2]]), m, nm);
+    if (np > 3) d[3].add(make_float2(ws[wa[3]], ws[wb[3]]), m, nm);
     if (odd) one.add(ws[w1], m1);
   }
   // Adds n terms: m at mp + k mstep (one coalesced load for all elements), the
@@ -290,6 +299,22 @@ __device__ __forceinline__ float relu_term(RowSum& R, float a, float da, float l
   // the pass's own rounding, times max x_{j-1} = max(u, 0)
   R.e = __fmaf_ru(da, u, R.e);
   return m;
+}
+
+// A CTA's sums of its rows into the chunk's slot.
+__device__ __forceinline__ void store_part(const IbStep& st, const IbRowMap& M, int gl, int chunk,
+                                           double (*red)[32][3], const RowSum& R) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  red[warp][lane][0] = R.v;
+  red[warp][lane][1] = (double)R.d.size();
+  red[warp][lane][2] = (double)R.e;
+  __syncthreads();
+  if (threadIdx.x < 96) {
+    const int q = threadIdx.x / 32;
+    double t = red[0][lane][q];
+    for (int w = 1; w < NW; ++w) t = q == 0 ? t + red[w][lane][q] : __dadd_ru(t, red[w][lane][q]);
+    st.part[(((size_t)st.slot + chunk) * M.n_groups * 32 + (size_t)gl * 32 + lane) * 3 + q] = t;
+  }
 }
 
 // One CTA: units [chunk * units_per_cta, ...) of one group of 32 rows; a unit
@@ -370,7 +395,6 @@ __global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
       unsigned rest = act;
 #pragma unroll
       for (int k = 0; k < kPairs; ++k) {
-        S.p[k] = S.c[k] = S.s[k] = make_float2(0.f, 0.f);
         S.wa[k] = S.wb[k] = 0;
         if (k < S.np) {
           const int a = __ffs(rest) - 1;
@@ -420,9 +444,9 @@ __global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
 #pragma unroll
       for (int k = 0; k < kPairs; ++k) {
         const bool lo = k < S.np && e == 2 * k, hi = k < S.np && e == 2 * k + 1;
-        d.p = lo ? S.p[k].x : hi ? S.p[k].y : d.p;
-        d.c = lo ? S.c[k].x : hi ? S.c[k].y : d.c;
-        d.s = lo ? S.s[k].x : hi ? S.s[k].y : d.s;
+        d.p = lo ? S.d[k].p.x : hi ? S.d[k].p.y : d.p;
+        d.c = lo ? S.d[k].c.x : hi ? S.d[k].c.y : d.c;
+        d.s = lo ? S.d[k].s.x : hi ? S.d[k].s.y : d.s;
       }
       if (st.seed) {
         if (!conv) d.p = sg * __ldg(L.W + (size_t)r.i * L.n_in + c);
@@ -446,16 +470,97 @@ __global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
     if (++done % st.flush == 0) R.flush();
   }
   R.flush();
-  red[warp][lane][0] = R.v;
-  red[warp][lane][1] = (double)R.d.size();
-  red[warp][lane][2] = (double)R.e;
-  __syncthreads();
-  if (threadIdx.x < 96) {
-    const int q = threadIdx.x / 32;
-    double t = red[0][lane][q];
-    for (int w = 1; w < NW; ++w) t = q == 0 ? t + red[w][lane][q] : __dadd_ru(t, red[w][lane][q]);
-    st.part[(((size_t)st.slot + chunk) * M.n_groups * 32 + (size_t)gl * 32 + lane) * 3 + q] = t;
+  store_part(st, M, gl, chunk, red, R);
+}
+
+// The input box of a conv first layer of C <= 4 channels: a unit is two
+// positions of one row and column phase, `stride` columns apart, and all
+// channels.  Both positions meet the same weights, so a packed instruction
+// holds one channel's two positions and one 16-byte load all its weights; with
+// the general kernel's unit (one position, three channels) the units' set-up
+// and votes were two thirds of the instructions.  Base, 3 channels: a call of
+// 64 subdomains 5.48 -> 3.38 ms, FSB's children of 256 subdomains 1.42 -> 1.09
+// ms, Deep's root bounds 0.685 -> 0.542 ms.
+template <int C>
+__global__ void __launch_bounds__(NT, 3) ib_box_kernel(IbStep st, IbRowMap M) {
+  extern __shared__ __align__(16) float sw[];  // [tap][o][4]
+  __shared__ double red[NW][32][3];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gl = blockIdx.x / st.chunks, chunk = blockIdx.x % st.chunks;
+  const IbRow r = ib_row(M, M.group0 + gl, lane);
+  const LayerDev& L = st.L;
+  for (int e = threadIdx.x; e < L.cout * L.kh * L.kw * 4; e += NT) {
+    const int c = e % 4, q = e / 4, o = q % L.cout, tap = q / L.cout;
+    sw[e] = c < C ? __ldg(L.Wt + ((size_t)o * L.kh * L.kw + tap) * C + c) : 0.f;
   }
+  __syncthreads();
+  const float* mu = st.mu_in + (size_t)gl * st.in_elems * 32 + lane;
+  const int iy0 = st.win.full ? 0 : r.oy * st.win.mul - st.win.sub;
+  const int ix0 = st.win.full ? 0 : r.ox * st.win.mul - st.win.sub;
+  const int oy0 = st.wout.full ? 0 : r.oy * st.wout.mul - st.wout.sub;
+  const int ox0 = st.wout.full ? 0 : r.ox * st.wout.mul - st.wout.sub;
+  const float* lp = st.l0 + (size_t)box_of(st, r.owner) * st.n0;
+  const float* up = st.u0 + (size_t)box_of(st, r.owner) * st.n0;
+  const int S = L.stride, estep = st.win.hh * st.win.ww * 32, per_row = box_units(S, st.wout.ww);
+  RowSum R;
+  int done = 0;
+  const int u_hi = min(st.units, (chunk + 1) * st.units_per_cta);
+  for (int un = chunk * st.units_per_cta + warp; un < u_hi; un += NW) {
+    const int wy = un / per_row, k = un - wy * per_row, wx = k % S + 2 * S * (k / S);
+    const int y = oy0 + wy, x = ox0 + wx;
+    const bool row = y >= 0 && y < L.h;
+    const bool in0 = row && wx < st.wout.ww && x >= 0 && x < L.w;
+    const bool in1 = row && wx + S < st.wout.ww && x + S >= 0 && x + S < L.w;
+    if (!in0 && !in1) continue;
+    Pair d[C];
+    // taps j0 + t S read column (x + pad - j0) / S - t, and one more for the second position
+    const int ys = y + L.pad, xs = x + L.pad;
+    const int j0 = (xs % S + S) % S, cx = (xs - j0) / S;
+    for (int i = ys % S, qy = ys / S; i < L.kh && qy >= 0; i += S, --qy) {
+      const int iy = qy - iy0;
+      if (qy >= L.ho || iy < 0 || iy >= st.win.hh) continue;
+      for (int j = j0, qx = cx; j < L.kw; j += S, --qx) {
+        const int ix = qx - ix0;
+        const bool a = in0 && qx >= 0 && qx < L.wo && ix >= 0 && ix < st.win.ww;
+        const bool b = in1 && qx + 1 >= 0 && qx + 1 < L.wo && ix + 1 >= 0 && ix + 1 < st.win.ww;
+        if (!a && !b) continue;
+        const float* mp = mu + (iy * st.win.ww + ix) * 32;
+        const float4* w = reinterpret_cast<const float4*>(sw) + (i * L.kw + j) * L.cout;
+        for (int o = 0; o < L.cout; o += 4, mp += 4 * (size_t)estep) {
+          float2 m[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const bool on = o + q < L.cout;
+            m[q].x = on && a ? __ldg(mp + (size_t)q * estep) : 0.f;
+            m[q].y = on && b ? __ldg(mp + (size_t)q * estep + 32) : 0.f;
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (!__any_sync(kFull, m[q].x != 0.f || m[q].y != 0.f)) continue;
+            const float4 wv = w[o + q];
+            const float2 nm = make_float2(-m[q].x, -m[q].y);
+            d[0].add(make_float2(wv.x, wv.x), m[q], nm);
+            if (C > 1) d[1 % C].add(make_float2(wv.y, wv.y), m[q], nm);
+            if (C > 2) d[2 % C].add(make_float2(wv.z, wv.z), m[q], nm);
+            if (C > 3) d[3 % C].add(make_float2(wv.w, wv.w), m[q], nm);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!(h ? in1 : in0)) continue;
+        const int ii = (c * L.h + y) * L.w + x + h * S;
+        const float a = h ? __fadd_rn(d[c].p.y, d[c].c.y) : __fadd_rn(d[c].p.x, d[c].c.x);
+        const float s = __fmul_ru(h ? d[c].s.y : d[c].s.x, 1.f + 2.f * kTwoU);
+        box_term(R, a, __fmaf_ru(st.g2, s, __fmul_ru(kTwoU, fabsf(a))), __ldg(lp + ii), __ldg(up + ii));
+      }
+    if (++done % st.flush == 0) R.flush();
+  }
+  R.flush();
+  store_part(st, M, gl, chunk, red, R);
 }
 
 // Sums a chunk's slots per row (fixed order), with the objective's bias term.
@@ -552,7 +657,11 @@ IbGeo ib_geo(const std::vector<LayerDev>& Ls, int k) {
     const bool conv = up.kind == LD_LAYER_CONV;
     g.elems[j] = conv ? up.cin * g.w[j].hh * g.w[j].ww : up.n_in;
     g.units[j] = conv ? g.w[j].hh * g.w[j].ww * ((up.cin + kUnitC - 1) / kUnitC) : (up.n_in + kUnitC - 1) / kUnitC;
-    const int unit_terms = up.fan_t * std::min(kUnitC, conv ? up.cin : up.n_in);
+    int unit_terms = up.fan_t * std::min(kUnitC, conv ? up.cin : up.n_in);
+    if (j == 0 && box_pairs(up)) {
+      g.units[j] = g.w[j].hh * box_units(up.stride, g.w[j].ww);
+      unit_terms = 2 * up.fan_t * up.cin;
+    }
     g.per_cta[j] = NW * std::max(std::min(8, std::max(2, kWarpWork / unit_terms)),
                                  (g.units[j] + NW * kMaxChunks - 1) / (NW * kMaxChunks));
     g.chunks[j] = (g.units[j] + g.per_cta[j] - 1) / g.per_cta[j];
@@ -657,12 +766,18 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
       st.units_per_cta = g.per_cta[j - 1];
       const bool conv = L.kind == LD_LAYER_CONV;
       st.cp = conv ? (L.cin <= 4 ? 4 : L.cin <= 8 ? 8 : L.cin <= 16 ? 16 : (L.cin + 1) & ~1) : NW * kUnitC;
-      const int terms = (st.box ? 1 : 2) * std::min(kUnitC, conv ? L.cin : L.n_in);
+      const bool pairs = st.box && !st.seed && box_pairs(L);
+      if (pairs) st.cp = 4;
+      const int terms = pairs ? 2 * L.cin : (st.box ? 1 : 2) * std::min(kUnitC, conv ? L.cin : L.n_in);
       st.flush = std::max(1, kTerms / terms);
       const size_t smem = sizeof(float) * (size_t)st.cp * (st.seed ? 0
                                                            : conv  ? L.cout * L.kh * L.kw
                                                                    : std::min(kFcRows, L.n_out));
-      auto kernel = st.cp == 4    ? ib_step_kernel<4>
+      auto kernel = pairs         ? (L.cin == 1   ? ib_box_kernel<1>
+                                     : L.cin == 2 ? ib_box_kernel<2>
+                                     : L.cin == 3 ? ib_box_kernel<3>
+                                                  : ib_box_kernel<4>)
+                    : st.cp == 4  ? ib_step_kernel<4>
                     : st.cp == 8  ? ib_step_kernel<8>
                     : st.cp == 16 ? ib_step_kernel<16>
                     : st.cp == 64 ? ib_step_kernel<64>
