@@ -142,6 +142,56 @@ __device__ __forceinline__ void argmin8(const Problem& P, const float* rho, floa
   }
 }
 
+// ------------------------------------------------------------------ halo tiles
+// The A operand of a conv pass from one halo tile: a tile is 16 (row, subdomain)
+// pairs x 8 consecutive columns of the output grid, and its operand pixels, with
+// the halo the taps reach, are loaded once per channel group (and input stride
+// phase) into a plane [y][subdomain][x] of 16-byte pixels (8 channels: one row of
+// a core matrix).  The 8-row groups of the tile then sit `sbo` apart for every
+// tap, so a tap is a shifted descriptor over the plane, and an MMA's two K
+// chunks are a second offset (lbo) apart.  A 128-pixel box per tap and channel
+// group instead made the TMA's 16-byte rows the limit (36 boxes a tile where 4
+// halo boxes hold the same pixels, Wide's second conv transposed).  Wide, 2048
+// subdomains, us before and after: transposed convs 68 -> 63 and 47 -> 31,
+// forward 37 -> 31 (the first layer's, 66, is bound by its Adam epilogue); a
+// call of 100 iterations 29.5 -> 27.0 ms.
+constexpr int kHaloSteps = 64;
+struct Halo {
+  int on;                       // 0: one box per tap and channel group (geometries without such tiles)
+  int rows_y, nsub, rblk, cblk; // rows x subdomains of a tile (16 pairs), tiles along y and x
+  int kq, n_planes;             // channel groups, planes (stride phases x channel groups)
+  int x_lo, y_lo;               // halo: first column / row relative to the tile's
+  uint32_t plane, box_bytes, sbo;
+  int steps;                    // MMAs of a tile
+  uint32_t tab[kHaloSteps];     // per MMA: operand offset (low half) and lbo (high half), in 16-byte units
+  __device__ __forceinline__ void tile(int t, int& b0, int& y0, int& x0) const {
+    const int cb = t % cblk;
+    t /= cblk;
+    const int rb = t % rblk;
+    b0 = t / rblk * nsub;
+    y0 = rb * rows_y;
+    x0 = cb * 8;
+  }
+  // subdomain and position of row r of tile t
+  __device__ __forceinline__ void row(int t, int r, int& b, int& y, int& x) const {
+    tile(t, b, y, x);
+    const int g = r >> 3, yy = g / nsub;
+    y += yy;
+    b += g - yy * nsub;
+    x += r & 7;
+  }
+  // The MMAs of a tile whose planes start at sst; B operand at sres (R columns).
+  __device__ __forceinline__ void mma(uint32_t sst, uint32_t sres, uint32_t tmem, uint32_t id, int R) const {
+    uint64_t db = op_desc(sres, 0, R);
+    const uint64_t d0 = ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
+    for (int s = 0; s < steps; ++s) {
+      const uint32_t e = tab[s];
+      mma_bf16(tmem, d0 | ((sst >> 4) + (e & 0xffffu)) | ((uint64_t)(e >> 16) << 16), db, id, s > 0 ? 1u : 0u);
+      db += (uint64_t)(2 * R * 16 >> 4);
+    }
+  }
+};
+
 // ------------------------------------------------------------------ ops
 // Common fields of one tensor-core launch.
 struct TcCommon {
@@ -158,8 +208,10 @@ struct TcCommon {
 struct alignas(128) ConvFwdOp {
   static constexpr bool kStageBulk = false;
   static constexpr bool kTma = true;
-  CUtensorMap mx[4];           // x_{k-1} shadow by input stride phase (py, px): (c, x', y', b)
+  CUtensorMap mx[4];           // x_{k-1} shadow by input stride phase (py, px): (c, x', y', b); halo: (c, x', b, y'),
+                               // phases in the order of the halo planes
   TcCommon c;
+  Halo hl;
   int nf, kf, KC, kq;          // N, K, K per stage (the last stage may be shorter), channel groups per tap
   int nsub, rows_y, tiles_b;   // tile = nsub subdomains x rows_y output rows (x all columns), or 1/tiles_b of one
   const uint16_t* W;
@@ -173,7 +225,6 @@ struct alignas(128) ConvFwdOp {
   const float* c1;
   AdamArgs ad;
 
-  __device__ void prepare(int4*) const {}
   __device__ void load_resident(uint32_t sres, uint32_t bar) const {
     mbar_expect_tx(bar, c.res_bytes);
     bulk_g2s(sres, W, c.res_bytes, bar);
@@ -184,8 +235,18 @@ struct alignas(128) ConvFwdOp {
   // lanes of the producer warp share the boxes.  Output (yo, xo) of tap (i, j)
   // reads input (S yo + i - pad, S xo + j - pad) = phase (py, px) position
   // (yo + dy, xo + dx): a contiguous box of that phase's map.
-  __device__ uint32_t stage_bytes_of(int chunk) const { return (uint32_t)((min(kf, (chunk + 1) * KC) - chunk * KC) / 8) * 2048u; }
+  __device__ uint32_t stage_bytes_of(int chunk) const {
+    if (hl.on) return (uint32_t)hl.n_planes * hl.box_bytes;
+    return (uint32_t)((min(kf, (chunk + 1) * KC) - chunk * KC) / 8) * 2048u;
+  }
   __device__ void produce(int tile, int chunk, uint32_t sst, uint32_t bar, int lane) const {
+    if (hl.on) {
+      int b0, y0, x0;
+      hl.tile(tile, b0, y0, x0);
+      for (int p = lane; p < hl.n_planes; p += 32)
+        tma_load_4d(sst + (uint32_t)p * hl.plane, &mx[p / hl.kq], 8 * (p % hl.kq), x0 + hl.x_lo, b0, y0 + hl.y_lo, bar);
+      return;
+    }
     const int k8_lo = chunk * KC / 8, k8_hi = min(kf, (chunk + 1) * KC) / 8;
     const int b0 = tiles_b > 1 ? tile / tiles_b : tile * nsub;
     const int yo0 = tiles_b > 1 ? (tile % tiles_b) * rows_y : 0;
@@ -204,6 +265,10 @@ struct alignas(128) ConvFwdOp {
   }
   __device__ void issue_mma(int, int chunk, uint32_t sres, uint32_t sst, uint32_t tmem) const {
     const uint32_t id = idesc_bf16(kRows, nf);
+    if (hl.on) {
+      hl.mma(sst, sres, tmem, id, nf);
+      return;
+    }
     const int s0 = chunk * KC / 16, ns = (min(kf, (chunk + 1) * KC) - chunk * KC) / 16;
     uint64_t da = op_desc(sst, 0, kRows), db = op_desc(sres, s0, nf);
     for (int s = 0; s < ns; ++s) {
@@ -215,7 +280,12 @@ struct alignas(128) ConvFwdOp {
   __device__ void epilogue(int tile, uint32_t tmem) const {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
     const int r = q * 32 + lane, R = tile * kRows + r, hw = ho * wo;
-    const int b = R / hw, p = R - b * hw;
+    int b = R / hw, p = R - b * hw;
+    if (hl.on) {
+      int y, x;
+      hl.row(tile, r, b, y, x);
+      p = y * wo + x;
+    }
     const bool row_ok = b < B && !P.empty[b];
     const int prop = row_ok ? prop_of(P, b) : 0;
     const int cols = nf / 2, lo = half * cols;
@@ -253,8 +323,9 @@ template <int SS>  // stride (1 or 2)
 struct alignas(128) ConvTOp {
   static constexpr bool kStageBulk = false;
   static constexpr bool kTma = true;
-  CUtensorMap mr;              // rho_k shadow: (c, x, y, b)
+  CUtensorMap mr;              // rho_k shadow: (c, x, y, b); halo: (c, x, b, y)
   TcCommon c;
+  Halo hl;
   int nt, kt, KC, cg, na, nb, dmy, dmx, kq;
   int nsub, rows_y, tiles_b;   // tile = nsub subdomains x rows_y phase rows, or 1/tiles_b of one
   const uint16_t* W;
@@ -270,19 +341,26 @@ struct alignas(128) ConvTOp {
   int rhb_off, rhb_conv, rhb_hw, rhb_cp;  // layout of the shadow of rho_kb
   int pairs;                   // S == 2 and every flat index of an x-pair even (float2 accesses)
 
-  __device__ void prepare(int4*) const {}
   __device__ void load_resident(uint32_t sres, uint32_t bar) const {
     mbar_expect_tx(bar, c.res_bytes);
     bulk_g2s(sres, W, c.res_bytes, bar);
   }
   __device__ void load_stage(int, int, uint32_t, uint32_t, const int4*) const {}
   __device__ uint32_t stage_bytes_of(int chunk) const {
+    if (hl.on) return (uint32_t)hl.n_planes * hl.box_bytes;
     return (uint32_t)((min(kt, (chunk + 1) * KC) - chunk * KC) / 8) * 2048u;
   }
   // TMA loads of one stage: per k-group (neighbourhood pixel, channel group)
   // one box of 8 channels x the tile's 128 positions of rho_k at
   // (qy + dmy + ty, qx + dmx + tx); out-of-range pixels read zero.
   __device__ void produce(int tile, int chunk, uint32_t sst, uint32_t bar, int lane) const {
+    if (hl.on) {
+      int b0, y0, x0;
+      hl.tile(tile, b0, y0, x0);
+      for (int p = lane; p < hl.n_planes; p += 32)
+        tma_load_4d(sst + (uint32_t)p * hl.plane, &mr, 8 * p, x0 + hl.x_lo, b0, y0 + hl.y_lo, bar);
+      return;
+    }
     const int k8_lo = chunk * KC / 8, k8_hi = min(kt, (chunk + 1) * KC) / 8;
     const int b0 = tiles_b > 1 ? tile / tiles_b : tile * nsub;
     const int qy0 = tiles_b > 1 ? (tile % tiles_b) * rows_y : 0;
@@ -297,6 +375,10 @@ struct alignas(128) ConvTOp {
   }
   __device__ void issue_mma(int, int chunk, uint32_t sres, uint32_t sst, uint32_t tmem) const {
     const uint32_t id = idesc_bf16(kRows, nt);
+    if (hl.on) {
+      hl.mma(sst, sres, tmem, id, nt);
+      return;
+    }
     const int s0 = chunk * KC / 16, ns = (min(kt, (chunk + 1) * KC) - chunk * KC) / 16;
     uint64_t da = op_desc(sst, 0, kRows), db = op_desc(sres, s0, nt);
     for (int s = 0; s < ns; ++s) {
@@ -431,7 +513,8 @@ struct alignas(128) ConvTOp {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
     const int PW = w / SS, PP = (h / SS) * PW;
     const int R = tile * kRows + q * 32 + lane;
-    const int b = R / PP, qq = R - b * PP, qy = qq / PW, qx = qq - qy * PW;
+    int b = R / PP, qq = R - b * PP, qy = qq / PW, qx = qq - qy * PW;
+    if (hl.on) hl.row(tile, q * 32 + lane, b, qy, qx);
     const bool row_ok = b < B;
     const int prop = row_ok ? prop_of(P, b) : 0;
     const uint32_t lanes = (uint32_t)(q * 32) << 16;
@@ -493,7 +576,6 @@ struct FcFwdOp {
   const float* c1;
   AdamArgs ad;
 
-  __device__ void prepare(int4*) const {}
   __device__ void load_resident(uint32_t, uint32_t) const {}
   __device__ uint32_t stage_bytes_of(int) const { return 0; }
   __device__ void produce(int, int, uint32_t, uint32_t, int) const {}
@@ -569,7 +651,6 @@ struct FcTOp {
 
   // the grid is a multiple of n_mt, so every tile of a CTA has the same 128-row
   // block of W^T (mt = blockIdx.x % n_mt): it stays resident
-  __device__ void prepare(int4*) const {}
   __device__ void load_resident(uint32_t sres, uint32_t bar) const {
     mbar_expect_tx(bar, a_bytes);
     bulk_g2s(sres, W + (size_t)(blockIdx.x % n_mt) * kRows * kt, a_bytes, bar);
@@ -726,7 +807,6 @@ __global__ void __launch_bounds__(kCtaThreads, 2) tc_kernel(const __grid_constan
     tmem_alloc(smem_u32(&tmem_slot), op.c.tmem_cols);
     tmem_relinquish();
   }
-  if (tid < kThreads) op.prepare(tab);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1070,6 +1150,64 @@ bool plane_tiling(int PH, int PW, int& nsub, int& rows_y, int& tiles_b) {
   return false;
 }
 
+// Halo tiles over an output grid of PH x PW positions per subdomain: operand
+// pixel of tap (i, j) at (y + dy(i), x + dx(j)) of stride phase (py(i), px(j))
+// (ph_y, ph_x phases in y and x, 1 without strides), kq channel groups, K =
+// taps x 8 kq rounded up to 16.  An odd number of chunks leaves the last MMA a
+// second chunk of zero weights: it reads the pixel to the right of the first's,
+// for which the halo is a column wider (a neighbouring subdomain's pixel there
+// could carry a NaN over).  False where the grid does not divide into such
+// tiles, a step's chunks lie in descending order, or two stages do not fit
+// beside the resident weights.
+struct HaloTap {
+  int d, ph;
+};
+bool halo_plan(int PH, int PW, const std::vector<HaloTap>& ty, const std::vector<HaloTap>& tx, int ph_y, int ph_x,
+               int kq, size_t res_bytes, uint32_t tmem_cols, Halo& h) {
+  h = Halo{};
+  h.rows_y = PH < 16 ? PH : 16;
+  if (PW % 8 || PH % h.rows_y || 16 % h.rows_y) return false;
+  h.nsub = 16 / h.rows_y;
+  h.rblk = PH / h.rows_y;
+  h.cblk = PW / 8;
+  int y_hi = ty[0].d, x_hi = tx[0].d;
+  h.y_lo = ty[0].d;
+  h.x_lo = tx[0].d;
+  for (const HaloTap& t : ty) {
+    h.y_lo = std::min(h.y_lo, t.d);
+    y_hi = std::max(y_hi, t.d);
+  }
+  for (const HaloTap& t : tx) {
+    h.x_lo = std::min(h.x_lo, t.d);
+    x_hi = std::max(x_hi, t.d);
+  }
+  const int odd = (int)(ty.size() * tx.size() * kq) % 2;
+  const int Wp = 8 + x_hi - h.x_lo + odd, Hp = h.rows_y + y_hi - h.y_lo;
+  h.kq = kq;
+  h.n_planes = ph_y * ph_x * kq;
+  h.box_bytes = (uint32_t)(16 * Wp * Hp * h.nsub);
+  h.plane = (h.box_bytes + 127u) / 128u * 128u;
+  h.sbo = (uint32_t)(16 * Wp);
+  if (Wp > 256 || Hp > 256 || launch_smem(res_bytes + 2 * (size_t)h.n_planes * h.plane, tmem_cols) > kSmemBudget)
+    return false;
+  // chunk addresses in the order of K: tap-major, channel group, then the padding
+  std::vector<uint32_t> at;
+  for (const HaloTap& a : ty)
+    for (const HaloTap& b : tx)
+      for (int g = 0; g < kq; ++g)
+        at.push_back((uint32_t)(((a.ph * ph_x + b.ph) * kq + g) * (int)h.plane +
+                                (((a.d - h.y_lo) * h.nsub) * Wp + b.d - h.x_lo) * 16));
+  if (odd) at.push_back(at.back() + 16);
+  h.steps = (int)at.size() / 2;
+  if (h.steps > kHaloSteps) return false;
+  for (int s = 0; s < h.steps; ++s) {
+    if (at[2 * s + 1] <= at[2 * s]) return false;
+    h.tab[s] = (at[2 * s] >> 4) | ((at[2 * s + 1] - at[2 * s]) >> 4) << 16;
+  }
+  h.on = 1;
+  return true;
+}
+
 }  // namespace
 
 ld_status build_tc_net(const std::vector<LayerDev>& Ls, TcNet* out) {
@@ -1269,11 +1407,21 @@ void launch_conv_t(TcNet& t, int k, const TcLayer& T, const LayerDev& L, const P
   ConvTOp<SS> op{};
   const int PH = L.h / SS, PW = L.w / SS;
   if (!plane_tiling(PH, PW, op.nsub, op.rows_y, op.tiles_b)) return;
+  std::vector<HaloTap> ty, tx;
+  for (int i = 0; i < T.na; ++i) ty.push_back({T.dmy + i, 0});
+  for (int j = 0; j < T.nb; ++j) tx.push_back({T.dmx + j, 0});
+  const bool halo = halo_plan(PH, PW, ty, tx, 1, 1, T.cp_out / 8, (size_t)2 * T.nt * T.kt,
+                              tmem_cols_for(2 * T.nt), op.hl);
   TcMaps& mc = t.tr[k - 1];
   if (mc.base != S.rh || mc.B != P.B) {
     // rho_k shadow of this layer: (cp_out, wo, ho, B), subdomain rows RH apart
-    if (!encode_map(&mc.m[0], S.rh + T.rh_off, T.cp_out, L.wo, L.ho, P.B, (uint64_t)T.cp_out * 2,
-                    (uint64_t)L.wo * T.cp_out * 2, (uint64_t)t.RH * 2, PW, op.rows_y, op.nsub)) {
+    // (halo tiles: (cp_out, wo, B, ho))
+    const uint64_t sx = (uint64_t)T.cp_out * 2, sy = (uint64_t)L.wo * T.cp_out * 2, sb = (uint64_t)t.RH * 2;
+    const bool ok = halo ? encode_map(&mc.m[0], S.rh + T.rh_off, T.cp_out, L.wo, P.B, L.ho, sx, sb, sy,
+                                      op.hl.sbo / 16, op.hl.nsub, op.hl.box_bytes / (op.hl.sbo * op.hl.nsub))
+                         : encode_map(&mc.m[0], S.rh + T.rh_off, T.cp_out, L.wo, L.ho, P.B, sx, sy, sb, PW, op.rows_y,
+                                      op.nsub);
+    if (!ok) {
       atomic_status_host(S.status);
       return;
     }
@@ -1287,6 +1435,11 @@ void launch_conv_t(TcNet& t, int k, const TcLayer& T, const LayerDev& L, const P
   op.c.n_chunks = (T.kt + op.KC - 1) / op.KC;
   op.c.res_bytes = (uint32_t)(2 * T.nt * T.kt);
   op.c.stage_bytes = (uint32_t)(2 * kRows * op.KC);
+  if (halo) {
+    op.c.n_tiles = (P.B + op.hl.nsub - 1) / op.hl.nsub * op.hl.rblk * op.hl.cblk;
+    op.c.n_chunks = 1;
+    op.c.stage_bytes = (uint32_t)op.hl.n_planes * op.hl.plane;
+  }
   op.c.tmem_cols = tmem_cols_for(2 * T.nt);
   op.c.grid_multiple = 1;
   op.c.status = S.status;
@@ -1394,10 +1547,35 @@ void launch_tc_forward(TcNet& t, const std::vector<LayerDev>& Ls, int k, const P
     ConvFwdOp op{};
     if (!plane_tiling(L.ho, L.wo, op.nsub, op.rows_y, op.tiles_b)) return;
     const int SS = L.stride;
+    // the phase of tap 0 first, so that consecutive taps' planes ascend
+    std::vector<HaloTap> ty, tx;
+    const int p0 = ((-L.pad) % SS + SS) % SS;
+    for (int i = 0; i < L.kh; ++i) {
+      const int d = floor_div(i - L.pad, SS);
+      ty.push_back({d, (i - L.pad - d * SS - p0 + SS) % SS});
+    }
+    for (int j = 0; j < L.kw; ++j) {
+      const int d = floor_div(j - L.pad, SS);
+      tx.push_back({d, (j - L.pad - d * SS - p0 + SS) % SS});
+    }
+    const bool halo = halo_plan(L.ho, L.wo, ty, tx, SS, SS, T.cp_in / 8, (size_t)2 * T.nf * T.kf,
+                                tmem_cols_for(2 * T.nf), op.hl);
     TcMaps& mc = t.fwd[k - 1];
     if (mc.base != S.xh || mc.B != P.B) {
       // x_{k-1} shadow by input stride phase (py, px): positions (S y' + py, S x' + px)
-      for (int py = 0; py < SS; ++py)
+      for (int py = 0; py < SS && halo; ++py)
+        for (int px = 0; px < SS; ++px) {
+          const int fy = (py + p0) % SS, fx = (px + p0) % SS;
+          const Halo& h = op.hl;
+          if (!encode_map(&mc.m[py * SS + px], S.xh + T.xh_off + (size_t)(fy * L.w + fx) * T.cp_in, T.cp_in,
+                          (L.w - fx + SS - 1) / SS, P.B, (L.h - fy + SS - 1) / SS, (uint64_t)SS * T.cp_in * 2,
+                          (uint64_t)t.XH * 2, (uint64_t)SS * L.w * T.cp_in * 2, h.sbo / 16, h.nsub,
+                          h.box_bytes / (h.sbo * h.nsub))) {
+            atomic_status_host(S.status);
+            return;
+          }
+        }
+      for (int py = 0; py < SS && !halo; ++py)
         for (int px = 0; px < SS; ++px)
           if (!encode_map(&mc.m[py * SS + px], S.xh + T.xh_off + (size_t)(py * L.w + px) * T.cp_in, T.cp_in,
                           (L.w - px + SS - 1) / SS, (L.h - py + SS - 1) / SS, P.B, (uint64_t)SS * T.cp_in * 2,
@@ -1415,6 +1593,11 @@ void launch_tc_forward(TcNet& t, const std::vector<LayerDev>& Ls, int k, const P
     op.c.n_chunks = (T.kf + op.KC - 1) / op.KC;
     op.c.res_bytes = (uint32_t)(2 * T.nf * T.kf);
     op.c.stage_bytes = (uint32_t)(2 * kRows * op.KC);
+    if (halo) {
+      op.c.n_tiles = (P.B + op.hl.nsub - 1) / op.hl.nsub * op.hl.rblk * op.hl.cblk;
+      op.c.n_chunks = 1;
+      op.c.stage_bytes = (uint32_t)op.hl.n_planes * op.hl.plane;
+    }
     op.c.tmem_cols = tmem_cols_for(2 * T.nf);
     op.c.status = S.status;
     op.nf = T.nf;
