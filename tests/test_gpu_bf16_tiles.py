@@ -42,7 +42,7 @@ def _built():
     ldb.load_library()
 
 
-def _problem(name):
+def _problem(name, props=1):
     shape, convs, B = NETS[name]
     rng = np.random.default_rng(sorted(NETS).index(name) + 70)
     c0 = rng.uniform(-0.5, 0.5, int(np.prod(shape)))
@@ -59,18 +59,20 @@ def _problem(name):
         n = m
     on = oracle.Net([oracle.Layer("fc", s.W, s.b) if s.kind == "fc" else
                      oracle.Layer("conv", s.W, s.b, in_shape=s.in_shape, stride=s.stride, pad=s.pad) for s in specs])
-    l0, u0 = (c0 - 0.02).astype(np.float32)[None], (c0 + 0.02).astype(np.float32)[None]
+    c0 = c0 + rng.uniform(-0.05, 0.05, (props, c0.size)) * (np.arange(props) > 0)[:, None]
+    l0, u0 = (c0 - 0.02).astype(np.float32), (c0 + 0.02).astype(np.float32)
     fl, fu = oracle.ibp_bounds(on, l0.astype(np.float64), u0.astype(np.float64))
     flat = [np.concatenate([f[k] for k in range(1, on.n)], axis=1) for f in (fl, fu)]
     lbk, ubk = outward_f32(*flat)
     amb = np.nonzero((lbk[0] < 0) & (ubk[0] > 0))[0]
     masks = synth.split_masks(lbk.shape[1], B, amb, (0, 4), block=3)
-    return specs, on, l0, u0, lbk, ubk, np.zeros(B, np.int32), masks
+    return specs, on, l0, u0, lbk, ubk, (np.arange(B) % props).astype(np.int32), masks
 
 
-@pytest.mark.parametrize("name", sorted(NETS))
-def test_short_runs_match_bf16_oracle(name):
-    specs, on, l0, u0, lbk, ubk, prop, masks = _problem(name)
+# subdomains of one property, and of several in turn (every tile of columns mixes them)
+@pytest.mark.parametrize("name,props", [(n, 1) for n in sorted(NETS)] + [("odd_chunks", 2), ("cols_4", 3)])
+def test_short_runs_match_bf16_oracle(name, props):
+    specs, on, l0, u0, lbk, ubk, prop, masks = _problem(name, props)
     net = ldb.Net(specs)
     opts = ldb.Options(precision="bf16", engine="layerwise")
     for T in (1, 3):
