@@ -124,6 +124,20 @@ __device__ __forceinline__ void relu_argmin(T r, T c, T l, T u, T& xb, T& xk, in
   }
 }
 
+// relu_argmin without branches: the same comparisons on the same products, so
+// the same vertex for every input, NaN and infinite bounds included.
+__device__ __forceinline__ void relu_argmin_flat(float r, float c, float l, float u, float& xb, float& xk) {
+  const float d = r - c, mag = kTieRel * (fabsf(r) + fabsf(c));
+  const bool blk = u <= 0.f, pas = l >= 0.f;
+  const float v0 = r * l;
+  const bool zero = 0.f < v0;
+  const float best = zero ? 0.f : v0;
+  const bool uu = d * u < best - mag * fmaxf(-l, u);
+  const bool up = blk ? r <= 0.f : (pas ? d <= mag : uu);
+  xb = up ? u : (!blk && !pas && zero ? 0.f : l);
+  xk = blk ? 0.f : (pas || uu ? xb : 0.f);
+}
+
 // ---------------------------------------------------------------- epilogues
 // Transposed-pass epilogues receive (b, i, g) with g = (W_{k+1}^T rho_{k+1})[i]
 // for neuron i of layer k.  Forward-pass epilogues receive (b, j, acc) with
