@@ -39,6 +39,42 @@ __device__ __forceinline__ void stage_floats(float* dst, const float* src, int n
   for (int e = (n & ~3) + threadIdx.x; e < n; e += nt) stage4(dst + e, src + e, true);
 }
 
+// A division by a number the whole launch shares: a shift for a power of two.
+struct SharedDiv {
+  int d, sh;
+  __device__ __forceinline__ int of(int n) const { return sh >= 0 ? n >> sh : n / d; }
+};
+__device__ __forceinline__ SharedDiv shared_div(int d) { return SharedDiv{d, (d & (d - 1)) == 0 ? __ffs(d) - 1 : -1}; }
+
+// f(e, c, y, x) for the elements e = (c rows + y) pitch + x of a staged tile,
+// thread t taking e = t, t + nt, ...: the coordinates move on by those of nt
+// with two carries.  Two divisions an element made staging a tile as many
+// instructions as its products; with these, shifts in the items' indices and
+// pointers that step through the taps, 512 Wide subdomains: a transposed pass
+// into the image 27 -> 22 us, the evaluation call 376 -> 354 us; a proximal call
+// (256 Base subdomains, T = 100) 16.7 -> 16.3 ms.
+template <class F>
+__device__ __forceinline__ void tile_elements(int channels, int rows, int pitch, int nt, F f) {
+  const int plane = rows * pitch, n = channels * plane;
+  const int dc = nt / plane, dr = (nt - dc * plane) / pitch, dx = nt - dc * plane - dr * pitch;
+  int e = threadIdx.x, c = e / plane, y = (e - c * plane) / pitch, x = e - c * plane - y * pitch;
+  while (e < n) {
+    f(e, c, y, x);
+    e += nt;
+    x += dx;
+    y += dr;
+    c += dc;
+    if (x >= pitch) {
+      x -= pitch;
+      ++y;
+    }
+    if (y >= rows) {
+      y -= rows;
+      ++c;
+    }
+  }
+}
+
 // Weights of the transposed pass: [o][i][j][wc].
 __device__ __forceinline__ void conv_t_weights(const LayerDev& L, const ConvTile& T, float* sW, int nt) {
   const int nw = L.cout * L.cin * L.kh * L.kw;
@@ -52,13 +88,12 @@ __device__ __forceinline__ void conv_t_weights(const LayerDev& L, const ConvTile
 // The rows of r (one subdomain's [cout, ho, wo]) read by the band from phase row q0.
 __device__ __forceinline__ void conv_t_rows(const LayerDev& L, const ConvTile& T, float* sR, const float* rb, int q0,
                                             int nt) {
-  const int plane = T.rows * T.pitch, n = L.cout * plane, hw_o = L.ho * L.wo;
-  for (int e = threadIdx.x; e < n; e += nt) {
-    const int o = e / plane, rem = e - o * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
+  const int hw_o = L.ho * L.wo;
+  tile_elements(L.cout, T.rows, T.pitch, nt, [&](int e, int o, int yy, int xx) {
     const int y = q0 + yy + T.y_off, x = xx + T.x_off;
     const bool in = y >= 0 && y < L.ho && x >= 0 && x < L.wo;
     stage4(sR + e, rb + (in ? o * hw_o + y * L.wo + x : 0), in);
-  }
+  });
 }
 
 // f(channel, y, x, g) for every output of the band: a thread takes one
@@ -69,15 +104,13 @@ template <int KH, int KW, int ST, int G, class F>
 __device__ __forceinline__ void conv_t_items(const LayerDev& L, const ConvTile& T, const float* sW, const float* sR,
                                              int q0, int nq, int nt, F f) {
   const int qw = L.w / ST, ncg = L.cin / G, plane = T.rows * T.pitch;
-  const int items = ST * ST * ncg * nq * qw;
+  const int items = ST * ST * ncg * nq * qw, wstep = KH * KW * T.wc;
+  const SharedDiv d_qw = shared_div(qw), d_nq = shared_div(nq);
   for (int e = threadIdx.x; e < items; e += nt) {
-    int q = e;
-    const int rx = q % ST;
-    q /= ST;
-    const int qx = q % qw;
-    q /= qw;
-    const int qy = q % nq;
-    q /= nq;
+    int q = e / ST, r = d_qw.of(q);
+    const int rx = e - q * ST, qx = q - r * qw;
+    q = d_nq.of(r);
+    const int qy = r - q * nq;
     const int ry = q % ST;
     const int cg = q / ST;
     const int i0 = (ry + L.pad) % ST, j0 = (rx + L.pad) % ST;
@@ -94,9 +127,9 @@ __device__ __forceinline__ void conv_t_items(const LayerDev& L, const ConvTile& 
         const float* ra = rp - a * T.pitch - bb;
         const float* wa = wp + (ST * a * KW + ST * bb) * T.wc;
 #pragma unroll 8
-        for (int o = 0; o < L.cout; ++o) {
-          const float rv = ra[o * plane];
-          const float4 w = *reinterpret_cast<const float4*>(wa + o * KH * KW * T.wc);
+        for (int o = 0; o < L.cout; ++o, ra += plane, wa += wstep) {
+          const float rv = *ra;
+          const float4 w = *reinterpret_cast<const float4*>(wa);
           acc[0] = fmaf(w.x, rv, acc[0]);
           acc[1] = fmaf(w.y, rv, acc[1]);
           acc[2] = fmaf(w.z, rv, acc[2]);
@@ -121,33 +154,31 @@ template <int KH, int KW, int ST, int GF, class F>
 __device__ __forceinline__ void conv_f_items(const LayerDev& L, const ConvTile& T, const float* sW, const float* sX,
                                              int y0, int ny, int nt, F f) {
   const int nog = L.cout / GF, items = nog * ny * L.wo, plane = T.rows * T.pitch, half = T.pitch / ST;
+  const SharedDiv d_wo = shared_div(L.wo), d_ny = shared_div(ny);
   for (int e = threadIdx.x; e < items; e += nt) {
-    int r = e;
-    const int xo = r % L.wo;
-    r /= L.wo;
-    const int yo = r % ny;
-    const int og = r / ny;
+    const int r = d_wo.of(e), xo = e - r * L.wo;
+    const int og = d_ny.of(r), yo = r - og * ny;
     float acc[GF];
 #pragma unroll
     for (int g = 0; g < GF; ++g) acc[g] = 0.f;
     const float* xc = sX + yo * ST * T.pitch + xo;
     const float* wc = sW + og * GF;
 #pragma unroll 2
-    for (int c = 0; c < L.cin; ++c, xc += plane, wc += KH * KW * L.cout) {
+    for (int c = 0; c < L.cin; ++c, xc += plane) {
+      const float* xr = xc;
 #pragma unroll
-      for (int i = 0; i < KH; ++i)
+      for (int i = 0; i < KH; ++i, xr += T.pitch)
 #pragma unroll
-        for (int j = 0; j < KW; ++j) {
-          const float xv = xc[i * T.pitch + (j % ST) * half + j / ST];
-          const float* w = wc + (i * KW + j) * L.cout;
+        for (int j = 0; j < KW; ++j, wc += L.cout) {
+          const float xv = (j % ST ? xr + half : xr)[j / ST];
           if (GF == 4) {
-            const float4 w4 = *reinterpret_cast<const float4*>(w);
+            const float4 w4 = *reinterpret_cast<const float4*>(wc);
             acc[0] = fmaf(w4.x, xv, acc[0]);
             acc[1] = fmaf(w4.y, xv, acc[1]);
             acc[GF - 2] = fmaf(w4.z, xv, acc[GF - 2]);
             acc[GF - 1] = fmaf(w4.w, xv, acc[GF - 1]);
           } else {
-            const float2 w2 = *reinterpret_cast<const float2*>(w);
+            const float2 w2 = *reinterpret_cast<const float2*>(wc);
             acc[0] = fmaf(w2.x, xv, acc[0]);
             acc[1] = fmaf(w2.y, xv, acc[1]);
           }

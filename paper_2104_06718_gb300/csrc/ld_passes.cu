@@ -238,13 +238,12 @@ __global__ void __launch_bounds__(NT) conv_fwd_fast_kernel(LayerDev L, ConvTile 
   const int b = blockIdx.x / T.bands, y0 = (blockIdx.x % T.bands) * T.bh, ny = min(T.bh, L.ho - y0);
   stage_floats(sm, L.Wf, L.cout * L.cin * KH * KW, NT);
   const float* xb = x + (size_t)b * xs;
-  const int hw_i = L.h * L.w, plane = T.rows * T.pitch, n = L.cin * plane;
-  for (int e = threadIdx.x; e < n; e += NT) {
-    const int c = e / plane, rem = e - c * plane, yy = rem / T.pitch, xx = rem - yy * T.pitch;
+  const int hw_i = L.h * L.w;
+  tile_elements(L.cin, T.rows, T.pitch, NT, [&](int, int c, int yy, int xx) {
     const int y = y0 * ST + yy + T.y_off, xi = xx + T.x_off;
     const bool in = y >= 0 && y < L.h && xi >= 0 && xi < L.w;
     stage4(sX + conv_f_at(T, ST, c, yy, xx), xb + (in ? c * hw_i + y * L.w + xi : 0), in);
-  }
+  });
   stage_wait();
   double q = 0.0;
   conv_f_items<KH, KW, ST, GF>(L, T, sm, sX, y0, ny, NT, [&](int o, int y, int xo, float acc) {
