@@ -115,9 +115,8 @@ __device__ __forceinline__ void conv_t_items(const LayerDev& L, const ConvTile& 
     const int cg = q / ST;
     const int i0 = (ry + L.pad) % ST, j0 = (rx + L.pad) % ST;
     const int dy0 = (ry + L.pad - i0) / ST, dx0 = (rx + L.pad - j0) / ST;
-    float acc[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) acc[g] = 0.f;
+    // channel pairs in packed FMAs (two round-to-nearest FMAs each)
+    float2 a01 = make_float2(0.f, 0.f), a23 = a01;
     const float* rp = sR + (qy + dy0 - T.y_off) * T.pitch + qx + dx0 - T.x_off;
     const float* wp = sW + (i0 * KW + j0) * T.wc + cg * G;
 #pragma unroll
@@ -130,13 +129,16 @@ __device__ __forceinline__ void conv_t_items(const LayerDev& L, const ConvTile& 
         for (int o = 0; o < L.cout; ++o, ra += plane, wa += wstep) {
           const float rv = *ra;
           const float4 w = *reinterpret_cast<const float4*>(wa);
-          acc[0] = fmaf(w.x, rv, acc[0]);
-          acc[1] = fmaf(w.y, rv, acc[1]);
-          acc[2] = fmaf(w.z, rv, acc[2]);
-          if (G == 4) acc[G - 1] = fmaf(w.w, rv, acc[G - 1]);
+          const float2 rr = make_float2(rv, rv);
+          a01 = __ffma2_rn(make_float2(w.x, w.y), rr, a01);
+          if (G == 4)
+            a23 = __ffma2_rn(make_float2(w.z, w.w), rr, a23);
+          else
+            a23.x = fmaf(w.z, rv, a23.x);
         }
       }
     const int yy = ry + ST * (q0 + qy), xx = rx + ST * qx;
+    const float acc[4] = {a01.x, a01.y, a23.x, a23.y};
 #pragma unroll
     for (int g = 0; g < G; ++g) f(cg * G + g, yy, xx, acc[g]);
   }
@@ -158,9 +160,7 @@ __device__ __forceinline__ void conv_f_items(const LayerDev& L, const ConvTile& 
   for (int e = threadIdx.x; e < items; e += nt) {
     const int r = d_wo.of(e), xo = e - r * L.wo;
     const int og = d_ny.of(r), yo = r - og * ny;
-    float acc[GF];
-#pragma unroll
-    for (int g = 0; g < GF; ++g) acc[g] = 0.f;
+    float2 a01 = make_float2(0.f, 0.f), a23 = a01;  // channel pairs, as above
     const float* xc = sX + yo * ST * T.pitch + xo;
     const float* wc = sW + og * GF;
 #pragma unroll 2
@@ -173,17 +173,15 @@ __device__ __forceinline__ void conv_f_items(const LayerDev& L, const ConvTile& 
           const float xv = (j % ST ? xr + half : xr)[j / ST];
           if (GF == 4) {
             const float4 w4 = *reinterpret_cast<const float4*>(wc);
-            acc[0] = fmaf(w4.x, xv, acc[0]);
-            acc[1] = fmaf(w4.y, xv, acc[1]);
-            acc[GF - 2] = fmaf(w4.z, xv, acc[GF - 2]);
-            acc[GF - 1] = fmaf(w4.w, xv, acc[GF - 1]);
+            a01 = __ffma2_rn(make_float2(w4.x, w4.y), make_float2(xv, xv), a01);
+            a23 = __ffma2_rn(make_float2(w4.z, w4.w), make_float2(xv, xv), a23);
           } else {
             const float2 w2 = *reinterpret_cast<const float2*>(wc);
-            acc[0] = fmaf(w2.x, xv, acc[0]);
-            acc[1] = fmaf(w2.y, xv, acc[1]);
+            a01 = __ffma2_rn(w2, make_float2(xv, xv), a01);
           }
         }
     }
+    const float acc[4] = {a01.x, a01.y, a23.x, a23.y};
 #pragma unroll
     for (int g = 0; g < GF; ++g) f(og * GF + g, y0 + yo, xo, acc[g]);
   }
