@@ -222,7 +222,8 @@ ld_status ld_intermediate_bounds_split(ld_net* net, const float* lb0, const floa
  *   CROWN / WK bounds (and hence every reachable pre-activation).
  * The call grows a workspace of its own on first use (up to ~24 bytes per
  * objective row, rows = n_rows x rules x 2 x the widest layer, plus 256 MB
- * of coefficient buffers), like ld_net_reserve; LD_ERR_NOMEM if that fails.
+ * of coefficient buffers and, for the 32-row groups these hold, 768 bytes per
+ * group and partial-sum slot), like ld_net_reserve; LD_ERR_NOMEM if that fails.
  * Errors: LD_ERR_ARG (nulls, n_props < 1, n_rows < 0, bad rules, prop NULL
  * with n_rows != n_props and n_props > 1); LD_ERR_UNSUPPORTED (n_rows >
  * 65535); LD_ERR_NONFINITE via the status word as ld_intermediate_bounds. */
