@@ -818,12 +818,12 @@ ld_status ensure_ball_ws(ld_net* net, int B) {
 
 // q in FP32 terms (FP64 sum) via the forward form, +inf for empty subdomains.
 void final_fp32(ld_net* net, const Problem& P, double* out, float* sg, int8_t* vtx, cudaStream_t s) {
-  cudaMemsetAsync(net->acc, 0, sizeof(double) * (size_t)P.B, s);
+  cudaMemsetAsync(net->acc, 0, 2 * sizeof(double) * (size_t)P.B, s);
   ld::AdamStep st{};
   ld_opts o;
   ld_opts_default(&o);
   sweep(net, P, 1, o, st, sg, net->acc, vtx, nullptr, s);
-  if (out) ld::launch_record_finish(P, net->acc, out, s);
+  if (out) ld::launch_record_finish(P, net->acc, net->acc + P.B, out, s);
 }
 
 // T iterations of the FP32 layer-wise engine with q(rho_t) recorded before
@@ -1442,7 +1442,7 @@ ld_status ld_bound_dsg(ld_net* net, const float* lb0, const float* ub0, const fl
     if (out_dsg) {
       cudaMemsetAsync(D.dval, 0, sizeof(double) * B, s);
       dsg_sweep(net, P, D, 1, o, ld::AdamStep{}, s);
-      ld::launch_record_finish(P, D.dval, out_dsg, s);
+      ld::launch_record_finish(P, D.dval, nullptr, out_dsg, s);
     }
   }
   if (mu_out) cudaMemcpyAsync(mu_out, net->rho, sizeof(float) * BN, cudaMemcpyDeviceToDevice, s);

@@ -265,7 +265,7 @@ struct EpiRecord {
   const float* xB;
   const float* rho;
   float* sg;           // [B, N] or nullptr
-  double* q;           // [B] or nullptr
+  double* q;           // [2, B] (see finish) or nullptr
   __device__ __forceinline__ double operator()(int b, int jj, float acc) const {
     const float xa = acc + bias[jj / plane];
     if (last) return (double)xa;
@@ -274,8 +274,19 @@ struct EpiRecord {
     if (sg) sg[j] = s;
     return q ? (double)(rho[j] * s) : 0.0;
   }
+  // The CTAs of a subdomain arrive in any order, so a sum goes in as two: its
+  // multiple of 2^-20, added exactly (sums below 2^32), and the rest, at most
+  // 2^-21, whose own rounding is far below the last bit of q.
   __device__ __forceinline__ void finish(int b, double t) const {
-    if (q) atomicAdd(&q[b], t);
+    if (!q) return;
+    constexpr double kGrid = 6442450944.0;  // 1.5 2^32: ulp 2^-20
+    if (!(fabs(t) < 2147483648.0)) {  // as well infinities and NaN
+      atomicAdd(&q[b], t);
+      return;
+    }
+    const double hi = __dsub_rn(__dadd_rn(t, kGrid), kGrid);
+    atomicAdd(&q[b], hi);
+    atomicAdd(&q[P.B + b], __dsub_rn(t, hi));
   }
 };
 
@@ -781,7 +792,7 @@ struct FinalAcc {
   int slot;            // first slot of the launch
 };
 int final_slots(const LayerDev& Lnext, int top);
-void launch_record_finish(const Problem& P, const double* q, double* out, cudaStream_t s);
+void launch_record_finish(const Problem& P, const double* q, const double* rest, double* out, cudaStream_t s);
 // l2-ball input domains (Sec. 3.2.1, ld_ball.cu).
 // P0 over the ball: x0 = c + eps g_0 / ||g_0|| per subdomain, from g_0 left in
 // x[b, 0..n0) by the layer-0 transposed epilogue (EpiArgmin).

@@ -556,9 +556,9 @@ __global__ void final_combine_kernel(Problem P, FinalAcc a, double bn, double bn
   }
 }
 
-__global__ void record_finish_kernel(Problem P, const double* q, double* out) {
+__global__ void record_finish_kernel(Problem P, const double* q, const double* rest, double* out) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < P.B; b += gridDim.x * blockDim.x)
-    out[b] = P.empty[b] ? __longlong_as_double(0x7ff0000000000000LL) : q[b];
+    out[b] = P.empty[b] ? __longlong_as_double(0x7ff0000000000000LL) : (rest ? q[b] + rest[b] : q[b]);
 }
 
 }  // namespace
@@ -664,10 +664,10 @@ void launch_final_combine_bn(const Problem& P, FinalAcc acc, double bn, double b
 
 double final_gamma(double K) { return gamma_of(K); }
 
-void launch_record_finish(const Problem& P, const double* q, double* out, cudaStream_t s) {
+void launch_record_finish(const Problem& P, const double* q, const double* rest, double* out, cudaStream_t s) {
   if (P.B == 0) return;
   count_launch();
-  record_finish_kernel<<<(P.B + 255) / 256, 256, 0, s>>>(P, q, out);
+  record_finish_kernel<<<(P.B + 255) / 256, 256, 0, s>>>(P, q, rest, out);
 }
 
 // Slots used by the final pass of layer k+1 (transposed pass into layer k).
