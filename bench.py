@@ -67,14 +67,14 @@ METRIC = "LD subdomain bounds/s on Base/Wide/Deep convnets, bf16 vs fp32 at ≤1
 TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum of one launch of the fused kernels
     # (fused_kernel<2, 512, 0|1> on Base, <1, 512, 0|1> on Wide and Deep): read + write
-    ("base", "fp32", "fused", 2, 512, 256, 100): ("f3512387ae4d", 8013568),
-    ("base", "bf16", "fused tensor-core bf16", 2, 512, 256, 100): ("b20cd24da710", 8575232),
+    ("base", "fp32", "fused", 2, 512, 256, 100): ("40151aec76f4", 8019968),
+    ("base", "bf16", "fused tensor-core bf16", 2, 512, 256, 100): ("5f54da708e5e", 8312064),
     ("wide", "fp32", "fused", 1, 512, 2048, 100): ("f3512387ae4d", 119097600 + 98118144),
-    ("deep", "fp32", "fused", 1, 512, 128, 100): ("f3512387ae4d", 8338688),
-    ("deep", "bf16", "fused tensor-core bf16", 1, 512, 128, 100): ("b20cd24da710", 8386560),
+    ("deep", "fp32", "fused", 1, 512, 128, 100): ("40151aec76f4", 8330240),
+    ("deep", "bf16", "fused tensor-core bf16", 1, 512, 128, 100): ("5f54da708e5e", 8346368),
     # the same metrics over the 7 launches of one iteration of the layer-wise tensor-core engine
-    # (read 359.94 MB + write 75.89 MB) x the 100 iterations of its graph launch
-    ("wide", "bf16", "tensor-core bf16", 0, 0, 2048, 100): ("81ea16f36381", (359940352 + 75886592) * 100),
+    # (read 367.56 MB + write 71.45 MB) x the 100 iterations of its graph launch
+    ("wide", "bf16", "tensor-core bf16", 0, 0, 2048, 100): ("253437eea2ec", (367555584 + 71448320) * 100),
 }
 
 # The sources each timed engine is compiled from (besides the shared header
