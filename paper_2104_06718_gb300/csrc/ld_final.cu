@@ -62,8 +62,8 @@ __device__ __forceinline__ void add_term(TermSum& s, double t, float e) {
 // One per-neuron minimum, g within delta of the exact value.  box: P0 term
 // with coefficient -g on [l, u]; otherwise the Pk neuron with rho r.
 __device__ __forceinline__ void final_term(TermSum& s, bool box, float r, double g, float delta, float l, float u) {
-  if (!box && u <= 0.f) {             // blocking: min r*xB over [l,u], exact products
-    add_term(s, widen(r) * widen(r >= 0.f ? l : u), 0.f);
+  if (!box && u <= 0.f) {             // blocking: min r*xB over [l,u], exact products (r = 0: 0, also with l = -inf)
+    add_term(s, widen(r) * widen(r > 0.f ? l : u), 0.f);
     return;
   }
   const double d = box ? -g : widen(r) - g;  // coefficient of xB (and of x) in the box/passing/(u,u) cases
