@@ -17,8 +17,8 @@
 // started at 1.5 2^b with 2^(b-1) >= (k + 1) 2^(a-24), whose errors, at most
 // 2^(b-24) each, level 3 sums plainly; levels 2 and 3 are added in FP64 after
 // each block.  So |g - exact| <= delta = (k + k^2) 2^(b-47) a block + 2^-52 |g|,
-// below 2^-48 sum|W||rho| a block, where an FP64 sum has the bound gamma_k =
-// 2^-47 sum|W||rho| for 64 terms.  15 FP32 operations a term take the place of
+// at most 1.02 2^-48 sum|W||rho| a block (2^a <= 8 sum), where an FP64 sum has
+// the bound gamma_k = 2^-47 sum|W||rho| for 64 terms.  15 FP32 operations a term take the place of
 // one FP64 one (64 FP32 slots).  Geometries without a blocked path
 // sum in FP64 (the products are exact there) with delta = gamma_K A_i,
 // A_i >= sum |W||rho| in FP32 rounded up (Higham, gamma_K = K u / (1 - K u),
@@ -26,8 +26,10 @@
 // bound e on its error (from delta_i and the rounding of one subtraction and
 // one product) are summed per subdomain; the bound returned is
 //   S - E - gamma_M * sum|t|   (S = sum t, E = sum e, M = number of terms),
-// with t and S in FP64, and E and sum|t| summed (in FP32 within a block) rounding upward and scaled by 1 + 2 gamma_M as a
-// margin.  Partial sums go to fixed slots that one kernel adds in a fixed
+// with t and S in FP64, and E and sum|t| summed rounding upward (within a
+// block in FP32, values outside its middle range in FP64) and scaled by
+// 1 + 2 gamma_M as a margin.  Sums |W||rho| below 2^-59 or from 2^117 on, which
+// the levels do not hold, are formed again in FP64.  Partial sums go to fixed slots that one kernel adds in a fixed
 // order, so the bound does not depend on the order in which blocks run.
 #include <cmath>
 
@@ -39,10 +41,12 @@ namespace {
 constexpr int BN = 64, NT = 256;
 constexpr float kU52 = 2.220446049250313e-16f;  // 2^-52
 
-// Sums of a thread's terms: values, error bounds (up), |values| (up).
+// Sums of a thread's terms: values, error bounds (up), |values| (up); the last
+// two in FP32, with the terms outside its middle range in eo and ao.
 struct TermSum {
   double t = 0.0;
   float e = 0.f, a = 0.f;
+  double eo = 0.0, ao = 0.0;
 };
 
 // |x| rounded up to FP32, by integer instructions (at least 2^-126).
@@ -53,32 +57,77 @@ __device__ __forceinline__ float abs_up(double x) {
   return __uint_as_float(((hi - 0x38000000u) << 3 | lo >> 29) + 1u);
 }
 
-__device__ __forceinline__ void add_term(TermSum& s, double t, float e) {
-  s.t += t;
-  s.e = __fadd_ru(s.e, e);
-  s.a = __fadd_ru(s.a, abs_up(t));
+// Whether a sum or a term of this size is kept in FP32: 2^-80 to 2^100, or 0.
+__device__ __forceinline__ bool middle(float x) {
+  return x < 1.2676506002282294e30f && (x > 8.271806125530277e-25f || x == 0.f);
 }
 
-// One per-neuron minimum, g within delta of the exact value.  box: P0 term
+// Adds t, the minimum of exact values and of the product tx = c x, c within
+// delta of its exact value: e = |x| (delta + 2^-52 |c|) + 2^-52 |tx| (none where
+// c is exactly 0, also beside an infinite x).
+__device__ __noinline__ double term_error_fp64(double tx, double c, double x, double delta) {
+  const double ec = __dadd_ru(delta, __dmul_ru((double)kU52, fabs(c)));
+  return ec == 0.0 ? 0.0 : __dadd_ru(__dmul_ru(fabs(x), ec), __dmul_ru((double)kU52, fabs(tx)));
+}
+__device__ __forceinline__ void add_term(TermSum& s, double t, double tx, double c, float x, double delta) {
+  s.t += t;
+  s.eo = __dadd_ru(s.eo, term_error_fp64(tx, c, (double)x, delta));
+  s.ao = __dadd_ru(s.ao, fabs(t));
+}
+__device__ __forceinline__ void add_term(TermSum& s, double t, double tx, double c, float x, float delta) {
+  const float at = abs_up(t);
+  const float e = __fmaf_ru(x, __fmaf_ru(kU52, abs_up(c), delta), __fmul_ru(kU52, abs_up(tx)));
+  if (middle(at) && e < 1.2676506002282294e30f) {
+    s.t += t;
+    s.e = __fadd_ru(s.e, e);
+    s.a = __fadd_ru(s.a, at);
+  } else {
+    add_term(s, t, tx, c, x, (double)delta);
+  }
+}
+// A term without an error.
+__device__ __forceinline__ void add_exact(TermSum& s, double t) {
+  const float at = abs_up(t);
+  s.t += t;
+  if (middle(at))
+    s.a = __fadd_ru(s.a, at);
+  else
+    s.ao = __dadd_ru(s.ao, fabs(t));
+}
+
+// Sums over the lanes of each group of 2 * top lanes (all 32 lanes take part).
+__device__ __forceinline__ void reduce_terms(TermSum& s, int top) {
+  for (int off = top; off > 0; off >>= 1) {
+    s.t += __shfl_xor_sync(0xffffffffu, s.t, off);
+    s.e = __fadd_ru(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
+    s.a = __fadd_ru(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
+  }
+  if (__any_sync(0xffffffffu, s.eo != 0.0 || s.ao != 0.0))
+    for (int off = top; off > 0; off >>= 1) {
+      s.eo = __dadd_ru(s.eo, __shfl_xor_sync(0xffffffffu, s.eo, off));
+      s.ao = __dadd_ru(s.ao, __shfl_xor_sync(0xffffffffu, s.ao, off));
+    }
+}
+
+// One per-neuron minimum, g within delta of the exact value (D: float, or
+// double where delta may lie outside FP32's middle range).  box: P0 term
 // with coefficient -g on [l, u]; otherwise the Pk neuron with rho r.
-__device__ __forceinline__ void final_term(TermSum& s, bool box, float r, double g, float delta, float l, float u) {
+template <class D>
+__device__ __forceinline__ void final_term(TermSum& s, bool box, float r, double g, D delta, float l, float u) {
   if (!box && u <= 0.f) {             // blocking: min r*xB over [l,u], exact products (r = 0: 0, also with l = -inf)
-    add_term(s, widen(r) * widen(r > 0.f ? l : u), 0.f);
+    add_exact(s, widen(r) * widen(r > 0.f ? l : u));
     return;
   }
   const double d = box ? -g : widen(r) - g;  // coefficient of xB (and of x) in the box/passing/(u,u) cases
-  const float ed = __fmaf_ru(kU52, abs_up(d), delta);
   if (box || l >= 0.f) {              // P0 box, or passing: min d*xB over [l,u]
-    const double t = d * widen(d >= 0.0 ? l : u);
     // within delta of d the other end may be the minimum: either product is then within |d|_up max|x| of 0
-    const float xm = fmaxf(fabsf(l), fabsf(u));
-    add_term(s, t, __fmaf_ru(xm, ed, __fmul_ru(kU52, abs_up(t))));
+    const double t = d * widen(d >= 0.0 ? l : u);
+    add_term(s, t, t, d, fmaxf(fabsf(l), fabsf(u)), delta);
     return;
   }
   // ambiguous: vertices (l,0) -> r*l (exact), (0,0) -> 0, (u,u) -> d*u
   const double tuu = d * widen(u);
-  add_term(s, fmin(fmin(widen(r) * widen(l), 0.0), tuu),
-           __fmaf_ru(fabsf(u), ed, __fmul_ru(kU52, abs_up(tuu))));
+  add_term(s, fmin(fmin(widen(r) * widen(l), 0.0), tuu), tuu, d, fabsf(u), delta);
 }
 
 struct FinalEpi {
@@ -90,15 +139,16 @@ struct FinalEpi {
   int ball_norm;       // layer 0, l2 ball: the term is an upper bound on g_0[i]^2 (for ||g_0||)
   // abs_sum: bound on sum |W||rho| of an FP64 sum g
   __device__ __forceinline__ void term(int b, int i, double g, float abs_sum, TermSum& s) const {
-    term_delta(b, i, g, __fmul_ru(__double2float_ru(gamma_K), abs_sum), s);
+    term_delta(b, i, g, __dmul_ru(gamma_K, (double)abs_sum), s);
   }
   // delta: bound on |g - exact g|
-  __device__ __forceinline__ void term_delta(int b, int i, double g, float delta, TermSum& s) const {
+  template <class D>
+  __device__ __forceinline__ void term_delta(int b, int i, double g, D delta, TermSum& s) const {
     if (layer == 0) {
       if (ball_norm) {
         // |exact g_0[i]| <= |g| + delta: its square, rounded up
         const double a = __dadd_ru(fabs(g), (double)delta);
-        add_term(s, __dmul_ru(a, a), 0.f);
+        add_exact(s, __dmul_ru(a, a));
         return;
       }
       // the box; over an l2 ball l0 = u0 = the centre, which gives the
@@ -114,6 +164,25 @@ struct FinalEpi {
     final_term(s, false, rho[(size_t)b * P.N + j], g, delta, l, u);
   }
 };
+
+// FP64 sum of products and the FP32 sum of their sizes (up), for the sums that
+// the levels below do not hold; n more products.  Runs with no nonzero product
+// (duals that are all 0) cost no FP64 instruction.
+struct Sum64 {
+  double g;
+  float abs_sum;
+};
+__device__ __noinline__ Sum64 sum_fp64(Sum64 t, const float* w, size_t ws, const float* r, size_t rs, int n) {
+  bool any = false;
+  for (int i = 0; i < n; ++i) any = any || (w[i * ws] != 0.f && r[i * rs] != 0.f);
+  if (!any) return t;
+  for (int i = 0; i < n; ++i) {
+    const float wv = w[i * ws], rv = r[i * rs];
+    t.g = fma((double)wv, (double)rv, t.g);
+    t.abs_sum = __fmaf_ru(fabsf(wv), fabsf(rv), t.abs_sum);
+  }
+  return t;
+}
 
 // ---------------------------------------------------------------- three-level sums
 // b - a by one packed instruction (the product with -1 is exact).
@@ -132,9 +201,9 @@ struct Sum3x2 {
   }
   // 2^a from the sum of |rounded products|: 2^(a-1) is more than twice the sum,
   // which leaves room for the products' rounding and the level's own errors;
-  // sums below 2^-40 take that a (their errors are then far below any term's)
+  // sums below 2^-60 take that a (see result)
   static __device__ __forceinline__ float top(float s) {
-    const unsigned e = __float_as_uint(fmaxf(s, 9.094947017729282e-13f)) & 0x7f800000u;
+    const unsigned e = __float_as_uint(fmaxf(s, 8.673617379884035e-19f)) & 0x7f800000u;
     return __uint_as_float(e) * 8.f;
   }
   static __device__ __forceinline__ float binade(float p) { return __uint_as_float(__float_as_uint(p) & 0x7f800000u); }
@@ -166,16 +235,14 @@ struct Sum3x2 {
     q = t3;
     c = __fadd2_rn(c, sub2(e3, n2));
   }
-  // Value and bound of half h after the last block.
-  __device__ __forceinline__ void result(int h, float kk, double& g, float& delta) const {
+  // Value and bound of half h after the last block.  False for sums of sizes
+  // below 2^-59 (the bound would be an absolute one, and a product's low part
+  // could underflow), from 2^117 on, and NaN.
+  __device__ __forceinline__ bool result(int h, float kk, double& g, float& delta) const {
     const float ph = h ? p.y : p.x, two_a = binade(ph);
-    if (!(two_a < 1.329227995784916e36f)) {          // sums beyond 2^117: no value, an infinite bound (NaN stays)
-      g = ph == ph ? 0.0 : (double)ph;
-      delta = INFINITY;
-      return;
-    }
     g = widen(ph - 1.5f * two_a) + (h ? g1 : g0);
     delta = __fmaf_ru(kk, two_a, __fmul_ru(kU52, abs_up(g)));
+    return two_a > 6.938893903907228e-18f && two_a < 1.329227995784916e36f;  // 2^-57, 2^120
   }
 };
 // 2^(b-a) of level 2, 2^(b-1) >= (k + 1) 2^(a-24) for blocks of at most k =
@@ -223,7 +290,7 @@ __device__ __forceinline__ void acc_add(FinalAcc a, int slot, int b, double t, d
 // 64-row grid would leave SMs idle; the column blocks, and so the partial-sum
 // slots, are the same either way), a thread TM x 4 of it; up to KS rows of K
 // staged at once.
-constexpr int KS = 128;
+constexpr int KS = 128;  // a multiple of kBlk: blocks end where rounds do
 template <int TM>
 __global__ void __launch_bounds__(NT) final_fc_kernel(int M, int Ncol, int K, const float* __restrict__ A, int lda,
                                                       const float* __restrict__ W, int ldw, FinalEpi epi,
@@ -305,45 +372,37 @@ __global__ void __launch_bounds__(NT) final_fc_kernel(int M, int Ncol, int K, co
         if (n >= Ncol) continue;
         double g;
         float delta;
-        acc[i][j / 2].result(j % 2, sc.kk, g, delta);
-        epi.term_delta(m, n, g, delta, s);
+        if (acc[i][j / 2].result(j % 2, sc.kk, g, delta)) {
+          epi.term_delta(m, n, g, delta, s);
+        } else {
+          const Sum64 v = sum_fp64(Sum64{0.0, 0.f}, W + n, ldw, A + (size_t)m * lda, 1, K);
+          epi.term(m, n, v.g, v.abs_sum, s);
+        }
       }
     }
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) {
-      s.t += __shfl_xor_sync(0xffffffffu, s.t, off);
-      s.e = __fadd_ru(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
-      s.a = __fadd_ru(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
-    }
-    if (tx == 0 && m < M) acc_add(acc_out, acc_out.slot + blockIdx.x, m, s.t, (double)s.e, (double)s.a);
+    reduce_terms(s, 8);
+    if (tx == 0 && m < M)
+      acc_add(acc_out, acc_out.slot + blockIdx.x, m, s.t, __dadd_ru((double)s.e, s.eo), __dadd_ru((double)s.a, s.ao));
   }
 }
 
 __device__ __forceinline__ void block_reduce_add(FinalAcc a, int slot, int b, TermSum s) {
-  __shared__ double rt[NT / 32];
-  __shared__ float re[NT / 32], ra[NT / 32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    s.t += __shfl_xor_sync(0xffffffffu, s.t, off);
-    s.e = __fadd_ru(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
-    s.a = __fadd_ru(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
-  }
+  __shared__ double red[3][NT / 32];
+  reduce_terms(s, 16);
   const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (lane == 0) {
-    rt[w] = s.t;
-    re[w] = s.e;
-    ra[w] = s.a;
+    red[0][w] = s.t;
+    red[1][w] = __dadd_ru((double)s.e, s.eo);
+    red[2][w] = __dadd_ru((double)s.a, s.ao);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    float e = 0.f, at = 0.f;
-    for (int i = 0; i < (int)(blockDim.x / 32); ++i) {
-      t += rt[i];
-      e = __fadd_ru(e, re[i]);
-      at = __fadd_ru(at, ra[i]);
+  if (threadIdx.x < 3) {  // a thread each for t, e and a
+    double v = red[threadIdx.x][0];
+    for (int i = 1; i < (int)(blockDim.x / 32); ++i) {
+      const double x = red[threadIdx.x][i];
+      v = threadIdx.x == 0 ? v + x : __dadd_ru(v, x);
     }
-    acc_add(a, slot, b, t, (double)e, (double)at);
+    a.slots[((size_t)b * a.n_slots + slot) * 3 + threadIdx.x] = v;
   }
 }
 
@@ -469,8 +528,16 @@ __global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, ConvTil
     for (int g = 0; g < G; ++g) {
       double gv;
       float delta;
-      (g / 2 ? a1 : a0).result(g % 2, sc.kk, gv, delta);
-      epi.term_delta(b, ((cg * G + g) * L.h + yy) * L.w + xx, gv, delta, s);
+      const int c = cg * G + g, i = (c * L.h + yy) * L.w + xx;
+      if ((g / 2 ? a1 : a0).result(g % 2, sc.kk, gv, delta)) {
+        epi.term_delta(b, i, gv, delta, s);
+      } else {
+        Sum64 v{0.0, 0.f};
+        for (int a = 0; a < KH / ST; ++a)
+          for (int bb = 0; bb < KW / ST; ++bb)
+            v = sum_fp64(v, wp + (ST * a * KW + ST * bb) * T.wc + g, KH * KW * T.wc, rp - a * T.pitch - bb, plane, L.cout);
+        epi.term(b, i, v.g, v.abs_sum, s);
+      }
     }
   }
   block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s);
@@ -503,9 +570,9 @@ __global__ void __launch_bounds__(NT) final_top_kernel(int n, const float* __res
   TermSum s;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     if (Wn64)
-      epi.term_delta(b, i, -Wn64[i], abs_up(Wn_err[i]), s);
+      epi.term_delta(b, i, -Wn64[i], Wn_err[i], s);
     else
-      epi.term_delta(b, i, -widen(Wn[i]), 0.f, s);
+      epi.term_delta(b, i, -widen(Wn[i]), 0.0, s);
   }
   block_reduce_add(acc_out, acc_out.slot, b, s);
 }
@@ -526,7 +593,7 @@ __global__ void __launch_bounds__(NT) final_bias_kernel(Problem P, BiasLayers BL
   for (int k = 0; k < BL.count; ++k)
 #pragma unroll 4
     for (int i = threadIdx.x; i < BL.n[k]; i += blockDim.x)
-      add_term(s, -widen(rho[(size_t)b * P.N + BL.r_off[k] + i]) * widen(__ldg(BL.bias[k] + i / BL.plane[k])), 0.f);
+      add_exact(s, -widen(rho[(size_t)b * P.N + BL.r_off[k] + i]) * widen(__ldg(BL.bias[k] + i / BL.plane[k])));
   block_reduce_add(acc_out, acc_out.slot, b, s);
 }
 
@@ -585,7 +652,7 @@ void launch_fc(const LayerDev& L, const Problem& P, const float* r, const FinalE
     cudaFuncSetAttribute(final_fc_kernel<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   dim3 grid((L.n_in + BN - 1) / BN, (P.B + BMt - 1) / BMt);
   final_fc_kernel<TM><<<grid, NT, smem, s>>>(P.B, L.n_in, L.n_out, r, P.N, L.W, L.n_in, epi,
-                                             sum3_const((L.n_out + kBlk - 1) / kBlk + L.n_out / KS, L.n_out), acc);
+                                             sum3_const((L.n_out + kBlk - 1) / kBlk, L.n_out), acc);
 }
 
 int sm_count() {
