@@ -146,9 +146,10 @@ struct FinalEpi {
   __device__ __forceinline__ void term_delta(int b, int i, double g, D delta, TermSum& s) const {
     if (layer == 0) {
       if (ball_norm) {
-        // |exact g_0[i]| <= |g| + delta: its square, rounded up
+        // |exact g_0[i]| <= |g| + delta: its square, rounded up (in FP64: the
+        // sum of these is the square of the norm itself, not a slack)
         const double a = __dadd_ru(fabs(g), (double)delta);
-        add_exact(s, __dmul_ru(a, a));
+        s.ao = __dadd_ru(s.ao, __dmul_ru(a, a));
         return;
       }
       // the box; over an l2 ball l0 = u0 = the centre, which gives the

@@ -93,3 +93,19 @@ def test_as_close_as_fp64_sums(name, case):
     lo, up, _ = oracle.apply_masks(on, oracle.layer_lists(on, rep(lbk)), oracle.layer_lists(on, rep(ubk)), masks)
     sol = oracle.inner_minimisation(on, rep(l0), rep(u0), lo, up, oracle.layer_lists(on, rho.astype(np.float64)))
     _check(got, sol.q, on, l0, u0, lbk, ubk, rho, sol.g)
+
+
+@pytest.mark.parametrize("name", sorted(NETS))
+def test_ball_norm(name):
+    """The l2 ball's term -eps ||g_0|| is as exact as the others: ||g_0||^2 is an FP64 sum, not an error bound."""
+    specs, on, l0, u0, lbk, ubk, rho = _problem(name, dual=1.0, zero_rows=True)
+    B, eps = rho.shape[0], np.float32(3.0)
+    masks = np.zeros(rho.shape, np.int8)
+    c = (l0 + u0) / 2
+    got = ldb.ld_bound_ball(ldb.Net(specs), c, [eps], lbk, ubk, np.zeros(B, np.int32), masks, n_iters=0, rho_in=rho,
+                            opts=ldb.Options(init="given", engine="layerwise")).cpu().numpy()
+    rep = lambda a: np.repeat(a.astype(np.float64), B, axis=0)
+    lo, up, _ = oracle.apply_masks(on, oracle.layer_lists(on, rep(lbk)), oracle.layer_lists(on, rep(ubk)), masks)
+    sol = oracle.inner_minimisation(on, rep(c), rep(c), lo, up, oracle.layer_lists(on, rho.astype(np.float64)),
+                                    ball_eps=np.full(B, np.float64(eps)))
+    _check(got, sol.q, on, c, c, lbk, ubk, rho, sol.g)
