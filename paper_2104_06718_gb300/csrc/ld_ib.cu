@@ -71,6 +71,8 @@ constexpr int kTerms = 16;         // most scalar terms of a row between two FP6
 constexpr int kMaxChunks = 64;     // CTAs of a group
 constexpr int kWarpWork = 1024;    // terms a warp should have (2 to 8 units): its fixed cost is a few hundred instructions
 constexpr int kFcRows = 128;       // FC weight rows staged at once (a CTA has one unit per warp)
+// Most staged weights of a conv: 12288 of them, one input channel padded to four.
+constexpr size_t kStageMost = sizeof(float) * 4 * 12288;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr float kTwoU = 1.1920928955078125e-07f;  // 2^-23, twice the FP32 unit roundoff
 
@@ -783,7 +785,7 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
                     : st.cp == 64 ? ib_step_kernel<64>
                                   : ib_step_kernel<0>;
       if (smem > 40 * 1024) {
-        const cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+        const cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageMost);
         if (ea != cudaSuccess) return ea;
       }
       count_launch();
