@@ -46,17 +46,24 @@
 // relaxation valid (a_bar upward, b_bar upward; any lower slope in [0,1] is
 // valid), and a rounded mu_j product lowers the bound by its rounding error
 // times max|x_hat_j|.  The scalar terms of a row (box, bias and intercept
-// products) are exact FP32 product pairs summed by the same Dot2 for one unit's
-// terms (at most 16), then added in FP64: GB300 runs 2 FP64 operations per clock
-// and SM against 128 FP32 ones, and an FP64 epilogue cost more than the sums.
-// The error of that is at most gamma_32^2 of a block's |terms| (FP32 gamma)
-// plus gamma_M (FP64) times the sum of |terms|; the error bounds and the sum
-// of |terms| themselves are FP32 sums rounded upward.  So the returned bounds
-// contain the exact CROWN/WK bounds (outward), like the interval bounds.
+// products) are exact FP32 product pairs summed by the same Dot2 in two halves of
+// at most 16 terms, then added in FP64: GB300 runs 2 FP64 operations per clock
+// and SM against 128 FP32 ones (64 Base subdomains: 6.1 ms with one FP64 FMA a
+// term, 4.7 with a third level of errors, 3.7 with Dot2).  That leaves at
+// most 16^2 2^-48 of a block's |terms| beside the gamma_M (FP64) of the sum of
+// |terms|; kErrA gives back more than that, so the bounds are no wider than with
+// FP64 sums.  Products below 2^-102, which have no exact low part (2^-150 each),
+// are covered by 2^-126 a row; a CTA whose terms or errors sum to 2^100 or more
+// runs its units again with FP64 terms (a test and a branch a term instead cost
+// that call 15 to 20%).  The error bounds are summed in FP32 over a block, in FP64
+// over the blocks, the sizes of the terms in FP32 over a thread's units, all
+// rounded upward.  So the returned bounds contain the exact CROWN/WK bounds
+// (outward), like the interval bounds.
 //
 // A row's value does not depend on the other rows of a call: the elements of a
 // layer are dealt to CTAs and warps by the layer's geometry alone.
 #include <algorithm>
+#include <cmath>
 
 #include "ld_common.cuh"
 
@@ -67,7 +74,7 @@ constexpr int NW = 8;              // warps per CTA
 constexpr int NT = 32 * NW;
 constexpr int kUnitC = 8;          // elements per unit (channels of a position / consecutive FC inputs)
 constexpr int kPairs = kUnitC / 2;
-constexpr int kTerms = 16;         // most scalar terms of a row between two FP64 flushes (a unit has up to 2 kUnitC)
+constexpr int kAdds = 16;          // most scalar terms of each half of a row's sum between two FP64 flushes
 constexpr int kMaxChunks = 64;     // CTAs of a group
 constexpr int kWarpWork = 1024;    // terms a warp should have (2 to 8 units): its fixed cost is a few hundred instructions
 constexpr int kFcRows = 128;       // FC weight rows staged at once (a CTA has one unit per warp)
@@ -75,6 +82,12 @@ constexpr int kFcRows = 128;       // FC weight rows staged at once (a CTA has o
 constexpr size_t kStageMost = sizeof(float) * 4 * 12288;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr float kTwoU = 1.1920928955078125e-07f;  // 2^-23, twice the FP32 unit roundoff
+// The rounding of p + c is at most 2^-24 |a|; 2^-23 (1 - 2^-13) is charged for it.
+// The 2^-13 is more than the bounds lose by FP32 scalar terms and error sums: a
+// box or intercept term is at most |a| times what its error multiplies, so it
+// gives back 2^-36 of their sizes (2^-40 are charged) and 2^-13 of the error.
+constexpr float kErrA = 1.1920928955078125e-07f * (1.f - 1.220703125e-04f);
+constexpr float kHuge = 1.2676506002282294e30f;   // 2^100
 
 // Window of a group's nonzero coefficients on a plane: full, or hh x ww from
 // (oy * mul - sub, ox * mul - sub) for the group's position (oy, ox).
@@ -260,29 +273,60 @@ struct UnitSums {
   }
 };
 
-// A row's scalar terms: the pair (d.p, d.c) of the current block, the FP64
-// sum of the finished ones, sum |terms| and the error bound (FP32, rounded up).
+// A row's scalar terms: the current block's sum (d, two halves) and error bound
+// e, with sum |terms| in d.s, and the finished blocks (v, ev); WIDE: all in FP64.
+template <bool WIDE>
 struct RowSum {
-  Dot2 d;
-  double v = 0.0;
+  Pair d;
   float e = 0.f;
-  __device__ __forceinline__ void flush() {
-    v += widen(d.p);
-    v += widen(d.c);
-    d.p = d.c = 0.f;
+  double v = 0.0, ev = 0.0, sv = 0.0;
+  __device__ __forceinline__ void add(float2 x, float2 a) {
+    if (WIDE) {
+      const double t0 = (double)x.x * (double)a.x, t1 = (double)x.y * (double)a.y;
+      v += t0;
+      v += t1;
+      sv = __dadd_ru(sv, __dadd_ru(fabs(t0), fabs(t1)));
+    } else {
+      d.add(x, a, make_float2(-a.x, -a.y));
+    }
   }
+  // An error of a coefficient times the size of what it multiplies.
+  __device__ __forceinline__ void error(float da, float x) {
+    if (WIDE)
+      ev = __dadd_ru(ev, __dmul_ru((double)da, (double)x));
+    else
+      e = __fmaf_ru(da, x, e);
+  }
+  __device__ __forceinline__ void flush() {
+    if (WIDE) return;
+    v += widen(d.p.x);
+    v += widen(d.p.y);
+    v += widen(d.c.x) + widen(d.c.y);
+    ev = __dadd_ru(ev, widen(e));
+    d.p = d.c = make_float2(0.f, 0.f);
+    e = 0.f;
+  }
+  __device__ __forceinline__ double size() const {
+    return WIDE ? sv : (double)__fmul_ru(__fadd_ru(d.s.x, d.s.y), 1.f + 2.f * kTwoU);
+  }
+  // Whether the sums left FP32's range (infinities and NaN among them), after the last flush.
+  __device__ __forceinline__ bool beyond() const { return !WIDE && !(size() < (double)kHuge && ev < (double)kHuge); }
 };
 
-// One element's contribution to the row and its coefficient for the next
-// pass: a with error bound da, on the input interval [l, u] (box) or through
-// the relaxation of a ReLU with bounds [l, u] and bias b.
-__device__ __forceinline__ void box_term(RowSum& R, float a, float da, float l, float u) {
-  const float x = a >= 0.f ? l : u;                 // min(a l, a u)
-  R.d.add(x, a);
-  R.e = __fmaf_ru(da, fmaxf(fabsf(l), fabsf(u)), R.e);
+// Two elements' contribution to the row: coefficients a with error bounds da on
+// the input intervals [l, u] (a = da = l = u = 0: none).
+template <bool WIDE>
+__device__ __forceinline__ void box_terms(RowSum<WIDE>& R, float2 a, float2 da, float2 l, float2 u) {
+  R.add(make_float2(a.x >= 0.f ? l.x : u.x, a.y >= 0.f ? l.y : u.y), a);  // min(a l, a u)
+  R.error(da.x, fmaxf(fabsf(l.x), fabsf(u.x)));
+  R.error(da.y, fmaxf(fabsf(l.y), fabsf(u.y)));
 }
 
-__device__ __forceinline__ float relu_term(RowSum& R, float a, float da, float l, float u, float b, int rule) {
+// The coefficient of the next pass: a with error bound da through the relaxation
+// of a ReLU with bounds [l, u]; ic: the intercept that multiplies a, or 0.
+template <bool WIDE>
+__device__ __forceinline__ float relu_coeff(RowSum<WIDE>& R, float a, float da, float l, float u, int rule, float& ic) {
+  ic = 0.f;
   if (u <= 0.f) return 0.f;                         // blocking: x = 0, nothing to relax
   float m = a;                                      // passing: x = x_hat
   if (l < 0.f) {
@@ -292,24 +336,26 @@ __device__ __forceinline__ float relu_term(RowSum& R, float a, float da, float l
       m = slo * a;
     } else {
       m = ab * a;
-      R.d.add(__fmul_ru(-l, ab), a);                // upper intercept, rounded up
+      ic = __fmul_ru(-l, ab);                       // upper intercept, rounded up
     }
     // rounding of the product mu = slope * a, times max |x_hat|
-    R.e = __fmaf_ru(__fmul_ru(kTwoU, fabsf(m)), fmaxf(-l, u), R.e);
+    R.error(__fmul_ru(kTwoU, fabsf(m)), fmaxf(-l, u));
   }
-  R.d.add(b, m);
   // the pass's own rounding, times max x_{j-1} = max(u, 0)
-  R.e = __fmaf_ru(da, u, R.e);
+  R.error(da, u);
   return m;
 }
 
-// A CTA's sums of its rows into the chunk's slot.
-__device__ __forceinline__ void store_part(const IbStep& st, const IbRowMap& M, int gl, int chunk,
-                                           double (*red)[32][3], const RowSum& R) {
+// A CTA's sums of its rows into the chunk's slot; false (nothing stored): some
+// left FP32's range.
+template <bool WIDE>
+__device__ __forceinline__ bool store_part(const IbStep& st, const IbRowMap& M, int gl, int chunk,
+                                           double (*red)[32][3], const RowSum<WIDE>& R) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (!WIDE && __syncthreads_or(R.beyond())) return false;
   red[warp][lane][0] = R.v;
-  red[warp][lane][1] = (double)R.d.size();
-  red[warp][lane][2] = (double)R.e;
+  red[warp][lane][1] = R.size();
+  red[warp][lane][2] = R.ev;
   __syncthreads();
   if (threadIdx.x < 96) {
     const int q = threadIdx.x / 32;
@@ -317,6 +363,7 @@ __device__ __forceinline__ void store_part(const IbStep& st, const IbRowMap& M, 
     for (int w = 1; w < NW; ++w) t = q == 0 ? t + red[w][lane][q] : __dadd_ru(t, red[w][lane][q]);
     st.part[(((size_t)st.slot + chunk) * M.n_groups * 32 + (size_t)gl * 32 + lane) * 3 + q] = t;
   }
+  return true;
 }
 
 // One CTA: units [chunk * units_per_cta, ...) of one group of 32 rows; a unit
@@ -328,10 +375,8 @@ __device__ __forceinline__ void store_part(const IbStep& st, const IbRowMap& M, 
 // loads, votes and addresses were most of the instructions.
 // CP: floats of a staged weight row where it is one of the usual sizes (the
 // four rows of an unrolled step are then immediate offsets), else 0.
-template <int CP>
-__global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
-  extern __shared__ float sw[];
-  __shared__ double red[NW][32][3];
+template <int CP, bool WIDE>
+__device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, float* sw, double (*red)[32][3]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gl = blockIdx.x / st.chunks, chunk = blockIdx.x % st.chunks;
   const IbRow r = ib_row(M, M.group0 + gl, lane);
@@ -358,7 +403,7 @@ __global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
   const int so = conv ? r.i / (L.ho * L.wo) : 0;
   const float sg = r.valid ? r.sign : 0.f;
   const int hw = conv ? L.h * L.w : 1, ostep = conv ? st.wout.hh * st.wout.ww : 1;
-  RowSum R;
+  RowSum<WIDE> R;
   int done = 0;
   const int u_lo = chunk * st.units_per_cta, u_hi = min(st.units, u_lo + st.units_per_cta);
   for (int ub = u_lo; ub < u_hi; ub += NW) {
@@ -438,41 +483,80 @@ __global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
       }
     }
     const int ky = y + L.pad - r.oy * L.stride, kx = x + L.pad - r.ox * L.stride;
-    for (int e = 0; act; ++e) {
-      const int c = c0 + __ffs(act) - 1, ii = ib + c * hw;
+    // the elements' sums in pairs, the odd one last with an empty second half
+    for (int k = 0; act; ++k) {
+      const bool two = k < S.np;
+      int c[2], ii[2];
+      c[0] = c0 + __ffs(act) - 1;
       act &= act - 1;
-      // the element's sum: half e % 2 of pair e / 2, or the odd one
-      Dot2 d = S.one;
+      c[1] = two ? c0 + __ffs(act) - 1 : c[0];
+      act &= act - (two ? 1u : 0u);
+      ii[0] = ib + c[0] * hw;
+      ii[1] = ib + c[1] * hw;
+      Pair D = S.d[0];
 #pragma unroll
-      for (int k = 0; k < kPairs; ++k) {
-        const bool lo = k < S.np && e == 2 * k, hi = k < S.np && e == 2 * k + 1;
-        d.p = lo ? S.d[k].p.x : hi ? S.d[k].p.y : d.p;
-        d.c = lo ? S.d[k].c.x : hi ? S.d[k].c.y : d.c;
-        d.s = lo ? S.d[k].s.x : hi ? S.d[k].s.y : d.s;
+      for (int q = 1; q < kPairs; ++q)
+        if (k == q) D = S.d[q];
+      if (!two) {
+        D.p = make_float2(S.one.p, 0.f);
+        D.c = make_float2(S.one.c, 0.f);
+        D.s = make_float2(S.one.s, 0.f);
       }
       if (st.seed) {
-        if (!conv) d.p = sg * __ldg(L.W + (size_t)r.i * L.n_in + c);
-        else if (ky >= 0 && ky < L.kh && kx >= 0 && kx < L.kw)
-          d.p = sg * __ldg(L.W + (((size_t)so * L.cin + c) * L.kh + ky) * L.kw + kx);
-        else
-          d.p = 0.f;
+        float w[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          w[h] = 0.f;
+          if (h && !two) continue;
+          if (!conv) w[h] = sg * __ldg(L.W + (size_t)r.i * L.n_in + c[h]);
+          else if (ky >= 0 && ky < L.kh && kx >= 0 && kx < L.kw)
+            w[h] = sg * __ldg(L.W + (((size_t)so * L.cin + c[h]) * L.kh + ky) * L.kw + kx);
+        }
+        D.p = make_float2(w[0], w[1]);
       }
-      const float l = __ldg(lp + ii), u = __ldg(up + ii);
-      const float a = d.value();
-      const float da = st.seed ? 0.f : __fmaf_ru(st.g2, d.size(), __fmul_ru(kTwoU, fabsf(a)));
+      const float2 l = make_float2(__ldg(lp + ii[0]), two ? __ldg(lp + ii[1]) : 0.f);
+      const float2 u = make_float2(__ldg(up + ii[0]), two ? __ldg(up + ii[1]) : 0.f);
+      const float2 a = __fadd2_rn(D.p, D.c);
+      float2 da = make_float2(0.f, 0.f);
+      if (!st.seed) {
+        da.x = __fmaf_ru(st.g2, __fmul_ru(D.s.x, 1.f + 2.f * kTwoU), __fmul_ru(kErrA, fabsf(a.x)));
+        da.y = __fmaf_ru(st.g2, __fmul_ru(D.s.y, 1.f + 2.f * kTwoU), __fmul_ru(kErrA, fabsf(a.y)));
+      }
       if (st.box) {
-        box_term(R, a, da, l, u);
+        box_terms(R, a, da, l, u);
       } else {
-        const float m = (a == 0.f && d.s == 0.f)
-                            ? 0.f
-                            : relu_term(R, a, da, l, u, __ldg(st.bias_prev + ii / st.plane_prev), r.rule);
-        out[(size_t)(eb + c * ostep) * 32] = m;
+        float2 m = make_float2(0.f, 0.f), ic = m, bias = m;
+        if (!(a.x == 0.f && D.s.x == 0.f)) {
+          m.x = relu_coeff(R, a.x, da.x, l.x, u.x, r.rule, ic.x);
+          bias.x = __ldg(st.bias_prev + ii[0] / st.plane_prev);
+        }
+        if (!(a.y == 0.f && D.s.y == 0.f)) {
+          m.y = relu_coeff(R, a.y, da.y, l.y, u.y, r.rule, ic.y);
+          bias.y = __ldg(st.bias_prev + ii[1] / st.plane_prev);
+        }
+        if (ic.x != 0.f || ic.y != 0.f) R.add(ic, a);
+        R.add(bias, m);
+        out[(size_t)(eb + c[0] * ostep) * 32] = m.x;
+        if (two) out[(size_t)(eb + c[1] * ostep) * 32] = m.y;
       }
     }
     if (++done % st.flush == 0) R.flush();
   }
   R.flush();
-  store_part(st, M, gl, chunk, red, R);
+  return store_part(st, M, gl, chunk, red, R);
+}
+
+// The FP64 form, out of line.
+template <int CP>
+__device__ __noinline__ void ib_step_wide(const IbStep& st, const IbRowMap& M, float* sw, double (*red)[32][3]) {
+  ib_step<CP, true>(st, M, sw, red);
+}
+template <int CP>
+__global__ void __launch_bounds__(NT, 3) ib_step_kernel(const __grid_constant__ IbStep st,
+                                                        const __grid_constant__ IbRowMap M) {
+  extern __shared__ __align__(16) float sw[];
+  __shared__ double red[NW][32][3];
+  if (!ib_step<CP, false>(st, M, sw, red)) ib_step_wide<CP>(st, M, sw, red);
 }
 
 // The input box of a conv first layer of C <= 4 channels: a unit is two
@@ -483,10 +567,9 @@ __global__ void __launch_bounds__(NT, 3) ib_step_kernel(IbStep st, IbRowMap M) {
 // and votes were two thirds of the instructions.  Base, 3 channels: a call of
 // 64 subdomains 5.48 -> 3.38 ms, FSB's children of 256 subdomains 1.42 -> 1.09
 // ms, Deep's root bounds 0.685 -> 0.542 ms.
-template <int C>
-__global__ void __launch_bounds__(NT, 3) ib_box_kernel(IbStep st, IbRowMap M) {
-  extern __shared__ __align__(16) float sw[];  // [tap][o][4]
-  __shared__ double red[NW][32][3];
+template <int C, bool WIDE>
+__device__ __forceinline__ bool ib_box(const IbStep& st, const IbRowMap& M, float* sw /* [tap][o][4] */,
+                                       double (*red)[32][3]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gl = blockIdx.x / st.chunks, chunk = blockIdx.x % st.chunks;
   const IbRow r = ib_row(M, M.group0 + gl, lane);
@@ -504,7 +587,7 @@ __global__ void __launch_bounds__(NT, 3) ib_box_kernel(IbStep st, IbRowMap M) {
   const float* lp = st.l0 + (size_t)box_of(st, r.owner) * st.n0;
   const float* up = st.u0 + (size_t)box_of(st, r.owner) * st.n0;
   const int S = L.stride, estep = st.win.hh * st.win.ww * 32, per_row = box_units(S, st.wout.ww);
-  RowSum R;
+  RowSum<WIDE> R;
   int done = 0;
   const int u_hi = min(st.units, (chunk + 1) * st.units_per_cta);
   for (int un = chunk * st.units_per_cta + warp; un < u_hi; un += NW) {
@@ -550,19 +633,41 @@ __global__ void __launch_bounds__(NT, 3) ib_box_kernel(IbStep st, IbRowMap M) {
       }
     }
 #pragma unroll
-    for (int c = 0; c < C; ++c)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (!(h ? in1 : in0)) continue;
-        const int ii = (c * L.h + y) * L.w + x + h * S;
-        const float a = h ? __fadd_rn(d[c].p.y, d[c].c.y) : __fadd_rn(d[c].p.x, d[c].c.x);
-        const float s = __fmul_ru(h ? d[c].s.y : d[c].s.x, 1.f + 2.f * kTwoU);
-        box_term(R, a, __fmaf_ru(st.g2, s, __fmul_ru(kTwoU, fabsf(a))), __ldg(lp + ii), __ldg(up + ii));
+    for (int c = 0; c < C; ++c) {
+      const int i0 = (c * L.h + y) * L.w + x, i1 = i0 + S;
+      float2 a = __fadd2_rn(d[c].p, d[c].c), da, l = make_float2(0.f, 0.f), u = l;
+      da.x = __fmaf_ru(st.g2, __fmul_ru(d[c].s.x, 1.f + 2.f * kTwoU), __fmul_ru(kErrA, fabsf(a.x)));
+      da.y = __fmaf_ru(st.g2, __fmul_ru(d[c].s.y, 1.f + 2.f * kTwoU), __fmul_ru(kErrA, fabsf(a.y)));
+      if (in0) {
+        l.x = __ldg(lp + i0);
+        u.x = __ldg(up + i0);
+      } else {
+        a.x = da.x = 0.f;
       }
+      if (in1) {
+        l.y = __ldg(lp + i1);
+        u.y = __ldg(up + i1);
+      } else {
+        a.y = da.y = 0.f;
+      }
+      box_terms(R, a, da, l, u);
+    }
     if (++done % st.flush == 0) R.flush();
   }
   R.flush();
-  store_part(st, M, gl, chunk, red, R);
+  return store_part(st, M, gl, chunk, red, R);
+}
+
+template <int C>
+__device__ __noinline__ void ib_box_wide(const IbStep& st, const IbRowMap& M, float* sw, double (*red)[32][3]) {
+  ib_box<C, true>(st, M, sw, red);
+}
+template <int C>
+__global__ void __launch_bounds__(NT, 3) ib_box_kernel(const __grid_constant__ IbStep st,
+                                                       const __grid_constant__ IbRowMap M) {
+  extern __shared__ __align__(16) float sw[];
+  __shared__ double red[NW][32][3];
+  if (!ib_box<C, false>(st, M, sw, red)) ib_box_wide<C>(st, M, sw, red);
 }
 
 // Sums a chunk's slots per row (fixed order), with the objective's bias term.
@@ -572,7 +677,7 @@ __global__ void __launch_bounds__(NT) ib_collect_kernel(IbRowMap M, int slots, c
   if (t >= (int64_t)M.n_groups * 32) return;
   const IbRow r = ib_row(M, M.group0 + t / 32, (int)(t % 32));
   if (!r.valid) return;
-  double v = (double)r.sign * (double)bias[r.i / plane], av = fabs(v), e = 0.0;
+  double v = (double)r.sign * (double)bias[r.i / plane], av = fabs(v), e = 1.1754943508222875e-38;  // 2^-126: see the top
   for (int s = 0; s < slots; ++s) {
     const double* p = part + ((size_t)s * M.n_groups * 32 + t) * 3;
     v += p[0];
@@ -730,6 +835,9 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
   st.box_row = A.box_row;
   st.n_boxes = A.n_boxes;
   st.part = A.part;
+  // FP64 sums, plus Dot2's errors in halves of n = kAdds terms: n^2 2^-48 of their
+  // |terms| (its c sums at most n 2^-24 of them in n steps of two roundings)
+  const double gamma_M = A.gamma_M + 1.001 * std::ldexp((double)kAdds * kAdds, -48);
   const int plane_k = Lk.kind == LD_LAYER_FC ? 1 : Lk.ho * Lk.wo;
   const int64_t chunk = ib_space(Ls, k, A.n_owners, A.n_rules, n_signs).chunk_groups;
   for (int64_t g0 = 0; g0 < groups; g0 += chunk) {
@@ -770,8 +878,8 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
       st.cp = conv ? (L.cin <= 4 ? 4 : L.cin <= 8 ? 8 : L.cin <= 16 ? 16 : (L.cin + 1) & ~1) : NW * kUnitC;
       const bool pairs = st.box && !st.seed && box_pairs(L);
       if (pairs) st.cp = 4;
-      const int terms = pairs ? 2 * L.cin : (st.box ? 1 : 2) * std::min(kUnitC, conv ? L.cin : L.n_in);
-      st.flush = std::max(1, kTerms / terms);
+      const int adds = pairs ? L.cin : (st.box ? 1 : 2) * ((std::min(kUnitC, conv ? L.cin : L.n_in) + 1) / 2);
+      st.flush = std::max(1, kAdds / adds);
       const size_t smem = sizeof(float) * (size_t)st.cp * (st.seed ? 0
                                                            : conv  ? L.cout * L.kh * L.kw
                                                                    : std::min(kFcRows, L.n_out));
@@ -799,9 +907,7 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
     ib_collect_kernel<<<(unsigned)((M.n_groups * 32LL + NT - 1) / NT), NT, 0, s>>>(M, g.slots, A.part, Lk.b, plane_k,
                                                                                  A.acc);
   }
-  // FP64 sums, plus Dot2's gamma_32^2 (FP32) of the blocks of at most kTerms terms
-  const double gd = gamma32(kTerms);
-  IbFinish f{A.n_owners, Lk.n_out, A.n_rules, n_signs, A.N, Lk.r_out_off, A.acc, A.gamma_M + 2.0 * gd * gd, A.mask,
+  IbFinish f{A.n_owners, Lk.n_out, A.n_rules, n_signs, A.N, Lk.r_out_off, A.acc, gamma_M, A.mask,
              A.lbk, A.ubk, A.out_lb};
   const int64_t total = (int64_t)A.n_owners * Lk.n_out;
   const int grid = (int)((total + 255) / 256 < 65535 ? (total + 255) / 256 : 65535);
