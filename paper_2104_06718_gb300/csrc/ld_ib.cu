@@ -73,7 +73,14 @@ namespace {
 constexpr int NW = 8;              // warps per CTA
 constexpr int NT = 32 * NW;
 constexpr int kUnitC = 8;          // elements per unit (channels of a position / consecutive FC inputs)
-constexpr int kPairs = kUnitC / 2;
+// Elements per unit of FC layers with fewer inputs than kWideFc.  Units of 8 leave
+// a small call one to three CTAs a group, each a chain of waits (two to five units
+// a warp in a row): CROWN/WK bounds of one row of a 400-20-20-20-1 net 203 us, with
+// units of 2 and one a warp 106; FSB of 128-128-1 157 and 84 us.  600 rows of such
+// nets take up to 1.7 times as long as with units of 8 (300-24-100-1), which is still
+// a tenth of a warp per row.  The inputs alone decide, so that a row's value stays
+// the same in any batch.
+constexpr int kUnitFc = 2, kWideFc = 1024;
 constexpr int kAdds = 16;          // most scalar terms of each half of a row's sum between two FP64 flushes
 constexpr int kMaxChunks = 64;     // CTAs of a group
 constexpr int kWarpWork = 1024;    // terms a warp should have (2 to 8 units): its fixed cost is a few hundred instructions
@@ -186,6 +193,8 @@ __device__ __forceinline__ IbRow ib_row(const IbRowMap& M, int64_t g, int lane) 
 __host__ __device__ __forceinline__ int box_units(int stride, int ww) {
   return stride * (((ww + stride - 1) / stride + 1) / 2);
 }
+// Elements of a unit of a_{j-1}, the inputs of layer L.
+inline int unit_elems(const LayerDev& L) { return L.kind == LD_LAYER_FC && L.n_in < kWideFc ? kUnitFc : kUnitC; }
 // Whether a_0 of first layer L goes through ib_box_kernel.
 inline bool box_pairs(const LayerDev& L) { return L.kind == LD_LAYER_CONV && L.cin <= 4; }
 
@@ -238,7 +247,9 @@ struct Pair {
 // The dot products of a unit's needed elements, two per packed instruction
 // (half the issue slots of two Dot2, which leaves them to loads and votes) and
 // a last odd one by itself; pairs past np are not touched.
+template <int UC>
 struct UnitSums {
+  static constexpr int kPairs = UC / 2;
   Pair d[kPairs];
   Dot2 one;
   int wa[kPairs], wb[kPairs], w1;    // the elements' places in a staged weight row
@@ -246,10 +257,9 @@ struct UnitSums {
   bool odd;
   __device__ __forceinline__ void add(const float* ws, float m1) {
     const float2 m = make_float2(m1, m1), nm = make_float2(-m1, -m1);
-    if (np > 0) d[0].add(make_float2(ws[wa[0]], ws[wb[0]]), m, nm);
-    if (np > 1) d[1].add(make_float2(ws[wa[1]], ws[wb[1]]), m, nm);
-    if (np > 2) d[2].add(make_float2(ws[wa[2]], ws[wb[2]]), m, nm);
-    if (np > 3) d[3].add(make_float2(ws[wa[3]], ws[wb[3]]), m, nm);
+#pragma unroll
+    for (int k = 0; k < kPairs; ++k)
+      if (np > k) d[k].add(make_float2(ws[wa[k]], ws[wb[k]]), m, nm);
     if (odd) one.add(ws[w1], m1);
   }
   // Adds n terms: m at mp + k mstep (one coalesced load for all elements), the
@@ -257,14 +267,15 @@ struct UnitSums {
   template <int CP>
   __device__ __forceinline__ void run(const float* __restrict__ mp, int mstep, const float* ws, int cp, int n) {
     const int wstep = CP ? CP : cp;
+    constexpr int U = UC == 2 ? 8 : 4;  // coefficients in flight
     int k = 0;
-    for (; k + 4 <= n; k += 4, mp += 4 * (size_t)mstep, ws += 4 * wstep) {
-      const float m0 = __ldg(mp), m1 = __ldg(mp + mstep), m2 = __ldg(mp + 2 * (size_t)mstep),
-                  m3 = __ldg(mp + 3 * (size_t)mstep);
-      if (__any_sync(kFull, m0 != 0.f)) add(ws, m0);
-      if (__any_sync(kFull, m1 != 0.f)) add(ws + wstep, m1);
-      if (__any_sync(kFull, m2 != 0.f)) add(ws + 2 * wstep, m2);
-      if (__any_sync(kFull, m3 != 0.f)) add(ws + 3 * wstep, m3);
+    for (; k + U <= n; k += U, mp += U * (size_t)mstep, ws += U * wstep) {
+      float m[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) m[q] = __ldg(mp + q * (size_t)mstep);
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (__any_sync(kFull, m[q] != 0.f)) add(ws + q * wstep, m[q]);
     }
     for (; k < n; ++k, mp += mstep, ws += wstep) {
       const float m = __ldg(mp);
@@ -367,7 +378,7 @@ __device__ __forceinline__ bool store_part(const IbStep& st, const IbRowMap& M, 
 }
 
 // One CTA: units [chunk * units_per_cta, ...) of one group of 32 rows; a unit
-// is kUnitC channels of one position (conv) or kUnitC consecutive inputs (FC).
+// is UC channels of one position (conv) or UC consecutive inputs (FC).
 // The elements that some row needs are summed together from one stream of
 // coefficients, the weights in shared memory (conv: [tap][o][cp] channels; FC:
 // up to kFcRows rows of the CTA's inputs at a time).  Bound by the FP32 pipe:
@@ -375,7 +386,7 @@ __device__ __forceinline__ bool store_part(const IbStep& st, const IbRowMap& M, 
 // loads, votes and addresses were most of the instructions.
 // CP: floats of a staged weight row where it is one of the usual sizes (the
 // four rows of an unrolled step are then immediate offsets), else 0.
-template <int CP, bool WIDE>
+template <int CP, int UC, bool WIDE>
 __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, float* sw, double (*red)[32][3]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gl = blockIdx.x / st.chunks, chunk = blockIdx.x % st.chunks;
@@ -395,7 +406,7 @@ __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, flo
   const int ix0 = st.win.full ? 0 : r.ox * st.win.mul - st.win.sub;
   const int oy0 = st.wout.full ? 0 : r.oy * st.wout.mul - st.wout.sub;
   const int ox0 = st.wout.full ? 0 : r.ox * st.wout.mul - st.wout.sub;
-  const int cb = conv ? (L.cin + kUnitC - 1) / kUnitC : 0;
+  const int cb = conv ? (L.cin + UC - 1) / UC : 0;
   const size_t lo_off = st.box ? (size_t)box_of(st, r.owner) * st.n0 : (size_t)r.owner * st.N + st.prev_r_off;
   const float* lp = (st.box ? st.l0 : st.lbk) + lo_off;
   const float* up = (st.box ? st.u0 : st.ubk) + lo_off;
@@ -409,12 +420,12 @@ __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, flo
   for (int ub = u_lo; ub < u_hi; ub += NW) {
     const int un = ub + warp;
     // element c (channel / input) of the unit: flat index ib + c hw, coefficient eb + c ostep
-    int y = 0, x = 0, c0 = un * kUnitC, nc = min(kUnitC, L.n_in - c0), ib = 0, eb = 0;
+    int y = 0, x = 0, c0 = un * UC, nc = min(UC, L.n_in - c0), ib = 0, eb = 0;
     bool in = un < u_hi;
     if (conv) {
       const int pos = un / cb, wy = pos / st.wout.ww, wx = pos - wy * st.wout.ww;
-      c0 = (un - pos * cb) * kUnitC;
-      nc = min(kUnitC, L.cin - c0);
+      c0 = (un - pos * cb) * UC;
+      nc = min(UC, L.cin - c0);
       y = oy0 + wy;
       x = ox0 + wx;
       in = in && y >= 0 && y < L.h && x >= 0 && x < L.w;
@@ -424,24 +435,24 @@ __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, flo
     unsigned act = in ? (1u << nc) - 1u : 0u;
     if (in && !st.box) {
       // elements blocking in every row relax to zero whatever their sum is
-      float u[kUnitC];
+      float u[UC];
 #pragma unroll
-      for (int q = 0; q < kUnitC; ++q) u[q] = q < nc ? __ldg(up + ib + (c0 + q) * hw) : 0.f;
+      for (int q = 0; q < UC; ++q) u[q] = q < nc ? __ldg(up + ib + (c0 + q) * hw) : 0.f;
 #pragma unroll
-      for (int q = 0; q < kUnitC; ++q)
+      for (int q = 0; q < UC; ++q)
         if (q < nc && !__any_sync(kFull, u[q] > 0.f)) {
           act &= ~(1u << q);
           out[(size_t)(eb + (c0 + q) * ostep) * 32] = 0.f;
         }
     }
-    UnitSums S;
+    UnitSums<UC> S;
     S.np = __popc(act) / 2;
     S.odd = __popc(act) & 1;
     {
-      const int wb = conv ? c0 : warp * kUnitC;   // the unit's first element in a staged weight row
+      const int wb = conv ? c0 : warp * UC;   // the unit's first element in a staged weight row
       unsigned rest = act;
 #pragma unroll
-      for (int k = 0; k < kPairs; ++k) {
+      for (int k = 0; k < UC / 2; ++k) {
         S.wa[k] = S.wb[k] = 0;
         if (k < S.np) {
           const int a = __ffs(rest) - 1;
@@ -470,12 +481,13 @@ __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, flo
           }
         }
     } else if (!st.seed) {
-      constexpr int kCols = NW * kUnitC;
+      constexpr int kCols = NW * UC;
       for (int o0 = 0; o0 < L.n_out; o0 += kFcRows) {
         const int nr = min(kFcRows, L.n_out - o0);
         __syncthreads();
+#pragma unroll 4
         for (int e = threadIdx.x; e < nr * kCols; e += NT) {
-          const int o = e / kCols, i = ub * kUnitC + e % kCols;
+          const int o = e / kCols, i = ub * UC + e % kCols;
           sw[e] = i < L.n_in ? __ldg(L.W + (size_t)(o0 + o) * L.n_in + i) : 0.f;
         }
         __syncthreads();
@@ -495,7 +507,7 @@ __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, flo
       ii[1] = ib + c[1] * hw;
       Pair D = S.d[0];
 #pragma unroll
-      for (int q = 1; q < kPairs; ++q)
+      for (int q = 1; q < UC / 2; ++q)
         if (k == q) D = S.d[q];
       if (!two) {
         D.p = make_float2(S.one.p, 0.f);
@@ -547,16 +559,16 @@ __device__ __forceinline__ bool ib_step(const IbStep& st, const IbRowMap& M, flo
 }
 
 // The FP64 form, out of line.
-template <int CP>
+template <int CP, int UC>
 __device__ __noinline__ void ib_step_wide(const IbStep& st, const IbRowMap& M, float* sw, double (*red)[32][3]) {
-  ib_step<CP, true>(st, M, sw, red);
+  ib_step<CP, UC, true>(st, M, sw, red);
 }
-template <int CP>
+template <int CP, int UC>
 __global__ void __launch_bounds__(NT, 3) ib_step_kernel(const __grid_constant__ IbStep st,
                                                         const __grid_constant__ IbRowMap M) {
   extern __shared__ __align__(16) float sw[];
   __shared__ double red[NW][32][3];
-  if (!ib_step<CP, false>(st, M, sw, red)) ib_step_wide<CP>(st, M, sw, red);
+  if (!ib_step<CP, UC, false>(st, M, sw, red)) ib_step_wide<CP, UC>(st, M, sw, red);
 }
 
 // The input box of a conv first layer of C <= 4 channels: a unit is two
@@ -763,14 +775,15 @@ IbGeo ib_geo(const std::vector<LayerDev>& Ls, int k) {
     g.w[j] = full ? IbWin{1, up.h, up.w, 0, 0} : IbWin{0, hh, ww, mul, sub};  // full: as layer j+1 sees it
     const bool conv = up.kind == LD_LAYER_CONV;
     g.elems[j] = conv ? up.cin * g.w[j].hh * g.w[j].ww : up.n_in;
-    g.units[j] = conv ? g.w[j].hh * g.w[j].ww * ((up.cin + kUnitC - 1) / kUnitC) : (up.n_in + kUnitC - 1) / kUnitC;
-    int unit_terms = up.fan_t * std::min(kUnitC, conv ? up.cin : up.n_in);
+    const int uc = unit_elems(up);
+    g.units[j] = conv ? g.w[j].hh * g.w[j].ww * ((up.cin + uc - 1) / uc) : (up.n_in + uc - 1) / uc;
+    int unit_terms = up.fan_t * std::min(uc, conv ? up.cin : up.n_in);
     if (j == 0 && box_pairs(up)) {
       g.units[j] = g.w[j].hh * box_units(up.stride, g.w[j].ww);
       unit_terms = 2 * up.fan_t * up.cin;
     }
-    g.per_cta[j] = NW * std::max(std::min(8, std::max(2, kWarpWork / unit_terms)),
-                                 (g.units[j] + NW * kMaxChunks - 1) / (NW * kMaxChunks));
+    const int per_warp = uc == kUnitFc ? 1 : std::min(8, std::max(2, kWarpWork / unit_terms));
+    g.per_cta[j] = NW * std::max(per_warp, (g.units[j] + NW * kMaxChunks - 1) / (NW * kMaxChunks));
     g.chunks[j] = (g.units[j] + g.per_cta[j] - 1) / g.per_cta[j];
     g.slots += g.chunks[j];
     if (j >= 1) g.width = std::max(g.width, g.elems[j]);
@@ -875,10 +888,11 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
       st.units = g.units[j - 1];
       st.units_per_cta = g.per_cta[j - 1];
       const bool conv = L.kind == LD_LAYER_CONV;
-      st.cp = conv ? (L.cin <= 4 ? 4 : L.cin <= 8 ? 8 : L.cin <= 16 ? 16 : (L.cin + 1) & ~1) : NW * kUnitC;
+      const int uc = unit_elems(L);
+      st.cp = conv ? (L.cin <= 4 ? 4 : L.cin <= 8 ? 8 : L.cin <= 16 ? 16 : (L.cin + 1) & ~1) : NW * uc;
       const bool pairs = st.box && !st.seed && box_pairs(L);
       if (pairs) st.cp = 4;
-      const int adds = pairs ? L.cin : (st.box ? 1 : 2) * ((std::min(kUnitC, conv ? L.cin : L.n_in) + 1) / 2);
+      const int adds = pairs ? L.cin : (st.box ? 1 : 2) * ((std::min(uc, conv ? L.cin : L.n_in) + 1) / 2);
       st.flush = std::max(1, kAdds / adds);
       const size_t smem = sizeof(float) * (size_t)st.cp * (st.seed ? 0
                                                            : conv  ? L.cout * L.kh * L.kw
@@ -887,11 +901,12 @@ cudaError_t launch_ib_layer(const std::vector<LayerDev>& Ls, int k, const IbLaye
                                      : L.cin == 2 ? ib_box_kernel<2>
                                      : L.cin == 3 ? ib_box_kernel<3>
                                                   : ib_box_kernel<4>)
-                    : st.cp == 4  ? ib_step_kernel<4>
-                    : st.cp == 8  ? ib_step_kernel<8>
-                    : st.cp == 16 ? ib_step_kernel<16>
-                    : st.cp == 64 ? ib_step_kernel<64>
-                                  : ib_step_kernel<0>;
+                    : uc == kUnitFc ? ib_step_kernel<NW * kUnitFc, kUnitFc>
+                    : st.cp == 4  ? ib_step_kernel<4, kUnitC>
+                    : st.cp == 8  ? ib_step_kernel<8, kUnitC>
+                    : st.cp == 16 ? ib_step_kernel<16, kUnitC>
+                    : st.cp == 64 ? ib_step_kernel<64, kUnitC>
+                                  : ib_step_kernel<0, kUnitC>;
       if (smem > 40 * 1024) {
         const cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageMost);
         if (ea != cudaSuccess) return ea;
