@@ -167,16 +167,18 @@ struct FinalEpi {
 };
 
 // FP64 sum of products and the FP32 sum of their sizes (up), for the sums that
-// the levels below do not hold; n more products.  Runs with no nonzero product
-// (duals that are all 0) cost no FP64 instruction.
+// the levels below do not hold; n more products.  Runs of duals that are all 0
+// (an ascent's zero start) cost one look at them.
 struct Sum64 {
   double g;
   float abs_sum;
 };
 __device__ __noinline__ Sum64 sum_fp64(Sum64 t, const float* w, size_t ws, const float* r, size_t rs, int n) {
   bool any = false;
-  for (int i = 0; i < n; ++i) any = any || (w[i * ws] != 0.f && r[i * rs] != 0.f);
+#pragma unroll 8
+  for (int i = 0; i < n; ++i) any |= r[i * rs] != 0.f;
   if (!any) return t;
+#pragma unroll 4
   for (int i = 0; i < n; ++i) {
     const float wv = w[i * ws], rv = r[i * rs];
     t.g = fma((double)wv, (double)rv, t.g);
