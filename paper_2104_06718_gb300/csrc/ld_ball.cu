@@ -115,13 +115,13 @@ __global__ void ball_first_layer_kernel(LayerDev L, int n_props, const float* __
   }
 }
 
-// Per subdomain: -eps sqrt(sum of the scratch slots' upper sums), rounded
+// Per subdomain: -eps sqrt(sum of the scratch slots' values, summed up), rounded
 // down, into slot `slot` of the main accumulator (value, error 0, |value|).
 __global__ void ball_final_kernel(Problem P, FinalAcc scratch, FinalAcc main, int slot) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < P.B; b += gridDim.x * blockDim.x) {
     const double* p = scratch.slots + (size_t)b * scratch.n_slots * 3;
     double q = 0.0;
-    for (int i = 0; i < scratch.n_slots; ++i) q = __dadd_ru(q, p[3 * i + 2]);
+    for (int i = 0; i < scratch.n_slots; ++i) q = __dadd_ru(q, p[3 * i]);
     const double t = -__dmul_ru((double)P.ball_eps[prop_of(P, b)], __dsqrt_ru(q));
     double* m = main.slots + ((size_t)b * main.n_slots + slot) * 3;
     m[0] = t;

@@ -26,10 +26,13 @@
 // bound e on its error (from delta_i and the rounding of one subtraction and
 // one product) are summed per subdomain; the bound returned is
 //   S - E - gamma_M * sum|t|   (S = sum t, E = sum e, M = number of terms),
-// with t and S in FP64, and E and sum|t| summed rounding upward (within a
-// block in FP32, values outside its middle range in FP64) and scaled by
-// 1 + 2 gamma_M as a margin.  Sums |W||rho| below 2^-59 or from 2^117 on, which
-// the levels do not hold, are formed again in FP64.  Partial sums go to fixed slots that one kernel adds in a fixed
+// with t and S in FP64, and E and sum|t| summed rounding upward (per thread and
+// warp in FP32) and scaled by 1 + 2 gamma_M as a margin.  A CTA in which a sum
+// |W||rho| is below 2^-59 (and not 0) or from 2^117 on, or a sum of errors or |t|
+// from 2^100 on, which FP32 does not hold, forms its terms again in FP64.  That
+// is one test a CTA and code behind the usual path: FP64 calls within it took the
+// conv kernels from 64 to 120 registers (2000 Base subdomains, duals given: 1054 us
+// then, 1003 so).  Partial sums go to fixed slots that one kernel adds in a fixed
 // order, so the bound does not depend on the order in which blocks run.
 #include <cmath>
 
@@ -41,12 +44,13 @@ namespace {
 constexpr int BN = 64, NT = 256;
 constexpr float kU52 = 2.220446049250313e-16f;  // 2^-52
 
-// Sums of a thread's terms: values, error bounds (up), |values| (up); the last
-// two in FP32, with the terms outside its middle range in eo and ao.
+// Sums of a thread's terms: values, error bounds (up), |values| (up).
 struct TermSum {
   double t = 0.0;
   float e = 0.f, a = 0.f;
-  double eo = 0.0, ao = 0.0;
+};
+struct WideSum {
+  double t = 0.0, e = 0.0, a = 0.0;
 };
 
 // |x| rounded up to FP32, by integer instructions (at least 2^-126).
@@ -57,63 +61,51 @@ __device__ __forceinline__ float abs_up(double x) {
   return __uint_as_float(((hi - 0x38000000u) << 3 | lo >> 29) + 1u);
 }
 
-// Whether a sum or a term of this size is kept in FP32: 2^-80 to 2^100, or 0.
-__device__ __forceinline__ bool middle(float x) {
-  return x < 1.2676506002282294e30f && (x > 8.271806125530277e-25f || x == 0.f);
-}
+constexpr float kHuge = 1.2676506002282294e30f;  // 2^100: FP32 sums of errors and sizes end here
+__device__ __forceinline__ bool beyond(const TermSum& s) { return !(s.e < kHuge && s.a < kHuge); }
 
 // Adds t, the minimum of exact values and of the product tx = c x, c within
 // delta of its exact value: e = |x| (delta + 2^-52 |c|) + 2^-52 |tx| (none where
 // c is exactly 0, also beside an infinite x).
-__device__ __noinline__ double term_error_fp64(double tx, double c, double x, double delta) {
-  const double ec = __dadd_ru(delta, __dmul_ru((double)kU52, fabs(c)));
-  return ec == 0.0 ? 0.0 : __dadd_ru(__dmul_ru(fabs(x), ec), __dmul_ru((double)kU52, fabs(tx)));
-}
-__device__ __forceinline__ void add_term(TermSum& s, double t, double tx, double c, float x, double delta) {
-  s.t += t;
-  s.eo = __dadd_ru(s.eo, term_error_fp64(tx, c, (double)x, delta));
-  s.ao = __dadd_ru(s.ao, fabs(t));
-}
 __device__ __forceinline__ void add_term(TermSum& s, double t, double tx, double c, float x, float delta) {
-  const float at = abs_up(t);
-  const float e = __fmaf_ru(x, __fmaf_ru(kU52, abs_up(c), delta), __fmul_ru(kU52, abs_up(tx)));
-  if (middle(at) && e < 1.2676506002282294e30f) {
-    s.t += t;
-    s.e = __fadd_ru(s.e, e);
-    s.a = __fadd_ru(s.a, at);
-  } else {
-    add_term(s, t, tx, c, x, (double)delta);
-  }
+  s.t += t;
+  s.e = __fadd_ru(s.e, __fmaf_ru(x, __fmaf_ru(kU52, abs_up(c), delta), __fmul_ru(kU52, abs_up(tx))));
+  s.a = __fadd_ru(s.a, abs_up(t));
+}
+__device__ __forceinline__ void add_term(WideSum& s, double t, double tx, double c, float x, double delta) {
+  const double ec = __dadd_ru(delta, __dmul_ru((double)kU52, fabs(c)));
+  s.t += t;
+  if (ec != 0.0) s.e = __dadd_ru(s.e, __dadd_ru(__dmul_ru((double)x, ec), __dmul_ru((double)kU52, fabs(tx))));
+  s.a = __dadd_ru(s.a, fabs(t));
 }
 // A term without an error.
 __device__ __forceinline__ void add_exact(TermSum& s, double t) {
-  const float at = abs_up(t);
   s.t += t;
-  if (middle(at))
-    s.a = __fadd_ru(s.a, at);
-  else
-    s.ao = __dadd_ru(s.ao, fabs(t));
+  s.a = __fadd_ru(s.a, abs_up(t));
+}
+__device__ __forceinline__ void add_exact(WideSum& s, double t) {
+  s.t += t;
+  s.a = __dadd_ru(s.a, fabs(t));
 }
 
-// Sums over the lanes of each group of 2 * top lanes (all 32 lanes take part).
-__device__ __forceinline__ void reduce_terms(TermSum& s, int top) {
+__device__ __forceinline__ float add_up(float a, float b) { return __fadd_ru(a, b); }
+__device__ __forceinline__ double add_up(double a, double b) { return __dadd_ru(a, b); }
+// Sums over the lanes of each group of 2 * top lanes (all 32 lanes take part);
+// up: t rounded upward too.
+template <class S>
+__device__ __forceinline__ void reduce_terms(S& s, int top, int up) {
   for (int off = top; off > 0; off >>= 1) {
-    s.t += __shfl_xor_sync(0xffffffffu, s.t, off);
-    s.e = __fadd_ru(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
-    s.a = __fadd_ru(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
+    const double t = __shfl_xor_sync(0xffffffffu, s.t, off);
+    s.t = up ? __dadd_ru(s.t, t) : s.t + t;
+    s.e = add_up(s.e, __shfl_xor_sync(0xffffffffu, s.e, off));
+    s.a = add_up(s.a, __shfl_xor_sync(0xffffffffu, s.a, off));
   }
-  if (__any_sync(0xffffffffu, s.eo != 0.0 || s.ao != 0.0))
-    for (int off = top; off > 0; off >>= 1) {
-      s.eo = __dadd_ru(s.eo, __shfl_xor_sync(0xffffffffu, s.eo, off));
-      s.ao = __dadd_ru(s.ao, __shfl_xor_sync(0xffffffffu, s.ao, off));
-    }
 }
 
-// One per-neuron minimum, g within delta of the exact value (D: float, or
-// double where delta may lie outside FP32's middle range).  box: P0 term
+// One per-neuron minimum, g within delta of the exact value.  box: P0 term
 // with coefficient -g on [l, u]; otherwise the Pk neuron with rho r.
-template <class D>
-__device__ __forceinline__ void final_term(TermSum& s, bool box, float r, double g, D delta, float l, float u) {
+template <class S, class D>
+__device__ __forceinline__ void final_term(S& s, bool box, float r, double g, D delta, float l, float u) {
   if (!box && u <= 0.f) {             // blocking: min r*xB over [l,u], exact products (r = 0: 0, also with l = -inf)
     add_exact(s, widen(r) * widen(r > 0.f ? l : u));
     return;
@@ -137,19 +129,15 @@ struct FinalEpi {
   const float* rho;
   double gamma_K;
   int ball_norm;       // layer 0, l2 ball: the term is an upper bound on g_0[i]^2 (for ||g_0||)
-  // abs_sum: bound on sum |W||rho| of an FP64 sum g
-  __device__ __forceinline__ void term(int b, int i, double g, float abs_sum, TermSum& s) const {
-    term_delta(b, i, g, __dmul_ru(gamma_K, (double)abs_sum), s);
-  }
   // delta: bound on |g - exact g|
-  template <class D>
-  __device__ __forceinline__ void term_delta(int b, int i, double g, D delta, TermSum& s) const {
+  template <class S, class D>
+  __device__ __forceinline__ void term(int b, int i, double g, D delta, S& s) const {
     if (layer == 0) {
       if (ball_norm) {
-        // |exact g_0[i]| <= |g| + delta: its square, rounded up (in FP64: the
-        // sum of these is the square of the norm itself, not a slack)
+        // |exact g_0[i]| <= |g| + delta: its square, summed rounding up (in the
+        // values: it is the square of the norm itself, not a slack)
         const double a = __dadd_ru(fabs(g), (double)delta);
-        s.ao = __dadd_ru(s.ao, __dmul_ru(a, a));
+        s.t = __dadd_ru(s.t, __dmul_ru(a, a));
         return;
       }
       // the box; over an l2 ball l0 = u0 = the centre, which gives the
@@ -166,25 +154,34 @@ struct FinalEpi {
   }
 };
 
-// FP64 sum of products and the FP32 sum of their sizes (up), for the sums that
-// the levels below do not hold; n more products.  Runs of duals that are all 0
-// (an ascent's zero start) cost one look at them.
-struct Sum64 {
-  double g;
-  float abs_sum;
-};
-__device__ __noinline__ Sum64 sum_fp64(Sum64 t, const float* w, size_t ws, const float* r, size_t rs, int n) {
-  bool any = false;
-#pragma unroll 8
-  for (int i = 0; i < n; ++i) any |= r[i * rs] != 0.f;
-  if (!any) return t;
-#pragma unroll 4
-  for (int i = 0; i < n; ++i) {
-    const float wv = w[i * ws], rv = r[i * rs];
-    t.g = fma((double)wv, (double)rv, t.g);
-    t.abs_sum = __fmaf_ru(fabsf(wv), fabsf(rv), t.abs_sum);
+// g of input element (c, yy, xx) of a conv in FP64 (exact products), and the FP32
+// sum of their sizes (up); W in its [o][c][i][j] layout, rb one subdomain's duals.
+__device__ __forceinline__ double conv_sum64(const LayerDev& L, const float* W, const float* rb, int c, int yy, int xx,
+                                             float& abs_sum) {
+  const int hw_o = L.ho * L.wo;
+  double acc = 0.0;
+  float aab = 0.f;
+  for (int i = 0; i < L.kh; ++i) {
+    const int ty = yy + L.pad - i;
+    if (ty < 0 || ty % L.stride) continue;
+    const int y = ty / L.stride;
+    if (y >= L.ho) continue;
+    for (int j = 0; j < L.kw; ++j) {
+      const int tx = xx + L.pad - j;
+      if (tx < 0 || tx % L.stride) continue;
+      const int xo = tx / L.stride;
+      if (xo >= L.wo) continue;
+      const float* wp = W + ((size_t)c * L.kh + i) * L.kw + j;
+      const float* rp = rb + y * L.wo + xo;
+      for (int o = 0; o < L.cout; ++o) {
+        const float wv = wp[(size_t)o * L.cin * L.kh * L.kw], rv = rp[(size_t)o * hw_o];
+        acc = fma((double)wv, (double)rv, acc);
+        aab = __fmaf_ru(fabsf(wv), fabsf(rv), aab);
+      }
+    }
   }
-  return t;
+  abs_sum = aab;
+  return acc;
 }
 
 // ---------------------------------------------------------------- three-level sums
@@ -197,6 +194,7 @@ constexpr int kBlk = 64;  // terms between two blocks
 struct Sum3x2 {
   float2 p, q, c;      // levels 1 to 3; p holds the sum of sizes until begin()
   double g0, g1;       // finished blocks
+  int zero;            // bit h: half h's products are all 0 (or below 2^-150)
   __device__ __forceinline__ void start() { p = make_float2(0.f, 0.f); }
   __device__ __forceinline__ void size(float2 w, float2 r) {
     const float2 h = __fmul2_rn(w, r);
@@ -211,6 +209,7 @@ struct Sum3x2 {
   }
   static __device__ __forceinline__ float binade(float p) { return __uint_as_float(__float_as_uint(p) & 0x7f800000u); }
   __device__ __forceinline__ void begin(float lvl2) {
+    zero = (p.x == 0.f ? 1 : 0) | (p.y == 0.f ? 2 : 0);
     p = make_float2(1.5f * top(p.x), 1.5f * top(p.y));
     q = make_float2(p.x * lvl2, p.y * lvl2);
     c = make_float2(0.f, 0.f);
@@ -238,13 +237,18 @@ struct Sum3x2 {
     q = t3;
     c = __fadd2_rn(c, sub2(e3, n2));
   }
-  // Value and bound of half h after the last block.  False for sums of sizes
-  // below 2^-59 (the bound would be an absolute one, and a product's low part
-  // could underflow), from 2^117 on, and NaN.
-  __device__ __forceinline__ bool result(int h, float kk, double& g, float& delta) const {
+  // Value and bound of half h of K products after the last block.  False for
+  // sums of sizes below 2^-59 (the bound would be an absolute one, and a product's
+  // low part could underflow) but not 0, from 2^117 on, and NaN.
+  __device__ __forceinline__ bool result(int h, float kk, int K, double& g, float& delta) const {
     const float ph = h ? p.y : p.x, two_a = binade(ph);
     g = widen(ph - 1.5f * two_a) + (h ? g1 : g0);
     delta = __fmaf_ru(kk, two_a, __fmul_ru(kU52, abs_up(g)));
+    if (zero >> h & 1) {
+      g = 0.0;
+      delta = (float)K * 1.401298464324817e-45f;
+      return true;
+    }
     return two_a > 6.938893903907228e-18f && two_a < 1.329227995784916e36f;  // 2^-57, 2^120
   }
 };
@@ -294,10 +298,35 @@ __device__ __forceinline__ void acc_add(FinalAcc a, int slot, int b, double t, d
 // slots, are the same either way), a thread TM x 4 of it; up to KS rows of K
 // staged at once.
 constexpr int KS = 128;  // a multiple of kBlk: blocks end where rounds do
+// The CTA's outputs in FP64, an output a thread at a time.
+template <int TM>
+__device__ __noinline__ void fc_wide(int M, int Ncol, int K, const float* A, int lda, const float* W, int ldw,
+                                     const FinalEpi& epi, const FinalAcc& acc_out) {
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  for (int i = 0; i < TM; ++i) {
+    const int m = blockIdx.y * 16 * TM + ty + 16 * i;
+    WideSum s;
+    for (int j = 0; j < 4; ++j) {
+      const int n = blockIdx.x * BN + 4 * tx + j;
+      if (m >= M || n >= Ncol) continue;
+      double g = 0.0;
+      float as = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        const float wv = W[(size_t)k * ldw + n], rv = A[(size_t)m * lda + k];
+        g = fma((double)wv, (double)rv, g);
+        as = __fmaf_ru(fabsf(wv), fabsf(rv), as);
+      }
+      epi.term(m, n, g, __dmul_ru(epi.gamma_K, (double)as), s);
+    }
+    reduce_terms(s, 8, epi.ball_norm);
+    if (tx == 0 && m < M) acc_add(acc_out, acc_out.slot + blockIdx.x, m, s.t, s.e, s.a);
+  }
+}
 template <int TM>
 __global__ void __launch_bounds__(NT) final_fc_kernel(int M, int Ncol, int K, const float* __restrict__ A, int lda,
-                                                      const float* __restrict__ W, int ldw, FinalEpi epi,
-                                                      Sum3Const sc, FinalAcc acc_out) {
+                                                      const float* __restrict__ W, int ldw, const __grid_constant__ FinalEpi epi,
+                                                      Sum3Const sc, const __grid_constant__ FinalAcc acc_out) {
   constexpr int BMt = 16 * TM;
   extern __shared__ __align__(16) float sm[];
   float* As = sm;                      // [k][BMt + 1]
@@ -364,88 +393,105 @@ __global__ void __launch_bounds__(NT) final_fc_kernel(int M, int Ncol, int K, co
         acc[i][1].begin(sc.lvl2);
       }
   }
+  TermSum sum[TM];
+  bool bad = false;
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int m = m0 + ty + 16 * i;
-    TermSum s;
-    if (m < M) {
+    if (m >= M) continue;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int n = n0 + 4 * tx + j;
-        if (n >= Ncol) continue;
-        double g;
-        float delta;
-        if (acc[i][j / 2].result(j % 2, sc.kk, g, delta)) {
-          epi.term_delta(m, n, g, delta, s);
-        } else {
-          const Sum64 v = sum_fp64(Sum64{0.0, 0.f}, W + n, ldw, A + (size_t)m * lda, 1, K);
-          epi.term(m, n, v.g, v.abs_sum, s);
-        }
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int n = n0 + 4 * tx + j;
+      if (n >= Ncol) continue;
+      double g;
+      float delta;
+      bad |= !acc[i][j / 2].result(j % 2, sc.kk, K, g, delta);
+      epi.term(m, n, g, delta, sum[i]);
     }
-    reduce_terms(s, 8);
-    if (tx == 0 && m < M)
-      acc_add(acc_out, acc_out.slot + blockIdx.x, m, s.t, __dadd_ru((double)s.e, s.eo), __dadd_ru((double)s.a, s.ao));
+    bad |= beyond(sum[i]);
+  }
+  if (__syncthreads_or(bad)) {
+    fc_wide<TM>(M, Ncol, K, A, lda, W, ldw, epi, acc_out);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int m = m0 + ty + 16 * i;
+    reduce_terms(sum[i], 8, epi.ball_norm);
+    if (tx == 0 && m < M) acc_add(acc_out, acc_out.slot + blockIdx.x, m, sum[i].t, (double)sum[i].e, (double)sum[i].a);
   }
 }
 
-__device__ __forceinline__ void block_reduce_add(FinalAcc a, int slot, int b, TermSum s) {
+template <class S>
+__device__ __forceinline__ void block_reduce_add(FinalAcc a, int slot, int b, S s, int up) {
   __shared__ double red[3][NT / 32];
-  reduce_terms(s, 16);
+  reduce_terms(s, 16, up);
   const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (lane == 0) {
     red[0][w] = s.t;
-    red[1][w] = __dadd_ru((double)s.e, s.eo);
-    red[2][w] = __dadd_ru((double)s.a, s.ao);
+    red[1][w] = (double)s.e;
+    red[2][w] = (double)s.a;
   }
   __syncthreads();
   if (threadIdx.x < 3) {  // a thread each for t, e and a
     double v = red[threadIdx.x][0];
     for (int i = 1; i < (int)(blockDim.x / 32); ++i) {
       const double x = red[threadIdx.x][i];
-      v = threadIdx.x == 0 ? v + x : __dadd_ru(v, x);
+      v = threadIdx.x == 0 && !up ? v + x : __dadd_ru(v, x);
     }
     a.slots[((size_t)b * a.n_slots + slot) * 3 + threadIdx.x] = v;
   }
 }
 
+// The elements of CTA blockIdx.x of a conv pass, as WideSum terms: `per` elements
+// per item (channels of one position, phase by phase for per > 1).
+__device__ __noinline__ WideSum conv_wide(const LayerDev& L, const float* rb, const FinalEpi& epi, int b, int per) {
+  WideSum s;
+  const int hw = L.h * L.w, ST = per > 1 ? L.stride : 1;
+  const int qh = L.h / ST, qw = L.w / ST, ncg = L.cin / per, items = ST * ST * ncg * qh * qw;
+  for (int e = blockIdx.x * NT + threadIdx.x; e < items; e += gridDim.x * NT) {
+    int q = e;
+    const int qx = q % qw;
+    q /= qw;
+    const int qy = q % qh;
+    q /= qh;
+    const int cg = q % ncg;
+    q /= ncg;
+    const int yy = q / ST + ST * qy, xx = q % ST + ST * qx;
+    for (int g = 0; g < per; ++g) {
+      const int c = cg * per + g;
+      float as;
+      const double v = conv_sum64(L, L.W, rb, c, yy, xx, as);
+      epi.term(b, c * hw + yy * L.w + xx, v, __dmul_ru(epi.gamma_K, (double)as), s);
+    }
+  }
+  return s;
+}
+
 // FP64 transposed conv pass; grid row = subdomain.
-__global__ void __launch_bounds__(NT) final_conv_kernel(LayerDev L, const float* __restrict__ r, int rs,
-                                                        FinalEpi epi, FinalAcc acc_out) {
+__global__ void __launch_bounds__(NT) final_conv_kernel(const __grid_constant__ LayerDev L, const float* __restrict__ r,
+                                                        int rs, const __grid_constant__ FinalEpi epi, FinalAcc acc_out) {
   extern __shared__ float sW[];
   const int nw = L.cout * L.cin * L.kh * L.kw;
   for (int e = threadIdx.x; e < nw; e += blockDim.x) sW[e] = L.W[e];
   __syncthreads();
   const int b = blockIdx.y;
   const float* rb = r + (size_t)b * rs;
-  const int hw_i = L.h * L.w, plane = L.cin * hw_i, hw_o = L.ho * L.wo;
+  const int hw_i = L.h * L.w, plane = L.cin * hw_i;
+  const float gamma_K = __double2float_ru(epi.gamma_K);
   TermSum s;
+  bool bad = false;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < plane; e += gridDim.x * blockDim.x) {
     const int c = e / hw_i, rem = e % hw_i, yy = rem / L.w, xx = rem % L.w;
-    double acc = 0.0;
-    float aab = 0.f;
-    for (int i = 0; i < L.kh; ++i) {
-      const int ty = yy + L.pad - i;
-      if (ty < 0 || ty % L.stride) continue;
-      const int y = ty / L.stride;
-      if (y >= L.ho) continue;
-      for (int j = 0; j < L.kw; ++j) {
-        const int tx = xx + L.pad - j;
-        if (tx < 0 || tx % L.stride) continue;
-        const int xo = tx / L.stride;
-        if (xo >= L.wo) continue;
-        const float* wp = sW + ((size_t)c * L.kh + i) * L.kw + j;
-        const float* rp = rb + y * L.wo + xo;
-        for (int o = 0; o < L.cout; ++o) {
-          const float wv = wp[(size_t)o * L.cin * L.kh * L.kw], rv = rp[(size_t)o * hw_o];
-          acc = fma((double)wv, (double)rv, acc);
-          aab = __fmaf_ru(fabsf(wv), fabsf(rv), aab);
-        }
-      }
-    }
-    epi.term(b, e, acc, aab, s);
+    float as;
+    const double g = conv_sum64(L, sW, rb, c, yy, xx, as);
+    bad |= as < 1e-18f && as != 0.f;  // delta too small for FP32
+    epi.term(b, e, g, __fmul_ru(gamma_K, as), s);
   }
-  block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s);
+  if (__syncthreads_or(bad || beyond(s)))
+    block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, conv_wide(L, rb, epi, b, 1), epi.ball_norm);
+  else
+    block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s, epi.ball_norm);
 }
 
 // Transposed conv by stride phase (k4 s2 / k3 s1) in three-level sums, G input
@@ -454,8 +500,10 @@ __global__ void __launch_bounds__(NT) final_conv_kernel(LayerDev L, const float*
 // rho[b, o, y, x], weights and the subdomain's rho_{k+1} (with its zero halo) in
 // shared memory.  The slots are this grid's blocks.
 template <int KH, int KW, int ST, int G>
-__global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, ConvTile T, const float* __restrict__ r, int rs,
-                                                             FinalEpi epi, Sum3Const sc, FinalAcc acc_out) {
+__global__ void __launch_bounds__(NT, 4) final_conv_fast_kernel(const __grid_constant__ LayerDev L, ConvTile T,
+                                                             const float* __restrict__ r, int rs,
+                                                             const __grid_constant__ FinalEpi epi, Sum3Const sc,
+                                                             FinalAcc acc_out) {
   extern __shared__ __align__(16) float sm[];
   float* sR = sm + T.w_floats;
   const int b = blockIdx.y;
@@ -466,7 +514,9 @@ __global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, ConvTil
   stage_wait();
   const int qh = L.h / ST, qw = L.w / ST, ncg = L.cin / G, plane = T.rows * T.pitch;
   const int items = ST * ST * ncg * qh * qw;
+  const int K = L.cout * (KH / ST) * (KW / ST);
   TermSum s;
+  bool bad = false;
   for (int e = blockIdx.x * NT + threadIdx.x; e < items; e += gridDim.x * NT) {
     int q = e;
     const int qx = q % qw;
@@ -532,18 +582,14 @@ __global__ void __launch_bounds__(NT) final_conv_fast_kernel(LayerDev L, ConvTil
       double gv;
       float delta;
       const int c = cg * G + g, i = (c * L.h + yy) * L.w + xx;
-      if ((g / 2 ? a1 : a0).result(g % 2, sc.kk, gv, delta)) {
-        epi.term_delta(b, i, gv, delta, s);
-      } else {
-        Sum64 v{0.0, 0.f};
-        for (int a = 0; a < KH / ST; ++a)
-          for (int bb = 0; bb < KW / ST; ++bb)
-            v = sum_fp64(v, wp + (ST * a * KW + ST * bb) * T.wc + g, KH * KW * T.wc, rp - a * T.pitch - bb, plane, L.cout);
-        epi.term(b, i, v.g, v.abs_sum, s);
-      }
+      bad |= !(g / 2 ? a1 : a0).result(g % 2, sc.kk, K, gv, delta);
+      epi.term(b, i, gv, delta, s);
     }
   }
-  block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s);
+  if (__syncthreads_or(bad || beyond(s)))
+    block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, conv_wide(L, r + (size_t)b * rs, epi, b, G), epi.ball_norm);
+  else
+    block_reduce_add(acc_out, acc_out.slot + blockIdx.x, b, s, epi.ball_norm);
 }
 
 // Geometry and channel blocking of the phase-split transposed conv, or 0.
@@ -570,14 +616,14 @@ __global__ void __launch_bounds__(NT) final_top_kernel(int n, const float* __res
                                                        const double* __restrict__ Wn_err, FinalEpi epi,
                                                        FinalAcc acc_out) {
   const int b = blockIdx.x;
-  TermSum s;
+  WideSum s;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     if (Wn64)
-      epi.term_delta(b, i, -Wn64[i], Wn_err[i], s);
+      epi.term(b, i, -Wn64[i], Wn_err[i], s);
     else
-      epi.term_delta(b, i, -widen(Wn[i]), 0.0, s);
+      epi.term(b, i, -widen(Wn[i]), 0.0, s);
   }
-  block_reduce_add(acc_out, acc_out.slot, b, s);
+  block_reduce_add(acc_out, acc_out.slot, b, s, epi.ball_norm);
 }
 
 struct BiasLayers {
@@ -592,12 +638,21 @@ struct BiasLayers {
 __global__ void __launch_bounds__(NT) final_bias_kernel(Problem P, BiasLayers BL, const float* __restrict__ rho,
                                                         FinalAcc acc_out) {
   const int b = blockIdx.x;
-  TermSum s;
-  for (int k = 0; k < BL.count; ++k)
+  const auto terms = [&](auto& s) {
+    for (int k = 0; k < BL.count; ++k)
 #pragma unroll 4
-    for (int i = threadIdx.x; i < BL.n[k]; i += blockDim.x)
-      add_exact(s, -widen(rho[(size_t)b * P.N + BL.r_off[k] + i]) * widen(__ldg(BL.bias[k] + i / BL.plane[k])));
-  block_reduce_add(acc_out, acc_out.slot, b, s);
+      for (int i = threadIdx.x; i < BL.n[k]; i += blockDim.x)
+        add_exact(s, -widen(rho[(size_t)b * P.N + BL.r_off[k] + i]) * widen(__ldg(BL.bias[k] + i / BL.plane[k])));
+  };
+  TermSum s;
+  terms(s);
+  if (__syncthreads_or(beyond(s))) {
+    WideSum w;
+    terms(w);
+    block_reduce_add(acc_out, acc_out.slot, b, w, 0);
+    return;
+  }
+  block_reduce_add(acc_out, acc_out.slot, b, s, 0);
 }
 
 // One warp per subdomain: lane i loads slot i of a round, the slots are added in order.

@@ -22,6 +22,7 @@ pytestmark = pytest.mark.gpu
 NETS = {
     "fc": ((40,), [], [130, 65, 1]),
     "conv": ((3, 12, 12), [(8, 4, 2, 1), (12, 3, 1, 1), (6, 5, 1, 2)], [33, 1]),
+    "channels": ((4, 6, 6), [(80, 3, 1, 1), (8, 4, 2, 1), (130, 3, 1, 1)], [9, 1]),  # more than a block of output channels
 }
 
 
