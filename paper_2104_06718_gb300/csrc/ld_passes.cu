@@ -22,10 +22,26 @@ namespace ld {
 namespace {
 
 constexpr int TM = 32, TN = 32, NT = 256;
-constexpr int TK = 128;    // K staged at once: the hidden FC widths and the split-K ranges of these nets in one round
+constexpr int kTK = 128;   // K staged at once: the hidden FC widths and the split-K ranges of these nets in one round
+constexpr int kNarrow = 16;
 constexpr int kSplitStep = 16;  // split-K ranges are multiples of this
 
-// Accumulates C[m0 + ty + 16r][n0 + 2 tx + c] (r, c in {0,1}) over k in [k_lo, k_hi):
+// How a launch stages and deals its outputs: TK of K at once, the least of 32, 64
+// and 128 that holds its K (loads past K are issued and thrown away), and a
+// thread's two columns side by side (the second one's state is in L1 when the first
+// one's epilogue is done with it) or, for at most kNarrow outputs, 16 apart, one a
+// thread instead of two in a row for half of them.  784-16-16-1, 20 iterations on one
+// subdomain: 549 us with 128 and side by side throughout, 486 so; 2400 subdomains:
+// 1272, 1095.  (Columns 16 apart throughout: 200-100-1, 2400 subdomains 860 -> 1035 us; the
+// choice made in the kernel: a proximal call 16.3 -> 17.7 ms.)
+template <int TK_, bool NARROW_>
+struct Tile {
+  static constexpr int TK = TK_;
+  static constexpr bool NARROW = NARROW_;
+  static __device__ __forceinline__ int col(int tx, int c) { return NARROW ? tx + 16 * c : 2 * tx + c; }
+};
+
+// Accumulates C[m0 + ty + 16r][n0 + T::col(tx, c)] (r, c in {0,1}) over k in [k_lo, k_hi):
 //   C[m, n] = sum_k A[m*lda + k] * Bop(k, n)
 //   W_KN:  Bop(k, n) = W[k*ldw + n]   (transposed pass: W[o, i], k = o, n = i)
 //   !W_KN: Bop(k, n) = W[n*ldw + k]   (forward pass:    W[o, i], k = i, n = o)
@@ -34,10 +50,11 @@ constexpr int kSplitStep = 16;  // split-K ranges are multiples of this
 // number of load rounds: all of K (up to TK) is staged in one round, every
 // thread's 32 loads in flight together (with 16 per round the 100 rows of the
 // Base FC layer took 7 rounds of load, barrier, 16 products).
-template <bool W_KN>
+template <bool W_KN, class T>
 __device__ __forceinline__ void gemm_tile(int m0, int n0, int M, int Ncol, int k_lo, int k_hi,
                                           const float* __restrict__ A, int lda, const float* __restrict__ W, int ldw,
                                           float acc[2][2]) {
+  constexpr int TK = T::TK;
   __shared__ float As[TM][TK + 1];
   __shared__ __align__(16) float Bs[TK][TN + 2];
   const int t = threadIdx.x, tx = t % 16, ty = t / 16;
@@ -66,7 +83,8 @@ __device__ __forceinline__ void gemm_tile(int m0, int n0, int M, int Ncol, int k
 #pragma unroll
     for (int e = 0; e < TN * TK / NT; ++e) {
       const int idx = t + e * NT;
-      Bs[W_KN ? idx / TN : idx % TK][W_KN ? idx % TN : idx / TK] = bv[e];
+      const int nn = W_KN ? idx % TN : idx / TK;  // a thread's two columns side by side
+      Bs[W_KN ? idx / TN : idx % TK][T::NARROW ? 2 * (nn % 16) + nn / 16 : nn] = bv[e];
     }
     __syncthreads();
 #pragma unroll 8
@@ -83,7 +101,7 @@ __device__ __forceinline__ void gemm_tile(int m0, int n0, int M, int Ncol, int k
 
 // Applies the epilogue to a thread's outputs of a tile; a reducing epilogue's
 // row sums are added over the 16 threads that share a row first.
-template <class Epi>
+template <class T, class Epi>
 __device__ __forceinline__ void gemm_epilogue(int m0, int n0, int M, int Ncol, const float (&acc)[2][2], const Epi& epi) {
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll
@@ -92,7 +110,7 @@ __device__ __forceinline__ void gemm_epilogue(int m0, int n0, int M, int Ncol, c
     double q = 0.0;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int n = n0 + 2 * tx + c;
+      const int n = n0 + T::col(tx, c);
       if (m < M && n < Ncol) {
         if constexpr (Epi::kReduce)
           q += epi(m, n, acc[r][c]);
@@ -108,13 +126,13 @@ __device__ __forceinline__ void gemm_epilogue(int m0, int n0, int M, int Ncol, c
 }
 
 // Full-K GEMM with the epilogue applied to every output.
-template <bool W_KN, class Epi>
+template <bool W_KN, class T, class Epi>
 __global__ void __launch_bounds__(NT) gemm_kernel(int M, int Ncol, int K, const float* __restrict__ A, int lda,
                                                   const float* __restrict__ W, int ldw, Epi epi) {
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
   float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  gemm_tile<W_KN>(m0, n0, M, Ncol, 0, K, A, lda, W, ldw, acc);
-  gemm_epilogue(m0, n0, M, Ncol, acc, epi);
+  gemm_tile<W_KN, T>(m0, n0, M, Ncol, 0, K, A, lda, W, ldw, acc);
+  gemm_epilogue<T>(m0, n0, M, Ncol, acc, epi);
 }
 
 // Ranges of the split-K forward pass of FC layer L for B subdomains: `splits`
@@ -138,17 +156,18 @@ void split_of(const LayerDev& L, const Problem& P, int& splits, int& kc) {
 
 // The partial sums alone: part[z][m][n] of every range z, for a consumer that
 // adds them itself in the order z = 0, 1, ...
+template <class T>
 __global__ void __launch_bounds__(NT) gemm_partials_kernel(int M, int Ncol, int K, int kc, const float* __restrict__ A,
                                                            int lda, const float* __restrict__ W, int ldw, float* part) {
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN, z = blockIdx.z;
   float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  gemm_tile<false>(m0, n0, M, Ncol, z * kc, min(K, (z + 1) * kc), A, lda, W, ldw, acc);
+  gemm_tile<false, T>(m0, n0, M, Ncol, z * kc, min(K, (z + 1) * kc), A, lda, W, ldw, acc);
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll
   for (int r = 0; r < 2; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int m = m0 + ty + 16 * r, n = n0 + 2 * tx + c;
+      const int m = m0 + ty + 16 * r, n = n0 + T::col(tx, c);
       if (m < M && n < Ncol) part[((size_t)z * M + m) * Ncol + n] = acc[r][c];
     }
 }
@@ -156,20 +175,20 @@ __global__ void __launch_bounds__(NT) gemm_partials_kernel(int M, int Ncol, int 
 // Split-K forward GEMM: block z covers K range [z*kc, (z+1)*kc); partial sums go
 // to part[z][m][n]; the last block to finish a tile sums the partials in the
 // order z = 0, 1, ... and applies the epilogue, then re-arms the tile counter.
-template <class Epi>
+template <class T, class Epi>
 __global__ void __launch_bounds__(NT) gemm_splitk_kernel(int M, int Ncol, int K, int kc, const float* __restrict__ A,
                                                          int lda, const float* __restrict__ W, int ldw, float* part,
                                                          int* count, Epi epi) {
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN, z = blockIdx.z, splits = gridDim.z;
   const int k_lo = z * kc, k_hi = min(K, k_lo + kc);
   float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  gemm_tile<false>(m0, n0, M, Ncol, k_lo, k_hi, A, lda, W, ldw, acc);
+  gemm_tile<false, T>(m0, n0, M, Ncol, k_lo, k_hi, A, lda, W, ldw, acc);
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll
   for (int r = 0; r < 2; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int m = m0 + ty + 16 * r, n = n0 + 2 * tx + c;
+      const int m = m0 + ty + 16 * r, n = n0 + T::col(tx, c);
       if (m < M && n < Ncol) part[((size_t)z * M + m) * Ncol + n] = acc[r][c];
     }
   __threadfence();
@@ -184,12 +203,12 @@ __global__ void __launch_bounds__(NT) gemm_splitk_kernel(int M, int Ncol, int K,
   for (int r = 0; r < 2; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int m = m0 + ty + 16 * r, n = n0 + 2 * tx + c;
+      const int m = m0 + ty + 16 * r, n = n0 + T::col(tx, c);
       acc[r][c] = 0.f;
       if (m < M && n < Ncol)
         for (int q = 0; q < splits; ++q) acc[r][c] += __ldcg(part + ((size_t)q * M + m) * Ncol + n);
     }
-  gemm_epilogue(m0, n0, M, Ncol, acc, epi);
+  gemm_epilogue<T>(m0, n0, M, Ncol, acc, epi);
   if (threadIdx.x == 0) count[tile] = 0;
 }
 
@@ -401,7 +420,7 @@ void launch_blocked(K kernel, unsigned grid, size_t smem, cudaStream_t s, A... a
 }
 
 // Rows per band of a blocked conv pass: the whole plane while the batch alone
-// gives every SM several CTAs; fewer (at least one round of items per CTA) for
+// gives each of 152 SMs four CTAs; fewer (at least one round of items per CTA) for
 // small batches, and what fits kConvSmem with the weights (row_bytes per
 // operand row; a band of bh rows stages bh * st + extra of them).  0: not even
 // one row fits.
@@ -412,6 +431,24 @@ int conv_band(int rows, int items_per_row, int B, size_t w_bytes, size_t row_byt
   return bh;
 }
 
+// Calls f(tile) for the Tile of a GEMM of n outputs over ranges of K inputs.
+template <bool NARROW, class F>
+void with_tk(int K, F f) {
+  if (K <= 32)
+    f(Tile<32, NARROW>{});
+  else if (K <= 64)
+    f(Tile<64, NARROW>{});
+  else
+    f(Tile<kTK, NARROW>{});
+}
+template <class F>
+void with_tile(int n, int K, F f) {
+  if (n <= kNarrow)
+    with_tk<true>(K, f);
+  else
+    with_tk<false>(K, f);
+}
+
 template <class Epi>
 void transposed(const LayerDev& L, const Problem& P, const float* rho, Epi epi, cudaStream_t s) {
   // g over the inputs of layer L (= the neurons of the layer below it).
@@ -419,7 +456,9 @@ void transposed(const LayerDev& L, const Problem& P, const float* rho, Epi epi, 
   const float* r = rho + L.r_out_off;
   if (L.kind == LD_LAYER_FC) {
     dim3 grid((L.n_in + TN - 1) / TN, (P.B + TM - 1) / TM);
-    gemm_kernel<true, Epi><<<grid, NT, 0, s>>>(P.B, L.n_in, L.n_out, r, P.N, L.W, L.n_in, epi);
+    with_tile(L.n_in, L.n_out, [&](auto t) {
+      gemm_kernel<true, decltype(t), Epi><<<grid, NT, 0, s>>>(P.B, L.n_in, L.n_out, r, P.N, L.W, L.n_in, epi);
+    });
     return;
   }
   const size_t smem = sizeof(float) * L.cout * L.cin * L.kh * L.kw;
@@ -460,11 +499,15 @@ void forward(const LayerDev& L, const Problem& P, const float* x, Epi epi, cudaS
     split_of(L, P, splits, kc);
     if (splits <= 1) {
       dim3 grid(tiles_n, tiles_m);
-      gemm_kernel<false, Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, xin, P.XS, L.W, L.n_in, epi);
+      with_tile(L.n_out, L.n_in, [&](auto t) {
+        gemm_kernel<false, decltype(t), Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, xin, P.XS, L.W, L.n_in, epi);
+      });
     } else {
       dim3 grid(tiles_n, tiles_m, splits);
-      gemm_splitk_kernel<Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, kc, xin, P.XS, L.W, L.n_in, P.splitk_part,
-                                                  P.splitk_count, epi);
+      with_tile(L.n_out, kc, [&](auto t) {
+        gemm_splitk_kernel<decltype(t), Epi><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, kc, xin, P.XS, L.W, L.n_in,
+                                                                 P.splitk_part, P.splitk_count, epi);
+      });
     }
     return;
   }
@@ -543,8 +586,10 @@ bool launch_forward_partials(const LayerDev& L, const Problem& P, const float* x
   if (!P.splitk_part || (size_t)k.splits * P.B * L.n_out > (size_t)P.splitk_part_cap) return false;
   count_launch();
   dim3 grid((L.n_out + TN - 1) / TN, (P.B + TM - 1) / TM, k.splits);
-  gemm_partials_kernel<<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, k.kc, x + L.x_in_off, P.XS, L.W, L.n_in,
-                                           P.splitk_part);
+  with_tile(L.n_out, k.kc, [&](auto t) {
+    gemm_partials_kernel<decltype(t)><<<grid, NT, 0, s>>>(P.B, L.n_out, L.n_in, k.kc, x + L.x_in_off, P.XS, L.W, L.n_in,
+                                                          P.splitk_part);
+  });
   return true;
 }
 
