@@ -276,7 +276,8 @@ struct EpiRecord {
   }
   // The CTAs of a subdomain arrive in any order, so a sum goes in as two: its
   // multiple of 2^-20, added exactly (sums below 2^32), and the rest, at most
-  // 2^-21, whose own rounding is far below the last bit of q.
+  // 2^-21, whose own rounding is far below the last bit of q (unless q is itself
+  // far below 1).  A CTA's sum from 2^31 on goes in as it is, in any order.
   __device__ __forceinline__ void finish(int b, double t) const {
     if (!q) return;
     constexpr double kGrid = 6442450944.0;  // 1.5 2^32: ulp 2^-20
@@ -521,6 +522,7 @@ cudaError_t launch_fused(const FusedNet& f, int code, const Problem& P, float* r
 // The same launch for nets of FC layers whose weights fit in shared memory
 // (ld_mlp.cu): bitwise the results of the launch shape `code`.
 bool mlp_covers(const FusedNet& f);
+bool mlp_faster(const FusedNet& f, int code, int B);
 cudaError_t launch_mlp(const FusedNet& f, int code, const Problem& P, float* rho, float* m, float* v,
                        const FusedIter& it, cudaStream_t s);
 

@@ -141,7 +141,7 @@ cudaError_t launch_fused(const FusedNet& f, int code, const Problem& P, float* r
                          const FusedIter& it, cudaStream_t s) {
   if (P.B == 0 || (it.T == 0 && !it.crown)) return cudaSuccess;
   // small FC nets (boxes): everything in shared memory, bitwise the same
-  if (!P.ball_eps && mlp_covers(f)) return launch_mlp(f, code, P, rho, m, v, it, s);
+  if (!P.ball_eps && mlp_covers(f) && mlp_faster(f, code, P.B)) return launch_mlp(f, code, P, rho, m, v, it, s);
   switch (code) {
     case 1: return launch_s<1, 256, false>(f, P, rho, m, v, it, s);
     case 2: return launch_s<2, 256, false>(f, P, rho, m, v, it, s);

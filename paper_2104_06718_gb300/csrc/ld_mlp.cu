@@ -259,6 +259,30 @@ bool mlp_covers(const FusedNet& f) {
   return f.n >= 2 && mlp_smem(make_mlp(f, NT)) <= kMlpSmem;
 }
 
+// Nets of one hidden layer and many inputs gain little: an iteration is one pass
+// over the same W_1 each way, which the general kernel also does in two phases, and
+// S >= 2 subdomains of its CTA share each weight it loads.  Its form is taken for
+//  * one subdomain an SM and 512 threads, W_1 over 64 KB of more than 640 inputs
+//    (784-24-1, T = 100, one subdomain: 478 us, 494 here; 784-10-1 423, 397), and
+//  * S >= 2 and 256 threads, more than 256 inputs and 1.5 times the subdomains that
+//    the GPU holds of this kernel (784-24-1, 1200 subdomains, T = 200: 2.9 ms, 4.2
+//    here; 300-60-1 3.8, 4.2; 300 subdomains of it 1.7, 1.1).
+bool mlp_faster(const FusedNet& f, int code, int B) {
+  const int S = code & ~kFusedWide, n0 = f.L[0].n_in;
+  const bool wide = (code & kFusedWide) != 0;
+  if (f.n != 2 || n0 <= 256 || (S > 1 && wide)) return true;
+  static int n_sm = 0;
+  if (!n_sm) {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    n_sm = v > 0 ? v : 1;
+  }
+  if (S == 1) return !(wide && n0 > 640 && n0 * f.L[0].n_out > 16384 && B <= n_sm);
+  const int per_sm = (int)std::min<size_t>(2048 / NT, (228 * 1024) / (mlp_smem(make_mlp(f, NT)) + 1024));
+  return B <= 3 * n_sm * per_sm / 2;
+}
+
 cudaError_t launch_mlp(const FusedNet& f, int code, const Problem& P, float* rho, float* m, float* v,
                        const FusedIter& it, cudaStream_t s) {
   const MlpNet net = make_mlp(f, (code & kFusedWide) ? 512 : 256);
