@@ -94,6 +94,16 @@ __device__ __forceinline__ void prefetch_state(const T* a, int b0, int nb, int B
     if (b0 + s < B) prefetch_l2(a + (size_t)(b0 + s) * N + off + lo, sizeof(T) * (size_t)(hi - lo));
 }
 
+// Whether the state (about 20 bytes a dual: rho, m, v, x_hat_B, masks) is too large
+// to stay in L2 from one pass to the next.  Smaller batches pay for the requests
+// alone: a call on a net with a 5x5 conv took 7% longer with them at 1 to 9
+// subdomains and 9% at 2048 (88 MB), Base 2% at 300 (19 MB).  At 2048 Base subdomains
+// (130 MB) a call takes 0.74 of the time that it took before the halo tiles, 0.80
+// without the requests; at 1000 of Deep (135 MB) 0.77 and 0.86, of Wide (125 MB) 0.69
+// and 0.72, of Base (63 MB) 0.78 and 0.79.
+constexpr double kStateInL2 = 100e6;
+inline int large_state(const Problem& P) { return 20.0 * P.B * P.N > kStateInL2; }
+
 // Adam on up to 8 duals: every load first (so that the 32 loads overlap
 // instead of forming 8 dependent round trips), then the updates and stores.
 // Same arithmetic as EpiAdam.
@@ -221,6 +231,7 @@ struct TcCommon {
   uint32_t res_bytes;      // resident operand (conv weights), 0 if none
   uint32_t stage_bytes;    // one pipeline stage (both operands of a K chunk)
   uint32_t tmem_cols;
+  int prefetch;            // ask for the epilogues' state ahead (large_state; launch_op picks the kernel)
   int* status;
 };
 
@@ -838,7 +849,7 @@ __device__ __forceinline__ void cp_wait_pending() {
 //                      free[s % NS] and, after a tile's last chunk, to acc_full
 // There is no CTA-wide barrier inside the loop; every wait is bounded and a
 // time-out anywhere makes every other wait give up (abort flag).
-template <class Op, int NS>
+template <class Op, int NS, bool PF>
 __global__ void __launch_bounds__(kCtaThreads, 2) tc_kernel(const __grid_constant__ Op op) {
   constexpr int LAG = NS - 1;
   extern __shared__ __align__(1024) uint8_t dyn_smem[];
@@ -904,7 +915,7 @@ __global__ void __launch_bounds__(kCtaThreads, 2) tc_kernel(const __grid_constan
       if (lane == 0) mbar_expect_tx(b_full + 8 * bi, op.stage_bytes_of(st % nch));
       __syncwarp();
       op.produce(tile_of(st), st % nch, sst0 + (uint32_t)bi * op.c.stage_bytes, b_full + 8 * bi, lane);
-      if (st % nch == 0) op.prefetch(tile_of(st), lane, 32);
+      if (PF && st % nch == 0) op.prefetch(tile_of(st), lane, 32);
       issued = st + 1;
     }
     // loads issued for stages never consumed must land before the CTA exits
@@ -921,7 +932,7 @@ __global__ void __launch_bounds__(kCtaThreads, 2) tc_kernel(const __grid_constan
         if (__any_sync(0xffffffffu, !fr)) break;
         op.load_stage(tile_of(i), i % nch, sst0 + (uint32_t)bi * op.c.stage_bytes, b_full + 8 * bi, tab);
         cp_arrive_noinc(b_full + 8 * bi);
-        if (i % nch == 0) op.prefetch(tile_of(i), tid, kThreads);
+        if (PF && i % nch == 0) op.prefetch(tile_of(i), tid, kThreads);
         issued = i + 1;
       }
       const int e = i - LAG;
@@ -1080,7 +1091,7 @@ size_t launch_smem(size_t need, uint32_t tmem_cols) {
 
 // Resident CTAs per SM from the kernel's registers and shared memory, the
 // thread limit and the TMEM columns (512 per SM).
-template <class Op, int NS>
+template <class Op, int NS, bool PF>
 const cudaFuncAttributes& kernel_attr();
 
 int ctas_per_sm(const cudaFuncAttributes& fa, size_t dyn_smem, uint32_t tmem_cols) {
@@ -1104,12 +1115,12 @@ int ctas_per_sm(const cudaFuncAttributes& fa, size_t dyn_smem, uint32_t tmem_col
 }
 
 // Registers and static shared memory of one kernel instantiation (queried once).
-template <class Op, int NS>
+template <class Op, int NS, bool PF>
 const cudaFuncAttributes& kernel_attr() {
   static cudaFuncAttributes fa{};
   static bool done = false;
   if (!done) {
-    if (cudaFuncGetAttributes(&fa, tc_kernel<Op, NS>) != cudaSuccess) {
+    if (cudaFuncGetAttributes(&fa, tc_kernel<Op, NS, PF>) != cudaSuccess) {
       cudaGetLastError();
       fa.numRegs = 0;
     }
@@ -1118,36 +1129,41 @@ const cudaFuncAttributes& kernel_attr() {
   return fa;
 }
 
-template <class Op, int NS>
+template <class Op, int NS, bool PF>
 cudaError_t launch_ns(const Op& op, size_t smem, int n_sm, cudaStream_t s) {
   static size_t attr_bytes = 0;  // dynamic shared memory opted in for this instantiation
   if (smem > attr_bytes) {
-    if (cudaFuncSetAttribute(tc_kernel<Op, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+    if (cudaFuncSetAttribute(tc_kernel<Op, NS, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return cudaGetLastError();
     attr_bytes = smem;
   }
-  const int per_sm = ctas_per_sm(kernel_attr<Op, NS>(), smem, op.c.tmem_cols);
+  const int per_sm = ctas_per_sm(kernel_attr<Op, NS, PF>(), smem, op.c.tmem_cols);
   int grid = n_sm * per_sm;
   if (grid > op.c.n_tiles) grid = op.c.n_tiles;
   const int gm = op.c.grid_multiple > 1 ? op.c.grid_multiple : 1;
   grid = grid / gm * gm;
   if (grid < gm) grid = gm;
   count_launch();
-  tc_kernel<Op, NS><<<grid, kCtaThreads, smem, s>>>(op);
+  tc_kernel<Op, NS, PF><<<grid, kCtaThreads, smem, s>>>(op);
   return cudaGetLastError();
 }
 
 // Three stage buffers unless two keep more CTAs resident on an SM.
-template <class Op>
-cudaError_t launch_op(const Op& op, int n_sm, cudaStream_t s) {
+template <class Op, bool PF>
+cudaError_t launch_stages(const Op& op, int n_sm, cudaStream_t s) {
   if (op.c.n_tiles <= 0) return cudaSuccess;
   const size_t m3 = launch_smem((size_t)op.c.res_bytes + 3 * (size_t)op.c.stage_bytes, op.c.tmem_cols);
   const size_t m2 = launch_smem((size_t)op.c.res_bytes + 2 * (size_t)op.c.stage_bytes, op.c.tmem_cols);
-  const int o3 = m3 <= kSmemBudget ? ctas_per_sm(kernel_attr<Op, 3>(), m3, op.c.tmem_cols) : 0;
-  const int o2 = ctas_per_sm(kernel_attr<Op, 2>(), m2, op.c.tmem_cols);
-  if (o3 >= o2) return launch_ns<Op, 3>(op, m3, n_sm, s);
-  return launch_ns<Op, 2>(op, m2, n_sm, s);
+  const int o3 = m3 <= kSmemBudget ? ctas_per_sm(kernel_attr<Op, 3, PF>(), m3, op.c.tmem_cols) : 0;
+  const int o2 = ctas_per_sm(kernel_attr<Op, 2, PF>(), m2, op.c.tmem_cols);
+  if (o3 >= o2) return launch_ns<Op, 3, PF>(op, m3, n_sm, s);
+  return launch_ns<Op, 2, PF>(op, m2, n_sm, s);
+}
+
+template <class Op>
+cudaError_t launch_op(const Op& op, int n_sm, cudaStream_t s) {
+  return op.c.prefetch ? launch_stages<Op, true>(op, n_sm, s) : launch_stages<Op, false>(op, n_sm, s);
 }
 
 AdamArgs adam_args(const TcState& S, AdamStep st) {
@@ -1519,6 +1535,7 @@ void launch_conv_t(TcNet& t, int k, const TcLayer& T, const LayerDev& L, const P
   op.c.tmem_cols = tmem_cols_for(2 * T.nt);
   op.c.grid_multiple = 1;
   op.c.status = S.status;
+  op.c.prefetch = large_state(P);
   op.nt = T.nt;
   op.kt = T.kt;
   op.cg = T.cg;
@@ -1593,6 +1610,7 @@ void launch_tc_transposed(TcNet& t, const std::vector<LayerDev>& Ls, int k, cons
   op.c.grid_multiple = op.n_mt;
   op.c.tmem_cols = tmem_cols_for(2 * op.BN);
   op.c.status = S.status;
+  op.c.prefetch = large_state(P);
   op.W = T.Wt;
   op.B = P.B;
   op.n_in = L.n_in;
@@ -1676,6 +1694,7 @@ void launch_tc_forward(TcNet& t, const std::vector<LayerDev>& Ls, int k, const P
     }
     op.c.tmem_cols = tmem_cols_for(2 * T.nf);
     op.c.status = S.status;
+    op.c.prefetch = large_state(P);
     op.nf = T.nf;
     op.kf = T.kf;
     op.W = T.Wf;
@@ -1717,6 +1736,7 @@ void launch_tc_forward(TcNet& t, const std::vector<LayerDev>& Ls, int k, const P
   op.c.stage_bytes = op.a_bytes + (uint32_t)(2 * op.BN * T.fc_kc);
   op.c.tmem_cols = tmem_cols_for(2 * op.BN);
   op.c.status = S.status;
+  op.c.prefetch = large_state(P);
   op.W = T.Wf;
   op.B = P.B;
   op.n_out = L.n_out;
