@@ -374,7 +374,7 @@ bool tile_fits(const ld_net* net, int code) { return ld::fused_smem_bytes(net->f
 // (Deep 8.9: 1024 subdomains, T = 50, 13.53 -> 12.37 ms; Wide 3.5 and Base 2.2
 // keep half: their FC passes are the longer ones with fewer threads).
 int fused_fc_threads(const ld_net* net, int code) {
-  constexpr double kConvHeavy = 6.0;
+  constexpr double kConvHeavy = 6.0;  // between those nets; nothing between 3.5 and 8.9 was measured
   double fc = 0, conv = 0;
   for (int k = 0; k + 1 < net->n; ++k) {
     const LayerDev& L = net->L[k];
@@ -765,8 +765,8 @@ void final_fp64(ld_net* net, const Problem& P, double* out, cudaStream_t s) {
   const int nfs = n_final_slots(net);
   const bool ball = P.ball_eps != nullptr;
   ld::FinalAcc acc{ball ? net->ball_ws : net->acc, nfs + (ball ? 1 : 0), 0};
-  // the per-layer passes on the side streams (FP64-pipe bound, each too
-  // small to fill the GPU alone), joined before the combine
+  // the per-layer passes on the side streams (each too small to fill the GPU
+  // alone), joined before the combine
   const bool fork = n >= 2 && net->aux_ok;
   if (fork) {
     cudaEventRecord(net->ev_fork, s);
