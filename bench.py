@@ -66,22 +66,21 @@ METRIC = "LD subdomain bounds/s on Base/Wide/Deep convnets, bf16 vs fp32 at ≤1
 # sources is not reported (the kernel changed since the capture).
 TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum of one launch of the fused kernels
-    # (fused_kernel<2, 512, 0|1> on Base, <1, 512, 0|1> on Wide and Deep): read + write
-    ("base", "fp32", "fused", 2, 512, 256, 100): ("40151aec76f4", 8019968),
-    ("base", "bf16", "fused tensor-core bf16", 2, 512, 256, 100): ("5f54da708e5e", 8312064),
-    ("wide", "fp32", "fused", 1, 512, 2048, 100): ("f3512387ae4d", 119097600 + 98118144),
-    ("deep", "fp32", "fused", 1, 512, 128, 100): ("40151aec76f4", 8330240),
-    ("deep", "bf16", "fused tensor-core bf16", 1, 512, 128, 100): ("5f54da708e5e", 8346368),
+    # (fused_kernel<2, 512, 0|1> on Base, <1, 512, 0|1> on Deep): read + write
+    ("base", "fp32", "fused", 2, 512, 256, 100): ("359e5e39c2de", 8003840),
+    ("base", "bf16", "fused tensor-core bf16", 2, 512, 256, 100): ("76147662f65d", 8306944),
+    ("deep", "fp32", "fused", 1, 512, 128, 100): ("359e5e39c2de", 8330240),
+    ("deep", "bf16", "fused tensor-core bf16", 1, 512, 128, 100): ("76147662f65d", 8348160),
     # the same metrics over the 7 launches of one iteration of the layer-wise tensor-core engine
-    # (read 367.56 MB + write 71.45 MB) x the 100 iterations of its graph launch
-    ("wide", "bf16", "tensor-core bf16", 0, 0, 2048, 100): ("253437eea2ec", (367555584 + 71448320) * 100),
+    # (read 367.47 MB + write 71.65 MB) x the 100 iterations of its graph launch
+    ("wide", "bf16", "tensor-core bf16", 0, 0, 2048, 100): ("70aa5b339d72", (367474176 + 71653888) * 100),
 }
 
 # The sources each timed engine is compiled from (besides the shared header
 # and the ABI header).
-ENGINE_SOURCES = {"fused": ["ld_fused.cu", "ld_fused_impl.cuh"],
+ENGINE_SOURCES = {"fused": ["ld_fused.cu", "ld_fused_impl.cuh", "ld_mlp.cu"],
                   "fused tensor-core bf16": ["ld_fused_tc.cu", "ld_fused_impl.cuh", "ld_tcgen05.cuh"],
-                  "tensor-core bf16": ["ld_tc.cu", "ld_tcgen05.cuh"], "layerwise": ["ld_passes.cu"]}
+                  "tensor-core bf16": ["ld_tc.cu", "ld_tcgen05.cuh"], "layerwise": ["ld_passes.cu", "ld_conv.cuh"]}
 
 
 def kernel_digest(engine=None) -> str:
