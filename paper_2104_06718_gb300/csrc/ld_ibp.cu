@@ -196,10 +196,12 @@ __global__ void ibp_out_kernel(LayerDev L, int n_rows, const float* __restrict__
 // neuron); lane q takes the inputs q, q + 32, ... (coalesced weight reads),
 // and the lanes' outward-rounded partial sums are added by a fixed shuffle
 // tree, rounding down for l_hat and up for u_hat, then the bias.  A lane waits
-// for its loads (weights from HBM or L2, once each), so kAhead rounds of them go
-// together: interval bounds of a net with 64 outputs of 16384 inputs, one subdomain,
-// 152 us with one round at a time, 108 so.
+// for its loads (weights from HBM or L2, once each), so from 1024 inputs on kAhead
+// rounds of them go together: interval bounds of a net with 64 outputs of 16384
+// inputs, one subdomain, 152 us with one round at a time, 109 so.  With fewer inputs
+// that costs large batches (100-100-100-1, 10000 subdomains 634 -> 818 us).
 constexpr int kAhead = 4;
+template <bool AHEAD>
 __global__ void ibp_fc_warp_kernel(LayerDev L, int first, int n_rows, const float* __restrict__ lin,
                                    const float* __restrict__ uin, int in_stride, float* lout, float* uout,
                                    int out_stride, int* status, IbpRows rows) {
@@ -214,28 +216,32 @@ __global__ void ibp_fc_warp_kernel(LayerDev L, int first, int n_rows, const floa
     const float* w = L.W + (size_t)o * L.n_in;
     float lo = 0.f, hi = 0.f;
     bool bad = false;
-    for (int i0 = lane; i0 < L.n_in; i0 += 32 * kAhead) {
-      float a[kAhead], c[kAhead], wi[kAhead];
-#pragma unroll
-      for (int q = 0; q < kAhead; ++q) {
-        const int i = min(i0 + 32 * q, L.n_in - 1);
-        a[q] = __ldg(lp + i);
-        c[q] = __ldg(up + i);
-        wi[q] = __ldg(w + i);
+    const auto add = [&](float a, float c, float wi) {
+      if (!first) {
+        a = fmaxf(a, 0.f);
+        c = fmaxf(c, 0.f);
+      } else if (!(isfinite(a) && isfinite(c) && a <= c)) {
+        bad = true;
       }
+      lo = __fmaf_rd(wi, wi >= 0.f ? a : c, lo);
+      hi = __fmaf_ru(wi, wi >= 0.f ? c : a, hi);
+    };
+    int i = lane;
+    if (AHEAD) {
+      const int full = L.n_in / (32 * kAhead) * (32 * kAhead);
+      for (; i < full; i += 32 * kAhead) {
+        float a[kAhead], c[kAhead], wi[kAhead];
 #pragma unroll
-      for (int q = 0; q < kAhead; ++q) {
-        if (i0 + 32 * q >= L.n_in) break;
-        if (!first) {
-          a[q] = fmaxf(a[q], 0.f);
-          c[q] = fmaxf(c[q], 0.f);
-        } else if (!(isfinite(a[q]) && isfinite(c[q]) && a[q] <= c[q])) {
-          bad = true;
+        for (int q = 0; q < kAhead; ++q) {
+          a[q] = __ldg(lp + i + 32 * q);
+          c[q] = __ldg(up + i + 32 * q);
+          wi[q] = __ldg(w + i + 32 * q);
         }
-        lo = __fmaf_rd(wi[q], wi[q] >= 0.f ? a[q] : c[q], lo);
-        hi = __fmaf_ru(wi[q], wi[q] >= 0.f ? c[q] : a[q], hi);
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) add(a[q], c[q], wi[q]);
       }
     }
+    for (; i < L.n_in; i += 32) add(lp[i], up[i], w[i]);
     if (bad) atomicCAS(status, 0, (int)LD_ERR_NONFINITE);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -266,8 +272,8 @@ void launch_ibp_layer(const LayerDev& L, int first, int last, int n_rows, const 
   if (L.kind == LD_LAYER_FC && L.n_in >= 64) {
     size_t g = (total + 7) / 8;  // 8 warps per block
     if (g > 65535 * 8) g = 65535 * 8;
-    ibp_fc_warp_kernel<<<(int)(g < 1 ? 1 : g), 256, 0, s>>>(L, first, n_rows, lin, uin, in_stride, lout, uout,
-                                                              out_stride, status, rows);
+    const auto k = L.n_in >= 1024 ? ibp_fc_warp_kernel<true> : ibp_fc_warp_kernel<false>;
+    k<<<(int)(g < 1 ? 1 : g), 256, 0, s>>>(L, first, n_rows, lin, uin, in_stride, lout, uout, out_stride, status, rows);
     return;
   }
   const int geo = L.kind != LD_LAYER_CONV ? 0 : (L.kh == 4 && L.kw == 4 && L.stride == 2) ? 1
