@@ -77,9 +77,9 @@ constexpr int kUnitC = 8;          // elements per unit (channels of a position 
 // a small call one to three CTAs a group, each a chain of waits (two to five units
 // a warp in a row): CROWN/WK bounds of one row of a 400-20-20-20-1 net 203 us, with
 // units of 2 and one a warp 106; FSB of 128-128-1 157 and 84 us.  600 rows of such
-// nets take up to 1.7 times as long as with units of 8 (300-24-100-1), which is still
-// a tenth of a warp per row.  The inputs alone decide, so that a row's value stays
-// the same in any batch.
+// nets take up to 1.7 times as long as with units of 8 (300-24-100-1; 80-80-80-80-1 3.0
+// -> 3.8 ms, 17.7 with a CTA per row).  The inputs alone decide, so that a row's value
+// stays the same in any batch.
 constexpr int kUnitFc = 2, kWideFc = 1024;
 constexpr int kAdds = 16;          // most scalar terms of each half of a row's sum between two FP64 flushes
 constexpr int kMaxChunks = 64;     // CTAs of a group

@@ -10,6 +10,7 @@
     and within 1e-4 of the oracle, a row the same alone and in a batch.
   * BF16 layer-wise passes with and without the state's prefetch (by batch size): the
     same subdomains, bitwise.
+  * DSG+ before and after a proximal call that grows the workspace of both.
 """
 import numpy as np
 import pytest
@@ -126,3 +127,13 @@ def test_bf16_passes_in_small_and_large_batches():
                                  return_rho=True)
     (a, ra), (b, rb) = run(12), run(large)
     assert torch.equal(ra, rb[:12]) and torch.equal(a, b[:12])
+
+
+def test_dsg_after_a_growing_proximal_call():
+    pb = conv_problem("base", 6, block=4)
+    net = ldb.Net(pb["specs"])
+    a = (net, pb["l0"], pb["u0"], pb["lbk"], pb["ubk"])
+    first = ldb.ld_bound_dsg(*a, None, pb["masks"], n_iters=5)
+    ldb.ld_bound_proximal(*a, None, np.zeros((64, pb["masks"].shape[1]), np.int8), n_iters=2)
+    again = ldb.ld_bound_dsg(*a, None, pb["masks"], n_iters=5)
+    assert torch.equal(first[0], again[0])
